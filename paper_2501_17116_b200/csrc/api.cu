@@ -131,6 +131,7 @@ int fp4_create(fp4_ctx** out, int device, size_t workspace_bytes) {
     ctx->workspace_bytes = workspace_bytes;
   }
   bool ok = true;
+  ok = ok && quantize_setup() == FP4_OK;
   // counters of the quantile selection (quantisation with clamping): cleared here, once
   ok = ok && cudaMalloc(reinterpret_cast<void**>(&ctx->occ_hist), quantize_persistent_bytes()) == cudaSuccess;
   ok = ok && cudaMemset(ctx->occ_hist, 0, quantize_persistent_bytes()) == cudaSuccess;

@@ -210,6 +210,7 @@ struct SparseOverlap {
 // E2M1 operand, 448 for an E4M3 one); 0: the vector is used as it is.  out->format selects E2M1 or E4M3.
 size_t quantize_scratch_bytes(int64_t rows, int64_t cols);
 size_t quantize_persistent_bytes();
+int quantize_setup();               // kernel attributes, once per device
 int launch_quantize(fp4_ctx* ctx, cudaStream_t stream, Arena& arena, const void* x_bf16, int64_t rows,
                     int64_t cols, int scale_axis, double alpha, const float* prescale,
                     float prescale_div, fp4_qtensor* out, int32_t* status,

@@ -3,7 +3,7 @@
 //
 // Passes over a [rows x cols] BF16 tensor:
 //   with outlier clamping (activations)
-//     1. hist_select      one read: 65536-bin histogram of the BF16 bit patterns (exact, in shared
+//     1. tail_select      one read: exact counts of the BF16 bit patterns in the two tails (shared
 //                         memory) + signed max / min of every row; the block that finishes last
 //     2.                  turns the cumulative counts into the two order statistics lo, hi
 //     3. encode           one read: clamp, per-row scale from the clamped row extremes, Q, both
@@ -16,16 +16,17 @@
 //     2. encode           one read
 // The "dual" mode serves the backward pass: one read of dY yields the token-wise codes of
 // dY (.) d_W[n] and the channel-wise codes of dY (.) d_A[m].
+#include <cmath>
 #include <mutex>
 
 #include "common.cuh"
 
 namespace {
 
-constexpr int HIST_THREADS = 1024;
 constexpr int ENC_TM = 64;                        // tile rows of the encoder (= one strip)
 constexpr int ENC_TK = 256;                       // tile columns
 constexpr int ENC_THREADS = 256;
+constexpr int SUPER = 16;                         // strips whose column counts are also kept as one sum
 
 enum Mode { MODE_ROWS = 0, MODE_COLS = 1, MODE_DUAL = 2 };
 
@@ -40,18 +41,31 @@ __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w 
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
 
 // ------------------------------------------------------------------------------------------
-// 1. + 2. histogram of bit patterns, row extremes, order statistics -- one kernel
+// 1. + 2. row extremes, histogram of the tails, order statistics -- one kernel
 // ------------------------------------------------------------------------------------------
-// Exact histogram with 32-bit shared-memory counters over a window of HIST_EXPS binary exponents
-// (both signs, all 128 mantissas): real tensors spread over far fewer exponents than BF16 offers.
-// Each block places its window HIST_HEADROOM binades above the largest magnitude of its first 8192
-// elements.  A vector of eight elements is tested against the window as a whole (four packed BF16
-// comparisons); if all eight are inside, each costs one extraction, one address and one increment.
-// Patterns outside the window (tiny values, later giants) go straight to the global histogram and
-// exact zeros are counted in registers, so every element is counted exactly once.  The window is
-// replicated HIST_COPIES times (one copy per group of warps) to thin out same-address conflicts;
-// the increments return no value and need no overflow handling.  What bounds the loop is the
-// shared-memory pipe: the increments of a warp fall into random banks.
+// The two thresholds are order statistics far out in the tails, so only the tails are counted value by
+// value.  Every block draws the same SEL_SAMPLES elements (stratified over the tensor, jittered by a hash
+// of the stratum) and takes from them a bracket Q < P that leaves slightly more than n_tail elements on
+// either side: the k-th smallest / largest sample, k six and a half standard deviations (plus eight)
+// above the expected n_tail * SEL_SAMPLES / n.  Elements strictly between Q and P are the bulk: a vector
+// of eight costs the packed maxima and minima that the row extremes need anyway and two packed
+// comparisons.  The others (2 to 6 % of the elements) are counted by pattern.  The number of bulk
+// elements B is n minus what was counted, so the rank r of the whole tensor is rank r of the counters
+// below the bulk and rank r - B above it.  The result is exact whatever the sample was: a rank that does
+// not fall into its tail (a sample that misleads, about one in 10^9) makes the last block count the whole
+// tensor by itself.
+//
+// What bounds it: a fixed chain of about 8 us (sample -> bracket, and flush -> ticket -> selection), then
+// HBM for light clamps and the counting loop for heavy ones.  A histogram of every element needed 180 KB
+// of shared memory (one block per SM) and 12 instructions per element; 8192 x 4096 at 0.1 % per tail
+// went from 28.8 to 24.5 us, 8192 x 5120 at 0.01 % from 34.7 to 27.6, 16384 x 13824 at 1 % from 130 to
+// 117 (L2 flushed by reads before each).  Samples are taken four adjacent elements at a time: one load
+// per thread; every block reading 2048 separate sectors cost 2 us more.
+//
+// Counters: 32-bit in shared memory over a window of SEL_EXPS binary exponents (both signs, all 128
+// mantissas), SEL_HEADROOM binades above the largest magnitude of the sample.  Counted elements outside
+// the window (tiny values of a bracket around zero, later giants) go to the global counters with
+// atomics and exact zeros are counted in registers, so every element is counted exactly once.
 //
 // A block owns whole rows (a contiguous range of them), so the signed max / min of a row are
 // reduced in shared memory and written with plain stores, as is the zero that starts the row's
@@ -64,290 +78,446 @@ __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w 
 // clears set 1 - p at its start (every block a slice, plain stores) and flips the parity at its
 // end, so the set a call counts into is always zero and no separate clearing pass exists.  With
 // `parity` null (the allocation-free entry point, which clears its one set itself) set 0 is used.
-constexpr int HIST_EXPS = 24;
-constexpr int HIST_WINDOW = HIST_EXPS * 128;       // 3072 magnitudes in the window, per sign
-constexpr int HIST_COPIES = 4;
-constexpr int HIST_HEADROOM = 1;                   // binades between the sample's maximum and the window's top
-constexpr int HIST_FLY = 4;                        // vectors a lane loads per unit
-constexpr int HIST_CHUNK = 32 * HIST_FLY;          // vectors of one row a warp takes at a time
-// Counter of pattern b in copy c: word c * HIST_WINDOW + (b - base).  The sign bit of b is left in
-// place, so the negative half of every copy lies 0x8000 words (128 KB) above its positive half and
-// the index of an element is its pattern minus a constant; the words between the halves are unused.
-constexpr int HIST_NEG_WORD = 0x8000;
-constexpr int HIST_SMEM_BYTES = (HIST_NEG_WORD + HIST_COPIES * HIST_WINDOW) * 4;
-constexpr int HIST_ROW_SLOTS = 512;                // rows whose extremes a block reduces at a time
+constexpr int SEL_THREADS = 512;
+constexpr int SEL_WARPS = SEL_THREADS / 32;
+constexpr int SEL_BLOCKS_PER_SM = 2;
+constexpr int SEL_SAMPLES = 4 * SEL_THREADS;        // one 8-byte load per thread
+constexpr int SEL_EXPS = 24;
+constexpr int SEL_WINDOW = SEL_EXPS * 128;         // 3072 magnitudes in the window, per sign
+constexpr int SEL_ALL = 8192;                       // elements per SM below which everything is counted
+constexpr int SEL_HEADROOM = 2;                    // binades between the sample's maximum and the window's top
+constexpr int SEL_FLY = 4;                         // vectors a lane loads per unit
+constexpr int SEL_DYN_SMEM = 2 * SEL_FLY * SEL_THREADS * 16;   // two units of every warp
+constexpr int SEL_ROW_SLOTS = 128;                 // rows whose extremes a block reduces at a time
+constexpr int SEL_BIN_SHIFT = 4;                   // sample histogram: 16 positions per bin
+constexpr int SEL_BINS = 65536 >> SEL_BIN_SHIFT;
 constexpr int HIST_COARSE = 32;                    // coarse counters: 2048 positions each
 constexpr int HIST_SET_WORDS = 65536 + HIST_COARSE; // one set: fine counters, then coarse counters
-
-// Inclusive scan of one value per thread over a block of 1024 threads.
-__device__ __forceinline__ long long block_scan_1024(long long v, long long* warp_tot /*[32] shared*/) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const long long up = __shfl_up_sync(0xFFFFFFFFu, v, off);
-    if (lane >= off) v += up;
-  }
-  if (lane == 31) warp_tot[warp] = v;
-  __syncthreads();
-  if (warp == 0) {
-    long long t = warp_tot[lane];
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const long long up = __shfl_up_sync(0xFFFFFFFFu, t, off);
-      if (lane >= off) t += up;
-    }
-    warp_tot[lane] = t;
-  }
-  __syncthreads();
-  if (warp > 0) v += warp_tot[warp - 1];
-  return v;
-}
 
 // Position p in ascending real order: p < 32768 are the negative patterns from 0xFFFF down to
 // 0x8000 (-0), p >= 32768 the non-negative patterns from 0x0000 up.
 __device__ __forceinline__ uint32_t pos_to_bits(int p) { return p < 32768 ? uint32_t(0xFFFF - p) : uint32_t(p - 32768); }
 __device__ __forceinline__ int bits_to_pos(uint32_t bits) { return (bits & 0x8000u) ? int(0xFFFFu - bits) : int(bits) + 32768; }
 
-__global__ void __launch_bounds__(HIST_THREADS, 1)
-hist_select_kernel(const uint4* __restrict__ x, int rows, int vec_per_row, uint32_t* sets, unsigned* parity,
-                   int* __restrict__ row_max, int* __restrict__ row_min, int* __restrict__ row_cnt, long long n,
-                   long long n_tail, float* __restrict__ thresholds, unsigned* ticket, int32_t* status, int abs_mode) {
-  extern __shared__ uint32_t h[];
-  __shared__ uint32_t s_top;
-  __shared__ int s_rmax[HIST_ROW_SLOTS], s_rmin[HIST_ROW_SLOTS];
-  __shared__ uint32_t s_coarse[HIST_COARSE];
-  __shared__ int s_last;
-  const int tid = threadIdx.x;
-  const int r_begin = int((long long)rows * blockIdx.x / gridDim.x);
-  const int r_end = int((long long)rows * (blockIdx.x + 1) / gridDim.x);
-  const int lane = tid & 31;
-  // sample for the window's top, issued first: its latency hides behind the clearing below
-  uint4 sample = make_uint4(0, 0, 0, 0);
-  {
-    const long long i0 = (long long)r_begin * vec_per_row + tid;
-    if (i0 < (long long)r_end * vec_per_row) sample = __ldg(&x[i0]);
-  }
-  const unsigned par = parity ? (*reinterpret_cast<volatile unsigned*>(parity) & 1u) : 0u;
-  uint32_t* ghist = sets + size_t(par) * HIST_SET_WORDS;
-  uint32_t* gcoarse = ghist + 65536;
-  if (parity) {
-    // this block's slice of the other set, for the next call
-    uint32_t* other = sets + size_t(par ^ 1u) * HIST_SET_WORDS;
-    const int per = (HIST_SET_WORDS + gridDim.x - 1) / gridDim.x;
-    const int w0 = blockIdx.x * per, w1 = min(HIST_SET_WORDS, w0 + per);
-    for (int i = w0 + tid; i < w1; i += HIST_THREADS) other[i] = 0;
-  }
-  {
-    uint4* pos4 = reinterpret_cast<uint4*>(h);
-    uint4* neg4 = reinterpret_cast<uint4*>(h + HIST_NEG_WORD);
-    for (int i = tid; i < HIST_WINDOW * HIST_COPIES / 4; i += HIST_THREADS)
-      pos4[i] = neg4[i] = make_uint4(0, 0, 0, 0);
-  }
-  if (tid < HIST_COARSE) s_coarse[tid] = 0;
-  if (tid == 0) s_top = 0;
-  __syncthreads();
-  {
-    // window top: largest exponent-and-mantissa field among this block's first vectors
-    const uint32_t w[4] = {sample.x, sample.y, sample.z, sample.w};
-    uint32_t m = 0;
+// Stratum i of SEL_THREADS over n elements -> the first of its four sampled elements (n is a multiple of 4).
+__device__ __forceinline__ long long sample_index(int i, long long n) {
+  const long long q = n >> 2, b = q * i / SEL_THREADS, e = q * (i + 1) / SEL_THREADS;
+  uint32_t h = uint32_t(i) * 2654435761u + 0x9E3779B9u;
+  h ^= h >> 15;
+  h *= 0x2C1B3C6Du;
+  h ^= h >> 13;
+  return 4 * (b + (long long)(h % uint32_t(e - b)));
+}
+
+__device__ __forceinline__ __nv_bfloat162 bf162_of(uint32_t bits) {
+  const __nv_bfloat16 v = __ushort_as_bfloat16((unsigned short)bits);
+  return __halves2bfloat162(v, v);
+}
+
+struct SelectArgs {
+  const uint4* x;
+  int rows, vec_per_row;
+  uint32_t* sets;               // global counters (two sets with `parity`, else one)
+  unsigned* parity;
+  unsigned* ticket;
+  int* row_max;
+  int* row_min;
+  int* row_cnt;                 // zeroed (or null)
+  int* clear;                   // `clear_words` ints that a later kernel adds to: zeroed (or null)
+  int clear_words;
+  long long n, n_tail;
+  int sample_rank;              // k: the bracket is the k-th smallest / largest sample (0-based); -1: none, count all
+  float* thresholds;
+  int32_t* status;
+  int abs_mode;
+};
+
+struct SelectShared {
+  union {
+    uint32_t window[2 * SEL_WINDOW];                // positive, then negative magnitudes
+    uint32_t bins[SEL_BINS];                        // histogram of the sample
+  };
+  int rmax[SEL_ROW_SLOTS], rmin[SEL_ROW_SLOTS];
+  uint32_t coarse[HIST_COARSE];
+  int warp_tot[SEL_WARPS];
+  uint32_t top;
+  int p_pos, q_pos;
+  int last, fail;
+  uint32_t step[2][8];
+};
+
+// Inclusive scan of one value per lane over the warp.
+template <typename T>
+__device__ __forceinline__ T warp_inclusive_scan(T v) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) m = max(m, max(w[q] & 0x7FFFu, (w[q] >> 16) & 0x7FFFu));
-    m = __reduce_max_sync(0xFFFFFFFFu, m);
-    if ((tid & 31) == 0 && m) atomicMax(&s_top, m);
+  for (int off = 1; off < 32; off <<= 1) {
+    const T up = __shfl_up_sync(0xFFFFFFFFu, v, off);
+    if (lane >= off) v += up;
   }
-  __syncthreads();
-  // window = exponents [e_top - HIST_EXPS + 1, e_top] with e_top HIST_HEADROOM binades above the sample's
-  // maximum (what lies above the window is counted in global memory like what lies below it)
-  const int e_top = min(254, int(s_top >> 7) + HIST_HEADROOM);
-  const uint32_t base = uint32_t(max(0, e_top - HIST_EXPS + 1)) << 7;
-  // The window's bounds as BF16 numbers (magnitudes order like their patterns; the upper bound is at
-  // most the pattern of infinity, and a NaN fails every comparison)
-  const __nv_bfloat162 lo_bf = __halves2bfloat162(__ushort_as_bfloat16((unsigned short)base),
-                                                  __ushort_as_bfloat16((unsigned short)base));
-  const __nv_bfloat162 hi_bf = __halves2bfloat162(__ushort_as_bfloat16((unsigned short)(base + HIST_WINDOW)),
-                                                  __ushort_as_bfloat16((unsigned short)(base + HIST_WINDOW)));
-  // this warp's copy: counter of pattern b at word b + my_off
-  const int my_off = ((tid >> 5) & (HIST_COPIES - 1)) * HIST_WINDOW - int(base);
+  return v;
+}
+
+// One counted element: into the window, or past it (rare) into the global counters.
+__device__ __forceinline__ void select_count(SelectShared& s, uint32_t bits, uint32_t base, uint32_t* ghist, uint32_t& zeros_pos,
+                                             uint32_t& zeros_neg, bool& nonfinite) {
+  const uint32_t m15 = bits & 0x7FFFu, off = m15 - base;
+  if (off < uint32_t(SEL_WINDOW)) {
+    atomicAdd(&s.window[off + (bits >> 15) * SEL_WINDOW], 1u);
+  } else if (m15 == 0) {
+    if (bits) ++zeros_neg; else ++zeros_pos;
+  } else {
+    atomicAdd(&ghist[bits], 1u);
+    atomicAdd(&s.coarse[bits_to_pos(bits) >> 11], 1u);
+    if (m15 >= 0x7F80u) nonfinite = true;             // infinity or NaN: always outside the window
+  }
+}
+
+// A unit is a stretch of consecutive vectors of one row, FLY per lane (vectors lane, lane + 32, ... of the
+// stretch); warp w takes units w, w + 16, ...  Units travel to shared memory (cp.async), two of a warp's in
+// flight; every lane reads only what it copied itself, so waiting for its own copies is all the
+// synchronisation there is.
+extern __shared__ __align__(16) unsigned char s_vec[];        // [2][SEL_FLY][SEL_THREADS] vectors
+template <int FLY>
+__device__ __forceinline__ void select_request(const SelectArgs& a, int u, int units, int r0, int stage) {
+  if (u < units) {
+    const int chunks_per_row = (a.vec_per_row + 32 * FLY - 1) / (32 * FLY), lane = threadIdx.x & 31;
+    const int row = u / chunks_per_row, v0 = (u - row * chunks_per_row) * 32 * FLY;
+    const uint4* px = a.x + ((long long)(r0 + row) * a.vec_per_row + v0 + lane);
+    const int mine = min(32 * FLY, a.vec_per_row - v0) - lane;             // vectors lane, lane + 32, ... below this
+    const uint32_t slot = uint32_t(__cvta_generic_to_shared(s_vec + (stage * SEL_FLY * SEL_THREADS + threadIdx.x) * 16));
+#pragma unroll
+    for (int k = 0; k < FLY; ++k)
+      if (32 * k < mine)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(slot + uint32_t(k * SEL_THREADS * 16)), "l"(px + 32 * k)
+                     : "memory");
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// Rows [r_begin, r_end): extremes of every row, and the counts of the elements outside (Q, P), or of all.
+// `requested`: the warp's first two units are on their way.
+template <bool ALL>
+__device__ __forceinline__ void select_count_rows(const SelectArgs& a, SelectShared& s, int r_begin, int r_end,
+                                                  uint32_t p_bits, uint32_t q_bits, uint32_t base, uint32_t* ghist,
+                                                  bool requested) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  const __nv_bfloat162 p2 = bf162_of(p_bits), q2 = bf162_of(q_bits);
+  // with everything counted a vector is work enough per lane
+  constexpr int FLY = ALL ? 1 : SEL_FLY, CHUNK = 32 * FLY;
+  const int chunks_per_row = (a.vec_per_row + CHUNK - 1) / CHUNK;
   uint32_t zeros_pos = 0, zeros_neg = 0;
   bool nonfinite = false;
-  for (int r0 = r_begin; r0 < r_end; r0 += HIST_ROW_SLOTS) {
-    const int r1 = min(r_end, r0 + HIST_ROW_SLOTS);
-    for (int r = tid; r < r1 - r0; r += HIST_THREADS) {
-      s_rmax[r] = INT_MIN;
-      s_rmin[r] = INT_MAX;
+  for (int r0 = r_begin; r0 < r_end; r0 += SEL_ROW_SLOTS) {
+    const int r1 = min(r_end, r0 + SEL_ROW_SLOTS);
+    for (int r = tid; r < r1 - r0; r += SEL_THREADS) {
+      s.rmax[r] = INT_MIN;
+      s.rmin[r] = INT_MAX;
     }
     __syncthreads();
-    // A unit is a stretch of up to HIST_CHUNK consecutive vectors of one row; warp w takes units
-    // w, w + 32, ...  A lane loads its HIST_FLY vectors of the unit (vectors lane, lane + 32, ... of
-    // the stretch) before it counts any of them, keeps the unit's extremes packed in two registers,
-    // and the warp reduces them once per unit.
-    const int chunks_per_row = (vec_per_row + HIST_CHUNK - 1) / HIST_CHUNK;
     const int units = (r1 - r0) * chunks_per_row;
-    for (int u = tid >> 5; u < units; u += HIST_THREADS / 32) {
-      const int row = u / chunks_per_row;
-      const int v0 = (u - row * chunks_per_row) * HIST_CHUNK;
-      const int mine = min(HIST_CHUNK, vec_per_row - v0) - lane;       // vectors lane, lane + 32, ... below this
-      const uint4* px = x + ((long long)(r0 + row) * vec_per_row + v0 + lane);
-      uint4 vv[HIST_FLY];
-#pragma unroll
-      for (int k = 0; k < HIST_FLY; ++k)
-        if (32 * k < mine) vv[k] = __ldg(px + 32 * k);
+    int u = tid >> 5, stage = 0;
+    if (r0 != r_begin || !requested) {
+      select_request<FLY>(a, u, units, r0, 0);
+      select_request<FLY>(a, u + SEL_WARPS, units, r0, 1);
+    }
+    for (; u < units; u += SEL_WARPS, stage ^= 1) {
+      const int row = u / chunks_per_row, v0 = (u - row * chunks_per_row) * CHUNK;
+      const int mine = min(CHUNK, a.vec_per_row - v0) - lane;
+      const unsigned char* slot = s_vec + (stage * SEL_FLY * SEL_THREADS + tid) * 16;
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+      // Extremes of the unit, packed (a NaN loses here: it is seen below), and one bit per element that
+      // is not strictly inside the bracket (a NaN never is): bit 4 k + q for the lower, 16 + 4 k + q for
+      // the upper half of word q of vector k.
       __nv_bfloat162 umax = __float2bfloat162_rn(-INFINITY), umin = __float2bfloat162_rn(INFINITY);
+      uint32_t tail = 0;
 #pragma unroll
-      for (int k = 0; k < HIST_FLY; ++k) {
+      for (int k = 0; k < FLY; ++k) {
         if (32 * k >= mine) break;
-        const uint32_t w[4] = {vv[k].x, vv[k].y, vv[k].z, vv[k].w};
+        const uint4 vv = *reinterpret_cast<const uint4*>(slot + k * SEL_THREADS * 16);
+        const uint32_t w[4] = {vv.x, vv.y, vv.z, vv.w};
         const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(w);
-        // all eight magnitudes inside the window?  (half-precision comparisons: they leave the
-        // integer pipe to the index arithmetic)
-        bool inside = true;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const __nv_bfloat162 mag = __habs2(p[q]);
-          inside = inside && __hbge2(mag, lo_bf) && __hblt2(mag, hi_bf);
-        }
-        if (inside) {
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            atomicAdd(&h[int(w[q] & 0xFFFFu) + my_off], 1u);
-            atomicAdd(&h[int(w[q] >> 16) + my_off], 1u);
-          }
-        } else {
-#pragma unroll 1
-          for (int e = 0; e < 8; ++e) {
-            const uint32_t word = (e & 4) ? ((e & 2) ? w[3] : w[2]) : ((e & 2) ? w[1] : w[0]);
-            const uint32_t bits = (e & 1) ? (word >> 16) : (word & 0xFFFFu);
-            const uint32_t m15 = bits & 0x7FFFu;
-            if (m15 - base < uint32_t(HIST_WINDOW)) {
-              atomicAdd(&h[int(bits) + my_off], 1u);
-            } else if (m15 == 0) {
-              if (bits) ++zeros_neg; else ++zeros_pos;
-            } else {
-              atomicAdd(&ghist[bits], 1u);
-              atomicAdd(&s_coarse[bits_to_pos(bits) >> 11], 1u);
-              if (m15 >= 0x7F80u) nonfinite = true;       // infinity or NaN: always outside the window
-            }
-          }
-        }
         umax = __hmax2(umax, __hmax2(__hmax2(p[0], p[1]), __hmax2(p[2], p[3])));
         umin = __hmin2(umin, __hmin2(__hmin2(p[0], p[1]), __hmin2(p[2], p[3])));
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (ALL) {
+            select_count(s, w[q] & 0xFFFFu, base, ghist, zeros_pos, zeros_neg, nonfinite);
+            select_count(s, w[q] >> 16, base, ghist, zeros_pos, zeros_neg, nonfinite);
+          } else {
+            tail |= ~(__hlt2_mask(p[q], p2) & __hgt2_mask(p[q], q2)) & (0x00010001u << (4 * k + q));
+          }
+        }
       }
+      if (!ALL) {
+        // Counted elements are picked out of shared memory rather than out of the registers by a chain of
+        // selections: the lanes hold few of them, and a lane's four vectors share one loop.
+        while (tail) {
+          const uint32_t b = 31u - __clz(tail);
+          tail ^= 1u << b;
+          const uint32_t at = ((b >> 2) & 3u) * (SEL_THREADS * 16) | ((b & 3u) << 2) | ((b >> 3) & 2u);
+          select_count(s, *reinterpret_cast<const unsigned short*>(slot + at), base, ghist, zeros_pos, zeros_neg, nonfinite);
+        }
+      }
+      select_request<FLY>(a, u + 2 * SEL_WARPS, units, r0, stage);
       int kmax = float_to_ordered(fmaxf(__low2float(umax), __high2float(umax)));
       int kmin = float_to_ordered(fminf(__low2float(umin), __high2float(umin)));
       kmax = __reduce_max_sync(0xFFFFFFFFu, kmax);
       kmin = __reduce_min_sync(0xFFFFFFFFu, kmin);
       if (lane == 0) {
-        atomicMax(&s_rmax[row], kmax);
-        atomicMin(&s_rmin[row], kmin);
+        atomicMax(&s.rmax[row], kmax);
+        atomicMin(&s.rmin[row], kmin);
       }
     }
     __syncthreads();
-    for (int r = tid; r < r1 - r0; r += HIST_THREADS) {
-      row_max[r0 + r] = s_rmax[r];
-      row_min[r0 + r] = s_rmin[r];
-      if (row_cnt) row_cnt[r0 + r] = 0;
+    for (int r = tid; r < r1 - r0; r += SEL_THREADS) {
+      a.row_max[r0 + r] = s.rmax[r];
+      a.row_min[r0 + r] = s.rmin[r];
+      if (a.row_cnt) a.row_cnt[r0 + r] = 0;
     }
     __syncthreads();
   }
-  if (__any_sync(0xFFFFFFFFu, nonfinite) && (tid & 31) == 0 && status) atomicOr(status, FP4_DEV_NONFINITE);
+  if (__any_sync(0xFFFFFFFFu, nonfinite) && lane == 0 && a.status) atomicOr(a.status, FP4_DEV_NONFINITE);
   zeros_pos = __reduce_add_sync(0xFFFFFFFFu, zeros_pos);
   zeros_neg = __reduce_add_sync(0xFFFFFFFFu, zeros_neg);
-  if ((tid & 31) == 0) {
-    if (zeros_pos) { atomicAdd(&ghist[0x0000], zeros_pos); atomicAdd(&s_coarse[bits_to_pos(0x0000u) >> 11], zeros_pos); }
-    if (zeros_neg) { atomicAdd(&ghist[0x8000], zeros_neg); atomicAdd(&s_coarse[bits_to_pos(0x8000u) >> 11], zeros_neg); }
+  if (lane == 0) {
+    if (zeros_pos) { atomicAdd(&ghist[0x0000], zeros_pos); atomicAdd(&s.coarse[bits_to_pos(0x0000u) >> 11], zeros_pos); }
+    if (zeros_neg) { atomicAdd(&ghist[0x8000], zeros_neg); atomicAdd(&s.coarse[bits_to_pos(0x8000u) >> 11], zeros_neg); }
   }
-  // Two neighbouring counters (an even pattern and the next one: same sign, same coarse range) leave
-  // with one 64-bit add; no 32-bit half can overflow into the other (n < 2^31).
-  for (int idx = tid; idx < HIST_WINDOW; idx += HIST_THREADS) {
-    const int neg = idx >= HIST_WINDOW / 2, off = 2 * (idx - neg * (HIST_WINDOW / 2));
-    uint32_t c0 = 0, c1 = 0;
+}
+
+// The block's counters (of the magnitudes from base + `from` up, `from` a multiple of 64) into the global
+// ones.  Two neighbouring counters (an even pattern and the next one: same sign, same coarse range) leave
+// with one 64-bit add; no 32-bit half can overflow into the other (n < 2^31).  A warp's 32 pairs lie in one
+// coarse range, whose counter gets one add per warp.
+__device__ __forceinline__ void select_flush(SelectShared& s, uint32_t base, uint32_t* ghist, int from) {
+  const int pairs = (SEL_WINDOW - from) / 2;         // per sign; a multiple of 32
+  for (int idx = threadIdx.x; idx < 2 * pairs; idx += SEL_THREADS) {
+    const int neg = idx >= pairs, off = from + 2 * (idx - neg * pairs);
+    const uint2 c = *reinterpret_cast<const uint2*>(&s.window[neg * SEL_WINDOW + off]);
+    const uint32_t bits = (uint32_t(neg) << 15) | (base + uint32_t(off));
+    if (c.x | c.y)
+      atomicAdd(reinterpret_cast<unsigned long long*>(&ghist[bits]), (unsigned long long)c.x | ((unsigned long long)c.y << 32));
+    const uint32_t t = __reduce_add_sync(0xFFFFFFFFu, c.x + c.y);
+    if ((threadIdx.x & 31) == 0 && t) atomicAdd(&s.coarse[bits_to_pos(bits) >> 11], t);
+  }
+}
+
+// The order statistics from the global counters, by all threads of one block.  `bulk` elements lie
+// between the tails and were not counted; a rank that falls inside them sets s.fail.
+__device__ __forceinline__ void select_ranks(const SelectArgs& a, SelectShared& s, const uint32_t* ghist,
+                                             const uint32_t* gcoarse, bool whole) {
+  // Rank q (0: lower, 1: upper) is served by warps 8 q .. 8 q + 7.  Every warp finds the rank's coarse
+  // range (one coarse counter per lane), then warp st of the 8 reads step st of the range's 2048 fine
+  // counters: 256 consecutive positions, 8 per lane.  The step totals meet in shared memory; the warp
+  // whose step holds the rank writes the threshold.
+  static_assert(SEL_WARPS == 16, "two ranks x eight steps, one warp each");
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = warp >> 3, st = warp & 7;
+  // abs_mode: one rank in the order of the magnitudes (both warp groups find it, the first writes
+  // -t and t): magnitude range c holds the positive range 16 + c and the negative range 15 - c.
+  // (counts and ranks fit 32 bits: n < 2^31)
+  const uint32_t raw = __ldcg(&gcoarse[lane]);
+  const uint32_t raw_mag = a.abs_mode && lane < 16 ? __ldcg(&gcoarse[16 + lane]) + __ldcg(&gcoarse[15 - lane]) : 0u;
+  const uint32_t n = uint32_t(a.n), n_tail = uint32_t(a.n_tail), bulk = n - __reduce_add_sync(0xFFFFFFFFu, raw);
+  const bool upper = a.abs_mode || q == 1;
+  const uint32_t rank = a.abs_mode ? n - 1 - 2 * n_tail - bulk : (q == 0 ? n_tail : n - 1 - n_tail - bulk);
+  const uint32_t cc = a.abs_mode ? raw_mag : raw;
+  const uint32_t sc = warp_inclusive_scan(cc);
+  const unsigned holds = __ballot_sync(0xFFFFFFFFu, rank >= sc - cc && rank < sc);   // at most one lane
+  const int region = holds ? __ffs(holds) - 1 : 0;
+  uint32_t run = __shfl_sync(0xFFFFFFFFu, sc - cc, region);                           // counts before the range
+  if (!holds && lane == 0) s.fail = 1;
+  // positions of the range in ascending order; in memory they ascend (region >= 16) or descend
+  const bool desc = !a.abs_mode && region < 16;
+  const uint32_t* first = a.abs_mode ? ghist + 2048 * region
+                                     : ghist + (desc ? (0xFFFF - 2048 * region - 2047) : 2048 * (region - 16));
+  const int word = desc ? (2048 - 256 * st - 8 * lane - 8) : (256 * st + 8 * lane);
+  uint32_t c[8];
 #pragma unroll
-    for (int r = 0; r < HIST_COPIES; ++r) {
-      const uint2 c = *reinterpret_cast<const uint2*>(&h[neg * HIST_NEG_WORD + r * HIST_WINDOW + off]);
-      c0 += c.x;
-      c1 += c.y;
+  for (int h = 0; h < 2; ++h) {
+    uint4 t = __ldcg(reinterpret_cast<const uint4*>(first + word) + h);
+    if (a.abs_mode) {                                 // the same magnitudes with the sign bit set
+      const uint4 tn = __ldcg(reinterpret_cast<const uint4*>(first + 0x8000 + word) + h);
+      t = make_uint4(t.x + tn.x, t.y + tn.y, t.z + tn.z, t.w + tn.w);
     }
-    if (c0 | c1) {
-      const uint32_t bits = (uint32_t(neg) << 15) | (base + uint32_t(off));
-      atomicAdd(reinterpret_cast<unsigned long long*>(&ghist[bits]), (unsigned long long)c0 | ((unsigned long long)c1 << 32));
-      atomicAdd(&s_coarse[bits_to_pos(bits) >> 11], c0 + c1);
+    const uint32_t tt[4] = {t.x, t.y, t.z, t.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {                     // in ascending position order
+      if (desc) c[7 - 4 * h - i] = tt[i]; else c[4 * h + i] = tt[i];
+    }
+  }
+  uint32_t mine = 0;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) mine += c[i];
+  const uint32_t incl = warp_inclusive_scan(mine);
+  if (lane == 31) s.step[q][st] = incl;
+  __syncthreads();
+  for (int j = 0; j < st; ++j) run += s.step[q][j];
+  uint32_t before = run + incl - mine;
+  if (holds && rank >= before && rank < before + mine) {
+    int k = 0;
+#pragma unroll
+    for (int i = 0; i < 7; ++i) {
+      if (k == i && rank >= before + c[i]) { before += c[i]; k = i + 1; }
+    }
+    const int at = 2048 * region + 256 * st + 8 * lane + k;
+    if (a.abs_mode) {
+      const uint32_t m15 = uint32_t(at);              // `at` counts magnitudes here
+      if (!whole && at + 32768 < s.p_pos) s.fail = 1;
+      if (q == 0) {
+        a.thresholds[1] = __uint_as_float(m15 << 16);
+        a.thresholds[0] = __uint_as_float(m15 ? (m15 | 0x8000u) << 16 : 0u);
+      }
+    } else {
+      if (!whole && (upper ? at < s.p_pos : at > s.q_pos)) s.fail = 1;
+      const uint32_t bits = pos_to_bits(at);
+      a.thresholds[q] = __uint_as_float((bits == 0x8000u ? 0u : bits) << 16);   // thresholds are real numbers: -0 is +0
     }
   }
   __syncthreads();
-  if (tid < HIST_COARSE && s_coarse[tid]) atomicAdd(&gcoarse[tid], s_coarse[tid]);
+}
+
+__global__ void __launch_bounds__(SEL_THREADS, SEL_BLOCKS_PER_SM)
+tail_select_kernel(const __grid_constant__ SelectArgs a) {
+  __shared__ SelectShared s;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int r_begin = int((long long)a.rows * blockIdx.x / gridDim.x);
+  const int r_end = int((long long)a.rows * (blockIdx.x + 1) / gridDim.x);
+  const unsigned par = a.parity ? (*reinterpret_cast<volatile unsigned*>(a.parity) & 1u) : 0u;
+  // loads issued first, so that their latency runs under the clearing below
+  const bool sampled = a.sample_rank >= 0;
+  uint2 sample = make_uint2(0, 0);
+  uint4 first = make_uint4(0, 0, 0, 0);
+  if (sampled) {
+    sample = __ldg(reinterpret_cast<const uint2*>(reinterpret_cast<const unsigned short*>(a.x) + sample_index(tid, a.n)));
+  } else if (tid < (long long)(r_end - r_begin) * a.vec_per_row) {
+    first = __ldg(&a.x[(long long)r_begin * a.vec_per_row + tid]);
+  }
+  {
+    const int rows0 = min(r_end - r_begin, SEL_ROW_SLOTS), v = a.vec_per_row;
+    if (sampled) {
+      const int units = rows0 * ((v + 32 * SEL_FLY - 1) / (32 * SEL_FLY));
+      select_request<SEL_FLY>(a, warp, units, r_begin, 0);
+      select_request<SEL_FLY>(a, warp + SEL_WARPS, units, r_begin, 1);
+    } else {
+      const int units = rows0 * ((v + 31) / 32);
+      select_request<1>(a, warp, units, r_begin, 0);
+      select_request<1>(a, warp + SEL_WARPS, units, r_begin, 1);
+    }
+  }
+  uint32_t* ghist = a.sets + size_t(par) * HIST_SET_WORDS;
+  uint32_t* gcoarse = ghist + 65536;
+  if (a.parity) {
+    // this block's slice of the other set, for the next call
+    uint32_t* other = a.sets + size_t(par ^ 1u) * HIST_SET_WORDS;
+    const int per = (HIST_SET_WORDS + gridDim.x - 1) / gridDim.x;
+    const int w0 = blockIdx.x * per, w1 = min(HIST_SET_WORDS, w0 + per);
+    for (int i = w0 + tid; i < w1; i += SEL_THREADS) other[i] = 0;
+  }
+  for (int i = blockIdx.x * SEL_THREADS + tid; i < a.clear_words; i += gridDim.x * SEL_THREADS) a.clear[i] = 0;
+  for (int i = tid; i < 2 * SEL_WINDOW / 4; i += SEL_THREADS) reinterpret_cast<uint4*>(s.window)[i] = make_uint4(0, 0, 0, 0);
+  if (tid < HIST_COARSE) s.coarse[tid] = 0;
+  if (tid == 0) { s.top = 0; s.fail = 0; }
+  __syncthreads();
+  // Everything is counted (no sample), or what lies outside the sample's bracket.
+  uint32_t p_bits = 0, q_bits = 0;
+  int p_pos = 0, q_pos = 65535;
+  if (!sampled) {
+    // the window's top: from the block's first vectors
+    const uint32_t w[4] = {first.x, first.y, first.z, first.w};
+    uint32_t m = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) m = max(m, max(w[q] & 0x7FFFu, (w[q] >> 16) & 0x7FFFu));
+    m = __reduce_max_sync(0xFFFFFFFFu, m);
+    if (lane == 0 && m) atomicMax(&s.top, m);
+  } else {
+    uint32_t m = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t w = i & 2 ? sample.y : sample.x, bits = i & 1 ? w >> 16 : w & 0xFFFFu;
+      atomicAdd(&s.bins[bits_to_pos(a.abs_mode ? bits & 0x7FFFu : bits) >> SEL_BIN_SHIFT], 1u);
+      m = max(m, bits & 0x7FFFu);
+    }
+    m = __reduce_max_sync(0xFFFFFFFFu, m);
+    if (lane == 0 && m) atomicMax(&s.top, m);
+    __syncthreads();
+    // bins 8 tid .. 8 tid + 7 of this thread; the thread whose bins hold a rank notes the bin
+    static_assert(SEL_BINS == 8 * SEL_THREADS, "eight bins per thread");
+    uint4* bins4 = reinterpret_cast<uint4*>(s.bins) + 2 * tid;
+    const uint4 b0 = bins4[0], b1 = bins4[1];
+    bins4[0] = bins4[1] = make_uint4(0, 0, 0, 0);      // the same words are the window's counters from here on
+    const int c[8] = {int(b0.x), int(b0.y), int(b0.z), int(b0.w), int(b1.x), int(b1.y), int(b1.z), int(b1.w)};
+    const int mine = c[0] + c[1] + c[2] + c[3] + c[4] + c[5] + c[6] + c[7];
+    const int incl = warp_inclusive_scan(mine);
+    if (lane == 31) s.warp_tot[warp] = incl;
+    __syncthreads();
+    int before = incl - mine;
+    for (int w = 0; w < warp; ++w) before += s.warp_tot[w];
+    const int k_lo = min(a.sample_rank, SEL_SAMPLES - 1), k_hi = SEL_SAMPLES - 1 - k_lo;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      if (k_lo >= before && k_lo < before + c[i]) s.q_pos = ((8 * tid + i) << SEL_BIN_SHIFT) + (1 << SEL_BIN_SHIFT) - 1;
+      if (k_hi >= before && k_hi < before + c[i]) s.p_pos = (8 * tid + i) << SEL_BIN_SHIFT;
+      before += c[i];
+    }
+    __syncthreads();
+    // The bracket as numbers.  Comparisons do not tell -0 from +0, so a bound at a zero takes in both; a
+    // bound among the NaN patterns (only with non-finite inputs) leaves no bulk.
+    p_pos = s.p_pos;
+    q_pos = a.abs_mode ? 65535 - p_pos : s.q_pos;
+    if (p_pos == bits_to_pos(0x0000u)) p_pos = bits_to_pos(0x8000u);
+    if (q_pos == bits_to_pos(0x8000u)) q_pos = bits_to_pos(0x0000u);
+    p_bits = pos_to_bits(p_pos);
+    q_bits = pos_to_bits(q_pos);
+  }
+  __syncthreads();
+  if (tid == 0) { s.p_pos = p_pos; s.q_pos = q_pos; }
+  const int e_top = min(254, int(s.top >> 7) + SEL_HEADROOM);
+  const uint32_t base = uint32_t(max(0, e_top - SEL_EXPS + 1)) << 7;
+  if (sampled)
+    select_count_rows<false>(a, s, r_begin, r_end, p_bits, q_bits, base, ghist, true);
+  else
+    select_count_rows<true>(a, s, r_begin, r_end, p_bits, q_bits, base, ghist, true);
+  __syncthreads();
+  // counted magnitudes start at the smaller bound where the bracket holds zero (else anywhere)
+  const uint32_t lowest = sampled && !(p_bits & 0x8000u) && (q_bits & 0x8000u) ? min(p_bits, q_bits & 0x7FFFu) : 0u;
+  select_flush(s, base, ghist, lowest > base ? int(lowest - base) & ~63 : 0);
+  __syncthreads();
+  if (tid < HIST_COARSE && s.coarse[tid]) atomicAdd(&gcoarse[tid], s.coarse[tid]);
   // ---- the last block to get here selects -------------------------------------------------
   __threadfence();
   __syncthreads();
-  if (tid == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  if (tid == 0) s.last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
   __syncthreads();
-  if (!s_last) return;
+  if (!s.last) return;
   __threadfence();
-  {
-    // Rank q (0: lower, 1: upper) is served by warps 16 q .. 16 q + 15.  Every warp finds the rank's
-    // coarse range (one coarse counter per lane), then warp st of the 16 reads step st of the range's
-    // 2048 fine counters: 128 consecutive positions, 4 per lane.  The step totals meet in shared
-    // memory; the warp whose step holds the rank writes the threshold.
-    static_assert(HIST_THREADS == 1024, "two ranks x sixteen steps, one warp each");
-    __shared__ long long s_step[2][16];
-    const int warp = tid >> 5, lane = tid & 31, q = warp >> 4, st = warp & 15;
-    // abs_mode: one rank in the order of the magnitudes (both warp groups find it, the first writes
-    // -t and t): magnitude range c holds the positive range 16 + c and the negative range 15 - c.
-    const long long rank = abs_mode ? n - 1 - 2 * n_tail : (q == 0 ? n_tail : n - 1 - n_tail);
-    const long long cc = !abs_mode ? (long long)__ldcg(&gcoarse[lane])
-                         : (lane < 16 ? (long long)__ldcg(&gcoarse[16 + lane]) + __ldcg(&gcoarse[15 - lane]) : 0ll);
-    long long sc = cc;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const long long up = __shfl_up_sync(0xFFFFFFFFu, sc, off);
-      if (lane >= off) sc += up;
-    }
-    const unsigned holds = __ballot_sync(0xFFFFFFFFu, rank >= sc - cc && rank < sc);   // exactly one lane
-    const int region = holds ? __ffs(holds) - 1 : 0;
-    long long run = __shfl_sync(0xFFFFFFFFu, sc - cc, region);                          // counts before the range
-    // positions of the range in ascending order; in memory they ascend (region >= 16) or descend
-    const bool desc = !abs_mode && region < 16;
-    const uint32_t* first = abs_mode ? ghist + 2048 * region
-                                     : ghist + (desc ? (0xFFFF - 2048 * region - 2047) : 2048 * (region - 16));
-    const int word = desc ? (2048 - 128 * st - 4 * lane - 4) : (128 * st + 4 * lane);
-    uint4 c = __ldcg(reinterpret_cast<const uint4*>(first + word));
-    if (abs_mode) {                                   // the same magnitudes with the sign bit set
-      const uint4 cn = __ldcg(reinterpret_cast<const uint4*>(first + 0x8000 + word));
-      c = make_uint4(c.x + cn.x, c.y + cn.y, c.z + cn.z, c.w + cn.w);
-    }
-    // in ascending position order
-    const long long v0 = desc ? c.w : c.x, v1 = desc ? c.z : c.y;
-    const long long v2 = desc ? c.y : c.z, v3 = desc ? c.x : c.w;
-    const long long mine = v0 + v1 + v2 + v3;
-    long long incl = mine;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const long long up = __shfl_up_sync(0xFFFFFFFFu, incl, off);
-      if (lane >= off) incl += up;
-    }
-    if (lane == 31) s_step[q][st] = incl;
+  select_ranks(a, s, ghist, gcoarse, false);
+  if (s.fail) {
+    // The bracket missed: count the whole tensor into the cleared set, nothing left out.
+    for (int i = tid; i < HIST_SET_WORDS; i += SEL_THREADS) ghist[i] = 0;
+    for (int i = tid; i < 2 * SEL_WINDOW; i += SEL_THREADS) s.window[i] = 0;
+    if (tid < HIST_COARSE) s.coarse[tid] = 0;
+    __threadfence();
     __syncthreads();
-    for (int j = 0; j < st; ++j) run += s_step[q][j];
-    const long long before = run + incl - mine;
-    if (holds && rank >= before && rank < before + mine) {
-      const int p0 = 2048 * region + 128 * st + 4 * lane;
-      const int k = rank < before + v0 ? 0 : (rank < before + v0 + v1 ? 1 : (rank < before + v0 + v1 + v2 ? 2 : 3));
-      if (abs_mode) {
-        const uint32_t m15 = uint32_t(p0 + k);          // p0 counts magnitudes here
-        if (q == 0) {
-          thresholds[1] = __uint_as_float(m15 << 16);
-          thresholds[0] = __uint_as_float(m15 ? (m15 | 0x8000u) << 16 : 0u);
-        }
-      } else {
-        const uint32_t bits = pos_to_bits(p0 + k);
-        thresholds[q] = __uint_as_float((bits == 0x8000u ? 0u : bits) << 16);   // thresholds are real numbers: -0 is +0
-      }
-    }
+    select_count_rows<true>(a, s, 0, a.rows, 0, 0, base, ghist, false);
+    __syncthreads();
+    select_flush(s, base, ghist, 0);
+    __syncthreads();
+    if (tid < HIST_COARSE) gcoarse[tid] = s.coarse[tid];
+    __threadfence();
+    __syncthreads();
+    select_ranks(a, s, ghist, gcoarse, true);
   }
-  __syncthreads();
   if (tid == 0) {
-    if (parity) *parity = par ^ 1u;
-    *ticket = 0;
+    if (a.parity) *a.parity = par ^ 1u;
+    *a.ticket = 0;
   }
+}
+
+// Sample rank of the bracket (see above): six and a half standard deviations of the sample count, plus eight.
+int select_sample_rank(long long n, long long n_tail) {
+  const double mean = double(n_tail) / double(n) * SEL_SAMPLES;
+  return int(mean + 6.5 * std::sqrt(mean) + 8.0);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -623,6 +793,7 @@ struct EncodeArgs {
   int* row_cnt;                 // clamp: clamped entries per row (zero-initialised)
   uint8_t* strip_cnt;           // clamp: [rows/64 x cols] clamped entries per (strip, column)
   int* col_cnt;                 // clamp: clamped entries per column (zero-initialised)
+  int* super_cnt;               // clamp: [groups of SUPER strips x cols] clamped entries (zero-initialised)
   float fmax;                   // FP8 encoder: the format's largest value (448 or 57344)
   int e5m2;                     // FP8 encoder: E5M2 bytes instead of E4M3 bytes
 };
@@ -733,6 +904,7 @@ encode_kernel(const EncodeArgs a) {
         f2[c] = __fmaf_rn(__fmul_rn(xv, prow), gc[c], 0.0f);
       }
     }
+    if (OCC && !in_cols) obits = 0;                   // beyond the tensor: its zeros may lie outside [lo, hi]
     word[r] = encode8(f);
     if constexpr (MODE == MODE_DUAL) word_t[r] = encode8(f2);
     if (in_cols) {
@@ -769,7 +941,10 @@ encode_kernel(const EncodeArgs a) {
   __syncthreads();
   if (OCC && col0 + tid < a.cols) {
     a.strip_cnt[(long long)blockIdx.y * a.cols + col0 + tid] = uint8_t(s_colcnt[tid]);
-    if (s_colcnt[tid]) atomicAdd(&a.col_cnt[col0 + tid], s_colcnt[tid]);     // integer sums: order-independent
+    if (s_colcnt[tid]) {                              // integer sums: order-independent
+      atomicAdd(&a.col_cnt[col0 + tid], s_colcnt[tid]);
+      atomicAdd(&a.super_cnt[(long long)(blockIdx.y / SUPER) * a.cols + col0 + tid], s_colcnt[tid]);
+    }
   }
   if (a.codes_t) {
     // thread (c = warp, j = lane) owns column col0 + 8 j + c: 64 rows = 8 words = 32 bytes
@@ -922,59 +1097,74 @@ encode_fp8_kernel(const EncodeArgs a) {
 // ------------------------------------------------------------------------------------------
 // 4. mask -> CSR / CSC
 // ------------------------------------------------------------------------------------------
-// The CSR and the CSC of the residual are built from the encoder's mask and counts in three launches
-// (formerly five, two of them single-block scans).
+// The CSR and the CSC of the residual are built from the encoder's mask and counts in three launches: the
+// two pointer arrays, then the two fills.
 //
 // Launch 1, sparse_prefix_kernel: block 0 turns the row counts into csr_rowptr (and nnz); every
-// other block owns 1024 columns: their column pointers -- the counts of all earlier columns are
-// summed by the block itself, so no block waits for another -- and, per column, the running offsets
-// of the 64-row strips (strip_off), from which the fill kernel places a strip's entries.
+// other block owns 1024 columns and their column pointers -- the counts of all earlier columns are
+// summed by the block itself, so no block waits for another.  (Where a strip's entries start inside a
+// column is worked out by the fill from the counts per strip and per SUPER strips.  A running sum over
+// the strips here was a serial loop on a handful of SMs: 14 us of 8192 x 4096.)
 // (A total cannot exceed the caller's capacity: the host refuses capacities below 2 n_tail, and at
-// most n_tail entries lie beyond either threshold.  The fill kernel still guards every write.)
+// most n_tail entries lie beyond either threshold.  The fill kernels still guard every write.)
+
+// Inclusive scan of one value per thread over a block of 1024 threads; the total is left in warp_tot[31].
+__device__ __forceinline__ int block_scan_1024(int v, int* warp_tot /*[32] shared*/) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  v = warp_inclusive_scan(v);
+  if (lane == 31) warp_tot[warp] = v;
+  __syncthreads();
+  if (warp == 0) warp_tot[lane] = warp_inclusive_scan(warp_tot[lane]);
+  __syncthreads();
+  if (warp > 0) v += warp_tot[warp - 1];
+  return v;
+}
+
 __global__ void __launch_bounds__(1024, 1)
 sparse_prefix_kernel(const int* __restrict__ row_cnt, int rows, int* __restrict__ rowptr, int* __restrict__ nnz_out,
-                     const int* __restrict__ col_cnt, const uint8_t* __restrict__ strip_cnt, int cols, int strips,
-                     int* __restrict__ colptr, int* __restrict__ strip_off) {
-  __shared__ long long warp_tot[32];
+                     const int* __restrict__ col_cnt, int cols, int* __restrict__ colptr) {
+  __shared__ int warp_tot[32];
   const int t = threadIdx.x;
   if (blockIdx.x == 0) {
-    const int per = (rows + 1023) / 1024;
-    const int b = min(rows, t * per), e = min(rows, b + per);
-    int s = 0;
-    for (int i = b; i < e; ++i) s += row_cnt[i];
-    const long long incl = block_scan_1024(s, warp_tot);
-    int run = int(incl) - s;
-    for (int i = b; i < e; ++i) {
-      rowptr[i] = run;
-      run += row_cnt[i];
+    // four rows per thread and round
+    int base = 0;
+    for (int r0 = 0; r0 < rows; r0 += 4096) {
+      const int r = r0 + 4 * t;
+      int4 c = make_int4(0, 0, 0, 0);
+      if (r < rows) c = *reinterpret_cast<const int4*>(row_cnt + r);
+      const int mine = c.x + c.y + c.z + c.w;
+      const int incl = block_scan_1024(mine, warp_tot);
+      const int at = base + incl - mine;
+      if (r < rows) {                                 // (the caller's pointer array is aligned to 4 bytes only)
+        rowptr[r] = at;
+        rowptr[r + 1] = at + c.x;
+        rowptr[r + 2] = at + c.x + c.y;
+        rowptr[r + 3] = at + c.x + c.y + c.z;
+      }
+      base += warp_tot[31];
+      __syncthreads();                                // warp_tot is written again in the next round
     }
-    if (t == 1023) {
-      rowptr[rows] = int(incl);
-      if (nnz_out) *nnz_out = int(incl);
+    if (t == 0) {
+      rowptr[rows] = base;
+      if (nnz_out) *nnz_out = base;
     }
     return;
   }
   const int c0 = (int(blockIdx.x) - 1) * 1024;
   // entries of all earlier columns
   int before = 0;
-  for (int i = t; i < c0; i += 1024) before += col_cnt[i];
-  const long long earlier = block_scan_1024(before, warp_tot);
-  __shared__ long long s_base;
-  if (t == 1023) s_base = earlier;
-  __syncthreads();
+  for (int i = 4 * t; i < c0; i += 4096) {
+    const int4 c = *reinterpret_cast<const int4*>(col_cnt + i);
+    before += c.x + c.y + c.z + c.w;
+  }
   const int k = c0 + t;
   const int mine = k < cols ? col_cnt[k] : 0;
-  const long long incl = block_scan_1024(mine, warp_tot);
-  if (k < cols) colptr[k] = int(s_base + incl) - mine;
-  if (k == cols - 1) colptr[cols] = int(s_base + incl);
-  if (k >= cols) return;
-  int run = 0;
-#pragma unroll 8
-  for (int s = 0; s < strips; ++s) {
-    const int c = strip_cnt[(long long)s * cols + k];
-    strip_off[(long long)s * cols + k] = run;
-    run += c;
-  }
+  block_scan_1024(before, warp_tot);
+  const int base = warp_tot[31];
+  __syncthreads();
+  const int incl = block_scan_1024(mine, warp_tot);
+  if (k < cols) colptr[k] = base + incl - mine;
+  if (k == cols - 1) colptr[cols] = base + incl;
 }
 
 __device__ __forceinline__ float residual_of(const __nv_bfloat16* x, long long idx, float lo, float hi) {
@@ -982,108 +1172,166 @@ __device__ __forceinline__ float residual_of(const __nv_bfloat16* x, long long i
   return __fsub_rn(v, v > hi ? hi : lo);
 }
 
-// CSR: one warp per row sweeps the row's mask words; a warp scan of the words' bit counts gives
-// every marked entry its place, columns ascending.
-__device__ __forceinline__ void csr_fill_block(int block, const uint32_t* __restrict__ mask,
-                                               const __nv_bfloat16* __restrict__ x, int rows, int cols,
-                                               const float* __restrict__ thresholds, int thr_per_row,
-                                               const int* __restrict__ rowptr, long long cap, int* __restrict__ csr_col,
-                                               float* __restrict__ csr_val) {
-  const int row = block * 8 + (threadIdx.x >> 5);
+// Both fills first list the marked positions of a warp's piece of the mask in shared memory, in output
+// order, and then fetch the values of the list 32 at a time: the scattered reads of x are independent of
+// one another, and the entries leave in order.  (Fetching each value where its bit was found made every
+// read wait for the previous one: csr 34 / csc 69 us of 8192 x 11008 at 1 % per tail.)
+constexpr int FILL_WARPS = 8;
+
+// CSR: one warp per row, 32 mask words (1024 columns) at a time; a warp scan of the words' bit counts
+// gives every marked entry its place, columns ascending.
+constexpr int CSR_LIST = 1024;                        // listed entries: at least the 1024 of one step
+__global__ void __launch_bounds__(32 * FILL_WARPS)
+csr_fill_kernel(const uint32_t* __restrict__ mask, const __nv_bfloat16* __restrict__ x, int rows, int cols,
+                const float* __restrict__ thresholds, int thr_per_row, const int* __restrict__ rowptr, long long cap,
+                int* __restrict__ csr_col, float* __restrict__ csr_val) {
+  __shared__ uint16_t s_list[FILL_WARPS][CSR_LIST];
+  const int row = blockIdx.x * FILL_WARPS + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= rows) return;
   int base = rowptr[row];
   if (rowptr[row + 1] == base) return;                // nothing clamped in this row
-  const int words_per_row = cols >> 5;
+  uint16_t* list = s_list[threadIdx.x >> 5];
+  const int words = cols >> 5;
+  const uint32_t* mrow = mask + (long long)row * words;
+  const __nv_bfloat16* xrow = x + (long long)row * cols;
   const float lo = thresholds[thr_per_row ? 2 * row : 0], hi = thresholds[thr_per_row ? 2 * row + 1 : 1];
-  for (int w0 = 0; w0 < words_per_row; w0 += 32) {
-    const int w = w0 + lane;
-    uint32_t m = w < words_per_row ? mask[(long long)row * words_per_row + w] : 0u;
-    const int c = __popc(m);
-    int incl = c;                                     // inclusive warp scan of the counts
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const int up = __shfl_up_sync(0xFFFFFFFFu, incl, off);
-      if (lane >= off) incl += up;
+  int n = 0;                                          // listed entries
+  int col0 = 0;                                       // list entries are columns less this (a multiple of 32768)
+  auto flush = [&]() {
+    __syncwarp();
+#pragma unroll 4
+    for (int i = lane; i < n; i += 32) {
+      const int col = col0 + list[i];
+      const float v = residual_of(xrow, col, lo, hi);
+      if (base + i < cap) {
+        csr_col[base + i] = col;
+        csr_val[base + i] = v;
+      }
     }
-    int pos = base + incl - c;
+    __syncwarp();
+    base += n;
+    n = 0;
+  };
+  uint32_t next = lane < words ? mrow[lane] : 0u;
+  for (int w0 = 0; w0 < words; w0 += 32) {
+    uint32_t m = next;
+    next = w0 + 32 + lane < words ? mrow[w0 + 32 + lane] : 0u;
+    const int c = __popc(m);
+    const int incl = warp_inclusive_scan(c), total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    if (n + total > CSR_LIST || 32 * w0 - col0 >= 32768) {
+      flush();
+      col0 = (32 * w0) & ~32767;
+    }
+    int pos = n + incl - c;
+    const int rel = 32 * (w0 + lane) - col0;
     while (m) {
       const int b = __ffs(m) - 1;
       m &= m - 1;
-      const int col = 32 * w + b;
-      if (pos < cap) {
-        csr_col[pos] = col;
-        csr_val[pos] = residual_of(x, (long long)row * cols + col, lo, hi);
-      }
-      ++pos;
+      list[pos++] = uint16_t(rel + b);
     }
-    base += __shfl_sync(0xFFFFFFFFu, incl, 31);
+    n += total;
   }
+  flush();
 }
 
-// CSC: one warp per (64-row strip, 32-column word of the mask).  Lane <-> row: each lane keeps the
-// mask word of its row.  For every column of the word that holds a marked entry (usually one or
-// two: the outlier channels), a ballot gives each marked row its rank inside the column, so all
-// gathers of a column are issued at once and the order is by row by construction.
-__device__ __forceinline__ void csc_fill_block(int bx, int strip, const uint32_t* __restrict__ mask,
-                                               const __nv_bfloat16* __restrict__ x, int rows, int cols,
-                                               const float* __restrict__ thresholds, int thr_per_row,
-                                               const int* __restrict__ colptr, const int* __restrict__ strip_off,
-                                               long long cap, int* __restrict__ csc_row, float* __restrict__ csc_val) {
-  const int q = bx * 8 + (threadIdx.x >> 5);
+// 32 x 32 bit transpose over a warp: bit c of lane r -> bit r of lane c.
+__device__ __forceinline__ uint32_t transpose_bits(uint32_t v) {
   const int lane = threadIdx.x & 31;
+  uint32_t keep = 0x0000FFFFu;
+#pragma unroll
+  for (int j = 16; j; j >>= 1) {
+    const uint32_t o = __shfl_xor_sync(0xFFFFFFFFu, v, j);
+    v = lane & j ? (v & ~keep) | ((o >> j) & keep) : (v & keep) | ((o << j) & ~keep);
+    keep ^= keep << (j >> 1);
+  }
+  return v;
+}
+
+// CSC: one warp per (64-row strip, 32-column word of the mask).  The word's two 32 x 32 blocks are
+// transposed, lane c then holds the marked rows of column c and lists them; a column with many of them
+// (an outlier channel) is listed by all lanes at once.
+constexpr int CSC_MANY = 8;
+__global__ void __launch_bounds__(32 * FILL_WARPS)
+csc_fill_kernel(const uint32_t* __restrict__ mask, const __nv_bfloat16* __restrict__ x, int rows, int cols,
+                const float* __restrict__ thresholds, int thr_per_row, const int* __restrict__ colptr,
+                const uint8_t* __restrict__ strip_cnt, const int* __restrict__ super_cnt, long long cap,
+                int* __restrict__ csc_row, float* __restrict__ csc_val) {
+  __shared__ uint16_t s_list[FILL_WARPS][2048];
+  __shared__ int s_delta[FILL_WARPS][32];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int q = blockIdx.x * FILL_WARPS + warp, strip = blockIdx.y;
   const int words_per_row = cols >> 5;
   if (q >= words_per_row) return;
   const int r0 = strip * ENC_TM;
   const uint32_t w0 = mask[(long long)(r0 + lane) * words_per_row + q];
   const uint32_t w1 = mask[(long long)(r0 + 32 + lane) * words_per_row + q];
-  const uint32_t any0 = __reduce_or_sync(0xFFFFFFFFu, w0);
-  const uint32_t any1 = __reduce_or_sync(0xFFFFFFFFu, w1);
-  if (!(any0 | any1)) return;
-  // lane c holds the next free position of column 32 q + c
-  int next = colptr[32 * q + lane] + strip_off[(long long)strip * cols + 32 * q + lane];
-  const uint32_t lt_mask = (1u << lane) - 1u;
+  if (!__any_sync(0xFFFFFFFFu, w0 | w1)) return;
+  // where this strip's entries of column 32 q + lane start: the column's pointer, whole groups of SUPER
+  // strips, then the strips of the own group
+  const int k = 32 * q + lane;
+  int at = colptr[k];
+  const int sup = strip / SUPER;
+  for (int g = 0; g < sup; ++g) at += super_cnt[(long long)g * cols + k];
 #pragma unroll
-  for (int half = 0; half < 2; ++half) {
-    const uint32_t w = half ? w1 : w0;
-    uint32_t any = half ? any1 : any0;
-    const int r = r0 + 32 * half + lane;
-    const float lo = thresholds[thr_per_row ? 2 * r : 0], hi = thresholds[thr_per_row ? 2 * r + 1 : 1];
-    while (any) {
-      const int c = __ffs(any) - 1;
-      any &= any - 1;
-      const bool mine = (w >> c) & 1u;
-      const uint32_t b = __ballot_sync(0xFFFFFFFFu, mine);
-      const int base = __shfl_sync(0xFFFFFFFFu, next, c);
-      if (mine) {
-        const int pos = base + __popc(b & lt_mask);
-        if (pos < cap) {
-          csc_row[pos] = r;
-          csc_val[pos] = residual_of(x, (long long)r * cols + 32 * q + c, lo, hi);
-        }
-      }
-      if (lane == c) next += __popc(b);
+  for (int g = 0; g < SUPER - 1; ++g)
+    if (sup * SUPER + g < strip) at += strip_cnt[(long long)(sup * SUPER + g) * cols + k];
+  const uint32_t t0 = transpose_bits(w0), t1 = transpose_bits(w1);       // rows 0..31 / 32..63 of column `lane`
+  const int c = __popc(t0) + __popc(t1);
+  const int incl = warp_inclusive_scan(c);
+  const int n = __shfl_sync(0xFFFFFFFFu, incl, 31);
+  uint16_t* list = s_list[warp];
+  int pos = incl - c;
+  s_delta[warp][lane] = at - pos;                     // output position of list entry i of this column: i + delta
+  unsigned many = __ballot_sync(0xFFFFFFFFu, c > CSC_MANY);
+  if (c <= CSC_MANY) {
+    int p = pos;
+    uint32_t m = t0;
+    while (m) {
+      const int b = __ffs(m) - 1;
+      m &= m - 1;
+      list[p++] = uint16_t((lane << 6) | b);
+    }
+    m = t1;
+    while (m) {
+      const int b = __ffs(m) - 1;
+      m &= m - 1;
+      list[p++] = uint16_t((lane << 6) | 32 | b);
+    }
+  }
+  while (many) {
+    const int src = __ffs(many) - 1;
+    many &= many - 1;
+    const uint32_t m0 = __shfl_sync(0xFFFFFFFFu, t0, src), m1 = __shfl_sync(0xFFFFFFFFu, t1, src);
+    const int p = __shfl_sync(0xFFFFFFFFu, pos, src);
+    const uint32_t lt = (1u << lane) - 1u;
+    if ((m0 >> lane) & 1u) list[p + __popc(m0 & lt)] = uint16_t((src << 6) | lane);
+    if ((m1 >> lane) & 1u) list[p + __popc(m0) + __popc(m1 & lt)] = uint16_t((src << 6) | 32 | lane);
+  }
+  __syncwarp();
+  const float lo = thresholds[0], hi = thresholds[1];
+#pragma unroll 4
+  for (int i = lane; i < n; i += 32) {
+    const int e = list[i], r = r0 + (e & 63), col = e >> 6;
+    const int to = i + s_delta[warp][col];
+    float l = lo, h = hi;
+    if (thr_per_row) { l = thresholds[2 * r]; h = thresholds[2 * r + 1]; }
+    const float v = residual_of(x, (long long)r * cols + 32 * q + col, l, h);
+    if (to < cap) {
+      csc_row[to] = r;
+      csc_val[to] = v;
     }
   }
 }
 
-// Launches 2 and 3 fill the CSR (8 rows per block) and the CSC (8 mask words of one strip per block).
-// They share only their inputs and run on two streams where the caller offers them: the forward's
-// compensation waits for the CSR alone.
-__global__ void __launch_bounds__(256)
-csr_fill_kernel(const uint32_t* __restrict__ mask, const __nv_bfloat16* __restrict__ x, int rows, int cols,
-                const float* __restrict__ thresholds, int thr_per_row, const int* __restrict__ rowptr, long long cap,
-                int* __restrict__ csr_col, float* __restrict__ csr_val) {
-  csr_fill_block(blockIdx.x, mask, x, rows, cols, thresholds, thr_per_row, rowptr, cap, csr_col, csr_val);
-}
-
-__global__ void __launch_bounds__(256)
-csc_fill_kernel(const uint32_t* __restrict__ mask, const __nv_bfloat16* __restrict__ x, int rows, int cols,
-                const float* __restrict__ thresholds, int thr_per_row, const int* __restrict__ colptr,
-                const int* __restrict__ strip_off, long long cap, int* __restrict__ csc_row,
-                float* __restrict__ csc_val) {
-  csc_fill_block(blockIdx.x, blockIdx.y, mask, x, rows, cols, thresholds, thr_per_row, colptr, strip_off, cap, csc_row,
-                 csc_val);
+// At most two blocks per SM, and as few as give no block more rows than that.  Small tensors (a block
+// holds a few thousand elements) are counted whole: the sample's chain would cost more than it saves.
+void launch_select(SelectArgs& a, int num_sms, cudaStream_t stream) {
+  const int most = SEL_BLOCKS_PER_SM * num_sms, per = (a.rows + most - 1) / most;
+  // abs mode has one bracket on the magnitudes, with both tails in it
+  const int k = select_sample_rank(a.n, a.abs_mode ? 2 * a.n_tail : a.n_tail);
+  a.sample_rank = a.n < (long long)SEL_ALL * num_sms ? -1 : k;
+  tail_select_kernel<<<(a.rows + per - 1) / per, SEL_THREADS, SEL_DYN_SMEM, stream>>>(a);
 }
 
 size_t r256(size_t b) { return (b + 255) & ~size_t(255); }
@@ -1097,11 +1345,14 @@ struct Scratch {
   int* row_cnt;
   int* col_cnt;
   uint8_t* strip_cnt;
-  int* strip_off;
+  int* super_cnt;               // directly behind col_cnt: cleared together
+  int count_words;              // of both
   float* pre_rows;
   float* pre_cols;
   bool ok;
 };
+
+int supers_of(int rows) { return (rows / ENC_TM + SUPER - 1) / SUPER; }
 
 Scratch carve(Arena& arena, int rows, int cols, bool occ) {
   Scratch s = {};
@@ -1110,13 +1361,14 @@ Scratch carve(Arena& arena, int rows, int cols, bool occ) {
   s.amax_rows = arena.take<uint32_t>(rows);
   s.amax_cols = arena.take<uint32_t>(cols);
   s.row_cnt = arena.take<int>(rows);
-  s.col_cnt = arena.take<int>(cols);
   s.pre_rows = arena.take<float>(rows);
   s.pre_cols = arena.take<float>(cols);
   if (occ) {
     s.mask = arena.take<uint8_t>(size_t(rows) * cols / 8);
     s.strip_cnt = arena.take<uint8_t>(size_t(rows / ENC_TM) * cols);
-    s.strip_off = arena.take<int>(size_t(rows / ENC_TM) * cols);
+    s.count_words = cols * (1 + supers_of(rows));
+    s.col_cnt = arena.take<int>(size_t(s.count_words));
+    s.super_cnt = s.col_cnt + cols;
   }
   s.ok = arena.ok;
   return s;
@@ -1124,15 +1376,23 @@ Scratch carve(Arena& arena, int rows, int cols, bool occ) {
 
 }  // namespace
 
+// Once per device, before the first launch there.
+int quantize_setup() {
+  FP4_CUDA_TRY(cudaFuncSetAttribute(tail_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SEL_DYN_SMEM));
+  // six blocks' lists side by side on an SM (the fills read nothing twice through L1)
+  FP4_CUDA_TRY(cudaFuncSetAttribute(csc_fill_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
+  return FP4_OK;
+}
+
 // Counters of the quantile selection that live as long as the context: two sets, parity, ticket.
 size_t quantize_persistent_bytes() { return (2 * size_t(HIST_SET_WORDS) + 64) * 4; }
 
 size_t quantize_scratch_bytes(int64_t rows, int64_t cols) {
   size_t b = 0;
-  b += 5 * r256(size_t(rows) * 4) + 4 * r256(size_t(cols) * 4);   // per-row / per-column vectors
+  b += 5 * r256(size_t(rows) * 4) + 2 * r256(size_t(cols) * 4);   // per-row / per-column vectors
   b += r256(size_t(rows) * size_t(cols) / 8);                    // outlier mask
   b += r256(size_t(rows / ENC_TM) * size_t(cols));               // per-strip column counts (bytes)
-  b += r256(size_t(rows / ENC_TM) * size_t(cols) * 4);           // per-strip column offsets
+  b += r256(size_t(cols) * size_t(1 + supers_of(int(rows))) * 4);   // column counts, whole and per SUPER strips
   return b;
 }
 
@@ -1166,6 +1426,7 @@ int launch_quantize(fp4_ctx* ctx, cudaStream_t stream, Arena& arena, const void*
   ea.row_cnt = sc.row_cnt;
   ea.strip_cnt = sc.strip_cnt;
   ea.col_cnt = sc.col_cnt;
+  ea.super_cnt = sc.super_cnt;
   ea.e5m2 = out->format == FP4_FORMAT_E5M2;
   ea.fmax = fp8_max(out->format);
   const dim3 tile_grid((cols + ENC_TK - 1) / ENC_TK, rows / ENC_TM);
@@ -1173,26 +1434,35 @@ int launch_quantize(fp4_ctx* ctx, cudaStream_t stream, Arena& arena, const void*
   const int per_token = occ && ctx->quantile_mode == FP4_QUANTILE_TOKEN;
   if (occ) {
     const long long n_tail = llround((1.0 - alpha) * double(n));
-    const long long n_vec = n / 8;
     if (per_token) {
       KernelScope scope(ctx, stream, KC_SELECT, 1);
       const int n_tail_row = int(llround((1.0 - alpha) * double(cols)));
+      FP4_CUDA_TRY(cudaMemsetAsync(sc.col_cnt, 0, size_t(sc.count_words) * 4, stream));     // the encoder adds to these
       row_select_kernel<<<rows, 256, 0, stream>>>(x, cols / 8, n_tail_row, sc.row_max, sc.row_min, sc.row_cnt,
                                                   out->thresholds, status);
     } else {
       // The two sets of global counters, their parity and the ticket belong to the context: the
       // kernel keeps the set it is about to use zero (see there), so nothing is cleared here.
       KernelScope scope(ctx, stream, KC_SELECT, 1);
-      FP4_CUDA_TRY(cudaFuncSetAttribute(hist_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        HIST_SMEM_BYTES));
-      long long blocks = (n_vec + HIST_THREADS - 1) / HIST_THREADS;
-      if (blocks > ctx->num_sms) blocks = ctx->num_sms;
-      unsigned* parity = reinterpret_cast<unsigned*>(ctx->occ_hist + 2 * HIST_SET_WORDS);
-      hist_select_kernel<<<int(blocks), HIST_THREADS, HIST_SMEM_BYTES, stream>>>(
-          x, rows, cols / 8, ctx->occ_hist, parity, sc.row_max, sc.row_min, sc.row_cnt, n, n_tail, out->thresholds,
-          parity + 1, status, ctx->quantile_mode == FP4_QUANTILE_ABS);
+      SelectArgs sa = {};
+      sa.x = x;
+      sa.rows = rows;
+      sa.vec_per_row = cols / 8;
+      sa.sets = ctx->occ_hist;
+      sa.parity = reinterpret_cast<unsigned*>(ctx->occ_hist + 2 * HIST_SET_WORDS);
+      sa.ticket = sa.parity + 1;
+      sa.row_max = sc.row_max;
+      sa.row_min = sc.row_min;
+      sa.row_cnt = sc.row_cnt;
+      sa.n = n;
+      sa.n_tail = n_tail;
+      sa.thresholds = out->thresholds;
+      sa.status = status;
+      sa.abs_mode = ctx->quantile_mode == FP4_QUANTILE_ABS;
+      sa.clear = sc.col_cnt;                          // the encoder adds to these
+      sa.clear_words = sc.count_words;
+      launch_select(sa, ctx->num_sms, stream);
     }
-    FP4_CUDA_TRY(cudaMemsetAsync(sc.col_cnt, 0, size_t(cols) * 4, stream));     // the encoder adds to it
     {
       KernelScope scope(ctx, stream, KC_ENCODE, 1);
       if (per_token)
@@ -1214,22 +1484,21 @@ int launch_quantize(fp4_ctx* ctx, cudaStream_t stream, Arena& arena, const void*
     {
       KernelScope scope(ctx, sp, KC_SPARSE, 2);
       sparse_prefix_kernel<<<1 + (cols + 1023) / 1024, 1024, 0, sp>>>(sc.row_cnt, rows, out->csr_rowptr, out->nnz,
-                                                                    sc.col_cnt, sc.strip_cnt, cols, strips,
-                                                                    out->csc_colptr, sc.strip_off);
+                                                                    sc.col_cnt, cols, out->csc_colptr);
       if (sp != stream && overlap->colptr_done) FP4_CUDA_TRY(cudaEventRecord(overlap->colptr_done, sp));
       if (sp != stream && overlap->stream_csc && overlap->colptr_done) {
         sc2 = overlap->stream_csc;
         FP4_CUDA_TRY(cudaStreamWaitEvent(sc2, overlap->colptr_done, 0));
       }
-      csr_fill_kernel<<<(rows + 7) / 8, 256, 0, sp>>>(mask32, xb, rows, cols, out->thresholds, per_token, out->csr_rowptr,
+      csr_fill_kernel<<<(rows + FILL_WARPS - 1) / FILL_WARPS, 32 * FILL_WARPS, 0, sp>>>(mask32, xb, rows, cols, out->thresholds, per_token, out->csr_rowptr,
                                                       out->sparse_cap, out->csr_col, out->csr_val);
     }
     if (sp != stream) FP4_CUDA_TRY(cudaEventRecord(overlap->csr_done, sp));
     {
       KernelScope scope(ctx, sc2, KC_SPARSE, 1);
-      const dim3 cgrid((cols / 32 + 7) / 8, strips);
-      csc_fill_kernel<<<cgrid, 256, 0, sc2>>>(mask32, xb, rows, cols, out->thresholds, per_token, out->csc_colptr, sc.strip_off,
-                                              out->sparse_cap, out->csc_row, out->csc_val);
+      const dim3 cgrid((cols / 32 + FILL_WARPS - 1) / FILL_WARPS, strips);
+      csc_fill_kernel<<<cgrid, 32 * FILL_WARPS, 0, sc2>>>(mask32, xb, rows, cols, out->thresholds, per_token, out->csc_colptr,
+                                                          sc.strip_cnt, sc.super_cnt, out->sparse_cap, out->csc_row, out->csc_val);
     }
     if (sp != stream && overlap->csc_done) FP4_CUDA_TRY(cudaEventRecord(overlap->csc_done, sc2));
   } else {
@@ -1383,8 +1652,8 @@ extern "C" int fp4_quantile_thresholds_static(void* stream, const void* x_bf16, 
     FP4_CUDA_TRY(cudaGetSymbolAddress(&ptr, g_static_scratch));
     int sms = 0;
     FP4_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device));
-    FP4_CUDA_TRY(cudaFuncSetAttribute(hist_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      HIST_SMEM_BYTES));
+    const int rc = quantize_setup();
+    if (rc != FP4_OK) return rc;
     sms_of_device[device] = sms;
     scratch_of_device[device] = ptr;
   }
@@ -1400,12 +1669,18 @@ extern "C" int fp4_quantile_thresholds_static(void* stream, const void* x_bf16, 
   // The array keeps what the previous call left (a call that was cut short may have left counts
   // behind): the histogram and the ticket are cleared; the row extremes are written before read.
   FP4_CUDA_TRY(cudaMemsetAsync(base, 0, STATIC_HIST_BYTES + STATIC_SELECT_BYTES, st));
-  const long long n_vec = n / 8;
-  long long blocks = (n_vec + HIST_THREADS - 1) / HIST_THREADS;
-  if (blocks > num_sms) blocks = num_sms;
-  hist_select_kernel<<<int(blocks), HIST_THREADS, HIST_SMEM_BYTES, st>>>(
-      static_cast<const uint4*>(x_bf16), int(rows), int(cols / 8), hist, nullptr, row_max, row_min, nullptr, n, n_tail,
-      thresholds, ticket, nullptr, 0);
+  SelectArgs sa = {};
+  sa.x = static_cast<const uint4*>(x_bf16);
+  sa.rows = int(rows);
+  sa.vec_per_row = int(cols / 8);
+  sa.sets = hist;
+  sa.ticket = ticket;
+  sa.row_max = row_max;
+  sa.row_min = row_min;
+  sa.n = n;
+  sa.n_tail = n_tail;
+  sa.thresholds = thresholds;
+  launch_select(sa, num_sms, st);
   FP4_CUDA_TRY(cudaGetLastError());
   return FP4_OK;
 }

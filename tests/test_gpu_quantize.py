@@ -221,6 +221,66 @@ def test_selection_on_tensors_whose_bulk_is_not_around_zero(lib, ctx, kind):
         _occ_equals_oracle(lib, ctx, bits, alpha)
 
 
+def _sample_positions(n, threads=512):
+    """The elements the selection samples from a tensor of n: four neighbours per stratum, at a hashed place."""
+    i = np.arange(threads, dtype=np.uint64)
+    q = n // 4
+    b, e = q * i // threads, q * (i + 1) // threads
+    h = (i.astype(np.uint32) * np.uint32(2654435761) + np.uint32(0x9E3779B9))
+    h ^= h >> np.uint32(15)
+    h *= np.uint32(0x2C1B3C6D)
+    h ^= h >> np.uint32(13)
+    at = 4 * (b + h.astype(np.uint64) % (e - b))
+    return (at[:, None] + np.arange(4, dtype=np.uint64)).ravel().astype(np.int64)
+
+
+@pytest.mark.parametrize("kind", ["plain", "misled_high", "misled_zero", "negative", "relu", "constant", "wide_rows"])
+@pytest.mark.parametrize("abs_mode", [False, True])
+def test_selection_that_counts_only_the_tails(lib, kind, abs_mode):
+    """Tensors large enough for the selection to sample first.  Thresholds and residual are exact
+    whatever the sample says: samples that are all large (the tails it announces are far too small, the
+    whole tensor is counted in a second pass) or all zero (everything is counted), one-signed tensors,
+    more zeros than the clamped share, one value only, and rows of more than 1024 clamped entries."""
+    rng = np.random.default_rng(41)
+    shape = (256, 36864) if kind == "wide_rows" else (1280, 1152)
+    a = rng.standard_normal(shape).astype(np.float32)
+    if kind == "negative":
+        a = -np.abs(a) * np.float32(100.0) - np.float32(1.0)
+    elif kind == "relu":
+        a = np.maximum(a, np.float32(0.0))
+    elif kind == "constant":
+        a[:] = np.float32(-1.5)
+    elif kind == "wide_rows":
+        a[:8] *= np.float32(30.0)
+    elif kind.startswith("misled"):
+        at = _sample_positions(a.size)
+        sign = np.where(np.arange(at.size) % 2, np.float32(-1.0), np.float32(1.0))
+        a.ravel()[at] = sign * np.float32(200.0 if kind == "misled_high" else 0.0)
+    bits = WL.to_bf16_bits(a)
+    c = lib.Context(0, 256 << 20)
+    if abs_mode:
+        c.set_quantile_mode(lib.FP4_QUANTILE_ABS)
+    for alpha in (0.99, 0.97) if kind != "wide_rows" else (0.97,):
+        q = lib.fp4_quantize(c, _dev(bits), 0, alpha=alpha)
+        torch.cuda.synchronize()
+        assert c.read_status() == 0
+        ref = O.occ_quantize(O.bf16_bits_to_f64(bits), alpha, quantile="abs" if abs_mode else "signed")
+        _check_sparse(q, ref)
+        _check_dense(q, ref)
+    c.close()
+
+
+@pytest.mark.parametrize("bad", [0x7F80, 0xFF80, 0x7FC0, 0xFFC0])
+def test_non_finite_inputs_of_a_sampled_tensor_raise_the_status_bit(lib, ctx, bad):
+    rng = np.random.default_rng(bad)
+    bits = WL.to_bf16_bits(rng.standard_normal((1280, 1152)).astype(np.float32))
+    bits[1279, 1151] = bad
+    ctx.status.zero_()
+    lib.fp4_quantize(ctx, _dev(bits), 0, alpha=0.999)
+    torch.cuda.synchronize()
+    assert ctx.read_status() & lib.FP4_DEV_NONFINITE
+
+
 def test_config0_activation_and_weight(lib, ctx):
     cfg = WL.CONFIGS[0]
     a_bits = WL.activations(cfg, 1024)
