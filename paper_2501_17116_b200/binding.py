@@ -127,11 +127,12 @@ def _check(rc: int):
 
 
 def _ptr(t):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    # the raw handle of the current stream: building a Stream object for it costs 3 us a call
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 class Context:

@@ -5,6 +5,7 @@
 #include <cmath>
 #include <new>
 
+#include "call_graph.cuh"
 #include "common.cuh"
 
 namespace {
@@ -98,6 +99,7 @@ int fp4_create(fp4_ctx** out, int device, size_t workspace_bytes) {
   ctx->overlap = 1;
   ctx->launch_count = 0;
   ctx->records = new (std::nothrow) std::vector<ProfRecord>();
+  ctx->graphs = nullptr;
   for (auto& s : ctx->side) s = nullptr;
   for (auto& e : ctx->ev) e = nullptr;
   ctx->copy_stream = ctx->compute_stream = ctx->return_stream = nullptr;
@@ -132,6 +134,8 @@ int fp4_create(fp4_ctx** out, int device, size_t workspace_bytes) {
   }
   bool ok = true;
   ok = ok && quantize_setup() == FP4_OK;
+  ctx->graphs = new (std::nothrow) CallGraphs();
+  ok = ok && ctx->graphs && ctx->graphs->init();
   // counters of the quantile selection (quantisation with clamping): cleared here, once
   ok = ok && cudaMalloc(reinterpret_cast<void**>(&ctx->occ_hist), quantize_persistent_bytes()) == cudaSuccess;
   ok = ok && cudaMemset(ctx->occ_hist, 0, quantize_persistent_bytes()) == cudaSuccess;
@@ -168,7 +172,8 @@ int fp4_destroy(fp4_ctx* ctx) {
   for (auto& e : ctx->host_step_copied)
     if (e) cudaEventDestroy(e);
   if (ctx->workspace) cudaFree(ctx->workspace);
-  if (ctx->occ_hist) cudaFree(ctx->occ_hist);
+  if (ctx->occ_hist) cudaFree(ctx->occ_hist);      // waits for the GPU, so no graph is running below
+  delete ctx->graphs;
   if (ctx->records) {
     fp4_profile_reset(ctx);
     delete ctx->records;
@@ -202,11 +207,24 @@ int fp4_quantize(fp4_ctx* ctx, void* stream, const void* x_bf16, int64_t rows, i
     if (rc != FP4_OK) return rc;
   }
   if (quantize_scratch_bytes(rows, cols) > ctx->workspace_bytes) return FP4_ERR_WORKSPACE;
-  Arena arena(ctx->workspace, ctx->workspace_bytes);
   out->rows = rows;
   out->cols = cols;
-  return launch_quantize(ctx, static_cast<cudaStream_t>(stream), arena, x_bf16, rows, cols, scale_axis, alpha,
-                         prescale, 0.0f, out, status);
+  CallKey key;
+  std::memset(&key, 0, sizeof(key));
+  key.kind = CALL_QUANTIZE;
+  key.quantile_mode = ctx->quantile_mode;
+  key.scale_axis = scale_axis;
+  key.alpha = alpha;
+  key.M = rows;
+  key.K = cols;
+  key.ptr[0] = x_bf16;
+  key.ptr[1] = prescale;
+  key.ptr[2] = status;
+  key.a = *out;
+  return ctx->graphs->run(ctx, static_cast<cudaStream_t>(stream), key, [&](cudaStream_t st) {
+    Arena arena(ctx->workspace, ctx->workspace_bytes);
+    return launch_quantize(ctx, st, arena, x_bf16, rows, cols, scale_axis, alpha, prescale, 0.0f, out, status);
+  });
 }
 
 int fp4_gemm(fp4_ctx* ctx, void* stream, const uint8_t* a_codes, const uint8_t* b_codes, int64_t I, int64_t J,
@@ -259,8 +277,31 @@ int fp4_linear_fwd(fp4_ctx* ctx, void* stream, const void* A_bf16, const void* W
     if (rc != FP4_OK) return rc;
   }
   if (fp4_workspace_bytes(M, K, N) > ctx->workspace_bytes) return FP4_ERR_WORKSPACE;
-  return linear_fwd_impl(ctx, static_cast<cudaStream_t>(stream), Arena(ctx->workspace, ctx->workspace_bytes), A_bf16,
-                         W_bf16, M, K, N, alpha, reuse, gemm_kind, Y, out_f32, savedA, savedW, status);
+  // (linear_fwd_impl sets these too, but does not run when the call is replayed)
+  if (!(reuse & FP4_REUSE_A)) { savedA->rows = M; savedA->cols = K; }
+  if (!(reuse & FP4_REUSE_W)) { savedW->rows = K; savedW->cols = N; }
+  CallKey key;
+  std::memset(&key, 0, sizeof(key));
+  key.kind = CALL_FWD;
+  key.flags = reuse;
+  key.gemm_kind = gemm_kind;
+  key.out_f32 = out_f32;
+  key.quantile_mode = ctx->quantile_mode;
+  key.overlap = ctx->overlap;
+  key.alpha = alpha;
+  key.M = M;
+  key.K = K;
+  key.N = N;
+  key.ptr[0] = A_bf16;
+  key.ptr[1] = W_bf16;
+  key.ptr[2] = Y;
+  key.ptr[3] = status;
+  key.a = *savedA;
+  key.w = *savedW;
+  return ctx->graphs->run(ctx, static_cast<cudaStream_t>(stream), key, [&](cudaStream_t st) {
+    return linear_fwd_impl(ctx, st, Arena(ctx->workspace, ctx->workspace_bytes), A_bf16, W_bf16, M, K, N, alpha, reuse,
+                           gemm_kind, Y, out_f32, savedA, savedW, status);
+  });
 }
 
 }  // extern "C"
@@ -376,8 +417,29 @@ int fp4_linear_bwd(fp4_ctx* ctx, void* stream, const void* dY_bf16, const void* 
   if (!savedA->codes_t || !savedA->amax || !savedW->codes || !savedW->amax) return FP4_ERR_NULL;
   if (!aligned16(dY_bf16) || !aligned16(W_bf16) || !aligned16(dA) || !aligned16(dW)) return FP4_ERR_ALIGN;
   if (fp4_workspace_bytes(M, K, N) > ctx->workspace_bytes) return FP4_ERR_WORKSPACE;
-  return linear_bwd_impl(ctx, static_cast<cudaStream_t>(stream), Arena(ctx->workspace, ctx->workspace_bytes), dY_bf16,
-                         W_bf16, savedA, savedW, M, K, N, dge_on, dge_k, dge_clip, gemm_kind, dA, dW, out_f32, status);
+  CallKey key;
+  std::memset(&key, 0, sizeof(key));
+  key.kind = CALL_BWD;
+  key.gemm_kind = gemm_kind;
+  key.out_f32 = out_f32;
+  key.dge_on = dge_on;
+  key.overlap = ctx->overlap;
+  key.dge_k = dge_k;
+  key.dge_clip = dge_clip;
+  key.M = M;
+  key.K = K;
+  key.N = N;
+  key.ptr[0] = dY_bf16;
+  key.ptr[1] = W_bf16;
+  key.ptr[2] = dA;
+  key.ptr[3] = dW;
+  key.ptr[4] = status;
+  key.a = *savedA;
+  key.w = *savedW;
+  return ctx->graphs->run(ctx, static_cast<cudaStream_t>(stream), key, [&](cudaStream_t st) {
+    return linear_bwd_impl(ctx, st, Arena(ctx->workspace, ctx->workspace_bytes), dY_bf16, W_bf16, savedA, savedW, M, K, N,
+                           dge_on, dge_k, dge_clip, gemm_kind, dA, dW, out_f32, status);
+  });
 }
 
 }  // extern "C"

@@ -33,6 +33,8 @@ struct ProfRecord {
 // of finished outputs for long).
 constexpr int HOST_STEP_SETS = 2;
 
+class CallGraphs;                     // call_graph.cuh
+
 struct fp4_ctx {
   int      device;
   int      num_sms;
@@ -57,6 +59,7 @@ struct fp4_ctx {
   int      profile;            // record CUDA events around every kernel class
   long long launch_count;      // kernels enqueued since the last reset
   std::vector<ProfRecord>* records;
+  CallGraphs* graphs;          // calls that repeat, as CUDA graphs
 };
 
 // Counts the kernels a launcher enqueues and, in profiling mode, brackets them with CUDA events

@@ -1167,72 +1167,80 @@ sparse_prefix_kernel(const int* __restrict__ row_cnt, int rows, int* __restrict_
   if (k == cols - 1) colptr[cols] = base + incl;
 }
 
-__device__ __forceinline__ float residual_of(const __nv_bfloat16* x, long long idx, float lo, float hi) {
-  const float v = __bfloat162float(x[idx]);
-  return __fsub_rn(v, v > hi ? hi : lo);
-}
-
-// Both fills first list the marked positions of a warp's piece of the mask in shared memory, in output
-// order, and then fetch the values of the list 32 at a time: the scattered reads of x are independent of
-// one another, and the entries leave in order.  (Fetching each value where its bit was found made every
-// read wait for the previous one: csr 34 / csc 69 us of 8192 x 11008 at 1 % per tail.)
+// Both fills hand the marked entries of a warp's piece of the mask out to the lanes, 32 at a time and in
+// output order: lane i finds the word that holds entry i by a binary search over the scanned bit counts,
+// and its bit by halving.  So all lanes fetch a value at once, and the entries leave in order.  (Fetching
+// every value by the lane that holds the word made the reads of a lane wait for one another: csr 12, csc 26
+// us of 1920 x 5504 at 3 % per tail, 8 and 10 now.)  No shared memory: a GEMM that runs beside the fills
+// leaves none on its SM, and blocks that need some would wait for its end.
 constexpr int FILL_WARPS = 8;
 
-// CSR: one warp per row, 32 mask words (1024 columns) at a time; a warp scan of the words' bit counts
-// gives every marked entry its place, columns ascending.
-constexpr int CSR_LIST = 1024;                        // listed entries: at least the 1024 of one step
+// Position of set bit number r (from 0, r < popc(m)) of m.
+__device__ __forceinline__ int nth_set_bit(uint32_t m, int r) {
+  int pos = 0;
+#pragma unroll
+  for (int s = 16; s; s >>= 1) {
+    const int c = __popc(m & ((1u << s) - 1u));
+    if (r >= c) { r -= c; m >>= s; pos += s; }
+  }
+  return pos;
+}
+
+// Lane that holds entry i, given every lane's inclusive count: the first lane whose count exceeds i.
+__device__ __forceinline__ int lane_of_entry(int i, int incl) {
+  int lane = 0;
+#pragma unroll
+  for (int s = 16; s; s >>= 1) {
+    const int c = __shfl_sync(0xFFFFFFFFu, incl, lane + s - 1);
+    if (i >= c) lane += s;
+  }
+  return lane;
+}
+
+// CSR: one warp per row, 32 mask words (1024 columns) at a time.  A round's values are stored in the next
+// round, so that their latency runs under its search.
 __global__ void __launch_bounds__(32 * FILL_WARPS)
 csr_fill_kernel(const uint32_t* __restrict__ mask, const __nv_bfloat16* __restrict__ x, int rows, int cols,
                 const float* __restrict__ thresholds, int thr_per_row, const int* __restrict__ rowptr, long long cap,
                 int* __restrict__ csr_col, float* __restrict__ csr_val) {
-  __shared__ uint16_t s_list[FILL_WARPS][CSR_LIST];
   const int row = blockIdx.x * FILL_WARPS + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= rows) return;
   int base = rowptr[row];
   if (rowptr[row + 1] == base) return;                // nothing clamped in this row
-  uint16_t* list = s_list[threadIdx.x >> 5];
   const int words = cols >> 5;
   const uint32_t* mrow = mask + (long long)row * words;
   const __nv_bfloat16* xrow = x + (long long)row * cols;
   const float lo = thresholds[thr_per_row ? 2 * row : 0], hi = thresholds[thr_per_row ? 2 * row + 1 : 1];
-  int n = 0;                                          // listed entries
-  int col0 = 0;                                       // list entries are columns less this (a multiple of 32768)
-  auto flush = [&]() {
-    __syncwarp();
-#pragma unroll 4
-    for (int i = lane; i < n; i += 32) {
-      const int col = col0 + list[i];
-      const float v = residual_of(xrow, col, lo, hi);
-      if (base + i < cap) {
-        csr_col[base + i] = col;
-        csr_val[base + i] = v;
-      }
+  int held_at = -1, held_col = 0;                     // the previous round's entry of this lane
+  __nv_bfloat16 held = __float2bfloat16(0.0f);
+  auto put = [&]() {
+    if (held_at >= 0 && held_at < cap) {
+      const float v = __bfloat162float(held);
+      csr_col[held_at] = held_col;
+      csr_val[held_at] = __fsub_rn(v, v > hi ? hi : lo);
     }
-    __syncwarp();
-    base += n;
-    n = 0;
   };
   uint32_t next = lane < words ? mrow[lane] : 0u;
   for (int w0 = 0; w0 < words; w0 += 32) {
-    uint32_t m = next;
+    const uint32_t m = next;
     next = w0 + 32 + lane < words ? mrow[w0 + 32 + lane] : 0u;
     const int c = __popc(m);
     const int incl = warp_inclusive_scan(c), total = __shfl_sync(0xFFFFFFFFu, incl, 31);
-    if (n + total > CSR_LIST || 32 * w0 - col0 >= 32768) {
-      flush();
-      col0 = (32 * w0) & ~32767;
+    for (int i0 = 0; i0 < total; i0 += 32) {
+      const int i = min(i0 + lane, total - 1);
+      const int src = lane_of_entry(i, incl);
+      const uint32_t word = __shfl_sync(0xFFFFFFFFu, m, src);
+      const int first = __shfl_sync(0xFFFFFFFFu, incl - c, src);
+      const int col = 32 * (w0 + src) + nth_set_bit(word, i - first);
+      put();
+      held_at = i0 + lane < total ? base + i : -1;
+      held_col = col;
+      held = xrow[col];
     }
-    int pos = n + incl - c;
-    const int rel = 32 * (w0 + lane) - col0;
-    while (m) {
-      const int b = __ffs(m) - 1;
-      m &= m - 1;
-      list[pos++] = uint16_t(rel + b);
-    }
-    n += total;
+    base += total;
   }
-  flush();
+  put();
 }
 
 // 32 x 32 bit transpose over a warp: bit c of lane r -> bit r of lane c.
@@ -1249,18 +1257,14 @@ __device__ __forceinline__ uint32_t transpose_bits(uint32_t v) {
 }
 
 // CSC: one warp per (64-row strip, 32-column word of the mask).  The word's two 32 x 32 blocks are
-// transposed, lane c then holds the marked rows of column c and lists them; a column with many of them
-// (an outlier channel) is listed by all lanes at once.
-constexpr int CSC_MANY = 8;
+// transposed: lane c holds the marked rows of column c.
 __global__ void __launch_bounds__(32 * FILL_WARPS)
 csc_fill_kernel(const uint32_t* __restrict__ mask, const __nv_bfloat16* __restrict__ x, int rows, int cols,
                 const float* __restrict__ thresholds, int thr_per_row, const int* __restrict__ colptr,
                 const uint8_t* __restrict__ strip_cnt, const int* __restrict__ super_cnt, long long cap,
                 int* __restrict__ csc_row, float* __restrict__ csc_val) {
-  __shared__ uint16_t s_list[FILL_WARPS][2048];
-  __shared__ int s_delta[FILL_WARPS][32];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int q = blockIdx.x * FILL_WARPS + warp, strip = blockIdx.y;
+  const int lane = threadIdx.x & 31;
+  const int q = blockIdx.x * FILL_WARPS + (threadIdx.x >> 5), strip = blockIdx.y;
   const int words_per_row = cols >> 5;
   if (q >= words_per_row) return;
   const int r0 = strip * ENC_TM;
@@ -1277,51 +1281,34 @@ csc_fill_kernel(const uint32_t* __restrict__ mask, const __nv_bfloat16* __restri
   for (int g = 0; g < SUPER - 1; ++g)
     if (sup * SUPER + g < strip) at += strip_cnt[(long long)(sup * SUPER + g) * cols + k];
   const uint32_t t0 = transpose_bits(w0), t1 = transpose_bits(w1);       // rows 0..31 / 32..63 of column `lane`
-  const int c = __popc(t0) + __popc(t1);
-  const int incl = warp_inclusive_scan(c);
-  const int n = __shfl_sync(0xFFFFFFFFu, incl, 31);
-  uint16_t* list = s_list[warp];
-  int pos = incl - c;
-  s_delta[warp][lane] = at - pos;                     // output position of list entry i of this column: i + delta
-  unsigned many = __ballot_sync(0xFFFFFFFFu, c > CSC_MANY);
-  if (c <= CSC_MANY) {
-    int p = pos;
-    uint32_t m = t0;
-    while (m) {
-      const int b = __ffs(m) - 1;
-      m &= m - 1;
-      list[p++] = uint16_t((lane << 6) | b);
-    }
-    m = t1;
-    while (m) {
-      const int b = __ffs(m) - 1;
-      m &= m - 1;
-      list[p++] = uint16_t((lane << 6) | 32 | b);
-    }
-  }
-  while (many) {
-    const int src = __ffs(many) - 1;
-    many &= many - 1;
-    const uint32_t m0 = __shfl_sync(0xFFFFFFFFu, t0, src), m1 = __shfl_sync(0xFFFFFFFFu, t1, src);
-    const int p = __shfl_sync(0xFFFFFFFFu, pos, src);
-    const uint32_t lt = (1u << lane) - 1u;
-    if ((m0 >> lane) & 1u) list[p + __popc(m0 & lt)] = uint16_t((src << 6) | lane);
-    if ((m1 >> lane) & 1u) list[p + __popc(m0) + __popc(m1 & lt)] = uint16_t((src << 6) | 32 | lane);
-  }
-  __syncwarp();
+  const int c0 = __popc(t0), c = c0 + __popc(t1);
+  const int incl = warp_inclusive_scan(c), total = __shfl_sync(0xFFFFFFFFu, incl, 31);
   const float lo = thresholds[0], hi = thresholds[1];
-#pragma unroll 4
-  for (int i = lane; i < n; i += 32) {
-    const int e = list[i], r = r0 + (e & 63), col = e >> 6;
-    const int to = i + s_delta[warp][col];
-    float l = lo, h = hi;
-    if (thr_per_row) { l = thresholds[2 * r]; h = thresholds[2 * r + 1]; }
-    const float v = residual_of(x, (long long)r * cols + 32 * q + col, l, h);
-    if (to < cap) {
-      csc_row[to] = r;
-      csc_val[to] = v;
+  int held_at = -1, held_row = 0;                     // the previous round's entry of this lane
+  __nv_bfloat16 held = __float2bfloat16(0.0f);
+  auto put = [&]() {
+    if (held_at >= 0 && held_at < cap) {
+      float l = lo, h = hi;
+      if (thr_per_row) { l = thresholds[2 * held_row]; h = thresholds[2 * held_row + 1]; }
+      const float v = __bfloat162float(held);
+      csc_row[held_at] = held_row;
+      csc_val[held_at] = __fsub_rn(v, v > h ? h : l);
     }
+  };
+  for (int i0 = 0; i0 < total; i0 += 32) {
+    const int i = min(i0 + lane, total - 1);
+    const int src = lane_of_entry(i, incl);
+    const uint32_t m0 = __shfl_sync(0xFFFFFFFFu, t0, src), m1 = __shfl_sync(0xFFFFFFFFu, t1, src);
+    const int n0 = __shfl_sync(0xFFFFFFFFu, c0, src), first = __shfl_sync(0xFFFFFFFFu, incl - c, src);
+    const int to = __shfl_sync(0xFFFFFFFFu, at, src);
+    const int j = i - first;                          // number of the entry inside its column
+    const int r = r0 + (j < n0 ? nth_set_bit(m0, j) : 32 + nth_set_bit(m1, j - n0));
+    put();
+    held_at = i0 + lane < total ? to + j : -1;
+    held_row = r;
+    held = x[(long long)r * cols + 32 * q + src];
   }
+  put();
 }
 
 // At most two blocks per SM, and as few as give no block more rows than that.  Small tensors (a block
@@ -1379,8 +1366,6 @@ Scratch carve(Arena& arena, int rows, int cols, bool occ) {
 // Once per device, before the first launch there.
 int quantize_setup() {
   FP4_CUDA_TRY(cudaFuncSetAttribute(tail_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SEL_DYN_SMEM));
-  // six blocks' lists side by side on an SM (the fills read nothing twice through L1)
-  FP4_CUDA_TRY(cudaFuncSetAttribute(csc_fill_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
   return FP4_OK;
 }
 
