@@ -111,24 +111,24 @@ struct Arena {
 
 // DGE derivative of Eq. 8 on a scaled weight, capped at `clip`.  The E2M1 grid has steps of 0.5
 // below 2, 1 on [2, 4) and 2 from 4 up, i.e. delta = 2^(max(e, 0) - 1) with e the binary exponent
-// of |w| (capped at the last interval, whose formula continues past 6).  With t = |w| / delta the
-// position inside the interval [g, g + delta], mapped to [-1, 1], is u = 2 (t - floor(t)) - 1.
-// Branch-free: the exponent arithmetic is done on the float's bit pattern.
-__device__ __forceinline__ float dge_factor(float ws, float expo, float inv_k, float clip) {
+// of |w| (capped at the last interval, whose formula continues past 6).  With g the interval's lower
+// end, the position inside it, mapped to [-1, 1], is u = (|w| - g) 2 / delta - 1, and the factor is
+// |u|^(1/k - 1) / k = 2^(expo log2 |u| + log2(1/k)).
+// Branch-free, 17 instructions (a fused epilogue evaluates it for every weight): delta and 2 / delta are
+// put together from the exponent bits; g comes from an addition of 2^23 delta rounded down (exact; floorf
+// would go to the pipe that also serves the two special functions).
+__device__ __forceinline__ float dge_factor(float ws, float expo, float log2_inv_k, float clip) {
   const float a = fabsf(ws);
-  int em = int(__float_as_uint(a) >> 23);
-  em = min(max(em, 127), 129);                                   // exponent 0, 1 or 2
-  const float inv_delta = __uint_as_float(uint32_t(255 - em) << 23);    // 2, 1 or 1/2
-  const float t = a * inv_delta;                                 // exact: a power of two
-  const float g = em == 129 ? 2.0f : floorf(t);                  // last interval starts at 4 = 2 delta
-  const float u = fabsf(fmaf(t - g, 2.0f, -1.0f));
-  // |u|^(1/k - 1) = 2^((1/k - 1) log2 |u|); u = 0 gives +inf, which the cap turns into `clip`
+  const uint32_t eb = min(max(__float_as_uint(a) & 0x7F800000u, 0x3F800000u), 0x40800000u);   // 1, 2 or 4
+  const float big = __uint_as_float(eb + (22u << 23));           // 2^23 delta
+  const float g = fminf(__fadd_rd(a, big) - big, 4.0f);          // the last interval starts at 4
+  const float u = fabsf(fmaf(a - g, __uint_as_float((256u << 23) - eb), -1.0f));
   // both special-function instructions as they are (2^-22 relative: far inside the tolerance of the
   // weight gradient): log2(0) = -inf, times the negative exponent +inf, 2^+inf = +inf, capped below
-  float p;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(p) : "f"(expo * __log2f(u)));
-  const float d = inv_k * p;
-  return fminf(d, clip);
+  float l, p;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l) : "f"(u));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(p) : "f"(fmaf(expo, l, log2_inv_k)));
+  return fminf(p, clip);
 }
 
 // Work fused into the epilogue of the weight-gradient GEMM (all null / zero: plain epilogue):

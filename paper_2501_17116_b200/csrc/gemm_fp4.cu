@@ -26,6 +26,8 @@
 // frees its tensor memory and returns.
 #include <cuda.h>
 
+#include <cmath>
+
 #include "common.cuh"
 #include "tc_ptx.cuh"
 
@@ -57,6 +59,7 @@ struct GemmArgs {
   int I, J;
   int num_k_blocks;
   int num_m_blocks, num_n_blocks;
+  int bn;                      // tile width: a multiple of 16, at most tile_n(kind)
   uint32_t tx_bytes;
   uint32_t idesc;              // instruction descriptor (operand formats differ per problem)
   float row_div, col_div;      // largest value of the row / column operand's format: 6 (E2M1) or 448 (E4M3)
@@ -68,9 +71,10 @@ struct GemmArgs {
   // fused weight-gradient epilogue (EPI_WGRAD)
   const float* addend;
   const int* slot_of_row;
-  const uint4* w;
+  const __nv_bfloat16* w;
+  bool w_aligned;              // `w` starts on a 32-byte boundary
   const float* w_amax;
-  float inv_k, expo, clip;
+  float log2_inv_k, expo, clip;
   // dense tail (single-problem launches only): after the FP4 k-blocks of a tile, 3 * ceil(*tail_count / 64)
   // k-blocks of 64 FP16 columns each from the maps that otherwise describe a second problem are
   // accumulated into the same tile with kind::f16 (null: no tail)
@@ -83,23 +87,20 @@ struct GemmArgs {
   int skip_fill;
 };
 
-// Instruction descriptors: M = 128, N = tile_n, both operands K-major, E2M1 x E2M1 -> fp32.
+// Instruction descriptors: M = 128, N = bn, both operands K-major, E2M1 x E2M1 -> fp32.
 // kind::f8f6f4 format fields: E4M3 = 0, E2M1 = 5
 // format field of the byte-container kind for an operand format of the C interface
 __host__ __device__ constexpr uint32_t f8f6f4_code(int format) {
   return format == FP4_FORMAT_E4M3 ? 0u : (format == FP4_FORMAT_E5M2 ? 1u : 5u);
 }
-__host__ __device__ constexpr uint32_t idesc_f8f6f4(int a_format = FP4_FORMAT_E2M1, int b_format = FP4_FORMAT_E2M1) {
-  return (1u << 4) | (f8f6f4_code(a_format) << 7) | (f8f6f4_code(b_format) << 10) |
-         (uint32_t(tile_n(FP4_GEMM_F8F6F4) >> 3) << 17) | (uint32_t(BM >> 4) << 24);
-}
-// kind::f16 with FP16 operands (format 0) and fp32 accumulators, M = 128, N = the kind's tile width
-__host__ __device__ constexpr uint32_t idesc_f16(int gemm_kind) {
-  return (1u << 4) | (uint32_t(tile_n(gemm_kind) >> 3) << 17) | (uint32_t(BM >> 4) << 24);
-}
-__host__ __device__ constexpr uint32_t idesc_mxf4() {
-  return (1u << 7) | (1u << 10) | (uint32_t(tile_n(FP4_GEMM_MXF4) >> 3) << 17) | (1u << 23) |
+constexpr uint32_t idesc_f8f6f4(int bn, int a_format, int b_format) {
+  return (1u << 4) | (f8f6f4_code(a_format) << 7) | (f8f6f4_code(b_format) << 10) | (uint32_t(bn >> 3) << 17) |
          (uint32_t(BM >> 4) << 24);
+}
+// kind::f16 with FP16 operands (format 0) and fp32 accumulators
+constexpr uint32_t idesc_f16(int bn) { return (1u << 4) | (uint32_t(bn >> 3) << 17) | (uint32_t(BM >> 4) << 24); }
+constexpr uint32_t idesc_mxf4(int bn) {
+  return (1u << 7) | (1u << 10) | (uint32_t(bn >> 3) << 17) | (1u << 23) | (uint32_t(BM >> 4) << 24);
 }
 
 // Where the bulk stores of the epilogue take their boxes from and how they are described.
@@ -180,15 +181,16 @@ __device__ __forceinline__ void descale_chunk(const uint32_t (&v)[32], float d_r
   }
 }
 
-// Plain epilogue of one 128 x BN block of accumulators for one warp (32 rows of it).  The warps
+// Plain epilogue of one 128 x bn block of accumulators for one warp (32 rows of it).  The warps
 // that share a lane quarter take the 32-column chunks in turn (`group` g of G: chunks g, g + G,
 // ...).  Chunks are read from tensor memory (the next one under the stores of the current one),
 // de-scaled and stored; `row_blk` is the index of the 128-row block.
-template <int BN, int G>
+template <int G>
 __device__ __forceinline__ void epilogue_tile_plain(const GemmArgs& args, int row_blk, int n_blk, uint32_t t_base,
                                                     float d_row, const float* dcol, uint8_t* stage, int quarter,
                                                     int group, int lane, const OutMaps& maps, uint32_t& seq) {
-  const int n_valid = min(BN, args.J - n_blk * BN);           // ragged last tile in N (multiple of 16)
+  const int n_col0 = n_blk * args.bn;
+  const int n_valid = min(args.bn, args.J - n_col0);          // ragged last tile in N (multiple of 16)
   const int row0 = row_blk * BM + quarter * 32;
   int c0 = 32 * group;
   if (c0 >= n_valid) return;
@@ -205,34 +207,45 @@ __device__ __forceinline__ void epilogue_tile_plain(const GemmArgs& args, int ro
       descale_chunk<32>(v, d_row, dcol + c0, y);
       if (next_width >= 32) tmem_ld_32x32(next_taddr, v);      // v is dead: fetch under the stores
       else if (next_width > 0) tmem_ld_32x16(next_taddr, v);
-      bulk_store_chunk<32, 2>(y, stage, args.out_f32, maps, row0, n_blk * BN + c0, lane, seq);
+      bulk_store_chunk<32, 2>(y, stage, args.out_f32, maps, row0, n_col0 + c0, lane, seq);
     } else {
       float y[16];
       descale_chunk<16>(v, d_row, dcol + c0, y);
-      bulk_store_chunk<16, 2>(y, stage, args.out_f32, maps, row0, n_blk * BN + c0, lane, seq);
+      bulk_store_chunk<16, 2>(y, stage, args.out_f32, maps, row0, n_col0 + c0, lane, seq);
     }
   }
 }
 
 // Operands of the fused weight-gradient epilogue for 16 columns of this thread's row: the BF16
 // weights that drive the DGE factor and the compensation row.  They are requested one chunk
-// ahead, right after the previous chunk's have been consumed.
+// ahead, right after the previous chunk's have been consumed, with 256-bit loads: a whole sector per
+// lane and request (as pairs of 128-bit loads the second one found its sector evicted every other time,
+// the kernel's shared memory leaves L1 a few KB).
 struct WgradOperands {
-  uint4 w[2];            // 16 BF16 weights
-  float4 add[4];         // 16 floats of the compensation row (zeros without one)
+  uint32_t w[8];         // 16 BF16 weights
+  float add[16];         // 16 floats of the compensation row (zeros without one)
 };
-__device__ __forceinline__ void wgrad_fetch(WgradOperands& op, const GemmArgs& args, int row, int slot, int col) {
-  if (args.w) {
-    const uint4* src = args.w + ((size_t(row) * size_t(args.J) + size_t(col)) >> 3);
-    op.w[0] = __ldg(src);
-    op.w[1] = __ldg(src + 1);
+__device__ __forceinline__ void ldg256(const void* p, uint32_t (&r)[8]) {
+  asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "l"(p));
+}
+__device__ __forceinline__ void wgrad_fetch(WgradOperands& op, const __nv_bfloat16* w, bool w_aligned, const float* add) {
+  if (w && w_aligned) {
+    ldg256(w, op.w);
+  } else if (w) {                                    // the caller's weights start on a 16-byte boundary only
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const uint4 q = __ldg(reinterpret_cast<const uint4*>(w) + h);
+      op.w[4 * h] = q.x; op.w[4 * h + 1] = q.y; op.w[4 * h + 2] = q.z; op.w[4 * h + 3] = q.w;
+    }
   }
 #pragma unroll
-  for (int j = 0; j < 4; ++j) op.add[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (slot >= 0) {
-    const float4* src = reinterpret_cast<const float4*>(args.addend + size_t(slot) * size_t(args.J) + size_t(col));
+  for (int h = 0; h < 2; ++h) {
+    uint32_t r[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    if (add) ldg256(add + 8 * h, r);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) op.add[j] = __ldg(src + j);
+    for (int j = 0; j < 8; ++j) op.add[8 * h + j] = __uint_as_float(r[j]);
   }
 }
 
@@ -240,14 +253,17 @@ __device__ __forceinline__ void wgrad_fetch(WgradOperands& op, const GemmArgs& a
 //   out[k, n] = store( (acc * d_col[n] + addend[slot[k], n]) * Q'(w[k, n] * 6 / w_amax[n]) ).
 // The thread-per-row layout of tensor memory is kept throughout: the weights and the
 // compensation row are read as whole 32-byte sectors per thread, the results leave through a
-// bulk store.  `first` holds the operands of the warp's first chunk, requested by the caller
+// bulk store.  `w` and `add` point to the row's weights and compensation at the tile's first column (null
+// without), `op` holds the operands of the warp's first chunk, requested by the caller
 // before the accumulators were awaited.
-template <int BN, int G>
+template <int G>
 __device__ __forceinline__ void epilogue_tile_wgrad(const GemmArgs& args, int row_blk, int n_blk, uint32_t t_base,
-                                                    float d_row, const float* dcol, const float* gcol, int slot,
+                                                    float d_row, const float* dcol, const float* gcol,
+                                                    const __nv_bfloat16* w, const float* add,
                                                     uint8_t* stage, int quarter, int group, int lane,
                                                     const OutMaps& maps, uint32_t& seq, WgradOperands& op) {
-  const int n_valid = min(BN, args.J - n_blk * BN);
+  const int n_col0 = n_blk * args.bn;
+  const int n_valid = min(args.bn, args.J - n_col0);
   const int row0 = row_blk * BM + quarter * 32;
   int c0 = 16 * group;
   if (c0 >= n_valid) return;
@@ -255,17 +271,14 @@ __device__ __forceinline__ void epilogue_tile_wgrad(const GemmArgs& args, int ro
   tmem_ld_32x16(t_base + uint32_t(c0), v);
 #pragma unroll 1
   for (; c0 < n_valid; c0 += 16 * G) {
-    const bool more = c0 + 16 * G < n_valid;
+    const int next = c0 + 16 * G;
     tmem_ld_wait();
     float y[16];
     descale_chunk<16>(v, d_row, dcol + c0, y);
-    if (more) tmem_ld_32x16(t_base + uint32_t(c0 + 16 * G), v);
+    if (next < n_valid) tmem_ld_32x16(t_base + uint32_t(next), v);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      y[4 * j + 0] += op.add[j].x; y[4 * j + 1] += op.add[j].y; y[4 * j + 2] += op.add[j].z; y[4 * j + 3] += op.add[j].w;
-    }
-    if (args.w) {
-      const uint32_t ww[8] = {op.w[0].x, op.w[0].y, op.w[0].z, op.w[0].w, op.w[1].x, op.w[1].y, op.w[1].z, op.w[1].w};
+    for (int j = 0; j < 16; ++j) y[j] += op.add[j];
+    if (w) {
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const float4 g4 = *reinterpret_cast<const float4*>(gcol + c0 + 4 * q);   // same address in every lane
@@ -273,13 +286,13 @@ __device__ __forceinline__ void epilogue_tile_wgrad(const GemmArgs& args, int ro
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const int c = 4 * q + e;
-          const float wf = __uint_as_float((c & 1) ? (ww[c >> 1] & 0xFFFF0000u) : (ww[c >> 1] << 16));
-          y[c] *= dge_factor(__fmul_rn(wf, g[e]), args.expo, args.inv_k, args.clip);
+          const float wf = __uint_as_float((c & 1) ? (op.w[c >> 1] & 0xFFFF0000u) : (op.w[c >> 1] << 16));
+          y[c] *= dge_factor(__fmul_rn(wf, g[e]), args.expo, args.log2_inv_k, args.clip);
         }
       }
     }
-    if (more) wgrad_fetch(op, args, row0 + lane, slot, n_blk * BN + c0 + 16 * G);
-    bulk_store_chunk<16, 1>(y, stage, args.out_f32, maps, row0, n_blk * BN + c0, lane, seq);
+    if (next < n_valid) wgrad_fetch(op, w ? w + next : nullptr, args.w_aligned, add ? add + next : nullptr);
+    bulk_store_chunk<16, 1>(y, stage, args.out_f32, maps, row0, n_col0 + c0, lane, seq);
   }
 }
 
@@ -292,7 +305,6 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
                 const __grid_constant__ CUtensorMap map_out_aux2, const __grid_constant__ GemmArgs args2) {
   constexpr int NACC = 2;
   constexpr int STAGES = stages_of(KIND);
-  constexpr int BN = tile_n(KIND);
   constexpr int B_STAGE_BYTES = b_stage_bytes(KIND);
   constexpr int STAGE_BYTES = stage_bytes(KIND);
   extern __shared__ uint8_t smem_raw[];
@@ -311,7 +323,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   float* s_dcol = reinterpret_cast<float*>(smem_misc + 256);                     // [2][256] column de-scales
   float* s_gcol = s_dcol + 2 * 256;                                              // [2][256] 6 / w_amax (DGE)
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = __shfl_sync(0xFFFFFFFFu, int(threadIdx.x >> 5), 0);    // known to be the same in all lanes
   const int lane = threadIdx.x & 31;
   // Two problems may share one launch (args2 with no tiles: one problem): the tiles of the first
   // come first, then those of the second, so that the epilogue of one problem's last tiles runs
@@ -319,7 +331,11 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   const int tiles_first = args.num_m_blocks * args.num_n_blocks;
   const int num_tiles = tiles_first + args2.num_m_blocks * args2.num_n_blocks;
 
-  int pre = 0;          // thread 0: k-blocks of its first tile already requested (see below)
+  int pre = 0;          // k-blocks of the first tile that thread 0 has requested already (see below)
+  if (int(blockIdx.x) < num_tiles) {
+    const int kbs = int(blockIdx.x) >= tiles_first ? args2.num_k_blocks : args.num_k_blocks;
+    pre = kbs < STAGES ? kbs : STAGES;
+  }
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(&full_bar[s], 1);
@@ -343,11 +359,10 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       const CUtensorMap* mb = second ? &map_b2 : &map_b;
       const int tt = second ? int(blockIdx.x) - tiles_first : int(blockIdx.x);
       const int m_blk = tt % pa.num_m_blocks, n_blk = tt / pa.num_m_blocks;
-      pre = pa.num_k_blocks < STAGES ? pa.num_k_blocks : STAGES;
       for (int kb = 0; kb < pre; ++kb) {
         mbar_arrive_expect_tx(&full_bar[kb], pa.tx_bytes);
         tma_load_2d(smem_a + kb * A_STAGE_BYTES, ma, &full_bar[kb], kb * 128, m_blk * BM);
-        tma_load_2d(smem_b + kb * B_STAGE_BYTES, mb, &full_bar[kb], kb * 128, n_blk * BN);
+        tma_load_2d(smem_b + kb * B_STAGE_BYTES, mb, &full_bar[kb], kb * 128, n_blk * pa.bn);
       }
     }
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_out) : "memory");
@@ -387,7 +402,10 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer -------
-    if (lane == 0) {
+    // One elected lane runs the loop, here and in the issuer's.  It has to be elect.sync that picks the lane:
+    // behind `lane == 0` the compiler does not take the code for single-threaded, and a k-block of four MMAs
+    // took 0.33 us to issue whatever its size (0.22 now; 8192 x 7680 x 8192: 178 -> 168 us).
+    if (elect_one()) {
       int stage = pre == STAGES ? 0 : pre;
       uint32_t phase = pre == STAGES ? 1u : 0u;
       uint32_t fills = uint32_t(pre);
@@ -407,7 +425,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           if (blockIdx.x != 0 || int(fills) != args.skip_fill) {      // a left-out fill: no copy, no arrival
             mbar_arrive_expect_tx(&full_bar[stage], pa.tx_bytes);
             tma_load_2d(smem_a + stage * A_STAGE_BYTES, ma, &full_bar[stage], kb * 128, m_blk * BM);
-            tma_load_2d(smem_b + stage * B_STAGE_BYTES, mb, &full_bar[stage], kb * 128, n_blk * BN);
+            tma_load_2d(smem_b + stage * B_STAGE_BYTES, mb, &full_bar[stage], kb * 128, n_blk * pa.bn);
           }
           ++fills;
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
@@ -417,7 +435,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           if (!ok) break;
           mbar_arrive_expect_tx(&full_bar[stage], args.tail_tx_bytes);
           tma_load_2d(smem_a + stage * A_STAGE_BYTES, &map_a2, &full_bar[stage], kb * 64, m_blk * BM);
-          tma_load_2d(smem_b + stage * B_STAGE_BYTES, &map_b2, &full_bar[stage], kb * 64, n_blk * BN);
+          tma_load_2d(smem_b + stage * B_STAGE_BYTES, &map_b2, &full_bar[stage], kb * 64, n_blk * args.bn);
           ++fills;
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
@@ -436,7 +454,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer ---------
-    if (lane == 0) {
+    if (elect_one()) {
       int stage = 0;
       uint32_t phase = 0;
       int acc = 0;
@@ -503,7 +521,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     const int quarter = warp & 3;               // the lane quarter of tensor memory this warp may read
     const int group = (warp - 2) >> 2;          // which of the G warps of this quarter
     const int et = threadIdx.x - 64;            // index among the epilogue threads
-    uint8_t* stage = s_out + (warp - 2) * (STAGE_OUT_BYTES / EW);
+    uint8_t* stage = s_out + (warp - 2) * (EPI == EPI_WGRAD ? 2048 : 4096);
     int acc = 0;
     uint32_t acc_phase = 0;
     uint32_t tile_parity = 0;
@@ -520,29 +538,35 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       const float d_row = pa.row_amax ? __fdiv_rn(__ldg(&pa.row_amax[row]), pa.row_div) : 1.0f;
       float* dcol = s_dcol + tile_parity * 256;
       float* gcol = s_gcol + tile_parity * 256;
-      for (int c = et; c < BN; c += 32 * EW) {
-        const int col = n_blk * BN + c;
+      for (int c = et; c < pa.bn; c += 32 * EW) {
+        const int col = n_blk * pa.bn + c;
         dcol[c] = (pa.col_amax && col < pa.J) ? __fdiv_rn(__ldg(&pa.col_amax[col]), pa.col_div) : 1.0f;
         if (EPI == EPI_WGRAD && pa.w) {
           const float am = col < pa.J ? __ldg(&pa.w_amax[col]) : 0.0f;
           gcol[c] = am > 0.0f ? __fdiv_rn(6.0f, am) : 0.0f;
         }
       }
-      int slot = -1;
+      const __nv_bfloat16* w_row = nullptr;
+      const float* add_row = nullptr;
       WgradOperands op;
       if (EPI == EPI_WGRAD) {
-        if (pa.slot_of_row) slot = __ldg(&pa.slot_of_row[row]);
-        if (n_blk * BN + 16 * group < pa.J) wgrad_fetch(op, pa, row, slot, n_blk * BN + 16 * group);
+        if (pa.w) w_row = pa.w + size_t(row) * size_t(pa.J) + size_t(n_blk * pa.bn);
+        if (pa.slot_of_row) {
+          const int slot = __ldg(&pa.slot_of_row[row]);
+          if (slot >= 0) add_row = pa.addend + size_t(slot) * size_t(pa.J) + size_t(n_blk * pa.bn);
+        }
+        if (16 * group < pa.bn && n_blk * pa.bn + 16 * group < pa.J)
+          wgrad_fetch(op, w_row ? w_row + 16 * group : nullptr, pa.w_aligned, add_row ? add_row + 16 * group : nullptr);
       }
       const bool ok = mbar_wait(&acc_full[acc], acc_phase, abort_flag, args.status, args.wait_limit_ns);
       if (epilogue_bar_any(!ok, 32 * EW)) break;   // also publishes dcol to the other warps
       tc_fence_after();
       const uint32_t t_base = tmem_base + (uint32_t(quarter * 32) << 16) + uint32_t(acc * ACC_STRIDE);
       if (EPI == EPI_WGRAD)
-        epilogue_tile_wgrad<BN, G>(pa, m_blk, n_blk, t_base, d_row, dcol, gcol, slot, stage, quarter, group, lane,
+        epilogue_tile_wgrad<G>(pa, m_blk, n_blk, t_base, d_row, dcol, gcol, w_row, add_row, stage, quarter, group, lane,
                                    out_maps, store_seq, op);
       else
-        epilogue_tile_plain<BN, G>(pa, m_blk, n_blk, t_base, d_row, dcol, stage, quarter, group, lane, out_maps,
+        epilogue_tile_plain<G>(pa, m_blk, n_blk, t_base, d_row, dcol, stage, quarter, group, lane, out_maps,
                                    store_seq);
       tc_fence_before();
       __syncwarp();
@@ -654,8 +678,63 @@ int launch_kernel(int grid, cudaStream_t stream, const Problem& p, const Problem
   return FP4_OK;
 }
 
+// Tile widths of a launch's problems (each a multiple of 16): the ones for which the CTA with the most work
+// ends soonest, under a model of the kernel.  Narrow tiles spread a small GEMM over all SMs and shorten the
+// epilogue that nothing hides; wide ones move fewer operand bytes per flop, so that they win as soon as
+// there are a few rounds.  The constants (ns) were fitted to sweeps of the width over 29 launches, in 27 of
+// which the choice is within 1.5 % of the best width: a tile costs 800, a k-block 170 + 0.85 per column, an
+// epilogue 10 per column (12 with fp32 outputs), with the fused weight gradient 500 + 40 per column.
+// Measured: 128 x 11008 x 4096 (width 80 instead of 240) 9.5 -> 7.1 us, 1024^3 (64) 6.2 -> 4.9, backward of
+// 256 x 1024 x 1024 (64 and 144) 12.0 -> 6.2.
+struct TileWidths {
+  int first, second;
+};
+struct TileCost {
+  long long tiles;
+  int steady, alone;           // time per tile in a row of tiles; what the last one adds
+};
+TileCost tile_cost(const Fp4GemmDesc& d, int gemm_kind, int bn) {
+  const int per_stage = gemm_kind == FP4_GEMM_F8F6F4 ? 128 : 256;
+  const int kbs = int((d.C + per_stage - 1) / per_stage);
+  const int mma = 800 + kbs * (170 + (17 * bn) / 20);
+  const bool dge = d.epilogue && d.epilogue->w_bf16;
+  const int epi = dge ? 500 + 40 * bn : (d.out_f32 ? 12 : 10) * bn;
+  return {(d.I / BM) * ((d.J + bn - 1) / bn), mma > epi ? mma : epi, mma > epi ? epi : mma};
+}
+TileWidths choose_bn(const fp4_ctx* ctx, const Fp4GemmDesc& p, const Fp4GemmDesc* q, int gemm_kind) {
+  constexpr int LEAST = 32, WIDTHS = 15;
+  const int most = tile_n(gemm_kind);
+  TileCost costs[2][WIDTHS];
+  int n = 0;
+  for (int bn = most; bn >= LEAST; bn -= 16, ++n) {
+    costs[0][n] = tile_cost(p, gemm_kind, bn);
+    costs[1][n] = q ? tile_cost(*q, gemm_kind, bn) : TileCost{0, 0, 0};
+  }
+  TileWidths best = {most, most};
+  long long best_cost = -1;
+  const long long G = ctx->num_sms;
+  for (int i = 0; i < n; ++i)
+    for (int j = 0; j < (q ? n : 1); ++j) {
+      const TileCost &c = costs[0][i], &d = costs[1][j];
+      // CTA r takes tiles r, r + G, ...: the counts change at r = tiles mod G of the first problem and of both
+      const long long all = c.tiles + d.tiles;
+      const long long at[3] = {0, c.tiles % G, all % G};
+      long long cost = 0;
+      for (const long long r : at) {
+        const long long n1 = (c.tiles - r + G - 1) / G, n2 = (all - r + G - 1) / G - n1;
+        const long long t = n1 * c.steady + n2 * d.steady + (n2 ? d.alone : n1 ? c.alone : 0);
+        if (t > cost) cost = t;
+      }
+      if (best_cost < 0 || cost < best_cost) {
+        best_cost = cost;
+        best = {most - 16 * i, q ? most - 16 * j : most};
+      }
+    }
+  return best;
+}
+
 // Tensor maps and arguments of one GEMM.
-int make_problem(fp4_ctx* ctx, Problem* p, const Fp4GemmDesc& d, int gemm_kind, int32_t* status) {
+int make_problem(fp4_ctx* ctx, Problem* p, const Fp4GemmDesc& d, int gemm_kind, int bn, int32_t* status) {
   if (gemm_kind != FP4_GEMM_MXF4 && gemm_kind != FP4_GEMM_F8F6F4) return FP4_ERR_ARG;
   const bool a8 = d.a_format != FP4_FORMAT_E2M1, b8 = d.b_format != FP4_FORMAT_E2M1;   // FP8 bytes
   if ((a8 || b8) && gemm_kind != FP4_GEMM_F8F6F4) return FP4_ERR_ARG;   // FP8 operands need the byte-container kind
@@ -666,8 +745,7 @@ int make_problem(fp4_ctx* ctx, Problem* p, const Fp4GemmDesc& d, int gemm_kind, 
     return FP4_ERR_ALIGN;
   int rc = make_codes_map(ctx, &p->map_a, d.a_codes, d.I, d.C, BM, gemm_kind, a8);
   if (rc != FP4_OK) return rc;
-  const int BN = tile_n(gemm_kind);
-  rc = make_codes_map(ctx, &p->map_b, d.b_codes, d.J, d.C, BN, gemm_kind, b8);
+  rc = make_codes_map(ctx, &p->map_b, d.b_codes, d.J, d.C, bn, gemm_kind, b8);
   if (rc != FP4_OK) return rc;
   if (reinterpret_cast<uintptr_t>(d.out) & 15) return FP4_ERR_ALIGN;
   rc = make_out_maps(ctx, &p->map_out, &p->map_out_aux, d.out, d.I, d.J, d.out_f32);
@@ -679,14 +757,15 @@ int make_problem(fp4_ctx* ctx, Problem* p, const Fp4GemmDesc& d, int gemm_kind, 
   const int k_per_stage = gemm_kind == FP4_GEMM_F8F6F4 ? 128 : 256;   // elements per 128-byte row
   args.num_k_blocks = int((d.C + k_per_stage - 1) / k_per_stage);
   args.num_m_blocks = int(d.I / BM);
-  args.num_n_blocks = int((d.J + BN - 1) / BN);
+  args.bn = bn;
+  args.num_n_blocks = int((d.J + bn - 1) / bn);
   // The transaction count of a copy is in bytes read from global memory: the byte-container form
   // fills a stage's 128-byte rows from 64 bytes of packed nibbles (E2M1) or from 128 bytes (E4M3).
   if (gemm_kind == FP4_GEMM_F8F6F4)
-    args.tx_bytes = uint32_t(A_STAGE_BYTES / (a8 ? 1 : 2) + b_stage_bytes(gemm_kind) / (b8 ? 1 : 2));
+    args.tx_bytes = uint32_t(A_STAGE_BYTES / (a8 ? 1 : 2) + 128 * bn / (b8 ? 1 : 2));
   else
-    args.tx_bytes = stage_bytes(gemm_kind);
-  args.idesc = gemm_kind == FP4_GEMM_F8F6F4 ? idesc_f8f6f4(d.a_format, d.b_format) : idesc_mxf4();
+    args.tx_bytes = uint32_t(A_STAGE_BYTES + 128 * bn);
+  args.idesc = gemm_kind == FP4_GEMM_F8F6F4 ? idesc_f8f6f4(bn, d.a_format, d.b_format) : idesc_mxf4(bn);
   args.row_div = fp8_max(d.a_format);
   args.col_div = fp8_max(d.b_format);
   args.row_amax = d.row_amax;
@@ -699,16 +778,18 @@ int make_problem(fp4_ctx* ctx, Problem* p, const Fp4GemmDesc& d, int gemm_kind, 
   p->fused = fused;
   args.addend = fused ? epi->addend : nullptr;
   args.slot_of_row = fused && epi->addend ? epi->slot_of_row : nullptr;
-  args.w = fused ? static_cast<const uint4*>(epi->w_bf16) : nullptr;
+  args.w = fused ? static_cast<const __nv_bfloat16*>(epi->w_bf16) : nullptr;
+  args.w_aligned = !(reinterpret_cast<uintptr_t>(args.w) & 31);
   args.w_amax = fused ? epi->w_amax : nullptr;
-  args.inv_k = fused && epi->w_bf16 ? 1.0f / epi->dge_k : 1.0f;
-  args.expo = args.inv_k - 1.0f;
+  const float inv_k = fused && epi->w_bf16 ? 1.0f / epi->dge_k : 1.0f;
+  args.log2_inv_k = std::log2(inv_k);
+  args.expo = inv_k - 1.0f;
   args.clip = fused ? epi->dge_clip : 0.0f;
   args.wait_limit_ns = ctx->debug_wait_limit_ns ? ctx->debug_wait_limit_ns : WAIT_LIMIT_NS;
   args.skip_fill = ctx->debug_skip_fill;
   args.tail_count = nullptr;
-  args.tail_tx_bytes = uint32_t(A_STAGE_BYTES + b_stage_bytes(gemm_kind));
-  args.tail_idesc = idesc_f16(gemm_kind);
+  args.tail_tx_bytes = uint32_t(A_STAGE_BYTES + 128 * bn);
+  args.tail_idesc = idesc_f16(bn);
   return FP4_OK;
 }
 
@@ -722,7 +803,8 @@ int launch_gemm_fp4(fp4_ctx* ctx, cudaStream_t stream, const uint8_t* a_codes, c
   d.a_format = a_format;
   d.b_format = b_format;
   Problem p;
-  int rc = make_problem(ctx, &p, d, gemm_kind, status);
+  const int bn = choose_bn(ctx, d, nullptr, gemm_kind).first;
+  int rc = make_problem(ctx, &p, d, gemm_kind, bn, status);
   if (rc != FP4_OK) return rc;
   // The dense tail's operands travel in the slots of a second problem that has no tiles.
   Problem with_tail;
@@ -731,7 +813,7 @@ int launch_gemm_fp4(fp4_ctx* ctx, cudaStream_t stream, const uint8_t* a_codes, c
     with_tail.args.num_m_blocks = with_tail.args.num_n_blocks = 0;
     rc = make_tail_map(ctx, &with_tail.map_a, tail->a, I, BM);
     if (rc != FP4_OK) return rc;
-    rc = make_tail_map(ctx, &with_tail.map_b, tail->b, J, tile_n(gemm_kind));
+    rc = make_tail_map(ctx, &with_tail.map_b, tail->b, J, bn);
     if (rc != FP4_OK) return rc;
     p.args.tail_count = tail->count;
   }
@@ -757,9 +839,10 @@ int launch_gemm_fp4(fp4_ctx* ctx, cudaStream_t stream, const uint8_t* a_codes, c
 int launch_gemm_fp4_two(fp4_ctx* ctx, cudaStream_t stream, const Fp4GemmDesc& first, const Fp4GemmDesc& second,
                         int gemm_kind, int32_t* status) {
   Problem p, q;
-  int rc = make_problem(ctx, &p, first, gemm_kind, status);
+  const TileWidths bn = choose_bn(ctx, first, &second, gemm_kind);
+  int rc = make_problem(ctx, &p, first, gemm_kind, bn.first, status);
   if (rc != FP4_OK) return rc;
-  rc = make_problem(ctx, &q, second, gemm_kind, status);
+  rc = make_problem(ctx, &q, second, gemm_kind, bn.second, status);
   if (rc != FP4_OK) return rc;
   const int tiles = p.args.num_m_blocks * p.args.num_n_blocks + q.args.num_m_blocks * q.args.num_n_blocks;
   const int grid = tiles < ctx->num_sms ? tiles : ctx->num_sms;

@@ -125,7 +125,7 @@ comp_wgrad_dense_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __g
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(final_bar + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xFFFFFFFFu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int tile = blockIdx.x % args.tiles, split = blockIdx.x / args.tiles;
   const int chunks_total = (args.M + DT_CHUNK - 1) / DT_CHUNK;
   const int c_begin = int((long long)chunks_total * split / args.splits);
@@ -161,7 +161,7 @@ comp_wgrad_dense_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __g
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer -------
-    if (lane == 0) {
+    if (elect_one()) {                            // (see the FP4 GEMM)
       int stage = 0;
       uint32_t phase = 0, fills = 0;
       bool ok = true;
@@ -194,7 +194,7 @@ comp_wgrad_dense_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __g
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer ---------
-    if (lane == 0) {
+    if (elect_one()) {                            // (see the FP4 GEMM)
       int stage = 0;
       uint32_t phase = 0;
       int acc = 0;

@@ -48,6 +48,22 @@ def test_accumulators_are_exact(lib, ctx, kind, shape):
 
 
 @pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("shape", [(128, 1024, 512), (128, 11008, 256), (1024, 1024, 128), (512, 5120, 128), (2304, 1408, 256),
+                                   (1152, 3200, 384), (640, 13824, 128), (2048, 2048, 256)])
+@pytest.mark.parametrize("f32", [True, False])
+def test_tile_widths(lib, ctx, kind, shape, f32):
+    """Shapes for which the launch picks tiles of 32 to 256 columns, most with a ragged last tile: fp32 exact,
+    BF16 the rounding of the exact sum."""
+    I, J, C = shape
+    rng = np.random.default_rng(I + J + C)
+    ca, cb = _codes(rng, I, C), _codes(rng, J, C)
+    got = _run(lib, ctx, ca, cb, kind, out_f32=f32).cpu()
+    val = torch.tensor([0, .5, 1, 1.5, 2, 3, 4, 6, 0, -.5, -1, -1.5, -2, -3, -4, -6], dtype=torch.float64)
+    want = val[torch.from_numpy(ca.astype(np.int64))] @ val[torch.from_numpy(cb.astype(np.int64))].T      # exact in double
+    assert torch.equal(got, want.float() if f32 else want.to(torch.bfloat16))
+
+
+@pytest.mark.parametrize("kind", KINDS)
 def test_extreme_codes_long_contraction(lib, ctx, kind):
     """All +-6 operands over the longest contraction of the workloads (16384): |acc| up to 589824."""
     rng = np.random.default_rng(5)

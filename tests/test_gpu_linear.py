@@ -400,3 +400,20 @@ def test_tensor_core_accumulation_stays_inside_its_floor(lib, ctx):
     # entries added per entry in fp32 (the scattered ones) get the ordinary summation bound on top
     allow_w += 64 * ulp * mags_w * b.dge
     assert (err_w <= allow_w).all(), f"weight gradient: {np.max(err_w / (TAIL_FLOOR * mags_w * b.dge + 1e-300)):.3f} of the floor"
+
+
+@pytest.mark.parametrize("M,K,N", [(128, 128, 128), (256, 1024, 1024), (640, 512, 1408)])
+def test_weights_on_a_16_byte_boundary(lib, M, K, N):
+    """The ABI asks for 16-byte alignment; the fused epilogue reads weights on a 32-byte boundary with wider loads."""
+    a, w, dy = (torch.from_numpy(b.view(np.int16)).cuda().view(torch.bfloat16) for b in WL.small_case(M, K, N, seed=9))
+    moved = torch.empty(K * N + 8, dtype=torch.bfloat16, device="cuda")[8:].view(K, N)
+    moved.copy_(w)
+    assert w.data_ptr() % 32 == 0 and moved.data_ptr() % 32 == 16
+    ctx = lib.Context.for_shape(M, K, N)
+    _, sa, sw = lib.fp4_linear_fwd(ctx, a, w, 0.99)
+    want = lib.fp4_linear_bwd(ctx, dy, w, sa, sw)
+    got = lib.fp4_linear_bwd(ctx, dy, moved, sa, sw)
+    torch.cuda.synchronize()
+    assert ctx.read_status() == 0
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+    ctx.close()
