@@ -108,13 +108,12 @@ int fp4_create(fp4_ctx** out, int device, size_t workspace_bytes) {
   for (auto& e : ctx->host_step_computed) e = nullptr;
   ctx->host_step_parity = 0;
   ctx->quantile_mode = FP4_QUANTILE_SIGNED;
-  cudaDeviceProp prop;
-  if (!ctx->records || cudaGetDeviceProperties(&prop, device) != cudaSuccess) {
+  // (one attribute: cudaGetDeviceProperties takes 3 ms)
+  if (!ctx->records || cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
     delete ctx->records;
     delete ctx;
     return FP4_ERR_CUDA;
   }
-  ctx->num_sms = prop.multiProcessorCount;
   cudaDriverEntryPointQueryResult qres;
   void* fn = nullptr;
   if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) != cudaSuccess ||
