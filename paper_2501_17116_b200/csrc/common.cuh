@@ -43,7 +43,7 @@ struct fp4_ctx {
   void*    encode_tiled;       // cuTensorMapEncodeTiled, fetched through the runtime
   uint32_t* occ_hist;          // quantile selection: two sets of global counters, parity, ticket
   cudaStream_t side[2];        // side streams for independent kernel chains inside one call
-  cudaEvent_t  ev[8];          // fork / join events of those chains
+  cudaEvent_t  ev[10];          // fork / join events of those chains
   // fp4_linear_step_host, pipelined over consecutive calls:
   cudaStream_t copy_stream;          // host-to-device copies of a call's inputs
   cudaStream_t compute_stream;       // its kernels
@@ -132,10 +132,10 @@ __device__ __forceinline__ float dge_factor(float ws, float expo, float log2_inv
 }
 
 // Work fused into the epilogue of the weight-gradient GEMM (all null / zero: plain epilogue):
-//   out[k, n] = store( (acc * d_col[n] + addend[slot_of_row[k], n]) * Q'(w[k, n] * 6 / w_amax[n]) )
+//   out[k, n] = store( (acc * d_col[n] + addend[k, n]) * Q'(w[k, n] * 6 / w_amax[n]) )
 struct GemmEpilogue {
-  const float* addend;        // compact [slots x J] fp32 rows, added before the DGE factor (or null)
-  const int*   slot_of_row;   // [I]: row of `addend` that belongs to output row i, -1 for none
+  const float* addend;        // [I x J] fp32, added before the DGE factor (or null)
+  const int*   slot_of_row;   // [I]: negative where `addend` has no row
   const void*  w_bf16;        // [I x J] BF16 weights whose scaled values drive the DGE factor (or null)
   const float* w_amax;        // [J]
   float dge_k, dge_clip;
@@ -206,7 +206,22 @@ struct SparseOverlap {
   cudaStream_t stream_csc;
   cudaEvent_t csc_done;
   cudaEvent_t colptr_done;    // csr_rowptr and csc_colptr are complete (or null: the CSC fill stays on `stream`)
+  struct CscFill* later;      // not null: the CSC fill is described here instead, for launch_csc_fill
 };
+struct CscFill {
+  const uint32_t* mask;
+  const void* x_bf16;
+  int rows, cols;
+  const float* thresholds;
+  int thr_per_row;
+  const int* colptr;
+  const uint8_t* strip_cnt;
+  const int* super_cnt;
+  long long cap;
+  int* csc_row;
+  float* csc_val;
+};
+int launch_csc_fill(fp4_ctx* ctx, cudaStream_t stream, const CscFill& f);
 
 // Quantiser pieces (quantize.cu)
 // `prescale_div` > 0: the prescale vector holds amax values and stands for amax / prescale_div (6 for an
@@ -240,12 +255,18 @@ size_t fwd_tail_scratch_bytes(int64_t M, int64_t K, int64_t N);
 int launch_fwd_tail(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, const void* w_bf16, const float* w_amax,
                     float w_div, Arena& scratch, int64_t M, int64_t K, int64_t N, GemmTail* tail,
                     const int** slot_of_col_out, const void** kept_out, const int** kept_end_out);
-// Weight-gradient compensation into a compact buffer: for every column k of the residual that
-// holds entries, comp[slot_of_col[k], :] = sum_{entries of column k} val * dy[row, :].
+// Weight-gradient compensation: for every column k of the residual that holds entries (slot_of_col[k] >= 0),
+// comp[k, :] = sum_{entries of column k} val * dy[row, :]; the other rows of `comp` are not written.
 // Lists, slots and the dense path's buffers are carved from `scratch` (comp_wgrad_scratch_bytes); the slot
-// vector is handed back for the GEMM's epilogue.  `a` is the saved activation (CSC; CSR for the dense path).
+// vector is handed back for the GEMM's epilogue.  `a` is the saved activation (its CSC).
+// With `overlap` the long columns run on `overlap->stream`, from `classified` to `long_done`.
+struct CompOverlap {
+  cudaStream_t stream;
+  cudaEvent_t classified, long_done;
+};
 int launch_comp_wgrad(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, const void* dy_bf16, Arena& scratch,
-                      int** slot_of_col_out, float* comp, int64_t M, int64_t K, int64_t N, int32_t* status);
+                      int** slot_of_col_out, float* comp, int64_t M, int64_t K, int64_t N, int32_t* status,
+                      const CompOverlap* overlap = nullptr);
 size_t comp_wgrad_scratch_bytes(int64_t M, int64_t K, int64_t N);
 
 // Dense columns of the residual in the weight gradient, on the tensor cores (wgrad_dense_tc.cu):
@@ -255,7 +276,7 @@ size_t comp_wgrad_scratch_bytes(int64_t M, int64_t K, int64_t N);
 constexpr int DENSE_TC_MAX = 128;
 int dense_tc_splits(const fp4_ctx* ctx, int64_t M, int64_t N);
 size_t dense_tc_scratch_bytes(int64_t M, int64_t N);
-int launch_comp_wgrad_dense_tc(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, const int* slot_of_col,
+int launch_comp_wgrad_dense_tc(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, const int* list_dense,
                                const int* counts, const void* dy_bf16, void* vt, float* partial, int splits,
                                int64_t M, int64_t N, int32_t* status);
 

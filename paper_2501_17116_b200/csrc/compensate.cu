@@ -2,13 +2,14 @@
 // forward fused with the final store, weight gradient (Eq. 6) as compact rows for the GEMM's epilogue.
 //
 //   forward   Y[m, :]  = store( Y1[m, :] + sum_{(m,k) in dA} dA[m,k] * W[k, :] )
-//   wgrad     C[slot(k), :] = sum_{(m,k) in dA} dA[m,k] * dY[m, :]   for the columns k that hold entries;
+//   wgrad     C[k, :] = sum_{(m,k) in dA} dA[m,k] * dY[m, :]   for the columns k that hold entries;
 //             the weight-gradient GEMM adds C and applies the DGE factor in its epilogue
 //
 // Both are "sparse row times dense BF16 matrix" with fp32 accumulation on the plain ALUs: a warp
 // owns one output row and 256 of its columns (8 per lane); the sparse entries of that row (CSR
 // for the forward, CSC for the weight gradient) are walked in order, so the result is
 // deterministic.  The FP4 branch and the compensation meet in fp32 and are rounded once.
+#include <cooperative_groups.h>
 #include <cuda_fp16.h>
 
 #include "common.cuh"
@@ -202,11 +203,34 @@ comp_fwd_kept_kernel(const float* __restrict__ y1, const int* __restrict__ rowpt
   store8(y, out_f32, off, y8);
 }
 
-constexpr int LONG_COLUMN = 512;           // entries from which a column gets a whole 1024-thread block
-constexpr int LONG_THREADS = 1024;
+// Columns of the residual by how many entries they hold.  LONG_COLUMN (and M / 4) entries make a column a
+// candidate for the dense class: an outlier channel that most tokens hit (Appendix D).
+constexpr int LONG_COLUMN = 512;
+// From how many entries a column's gathers are spread over a whole cluster of blocks instead of one warp:
+// LONG_FEW entries as long as at most LONG_FEW_MAX columns reach that, else LONG_COLUMN.  A warp walks eight
+// entries per round trip to L2, so the few outlier channels of a small batch (256 entries: 32 round trips)
+// are what everything waits for; thousands of columns with a hundred-odd entries each, as in the heavy
+// residuals of the 7B and 13B shapes, keep all warps busy as they are.
+constexpr int LONG_FEW = 64, LONG_FEW_MAX = 256;
 
-// Exclusive scan of one int per thread over a 1024-thread block; the block's total goes to *total.
-__device__ __forceinline__ int block_exclusive_scan_1024(int c, int* warp_tot, int* total) {
+struct ColumnClasses {
+  int* list_dense;             // [DENSE_TC_MAX] dense columns, ascending
+  int* list_long;              // [K]
+  int* list_short;             // [K]
+  int* counts;                 // numbers of dense, long and short columns
+  int* slot_of_col;            // [K] position among the dense columns; DENSE_TC_MAX for a long or short one; -1: empty
+};
+
+__device__ __forceinline__ int block_sum_1024(int v, int* warp_tot) {
+  v = __reduce_add_sync(0xFFFFFFFFu, v);
+  __syncthreads();                                   // warp_tot may still be read from the previous sum
+  if ((threadIdx.x & 31) == 0) warp_tot[threadIdx.x >> 5] = v;
+  __syncthreads();
+  return __reduce_add_sync(0xFFFFFFFFu, warp_tot[threadIdx.x & 31]);
+}
+
+// Exclusive scan of one int per thread over a 1024-thread block.
+__device__ __forceinline__ int block_exclusive_scan_1024(int c, int* warp_tot) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int incl = c;
 #pragma unroll
@@ -217,43 +241,68 @@ __device__ __forceinline__ int block_exclusive_scan_1024(int c, int* warp_tot, i
   __syncthreads();                                   // warp_tot may still be read from the previous scan
   if (lane == 31) warp_tot[warp] = incl;
   __syncthreads();
-  if (warp == 0) {
-    int v = warp_tot[lane];
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-      const int up = __shfl_up_sync(0xFFFFFFFFu, v, off);
-      if (lane >= off) v += up;
-    }
-    warp_tot[lane] = v;
-  }
-  __syncthreads();
-  *total = warp_tot[31];
-  return incl - c + (warp ? warp_tot[warp - 1] : 0);
+  int before = lane < warp ? warp_tot[lane] : 0;
+  before = __reduce_add_sync(0xFFFFFFFFu, before);
+  return before + incl - c;
 }
 
-// Hot columns of the residual for the forward GEMM's dense tail: the first TAIL_MAX_COLS columns, in
-// ascending order, that hold at least `hot_from` entries.  slot_of_col[k] is column k's position
-// among them or -1, list_hot the inverse, *count their number.
+// Dense columns: the first DENSE_TC_MAX, in ascending order, that hold at least `dense_from` entries (INT_MAX:
+// none).  With ALL the others are listed too, long and short ones, in ascending order.
+// A block owns 1024 columns and counts all earlier ones itself (coalesced reads of a few KB from L2), so no
+// block waits for another: one block walking all columns in stretches took 4.5 us of 2048 and 17.5 of 11008.
+template <bool ALL>
 __global__ void __launch_bounds__(1024, 1)
-hot_columns_kernel(const int* __restrict__ colptr, int K, int hot_from, int* __restrict__ list_hot,
-                   int* __restrict__ slot_of_col, int* __restrict__ count) {
+classify_columns_kernel(const int* __restrict__ colptr, int K, int dense_from, const ColumnClasses out) {
   __shared__ int warp_tot[32];
-  const int t = threadIdx.x;
-  const int per = (K + 1023) / 1024;
-  const int b = min(K, t * per), e = min(K, b + per);
-  int c = 0;
-  for (int k = b; k < e; ++k) c += (colptr[k + 1] - colptr[k] >= hot_from) ? 1 : 0;
-  int total;
-  int rank = block_exclusive_scan_1024(c, warp_tot, &total);
-  for (int k = b; k < e; ++k) {
-    int slot = -1;
-    if (colptr[k + 1] - colptr[k] >= hot_from) {
-      if (rank < TAIL_MAX_COLS) { slot = rank; list_hot[rank] = k; }
-      ++rank;
+  const int t = threadIdx.x, c0 = blockIdx.x * 1024;
+  int cand_b = 0, cand = 0, few = 0, few_b = 0, large = 0, large_b = 0, any = 0, any_b = 0;   // _b: before c0
+  for (int k = t; k < K; k += 1024) {
+    const int n = __ldg(&colptr[k + 1]) - __ldg(&colptr[k]);
+    const bool b = k < c0, c = n >= dense_from;
+    cand += c;
+    cand_b += c && b;
+    if (ALL) {
+      few += n >= LONG_FEW && !c;
+      few_b += n >= LONG_FEW && !c && b;
+      large += n >= LONG_COLUMN && !c;
+      large_b += n >= LONG_COLUMN && !c && b;
+      any += n > 0;
+      any_b += n > 0 && b;
     }
-    slot_of_col[k] = slot;
   }
-  if (t == 0) *count = min(total, TAIL_MAX_COLS);
+  cand = block_sum_1024(cand, warp_tot);
+  cand_b = block_sum_1024(cand_b, warp_tot);
+  const int n_dense = min(cand, DENSE_TC_MAX);
+  const int k = c0 + t;
+  const int n = k < K ? __ldg(&colptr[k + 1]) - __ldg(&colptr[k]) : 0;
+  const bool is_cand = n >= dense_from;
+  const int rank = cand_b + block_exclusive_scan_1024(is_cand, warp_tot);
+  const bool dense = is_cand && rank < DENSE_TC_MAX;
+  if (dense) out.list_dense[rank] = k;
+  if (!ALL) {
+    if (k < K) out.slot_of_col[k] = dense ? rank : -1;
+    if (k == 0) out.counts[0] = n_dense;
+    return;
+  }
+  few = block_sum_1024(few, warp_tot);
+  const bool use_few = few <= LONG_FEW_MAX;
+  const int long_from = use_few ? LONG_FEW : LONG_COLUMN;
+  // (candidates beyond DENSE_TC_MAX hold LONG_COLUMN entries or more: they are long)
+  large = (use_few ? few : block_sum_1024(large, warp_tot)) + cand - n_dense;
+  large_b = block_sum_1024(use_few ? few_b : large_b, warp_tot) + max(0, cand_b - DENSE_TC_MAX);
+  any = block_sum_1024(any, warp_tot);
+  any_b = block_sum_1024(any_b, warp_tot);
+  const bool is_long = !dense && n >= long_from, is_short = !dense && !is_long && n > 0;
+  const int at_long = large_b + block_exclusive_scan_1024(is_long, warp_tot);
+  const int at_short = any_b - large_b - min(cand_b, DENSE_TC_MAX) + block_exclusive_scan_1024(is_short, warp_tot);
+  if (is_long) out.list_long[at_long] = k;
+  if (is_short) out.list_short[at_short] = k;
+  if (k < K) out.slot_of_col[k] = dense ? rank : n > 0 ? DENSE_TC_MAX : -1;
+  if (k == 0) {
+    out.counts[0] = n_dense;
+    out.counts[1] = large;
+    out.counts[2] = any - n_dense - large;
+  }
 }
 
 // Two-term FP16 split of x: hi = RN16(x), lo = RN16(x - hi), stored for the cross products as
@@ -343,69 +392,26 @@ tail_b_kernel(const __nv_bfloat16* __restrict__ w, const int* __restrict__ list_
   }
 }
 
-// The columns of the residual that hold entries, by how full they are: "dense" (at least
-// `dense_from` entries, the first DENSE_TC_MAX of them: outlier channels that most tokens hit,
-// Appendix D), "long" (at least LONG_COLUMN entries) and "short".  The long and the short ones
-// are listed in ascending order; counts[0..2] are the three sizes.  Rows of the compact buffer:
-// dense columns first, then the long, then the short ones, each in ascending column order;
-// slot_of_col[k] is column k's row or -1.  dense_from = INT_MAX switches the dense class off.
-__global__ void __launch_bounds__(1024, 1)
-nonempty_columns_kernel(const int* __restrict__ colptr, int K, int dense_from, int* __restrict__ list_long,
-                        int* __restrict__ list_short, int* __restrict__ counts, int* __restrict__ slot_of_col) {
-  __shared__ int warp_tot[32];
-  const int t = threadIdx.x;
-  const int per = (K + 1023) / 1024;
-  const int b = min(K, t * per), e = min(K, b + per);
-  int c_cand = 0;
-  for (int k = b; k < e; ++k) c_cand += (colptr[k + 1] - colptr[k] >= dense_from) ? 1 : 0;
-  int n_cand;
-  int rank = block_exclusive_scan_1024(c_cand, warp_tot, &n_cand);     // dense candidates before this thread
-  const int n_dense = min(n_cand, DENSE_TC_MAX);
-  int c_long = 0, c_short = 0;
-  {
-    int r = rank;
-    for (int k = b; k < e; ++k) {
-      const int n = colptr[k + 1] - colptr[k];
-      if (n >= dense_from && r++ < DENSE_TC_MAX) continue;
-      if (n >= LONG_COLUMN) ++c_long;
-      else if (n > 0) ++c_short;
-    }
-  }
-  int n_long, n_short;
-  int pos_long = block_exclusive_scan_1024(c_long, warp_tot, &n_long);
-  int pos_short = block_exclusive_scan_1024(c_short, warp_tot, &n_short);
-  for (int k = b; k < e; ++k) {
-    const int n = colptr[k + 1] - colptr[k];
-    int slot = -1;
-    if (n >= dense_from && rank < DENSE_TC_MAX) slot = rank;
-    else if (n >= LONG_COLUMN) { slot = n_dense + pos_long; list_long[pos_long++] = k; }
-    else if (n > 0) { slot = n_dense + n_long + pos_short; list_short[pos_short++] = k; }
-    if (n >= dense_from) ++rank;
-    slot_of_col[k] = slot;
-  }
-  if (t == 0) {
-    counts[0] = n_dense;
-    counts[1] = n_long;
-    counts[2] = n_short;
-  }
-}
-
 // Dense columns (their partial sums come from the tensor-core kernel, one set per range of tokens):
-// C[slot, n] = sum over the ranges, in order.
+// C[column of slot s, n] = sum over the ranges, in order.
 __global__ void __launch_bounds__(256)
-dense_reduce_kernel(float* __restrict__ comp, const float* __restrict__ partial, const int* __restrict__ counts, int N,
-                    int chunks, long long chunk_stride) {
-  const long long total = (long long)counts[0] * N;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    float t = 0.0f;
-    for (int c0 = 0; c0 < chunks; c0 += 8) {            // eight loads in flight, added in chunk order
-      float p[8];
+dense_reduce_kernel(float* __restrict__ comp, const float* __restrict__ partial, const int* __restrict__ list_dense,
+                    const int* __restrict__ counts, int N, int chunks, long long chunk_stride) {
+  const int n4 = N >> 2;
+  const int total = counts[0] * n4;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
+    const int s = i / n4;
+    float4 t = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int c0 = 0; c0 < chunks; c0 += 4) {            // four loads in flight, added in chunk order
+      float4 p[4];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) p[u] = c0 + u < chunks ? __ldg(&partial[(long long)(c0 + u) * chunk_stride + i]) : 0.0f;
+      for (int u = 0; u < 4; ++u)
+        p[u] = c0 + u < chunks ? __ldg(reinterpret_cast<const float4*>(partial + (long long)(c0 + u) * chunk_stride) + i)
+                               : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
-      for (int u = 0; u < 8; ++u) t += p[u];
+      for (int u = 0; u < 4; ++u) { t.x += p[u].x; t.y += p[u].y; t.z += p[u].z; t.w += p[u].w; }
     }
-    comp[i] = t;
+    reinterpret_cast<float4*>(comp + (long long)list_dense[s] * N)[i - s * n4] = t;
   }
 }
 
@@ -448,37 +454,46 @@ __device__ __forceinline__ void store8_f32(float* dst, const float (&t)[8]) {
   *reinterpret_cast<float4*>(dst + 4) = make_float4(t[4], t[5], t[6], t[7]);
 }
 
-// Weight-gradient compensation, step 1: S[k, n-block] += sum over the entries of column k of
-// dA[m,k] * dY[m, n-block].  Outliers sit in a few channels (Appendix D): a handful of columns
-// hold thousands of entries, a few hundred hold one or two, most hold none.
-// Long columns: one 1024-thread block per (column, 256 outputs); its 32 warps take the entries
-// round-robin and their partial sums are added in warp order (independent of scheduling).
-__global__ void __launch_bounds__(LONG_THREADS, 1)
+// Weight-gradient compensation of the columns that are not dense:
+//   comp[k, :] = sum over the entries of column k of dA[m,k] * dY[m, :].
+// Long columns: a cluster of four blocks per (column, 256 outputs).  Its 32 warps take the entries
+// round-robin inside the block's quarter of them; partial sums are added in warp order, then in block order
+// (distributed shared memory), so the result does not depend on scheduling.  (One block of 32 warps
+// per item left ten outlier channels x 8 blocks of outputs with 80 blocks for 148 SMs.)
+constexpr int LONG_CLUSTER = 4, LONG_WARPS = 8;
+__global__ void __cluster_dims__(LONG_CLUSTER, 1, 1) __launch_bounds__(32 * LONG_WARPS, 4)
 comp_wgrad_long_kernel(float* __restrict__ comp, const int* __restrict__ colptr, const int* __restrict__ row,
                        const float* __restrict__ val, const uint4* __restrict__ dy, const int* __restrict__ list,
-                       const int* __restrict__ count, int N) {
-  __shared__ float part[32][32][9];                 // [warp][lane][8 (+1 pad)]
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n0 = blockIdx.x * COMP_COLS + 8 * lane;
-  const bool in_cols = n0 < N;
-  const int n_dense = count[0], n_cols = count[1];
-  for (int slot = blockIdx.y; slot < n_cols; slot += gridDim.y) {
-    const int k = list[slot];
+                       const int* __restrict__ counts, int N) {
+  static_assert(32 * LONG_WARPS == COMP_COLS, "one thread per output of the block sums");
+  __shared__ float part[LONG_WARPS][32][9];         // [warp][lane][8 (+1 pad)]
+  __shared__ float block_sum[COMP_COLS];
+  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int n_long = counts[1], n_blocks = (N + COMP_COLS - 1) / COMP_COLS;
+  const int clusters = gridDim.x / LONG_CLUSTER, rank = int(cluster.block_rank());
+  for (int it = blockIdx.x / LONG_CLUSTER; it < n_long * n_blocks; it += clusters) {
+    const int nb = it / n_long, k = list[it - nb * n_long];
+    const int n0 = nb * COMP_COLS + 8 * lane;
+    const int e0 = colptr[k], n = colptr[k + 1] - e0;
+    const int ea = e0 + int((long long)n * rank / LONG_CLUSTER), eb = e0 + int((long long)n * (rank + 1) / LONG_CLUSTER);
     float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    if (in_cols)
-      strided_entries_times_dense(acc, row, val, colptr[k] + warp, colptr[k + 1], 32, dy, N >> 3, n0 >> 3);
-    __syncthreads();                                // the previous column's partials have been read
+    if (n0 < N) strided_entries_times_dense(acc, row, val, ea + warp, eb, LONG_WARPS, dy, N >> 3, n0 >> 3);
 #pragma unroll
     for (int c = 0; c < 8; ++c) part[warp][lane][c] = acc[c];
     __syncthreads();
-    if (warp == 0 && in_cols) {
-      float t[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-      for (int w = 0; w < 32; ++w) {
+    float t = 0.0f;
 #pragma unroll
-        for (int c = 0; c < 8; ++c) t[c] += part[w][lane][c];
-      }
-      store8_f32(comp + (long long)(n_dense + slot) * N + n0, t);
+    for (int w = 0; w < LONG_WARPS; ++w) t += part[w][tid >> 3][tid & 7];
+    block_sum[tid] = t;
+    cluster.sync();
+    if (rank == 0 && nb * COMP_COLS + tid < N) {
+      t = 0.0f;
+#pragma unroll
+      for (int r = 0; r < LONG_CLUSTER; ++r) t += cluster.map_shared_rank(block_sum, r)[tid];
+      comp[(long long)k * N + nb * COMP_COLS + tid] = t;
     }
+    cluster.sync();                                 // the sums have been read
   }
 }
 
@@ -492,7 +507,7 @@ comp_wgrad_short_kernel(float* __restrict__ comp, const int* __restrict__ colptr
                         const float* __restrict__ val, const uint4* __restrict__ dy, const int* __restrict__ list,
                         const int* __restrict__ counts, int N) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n_before = counts[0] + counts[1], n_cols = counts[2];
+  const int n_cols = counts[2];
   const int groups = (n_cols + 7) >> 3;
   const int n_blocks = (N + COMP_COLS - 1) / COMP_COLS;
   const long long items = (long long)groups * n_blocks;
@@ -520,7 +535,7 @@ comp_wgrad_short_kernel(float* __restrict__ comp, const int* __restrict__ colptr
       }
       for (; e < e1; ++e) fma8(acc, __ldg(&val[e]), __ldg(&dy[(long long)__ldg(&row[e]) * vec_per_row + vcol]));
     }
-    store8_f32(comp + (long long)(n_before + slot) * N + n0, acc);
+    store8_f32(comp + (long long)k * N + n0, acc);
   }
 }
 
@@ -583,7 +598,7 @@ int launch_comp_fwd(fp4_ctx* ctx, cudaStream_t stream, const float* y1, const in
 
 size_t comp_wgrad_scratch_bytes(int64_t M, int64_t K, int64_t N) {
   auto r256 = [](size_t b) { return (b + 255) & ~size_t(255); };
-  size_t b = r256((2 * size_t(K) + 4) * 4) + r256(size_t(K) * 4);                     // lists + counters, slots
+  size_t b = r256((2 * size_t(K) + DENSE_TC_MAX + 4) * 4) + r256(size_t(K) * 4);                     // lists + counters, slots
   b += dense_tc_scratch_bytes(M, N);                                                  // BF16 terms, partial sums
   return b;
 }
@@ -617,7 +632,8 @@ int launch_fwd_tail(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, con
   *kept_end_out = kept_end;
   const int hot_from = int(M / 4 > LONG_COLUMN ? M / 4 : LONG_COLUMN);
   KernelScope scope(ctx, stream, KC_COMP_FWD, 3);
-  hot_columns_kernel<<<1, 1024, 0, stream>>>(a->csc_colptr, int(K), hot_from, list_hot, slot_of_col, count);
+  const ColumnClasses classes = {list_hot, nullptr, nullptr, count, slot_of_col};
+  classify_columns_kernel<false><<<unsigned((K + 1023) / 1024), 1024, 0, stream>>>(a->csc_colptr, int(K), hot_from, classes);
   FP4_CUDA_TRY(cudaMemsetAsync(tb, 0, size_t(N) * TAIL_WIDTH * 2, stream));
   tail_a_kernel<<<unsigned((M + 7) / 8), COMP_THREADS, 0, stream>>>(a->csr_rowptr, a->csr_col, a->csr_val, slot_of_col,
                                                                    count, a->amax, 6.0f, ta, int(M), kept, kept_end);
@@ -632,48 +648,56 @@ int launch_fwd_tail(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, con
 }
 
 int launch_comp_wgrad(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, const void* dy_bf16, Arena& scratch,
-                      int** slot_of_col_out, float* comp, int64_t M, int64_t K, int64_t N, int32_t* status) {
-  // lists: [K] long columns, [K] short columns, three counters
-  int* lists = scratch.take<int>(2 * size_t(K) + 4);
+                      int** slot_of_col_out, float* comp, int64_t M, int64_t K, int64_t N, int32_t* status,
+                      const CompOverlap* overlap) {
+  // lists: [K] long columns, [K] short columns, the dense columns, three counters
+  int* lists = scratch.take<int>(2 * size_t(K) + DENSE_TC_MAX + 4);
   int* slot_of_col = scratch.take<int>(size_t(K));
   const int splits = dense_tc_splits(ctx, M, N);
   void* vt = scratch.take<uint16_t>(size_t(3) * DENSE_TC_MAX * size_t(M));
   float* partial = scratch.take<float>(size_t(splits) * DENSE_TC_MAX * size_t(N));
   if (!scratch.ok) return FP4_ERR_WORKSPACE;
   *slot_of_col_out = slot_of_col;
-  int* list_long = lists;
-  int* list_short = lists + K;
-  int* counts = lists + 2 * K;
+  const ColumnClasses classes = {lists + 2 * K, lists, lists + K, lists + 2 * K + DENSE_TC_MAX, slot_of_col};
   // Columns that at least a quarter of the tokens hit (the outlier channels) form the dense class,
-  // whose product runs on the tensor cores; it needs the CSR.  It costs three launches, which pay
+  // whose product runs on the tensor cores.  It costs three launches, which pay
   // when the residual is heavy: when it may hold at least 1 % of the activation (alpha <= 0.995).
   // (No column can reach LONG_COLUMN entries with fewer tokens than that.)
   const bool dense = a->csr_rowptr != nullptr && a->sparse_cap * 100 >= M * K && M >= LONG_COLUMN;
   const int dense_from = dense ? int(M / 4 > LONG_COLUMN ? M / 4 : LONG_COLUMN) : INT_MAX;
-  const unsigned n_blocks = unsigned((N + COMP_COLS - 1) / COMP_COLS);
-  KernelScope scope(ctx, stream, KC_COMP_WGRAD, 3 + (dense ? (splits > 1 ? 3 : 2) : 0));
-  nonempty_columns_kernel<<<1, 1024, 0, stream>>>(a->csc_colptr, int(K), dense_from, list_long, list_short, counts,
-                                                  slot_of_col);
+  KernelScope scope(ctx, stream, KC_COMP_WGRAD, 3 + (dense ? 3 : 0));
+  classify_columns_kernel<true><<<unsigned((K + 1023) / 1024), 1024, 0, stream>>>(a->csc_colptr, int(K), dense_from, classes);
   const uint4* dy = static_cast<const uint4*>(dy_bf16);
-  if (dense) {
-    const int rc = launch_comp_wgrad_dense_tc(ctx, stream, a, slot_of_col, counts, dy_bf16, vt,
-                                              splits > 1 ? partial : comp, splits, M, N, status);
-    if (rc != FP4_OK) return rc;
-    if (splits > 1)
-      dense_reduce_kernel<<<unsigned(2 * ctx->num_sms), 256, 0, stream>>>(comp, partial, counts, int(N), splits,
-                                                                         (long long)DENSE_TC_MAX * N);
+  // The long columns (a few blocks, latency) run beside the others.
+  cudaStream_t sl = stream;
+  if (overlap) {
+    sl = overlap->stream;
+    FP4_CUDA_TRY(cudaEventRecord(overlap->classified, stream));
+    FP4_CUDA_TRY(cudaStreamWaitEvent(sl, overlap->classified, 0));
   }
-  unsigned gy = unsigned(4 * ctx->num_sms) / n_blocks;          // long columns: 2 resident blocks per SM
-  gy = gy < 1 ? 1 : (gy > unsigned(K) ? unsigned(K) : gy);
-  comp_wgrad_long_kernel<<<dim3(n_blocks, gy), LONG_THREADS, 0, stream>>>(comp, a->csc_colptr, a->csc_row, a->csc_val,
-                                                                         dy, list_long, counts, int(N));
+  if (dense) {
+    const int rc = launch_comp_wgrad_dense_tc(ctx, stream, a, classes.list_dense, classes.counts, dy_bf16, vt, partial, splits,
+                                              M, N, status);
+    if (rc != FP4_OK) return rc;
+    dense_reduce_kernel<<<unsigned(2 * ctx->num_sms), 256, 0, stream>>>(comp, partial, classes.list_dense, classes.counts,
+                                                                       int(N), splits, (long long)DENSE_TC_MAX * N);
+  }
+  const unsigned n_blocks = unsigned((N + COMP_COLS - 1) / COMP_COLS);
+  // long columns: up to four blocks per SM
+  const unsigned clusters = unsigned(4 * ctx->num_sms / LONG_CLUSTER);
+  comp_wgrad_long_kernel<<<clusters * LONG_CLUSTER, 32 * LONG_WARPS, 0, sl>>>(comp, a->csc_colptr, a->csc_row, a->csc_val, dy,
+                                                                             classes.list_long, classes.counts, int(N));
   {
     // short columns: 8 per block; about 32 blocks per SM in all, each taking work items in order
     const long long max_items = (long long)((K + 7) / 8) * n_blocks;
     long long g = 32LL * ctx->num_sms;
     g = g > max_items ? max_items : g;
     comp_wgrad_short_kernel<<<unsigned(g), COMP_THREADS, 0, stream>>>(comp, a->csc_colptr, a->csc_row, a->csc_val, dy,
-                                                                      list_short, counts, int(N));
+                                                                     classes.list_short, classes.counts, int(N));
+  }
+  if (sl != stream) {
+    FP4_CUDA_TRY(cudaEventRecord(overlap->long_done, sl));
+    FP4_CUDA_TRY(cudaStreamWaitEvent(stream, overlap->long_done, 0));
   }
   FP4_CUDA_TRY(cudaGetLastError());
   return FP4_OK;

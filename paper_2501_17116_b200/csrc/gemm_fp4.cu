@@ -250,7 +250,7 @@ __device__ __forceinline__ void wgrad_fetch(WgradOperands& op, const __nv_bfloat
 }
 
 // Fused weight-gradient epilogue for one warp: 16-column chunks, every thread keeps its own row
-//   out[k, n] = store( (acc * d_col[n] + addend[slot[k], n]) * Q'(w[k, n] * 6 / w_amax[n]) ).
+//   out[k, n] = store( (acc * d_col[n] + addend[k, n]) * Q'(w[k, n] * 6 / w_amax[n]) ).
 // The thread-per-row layout of tensor memory is kept throughout: the weights and the
 // compensation row are read as whole 32-byte sectors per thread, the results leave through a
 // bulk store.  `w` and `add` point to the row's weights and compensation at the tile's first column (null
@@ -553,7 +553,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         if (pa.w) w_row = pa.w + size_t(row) * size_t(pa.J) + size_t(n_blk * pa.bn);
         if (pa.slot_of_row) {
           const int slot = __ldg(&pa.slot_of_row[row]);
-          if (slot >= 0) add_row = pa.addend + size_t(slot) * size_t(pa.J) + size_t(n_blk * pa.bn);
+          if (slot >= 0) add_row = pa.addend + size_t(row) * size_t(pa.J) + size_t(n_blk * pa.bn);
         }
         if (16 * group < pa.bn && n_blk * pa.bn + 16 * group < pa.J)
           wgrad_fetch(op, w_row ? w_row + 16 * group : nullptr, pa.w_aligned, add_row ? add_row + 16 * group : nullptr);

@@ -1381,6 +1381,16 @@ size_t quantize_scratch_bytes(int64_t rows, int64_t cols) {
   return b;
 }
 
+int launch_csc_fill(fp4_ctx* ctx, cudaStream_t stream, const CscFill& f) {
+  KernelScope scope(ctx, stream, KC_SPARSE, 1);
+  const dim3 grid((f.cols / 32 + FILL_WARPS - 1) / FILL_WARPS, f.rows / ENC_TM);
+  csc_fill_kernel<<<grid, 32 * FILL_WARPS, 0, stream>>>(f.mask, static_cast<const __nv_bfloat16*>(f.x_bf16), f.rows, f.cols,
+                                                       f.thresholds, f.thr_per_row, f.colptr, f.strip_cnt, f.super_cnt, f.cap,
+                                                       f.csc_row, f.csc_val);
+  FP4_CUDA_TRY(cudaGetLastError());
+  return FP4_OK;
+}
+
 int launch_quantize(fp4_ctx* ctx, cudaStream_t stream, Arena& arena, const void* x_bf16, int64_t rows64,
                     int64_t cols64, int scale_axis, double alpha, const float* prescale, float prescale_div,
                     fp4_qtensor* out, int32_t* status, const SparseOverlap* overlap) {
@@ -1479,12 +1489,14 @@ int launch_quantize(fp4_ctx* ctx, cudaStream_t stream, Arena& arena, const void*
                                                       out->sparse_cap, out->csr_col, out->csr_val);
     }
     if (sp != stream) FP4_CUDA_TRY(cudaEventRecord(overlap->csr_done, sp));
-    {
-      KernelScope scope(ctx, sc2, KC_SPARSE, 1);
-      const dim3 cgrid((cols / 32 + FILL_WARPS - 1) / FILL_WARPS, strips);
-      csc_fill_kernel<<<cgrid, 32 * FILL_WARPS, 0, sc2>>>(mask32, xb, rows, cols, out->thresholds, per_token, out->csc_colptr,
-                                                          sc.strip_cnt, sc.super_cnt, out->sparse_cap, out->csc_row, out->csc_val);
+    const CscFill fill = {mask32, x_bf16, rows, cols, out->thresholds, per_token, out->csc_colptr,
+                          sc.strip_cnt, sc.super_cnt, out->sparse_cap, out->csc_row, out->csc_val};
+    if (sp != stream && overlap->later) {
+      *overlap->later = fill;
+      return FP4_OK;
     }
+    const int rc = launch_csc_fill(ctx, sc2, fill);
+    if (rc != FP4_OK) return rc;
     if (sp != stream && overlap->csc_done) FP4_CUDA_TRY(cudaEventRecord(overlap->csc_done, sc2));
   } else {
     if (prescale && prescale_div > 0.0f) {

@@ -55,44 +55,45 @@ __device__ __forceinline__ uint32_t idesc_dense(int n) {
 }
 
 // Vt[term][s][m]: the three BF16 terms of the dense columns' residual values, zero where a token has
-// no entry.  A block owns 64 tokens: its warps walk the tokens' CSR rows into a shared tile, which
-// then leaves as whole 128-byte rows.  Only rows of boxes the GEMM will load (64 per box) are written.
+// no entry.  A block owns SPLIT_TOK tokens of one column: it finds their entries in the column's list (one
+// sample per thread brackets the first one), scatters them into a shared tile and writes that out as whole
+// lines.  Only rows of boxes the GEMM will load (64 per box) are written.  (Walking the tokens' rows instead, one
+// dependent look-up per entry, took 46 us of 16384 x 5120 and 69 of 8192 x 11008; 6 and 5 now.)
+constexpr int SPLIT_TOK = 2048;
 __global__ void __launch_bounds__(256)
-dense_split_kernel(const int* __restrict__ rowptr, const int* __restrict__ col, const float* __restrict__ val,
-                   const int* __restrict__ slot_of_col, const int* __restrict__ counts,
-                   __nv_bfloat16* __restrict__ vt, int M) {
-  extern __shared__ __align__(16) uint8_t split_smem[];
-  __nv_bfloat16* tile = reinterpret_cast<__nv_bfloat16*>(split_smem);        // [3][DENSE_TC_MAX][64]
-  const int n_dense = min(counts[0], DENSE_TC_MAX);
-  if (n_dense == 0) return;
-  const int rows = ((n_dense + 63) / 64) * 64;
-  const int m0 = blockIdx.x * 64;
-  uint4* t4 = reinterpret_cast<uint4*>(tile);
-  for (int i = threadIdx.x; i < 3 * DENSE_TC_MAX * 64 * 2 / 16; i += blockDim.x) t4[i] = make_uint4(0, 0, 0, 0);
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int tl = warp; tl < 64; tl += 8) {
-    const int m = m0 + tl;
-    if (m >= M) break;
-    for (int e = rowptr[m] + lane; e < rowptr[m + 1]; e += 32) {
-      const int slot = slot_of_col[col[e]];
-      if (unsigned(slot) >= unsigned(n_dense)) continue;
-      const float v = val[e];
+dense_split_kernel(const int* __restrict__ colptr, const int* __restrict__ row, const float* __restrict__ val,
+                   const int* __restrict__ list_dense, const int* __restrict__ counts, __nv_bfloat16* __restrict__ vt,
+                   int M) {
+  __shared__ __align__(16) __nv_bfloat16 tile[3][SPLIT_TOK];
+  const int n_dense = min(counts[0], DENSE_TC_MAX), s = blockIdx.y, t = threadIdx.x;
+  if (s >= ((n_dense + 63) / 64) * 64) return;
+  const int m0 = blockIdx.x * SPLIT_TOK, m1 = min(M, m0 + SPLIT_TOK);
+  uint4* t4 = reinterpret_cast<uint4*>(&tile[0][0]);
+  for (int i = t; i < 3 * SPLIT_TOK / 8; i += 256) t4[i] = make_uint4(0, 0, 0, 0);
+  if (s < n_dense) {
+    const int e0 = colptr[list_dense[s]], n = colptr[list_dense[s] + 1] - e0;
+    // entries before the sample of the last thread whose sample lies before m0 are before m0 as well
+    const int before = __syncthreads_count(n > 0 && row[e0 + int((long long)n * t / 256)] < m0);
+    const int first = before ? int((long long)n * (before - 1) / 256) : 0;
+    for (int e = first + t; e < n; e += 256) {
+      const int m = row[e0 + e];
+      if (m >= m1) break;
+      if (m < m0) continue;
+      const float v = val[e0 + e];
       const __nv_bfloat16 b1 = __float2bfloat16_rn(v);
       const float r1 = v - __bfloat162float(b1);                 // exact
       const __nv_bfloat16 b2 = __float2bfloat16_rn(r1);
       const float r2 = r1 - __bfloat162float(b2);                // exact
-      const __nv_bfloat16 b3 = __float2bfloat16_rn(r2);          // exact: 24 bits in three terms of 8
-      tile[(0 * DENSE_TC_MAX + slot) * 64 + tl] = b1;
-      tile[(1 * DENSE_TC_MAX + slot) * 64 + tl] = b2;
-      tile[(2 * DENSE_TC_MAX + slot) * 64 + tl] = b3;
+      tile[0][m - m0] = b1;
+      tile[1][m - m0] = b2;
+      tile[2][m - m0] = __float2bfloat16_rn(r2);                 // exact: 24 bits in three terms of 8
     }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < 3 * rows * 8; i += blockDim.x) {
-    const int t = i / (rows * 8), r = (i / 8) % rows, c = i % 8;
-    const uint4 x = t4[((t * DENSE_TC_MAX + r) * 64 * 2) / 16 + c];
-    *reinterpret_cast<uint4*>(vt + (size_t(t * DENSE_TC_MAX + r) * size_t(M) + size_t(m0)) + 8 * c) = x;
+  for (int i = t; i < 3 * (SPLIT_TOK / 8); i += 256) {
+    const int term = i / (SPLIT_TOK / 8), c = i - term * (SPLIT_TOK / 8);
+    if (m0 + 8 * c < m1)
+      *reinterpret_cast<uint4*>(vt + size_t(term * DENSE_TC_MAX + s) * size_t(M) + size_t(m0) + 8 * c) = t4[i];
   }
 }
 
@@ -334,7 +335,7 @@ size_t dense_tc_scratch_bytes(int64_t M, int64_t N) {
 
 // C[s, :] for the dense columns s < counts[0] into `partial` ([splits][DENSE_TC_MAX][N]); the caller
 // adds the splits in order.  M must be a multiple of 128.
-int launch_comp_wgrad_dense_tc(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, const int* slot_of_col,
+int launch_comp_wgrad_dense_tc(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, const int* list_dense,
                                const int* counts, const void* dy_bf16, void* vt, float* partial, int splits,
                                int64_t M, int64_t N, int32_t* status) {
   CUtensorMap map_dy, map_vt;
@@ -342,8 +343,8 @@ int launch_comp_wgrad_dense_tc(fp4_ctx* ctx, cudaStream_t stream, const fp4_qten
   if (rc != FP4_OK) return rc;
   rc = make_bf16_map(ctx, &map_vt, vt, 3 * DENSE_TC_MAX, M);
   if (rc != FP4_OK) return rc;
-  dense_split_kernel<<<unsigned((M + 63) / 64), 256, 3 * DENSE_TC_MAX * 64 * 2, stream>>>(
-      a->csr_rowptr, a->csr_col, a->csr_val, slot_of_col, counts, static_cast<__nv_bfloat16*>(vt), int(M));
+  dense_split_kernel<<<dim3(unsigned((M + SPLIT_TOK - 1) / SPLIT_TOK), DENSE_TC_MAX), 256, 0, stream>>>(
+      a->csc_colptr, a->csc_row, a->csc_val, list_dense, counts, static_cast<__nv_bfloat16*>(vt), int(M));
   DenseTcArgs args;
   args.M = int(M);
   args.N = int(N);
