@@ -8,7 +8,7 @@
 //
 // Structure: persistent CTAs (one per SM), 128 x BN output tile per CTA:
 //   warp 0      TMA producer: cp.async.bulk.tensor loads into 128-byte-swizzled shared memory,
-//               a ring of STAGES stages guarded by full/empty mbarriers;
+//               a ring of 3 or 4 stages guarded by full/empty mbarriers;
 //   warp 1      allocates tensor memory and issues tcgen05.mma from one thread, fp32
 //               accumulators in tensor memory; tcgen05.commit releases stages and publishes tiles;
 //   warps 2..   epilogue (8 warps; 16 with the fused weight-gradient epilogue): tcgen05.ld the
@@ -39,27 +39,49 @@ constexpr int BM = 128;
 enum { EPI_PLAIN = 0, EPI_WGRAD = 1 };
 __host__ __device__ constexpr int epi_warps(int epi) { return epi == EPI_WGRAD ? 16 : 8; }
 __host__ __device__ constexpr int num_threads(int epi) { return 64 + 32 * epi_warps(epi); }
-__host__ __device__ constexpr int stages_of(int kind) { return kind == FP4_GEMM_F8F6F4 ? 3 : 4; }
 constexpr int A_STAGE_BYTES = BM * 128;
 constexpr int TMEM_COLS = 512;
 constexpr int ACC_STRIDE = 256;          // tensor-memory columns between the two accumulator stages
 constexpr int SF_COL_B = 240;            // MXF4 only: unit block scales in the gap behind stage 0
 constexpr int SF_COL_A = 248;
-constexpr int STAGE_OUT_BYTES = 32768;    // epilogue staging: 4 KB per warp (plain) or 2 KB (fused)
+constexpr int STAGE_OUT_BYTES = 4096;     // plain epilogue: staging of a warp, two buffers of 2 KB
+// Fused epilogue: a warp's chunk of weights and of compensation, and its staging (an fp32 chunk, or two of BF16)
+constexpr int IN_W_BYTES = 1024, IN_ADD_BYTES = 2048, FUSED_OUT_BYTES = 2048;
 
-__host__ __device__ constexpr int tile_n(int kind) { return kind == FP4_GEMM_F8F6F4 ? 256 : 240; }
-__host__ __device__ constexpr int b_stage_bytes(int kind) { return tile_n(kind) * 128; }
-__host__ __device__ constexpr int stage_bytes(int kind) { return A_STAGE_BYTES + b_stage_bytes(kind); }
-// operand ring, epilogue staging, barriers, column de-scales [2][256], DGE column scales [2][256]
-constexpr size_t smem_bytes(int kind) {
-  return 1024 + size_t(stages_of(kind)) * stage_bytes(kind) + 256 + 2 * 256 * 4 + STAGE_OUT_BYTES + 2 * 256 * 4;
+// Widest tile: what tensor memory holds twice (MXF4: beside the block scales) and the ring three times.
+__host__ __device__ constexpr int tile_n(int kind, int epi) {
+  return kind == FP4_GEMM_F8F6F4 && epi == EPI_PLAIN ? 256 : 240;
+}
+// Shared memory: operand ring, epilogue buffers, barriers, column de-scales [2][256], DGE column scales [2][256].
+// The ring has MAX_STAGES stages (A and B tile of one k-block) where they fit, else three.
+constexpr int MAX_STAGES = 4;
+constexpr int MISC_BYTES = 512;
+constexpr int FIXED_SMEM = 1024 + MISC_BYTES + 2 * 256 * 4 + 2 * 256 * 4;
+constexpr int MOST_SMEM = 227 * 1024;
+struct SmemPlan {
+  int stages, stage_bytes, out_bytes, in_bytes;      // out_bytes, in_bytes: per epilogue warp
+};
+SmemPlan plan_smem(int epi, int bn, bool has_w, bool has_add, bool f32) {
+  const int avail = MOST_SMEM - FIXED_SMEM, stage = A_STAGE_BYTES + 128 * bn, warps = epi_warps(epi);
+  SmemPlan p = {MAX_STAGES, stage, STAGE_OUT_BYTES, 0};
+  if (epi == EPI_WGRAD) {
+    p.out_bytes = FUSED_OUT_BYTES;
+    p.in_bytes = (has_w ? IN_W_BYTES : 0) + (has_add ? IN_ADD_BYTES : 0);
+    // a fourth stage is worth more than a second BF16 staging buffer
+    if (!f32 && p.stages * stage + warps * (p.out_bytes + p.in_bytes) > avail &&
+        p.stages * stage + warps * (p.out_bytes / 2 + p.in_bytes) <= avail)
+      p.out_bytes /= 2;
+  }
+  while (p.stages * stage + warps * (p.out_bytes + p.in_bytes) > avail) --p.stages;
+  return p;
 }
 
 struct GemmArgs {
   int I, J;
   int num_k_blocks;
   int num_m_blocks, num_n_blocks;
-  int bn;                      // tile width: a multiple of 16, at most tile_n(kind)
+  int bn;                      // tile width: a multiple of 16, at most tile_n
+  SmemPlan smem;               // (the same for both problems of a launch)
   uint32_t tx_bytes;
   uint32_t idesc;              // instruction descriptor (operand formats differ per problem)
   float row_div, col_div;      // largest value of the row / column operand's format: 6 (E2M1) or 448 (E4M3)
@@ -69,10 +91,8 @@ struct GemmArgs {
   int out_f32;
   int32_t* status;
   // fused weight-gradient epilogue (EPI_WGRAD)
-  const float* addend;
-  const int* slot_of_row;
-  const __nv_bfloat16* w;
-  bool w_aligned;              // `w` starts on a 32-byte boundary
+  const int* slot_of_row;      // rows with a compensation row: not negative (null: none)
+  bool has_w;                  // the DGE factor applies
   const float* w_amax;
   float log2_inv_k, expo, clip;
   // dense tail (single-problem launches only): after the FP4 k-blocks of a tile, 3 * ceil(*tail_count / 64)
@@ -118,14 +138,14 @@ struct OutMaps {
 // between two 2 KB buffers.
 template <int W, int NBUF>
 __device__ __forceinline__ void bulk_store_chunk(const float (&y)[W], uint8_t* stage, int out_f32, const OutMaps& maps,
-                                                 int row0, int col0, int lane, uint32_t& seq) {
+                                                 int row0, int col0, int lane, uint32_t& seq, bool two_small = true) {
   const int fx = (lane >> 1) & 3;
   if (out_f32) {
 #pragma unroll
     for (int u = 0; u < W / 16; ++u) {              // one box per 16 columns
       uint8_t* buf = stage + (NBUF == 2 ? (seq & 1u) * 2048 : 0);
       ++seq;
-      if (lane == 0) { if (NBUF == 2) tma_store_wait_read_1(); else tma_store_wait_read_0(); }
+      if (elect_one()) { if (NBUF == 2) tma_store_wait_read_1(); else tma_store_wait_read_0(); }
       __syncwarp();
       uint8_t* my_row = buf + lane * 64;
 #pragma unroll
@@ -134,7 +154,7 @@ __device__ __forceinline__ void bulk_store_chunk(const float (&y)[W], uint8_t* s
             make_float4(y[16 * u + 4 * j], y[16 * u + 4 * j + 1], y[16 * u + 4 * j + 2], y[16 * u + 4 * j + 3]);
       fence_async_smem();
       __syncwarp();
-      if (lane == 0) tma_store_2d(maps.unit, buf, col0 + 16 * u, row0);
+      if (elect_one()) tma_store_2d(maps.unit, buf, col0 + 16 * u, row0);
     }
   } else {
     uint4 packed[W / 8];
@@ -148,11 +168,11 @@ __device__ __forceinline__ void bulk_store_chunk(const float (&y)[W], uint8_t* s
       }
       packed[j] = make_uint4(w4[0], w4[1], w4[2], w4[3]);
     }
-    // a 16-column BF16 box is 1 KB: two of them always fit the 2 KB every warp has
-    constexpr bool two = NBUF == 2 || W == 16;
+    // a 16-column BF16 box is 1 KB: two of them fit the 2 KB a warp has, unless it has only one (two_small)
+    const bool two = NBUF == 2 || (W == 16 && two_small);
     uint8_t* buf = stage + (two ? (seq & 1u) * (W == 16 && NBUF == 1 ? 1024 : 2048) : 0);
     ++seq;
-    if (lane == 0) { if (two) tma_store_wait_read_1(); else tma_store_wait_read_0(); }
+    if (elect_one()) { if (two) tma_store_wait_read_1(); else tma_store_wait_read_0(); }
     __syncwarp();
     if (W == 32) {
       uint8_t* my_row = buf + lane * 64;
@@ -165,7 +185,7 @@ __device__ __forceinline__ void bulk_store_chunk(const float (&y)[W], uint8_t* s
     }
     fence_async_smem();
     __syncwarp();
-    if (lane == 0) tma_store_2d(W == 32 ? maps.unit : maps.half, buf, col0, row0);
+    if (elect_one()) tma_store_2d(W == 32 ? maps.unit : maps.half, buf, col0, row0);
   }
 }
 
@@ -216,57 +236,51 @@ __device__ __forceinline__ void epilogue_tile_plain(const GemmArgs& args, int ro
   }
 }
 
-// Operands of the fused weight-gradient epilogue for 16 columns of this thread's row: the BF16
-// weights that drive the DGE factor and the compensation row.  They are requested one chunk
-// ahead, right after the previous chunk's have been consumed, with 256-bit loads: a whole sector per
-// lane and request (as pairs of 128-bit loads the second one found its sector evicted every other time,
-// the kernel's shared memory leaves L1 a few KB).
-struct WgradOperands {
-  uint32_t w[8];         // 16 BF16 weights
-  float add[16];         // 16 floats of the compensation row (zeros without one)
+// Inputs of the fused weight-gradient epilogue: for a chunk of 32 rows x 16 columns the BF16 weights that drive
+// the DGE factor and the fp32 compensation.  A warp's next chunk travels by TMA into its own 3 KB while the
+// current one is computed.  (Read by the lanes themselves, a row each, every load touched 32 lines and the
+// requests, not the bytes, were the limit: 640 x 4096 x 4096, 55 us with weights and compensation, 22 with neither.
+// Prefetching deeper or to L2 made it worse; 45 us now, 4096 x 2048 x 5504 65 -> 54, 4096 x 5504 x 2048 68 -> 54.)
+struct WgradInput {
+  const CUtensorMap* map_w;    // boxes of 16 columns x 32 rows: 32-byte rows, 32-byte swizzle
+  const CUtensorMap* map_add;  // 64-byte rows, 64-byte swizzle
+  uint8_t* buf;                // [1 KB weights, if any][2 KB compensation]
+  uint64_t* bar;
+  uint32_t state;              // bytes of a chunk (IN_W_BYTES, IN_ADD_BYTES: any of the warp's rows has some) | flags
 };
-__device__ __forceinline__ void ldg256(const void* p, uint32_t (&r)[8]) {
-  asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "l"(p));
-}
-__device__ __forceinline__ void wgrad_fetch(WgradOperands& op, const __nv_bfloat16* w, bool w_aligned, const float* add) {
-  if (w && w_aligned) {
-    ldg256(w, op.w);
-  } else if (w) {                                    // the caller's weights start on a 16-byte boundary only
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const uint4 q = __ldg(reinterpret_cast<const uint4*>(w) + h);
-      op.w[4 * h] = q.x; op.w[4 * h + 1] = q.y; op.w[4 * h + 2] = q.z; op.w[4 * h + 3] = q.w;
-    }
+constexpr uint32_t IN_PHASE = 1, IN_PENDING = 2;     // parity of the next wait; a request has not been waited for
+__device__ __forceinline__ void wgrad_request(WgradInput& in, int w_bytes, int row0, int col) {
+  const uint32_t bytes = in.state & (IN_W_BYTES | IN_ADD_BYTES);
+  if (!bytes) return;
+  if (elect_one()) {
+    mbar_arrive_expect_tx(in.bar, bytes);
+    if (bytes & IN_W_BYTES) tma_load_2d(in.buf, in.map_w, in.bar, col, row0);
+    if (bytes & IN_ADD_BYTES) tma_load_2d(in.buf + w_bytes, in.map_add, in.bar, col, row0);
   }
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    uint32_t r[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    if (add) ldg256(add + 8 * h, r);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) op.add[8 * h + j] = __uint_as_float(r[j]);
-  }
+  __syncwarp();
+  in.state |= IN_PENDING;
 }
 
 // Fused weight-gradient epilogue for one warp: 16-column chunks, every thread keeps its own row
 //   out[k, n] = store( (acc * d_col[n] + addend[k, n]) * Q'(w[k, n] * 6 / w_amax[n]) ).
-// The thread-per-row layout of tensor memory is kept throughout: the weights and the
-// compensation row are read as whole 32-byte sectors per thread, the results leave through a
-// bulk store.  `w` and `add` point to the row's weights and compensation at the tile's first column (null
-// without), `op` holds the operands of the warp's first chunk, requested by the caller
-// before the accumulators were awaited.
+// The thread-per-row layout of tensor memory is kept throughout; the results leave through a
+// bulk store.  `add_row`: this thread's row has compensation.  The caller has requested the inputs of the warp's
+// first chunk before it awaited the accumulators.  False: a wait ran out (the tile is not finished).
 template <int G>
-__device__ __forceinline__ void epilogue_tile_wgrad(const GemmArgs& args, int row_blk, int n_blk, uint32_t t_base,
-                                                    float d_row, const float* dcol, const float* gcol,
-                                                    const __nv_bfloat16* w, const float* add,
+__device__ __forceinline__ bool epilogue_tile_wgrad(const GemmArgs& args, int row_blk, int n_blk, uint32_t t_base,
+                                                    float d_row, const float* dcol, const float* gcol, bool add_row,
+                                                    WgradInput& in, volatile int* abort_flag, uint64_t wait_limit_ns,
                                                     uint8_t* stage, int quarter, int group, int lane,
-                                                    const OutMaps& maps, uint32_t& seq, WgradOperands& op) {
+                                                    const OutMaps& maps, uint32_t& seq, bool two_out) {
   const int n_col0 = n_blk * args.bn;
   const int n_valid = min(args.bn, args.J - n_col0);
   const int row0 = row_blk * BM + quarter * 32;
   int c0 = 16 * group;
-  if (c0 >= n_valid) return;
+  if (c0 >= n_valid) return true;
+  const int w_bytes = args.has_w ? IN_W_BYTES : 0;
+  const uint8_t* w_smem = in.buf + lane * 32;
+  const uint8_t* add_smem = in.buf + w_bytes + lane * 64;
+  const int w_fx = (lane >> 2) & 1, add_fx = (lane >> 1) & 3;
   uint32_t v[32];
   tmem_ld_32x16(t_base + uint32_t(c0), v);
 #pragma unroll 1
@@ -274,11 +288,34 @@ __device__ __forceinline__ void epilogue_tile_wgrad(const GemmArgs& args, int ro
     const int next = c0 + 16 * G;
     tmem_ld_wait();
     float y[16];
+    uint32_t w[8];
     descale_chunk<16>(v, d_row, dcol + c0, y);
     if (next < n_valid) tmem_ld_32x16(t_base + uint32_t(next), v);
+    if (in.state & IN_PENDING) {
+      const bool ok = mbar_wait(in.bar, in.state & IN_PHASE, abort_flag, args.status, wait_limit_ns);
+      if (!__all_sync(0xFFFFFFFFu, ok)) return false;
+      in.state ^= IN_PHASE | IN_PENDING;
+      if (in.state & IN_ADD_BYTES) {
 #pragma unroll
-    for (int j = 0; j < 16; ++j) y[j] += op.add[j];
-    if (w) {
+        for (int q = 0; q < 4; ++q) {
+          const float4 a = *reinterpret_cast<const float4*>(add_smem + ((q ^ add_fx) * 16));
+          y[4 * q + 0] += add_row ? a.x : 0.0f;
+          y[4 * q + 1] += add_row ? a.y : 0.0f;
+          y[4 * q + 2] += add_row ? a.z : 0.0f;
+          y[4 * q + 3] += add_row ? a.w : 0.0f;
+        }
+      }
+      if (args.has_w) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const uint4 q = *reinterpret_cast<const uint4*>(w_smem + ((h ^ w_fx) * 16));
+          w[4 * h] = q.x; w[4 * h + 1] = q.y; w[4 * h + 2] = q.z; w[4 * h + 3] = q.w;
+        }
+      }
+      __syncwarp();                                    // every lane has its row
+      if (next < n_valid) wgrad_request(in, w_bytes, row0, n_col0 + next);
+    }
+    if (args.has_w) {
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const float4 g4 = *reinterpret_cast<const float4*>(gcol + c0 + 4 * q);   // same address in every lane
@@ -286,14 +323,14 @@ __device__ __forceinline__ void epilogue_tile_wgrad(const GemmArgs& args, int ro
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
           const int c = 4 * q + e;
-          const float wf = __uint_as_float((c & 1) ? (op.w[c >> 1] & 0xFFFF0000u) : (op.w[c >> 1] << 16));
+          const float wf = __uint_as_float((c & 1) ? (w[c >> 1] & 0xFFFF0000u) : (w[c >> 1] << 16));
           y[c] *= dge_factor(__fmul_rn(wf, g[e]), args.expo, args.log2_inv_k, args.clip);
         }
       }
     }
-    if (next < n_valid) wgrad_fetch(op, w ? w + next : nullptr, args.w_aligned, add ? add + next : nullptr);
-    bulk_store_chunk<16, 1>(y, stage, args.out_f32, maps, row0, n_col0 + c0, lane, seq);
+    bulk_store_chunk<16, 1>(y, stage, args.out_f32, maps, row0, n_col0 + c0, lane, seq, two_out);
   }
+  return true;
 }
 
 template <int KIND, int EPI>
@@ -302,25 +339,24 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
                 const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_out_aux,
                 const __grid_constant__ GemmArgs args, const __grid_constant__ CUtensorMap map_a2,
                 const __grid_constant__ CUtensorMap map_b2, const __grid_constant__ CUtensorMap map_out2,
-                const __grid_constant__ CUtensorMap map_out_aux2, const __grid_constant__ GemmArgs args2) {
+                const __grid_constant__ CUtensorMap map_out_aux2, const __grid_constant__ GemmArgs args2,
+                const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_add) {
   constexpr int NACC = 2;
-  constexpr int STAGES = stages_of(KIND);
-  constexpr int B_STAGE_BYTES = b_stage_bytes(KIND);
-  constexpr int STAGE_BYTES = stage_bytes(KIND);
+  const int STAGES = args.smem.stages, STAGE_BYTES = args.smem.stage_bytes;      // a stage: A tile, then B tile
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* smem_a = smem;
-  uint8_t* smem_b = smem + STAGES * A_STAGE_BYTES;
-  uint8_t* s_out = smem + STAGES * STAGE_BYTES;        // [8 warps][4096] staging, 1024-byte aligned
-  uint8_t* smem_misc = s_out + STAGE_OUT_BYTES;
+  uint8_t* s_in = smem + STAGES * STAGE_BYTES;         // fused epilogue: inputs of each warp, 1024-byte aligned
+  uint8_t* s_out = s_in + epi_warps(EPI) * args.smem.in_bytes;         // staging of each epilogue warp
+  uint8_t* smem_misc = s_out + epi_warps(EPI) * args.smem.out_bytes;
   uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem_misc);
-  uint64_t* empty_bar = full_bar + STAGES;
-  uint64_t* acc_full = empty_bar + STAGES;
+  uint64_t* empty_bar = full_bar + MAX_STAGES;
+  uint64_t* acc_full = empty_bar + MAX_STAGES;
   uint64_t* acc_empty = acc_full + 2;
-  uint64_t* final_bar = acc_empty + 2;
+  uint64_t* in_bar = acc_empty + 2;                    // [16]
+  uint64_t* final_bar = in_bar + 16;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(final_bar + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  float* s_dcol = reinterpret_cast<float*>(smem_misc + 256);                     // [2][256] column de-scales
+  float* s_dcol = reinterpret_cast<float*>(smem_misc + MISC_BYTES);              // [2][256] column de-scales
   float* s_gcol = s_dcol + 2 * 256;                                              // [2][256] 6 / w_amax (DGE)
 
   const int warp = __shfl_sync(0xFFFFFFFFu, int(threadIdx.x >> 5), 0);    // known to be the same in all lanes
@@ -345,6 +381,8 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       mbar_init(&acc_full[a], 1);
       mbar_init(&acc_empty[a], epi_warps(EPI));
     }
+    if (EPI == EPI_WGRAD)
+      for (int w = 0; w < epi_warps(EPI); ++w) mbar_init(&in_bar[w], 1);
     mbar_init(final_bar, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -361,11 +399,15 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       const int m_blk = tt % pa.num_m_blocks, n_blk = tt / pa.num_m_blocks;
       for (int kb = 0; kb < pre; ++kb) {
         mbar_arrive_expect_tx(&full_bar[kb], pa.tx_bytes);
-        tma_load_2d(smem_a + kb * A_STAGE_BYTES, ma, &full_bar[kb], kb * 128, m_blk * BM);
-        tma_load_2d(smem_b + kb * B_STAGE_BYTES, mb, &full_bar[kb], kb * 128, n_blk * pa.bn);
+        tma_load_2d(smem + kb * STAGE_BYTES, ma, &full_bar[kb], kb * 128, m_blk * BM);
+        tma_load_2d(smem + kb * STAGE_BYTES + A_STAGE_BYTES, mb, &full_bar[kb], kb * 128, n_blk * pa.bn);
       }
     }
     asm volatile("prefetch.tensormap [%0];" ::"l"(&map_out) : "memory");
+    if (EPI == EPI_WGRAD) {
+      asm volatile("prefetch.tensormap [%0];" ::"l"(&map_w) : "memory");
+      asm volatile("prefetch.tensormap [%0];" ::"l"(&map_add) : "memory");
+    }
     if (args.tail_count) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(&map_a2) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(&map_b2) : "memory");
@@ -424,8 +466,8 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           if (!ok) break;
           if (blockIdx.x != 0 || int(fills) != args.skip_fill) {      // a left-out fill: no copy, no arrival
             mbar_arrive_expect_tx(&full_bar[stage], pa.tx_bytes);
-            tma_load_2d(smem_a + stage * A_STAGE_BYTES, ma, &full_bar[stage], kb * 128, m_blk * BM);
-            tma_load_2d(smem_b + stage * B_STAGE_BYTES, mb, &full_bar[stage], kb * 128, n_blk * pa.bn);
+            tma_load_2d(smem + stage * STAGE_BYTES, ma, &full_bar[stage], kb * 128, m_blk * BM);
+            tma_load_2d(smem + stage * STAGE_BYTES + A_STAGE_BYTES, mb, &full_bar[stage], kb * 128, n_blk * pa.bn);
           }
           ++fills;
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
@@ -434,8 +476,8 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           ok = mbar_wait(&empty_bar[stage], phase ^ 1u, abort_flag, args.status, args.wait_limit_ns);
           if (!ok) break;
           mbar_arrive_expect_tx(&full_bar[stage], args.tail_tx_bytes);
-          tma_load_2d(smem_a + stage * A_STAGE_BYTES, &map_a2, &full_bar[stage], kb * 64, m_blk * BM);
-          tma_load_2d(smem_b + stage * B_STAGE_BYTES, &map_b2, &full_bar[stage], kb * 64, n_blk * args.bn);
+          tma_load_2d(smem + stage * STAGE_BYTES, &map_a2, &full_bar[stage], kb * 64, m_blk * BM);
+          tma_load_2d(smem + stage * STAGE_BYTES + A_STAGE_BYTES, &map_b2, &full_bar[stage], kb * 64, n_blk * args.bn);
           ++fills;
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
@@ -472,8 +514,8 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           ok = mbar_wait(&full_bar[stage], phase, abort_flag, args.status, args.wait_limit_ns);
           if (!ok) break;
           tc_fence_after();
-          const uint64_t a_desc = make_smem_desc(smem_u32(smem_a + stage * A_STAGE_BYTES));
-          const uint64_t b_desc = make_smem_desc(smem_u32(smem_b + stage * B_STAGE_BYTES));
+          const uint64_t a_desc = make_smem_desc(smem_u32(smem + stage * STAGE_BYTES));
+          const uint64_t b_desc = make_smem_desc(smem_u32(smem + stage * STAGE_BYTES + A_STAGE_BYTES));
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
             // 32 bytes of the swizzled 128-byte row per instruction: +2 in the (>>4) address field
@@ -492,8 +534,8 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           ok = mbar_wait(&full_bar[stage], phase, abort_flag, args.status, args.wait_limit_ns);
           if (!ok) break;
           tc_fence_after();
-          const uint64_t a_desc = make_smem_desc(smem_u32(smem_a + stage * A_STAGE_BYTES));
-          const uint64_t b_desc = make_smem_desc(smem_u32(smem_b + stage * B_STAGE_BYTES));
+          const uint64_t a_desc = make_smem_desc(smem_u32(smem + stage * STAGE_BYTES));
+          const uint64_t b_desc = make_smem_desc(smem_u32(smem + stage * STAGE_BYTES + A_STAGE_BYTES));
 #pragma unroll
           for (int k = 0; k < 4; ++k)          // 16 FP16 columns = 32 bytes of the 128-byte row per instruction
             mma_f16(d_tmem, a_desc + uint64_t(2 * k), b_desc + uint64_t(2 * k), args.tail_idesc, 1u);
@@ -521,11 +563,13 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     const int quarter = warp & 3;               // the lane quarter of tensor memory this warp may read
     const int group = (warp - 2) >> 2;          // which of the G warps of this quarter
     const int et = threadIdx.x - 64;            // index among the epilogue threads
-    uint8_t* stage = s_out + (warp - 2) * (EPI == EPI_WGRAD ? 2048 : 4096);
+    uint8_t* stage = s_out + (warp - 2) * args.smem.out_bytes;
     int acc = 0;
     uint32_t acc_phase = 0;
     uint32_t tile_parity = 0;
     uint32_t store_seq = 0;
+    WgradInput in = {&map_w, &map_add, s_in + (warp - 2) * args.smem.in_bytes, &in_bar[warp - 2], 0u};
+    bool dead = false;
     for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
       const bool second = t >= tiles_first;
       const GemmArgs& pa = second ? args2 : args;
@@ -541,30 +585,27 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       for (int c = et; c < pa.bn; c += 32 * EW) {
         const int col = n_blk * pa.bn + c;
         dcol[c] = (pa.col_amax && col < pa.J) ? __fdiv_rn(__ldg(&pa.col_amax[col]), pa.col_div) : 1.0f;
-        if (EPI == EPI_WGRAD && pa.w) {
+        if (EPI == EPI_WGRAD && pa.has_w) {
           const float am = col < pa.J ? __ldg(&pa.w_amax[col]) : 0.0f;
           gcol[c] = am > 0.0f ? __fdiv_rn(6.0f, am) : 0.0f;
         }
       }
-      const __nv_bfloat16* w_row = nullptr;
-      const float* add_row = nullptr;
-      WgradOperands op;
+      bool add_row = false;
       if (EPI == EPI_WGRAD) {
-        if (pa.w) w_row = pa.w + size_t(row) * size_t(pa.J) + size_t(n_blk * pa.bn);
-        if (pa.slot_of_row) {
-          const int slot = __ldg(&pa.slot_of_row[row]);
-          if (slot >= 0) add_row = pa.addend + size_t(row) * size_t(pa.J) + size_t(n_blk * pa.bn);
-        }
-        if (16 * group < pa.bn && n_blk * pa.bn + 16 * group < pa.J)
-          wgrad_fetch(op, w_row ? w_row + 16 * group : nullptr, pa.w_aligned, add_row ? add_row + 16 * group : nullptr);
+        add_row = pa.slot_of_row && __ldg(&pa.slot_of_row[row]) >= 0;
+        in.state = (in.state & (IN_PHASE | IN_PENDING)) | (pa.has_w ? IN_W_BYTES : 0u) |
+                   (__any_sync(0xFFFFFFFFu, add_row) ? IN_ADD_BYTES : 0u);
+        if (!dead && 16 * group < min(pa.bn, pa.J - n_blk * pa.bn))
+          wgrad_request(in, pa.has_w ? IN_W_BYTES : 0, m_blk * BM + quarter * 32, n_blk * pa.bn + 16 * group);
       }
       const bool ok = mbar_wait(&acc_full[acc], acc_phase, abort_flag, args.status, args.wait_limit_ns);
       if (epilogue_bar_any(!ok, 32 * EW)) break;   // also publishes dcol to the other warps
       tc_fence_after();
       const uint32_t t_base = tmem_base + (uint32_t(quarter * 32) << 16) + uint32_t(acc * ACC_STRIDE);
       if (EPI == EPI_WGRAD)
-        epilogue_tile_wgrad<G>(pa, m_blk, n_blk, t_base, d_row, dcol, gcol, w_row, add_row, stage, quarter, group, lane,
-                                   out_maps, store_seq, op);
+        dead = !epilogue_tile_wgrad<G>(pa, m_blk, n_blk, t_base, d_row, dcol, gcol, add_row, in, abort_flag,
+                                       args.wait_limit_ns, stage, quarter, group, lane, out_maps, store_seq,
+                                       args.smem.out_bytes == FUSED_OUT_BYTES);
       else
         epilogue_tile_plain<G>(pa, m_blk, n_blk, t_base, d_row, dcol, stage, quarter, group, lane, out_maps,
                                    store_seq);
@@ -574,7 +615,11 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       if (++acc == NACC) { acc = 0; acc_phase ^= 1u; }
       tile_parity ^= 1u;
     }
-    if (lane == 0) tma_store_wait_all();    // this warp's bulk stores have landed
+    if (elect_one()) tma_store_wait_all();    // this warp's bulk stores have landed
+    if (EPI == EPI_WGRAD && (in.state & IN_PENDING)) {        // gave up: let the inputs in flight land
+      const uint64_t t0 = global_timer_ns();
+      while (!mbar_try_wait(in.bar, in.state & IN_PHASE) && global_timer_ns() - t0 < 1000000ull) {}
+    }
   }
 
   tc_fence_before();
@@ -658,23 +703,41 @@ int make_out_maps(fp4_ctx* ctx, CUtensorMap* unit, CUtensorMap* aux, void* out, 
   return r == CUDA_SUCCESS ? FP4_OK : FP4_ERR_CUDA;
 }
 
+// Tensor map of an input of the fused epilogue, [I x J]: boxes of 16 columns x 32 rows.
+int make_in_map(fp4_ctx* ctx, CUtensorMap* map, const void* base, int64_t I, int64_t J, bool f32) {
+  EncodeTiledFn encode = reinterpret_cast<EncodeTiledFn>(ctx->encode_tiled);
+  if (!encode) return FP4_ERR_CUDA;
+  const cuuint64_t dims[2] = {cuuint64_t(J), cuuint64_t(I)};
+  const cuuint64_t strides[1] = {cuuint64_t(J) * (f32 ? 4 : 2)};
+  const cuuint32_t box[2] = {16, 32}, elem_strides[2] = {1, 1};
+  const CUresult r = encode(map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
+                            const_cast<void*>(base), dims, strides, box, elem_strides, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                            f32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? FP4_OK : FP4_ERR_CUDA;
+}
+
 struct Problem {
   CUtensorMap map_a, map_b, map_out, map_out_aux;
+  CUtensorMap map_w, map_add;       // fused epilogue (without one of them: a copy of map_out)
   GemmArgs args;
   bool fused;
 };
 
 template <int KIND, int EPI>
 int launch_kernel(int grid, cudaStream_t stream, const Problem& p, const Problem* second = nullptr) {
-  constexpr size_t kSmem = smem_bytes(KIND);
-  FP4_CUDA_TRY(cudaFuncSetAttribute(gemm_fp4_kernel<KIND, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    int(kSmem)));
+  FP4_CUDA_TRY(cudaFuncSetAttribute(gemm_fp4_kernel<KIND, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, MOST_SMEM));
   Problem none = p;
   none.args.num_m_blocks = none.args.num_n_blocks = 0;          // a second problem without tiles
   const Problem& q = second ? *second : none;
-  gemm_fp4_kernel<KIND, EPI><<<grid, num_threads(EPI), kSmem, stream>>>(p.map_a, p.map_b, p.map_out, p.map_out_aux,
-                                                                        p.args, q.map_a, q.map_b, q.map_out,
-                                                                        q.map_out_aux, q.args);
+  GemmArgs args = p.args;
+  args.smem = plan_smem(EPI, p.args.bn > q.args.bn ? p.args.bn : q.args.bn, args.has_w, args.slot_of_row != nullptr,
+                        args.out_f32 != 0);
+  const int smem = FIXED_SMEM + args.smem.stages * args.smem.stage_bytes +
+                   epi_warps(EPI) * (args.smem.out_bytes + args.smem.in_bytes);
+  gemm_fp4_kernel<KIND, EPI><<<grid, num_threads(EPI), smem, stream>>>(p.map_a, p.map_b, p.map_out, p.map_out_aux, args,
+                                                                       q.map_a, q.map_b, q.map_out, q.map_out_aux,
+                                                                       q.args, p.map_w, p.map_add);
   return FP4_OK;
 }
 
@@ -703,7 +766,8 @@ TileCost tile_cost(const Fp4GemmDesc& d, int gemm_kind, int bn) {
 }
 TileWidths choose_bn(const fp4_ctx* ctx, const Fp4GemmDesc& p, const Fp4GemmDesc* q, int gemm_kind) {
   constexpr int LEAST = 32, WIDTHS = 15;
-  const int most = tile_n(gemm_kind);
+  const bool fused = q || (p.epilogue && (p.epilogue->addend || p.epilogue->w_bf16));
+  const int most = tile_n(gemm_kind, fused ? EPI_WGRAD : EPI_PLAIN);
   TileCost costs[2][WIDTHS];
   int n = 0;
   for (int bn = most; bn >= LEAST; bn -= 16, ++n) {
@@ -776,10 +840,11 @@ int make_problem(fp4_ctx* ctx, Problem* p, const Fp4GemmDesc& d, int gemm_kind, 
   const GemmEpilogue* epi = d.epilogue;
   const bool fused = epi && (epi->addend || epi->w_bf16);
   p->fused = fused;
-  args.addend = fused ? epi->addend : nullptr;
   args.slot_of_row = fused && epi->addend ? epi->slot_of_row : nullptr;
-  args.w = fused ? static_cast<const __nv_bfloat16*>(epi->w_bf16) : nullptr;
-  args.w_aligned = !(reinterpret_cast<uintptr_t>(args.w) & 31);
+  args.has_w = fused && epi->w_bf16;
+  p->map_w = p->map_add = p->map_out;
+  if (args.has_w && (rc = make_in_map(ctx, &p->map_w, epi->w_bf16, d.I, d.J, false)) != FP4_OK) return rc;
+  if (args.slot_of_row && (rc = make_in_map(ctx, &p->map_add, epi->addend, d.I, d.J, true)) != FP4_OK) return rc;
   args.w_amax = fused ? epi->w_amax : nullptr;
   const float inv_k = fused && epi->w_bf16 ? 1.0f / epi->dge_k : 1.0f;
   args.log2_inv_k = std::log2(inv_k);
