@@ -32,6 +32,26 @@ size_t linear_scratch_bytes(int64_t M, int64_t K, int64_t N) {
   return b;
 }
 
+// Scratch of the heavy residual's dense product, forward or backward: used where the workspace has room for it.
+size_t full_scratch_bytes(int64_t M, int64_t K) {
+  const size_t f = residual_full_scratch_bytes(M, K), b = residual_full_scratch_bytes(K, M);
+  return f > b ? f : b;
+}
+
+// The least workspace that fp4_quantize / fp4_linear_fwd / fp4_linear_bwd accept.
+size_t least_workspace_bytes(int64_t M, int64_t K, int64_t N) {
+  // forward: A and W are quantised concurrently, each in its own scratch; backward: dY alone
+  size_t q = quantize_scratch_bytes(M, K) + quantize_scratch_bytes(K, N);
+  const size_t qg = quantize_scratch_bytes(M, N);
+  if (qg > q) q = qg;
+  return q + linear_scratch_bytes(M, K, N) + 4096;
+}
+
+// A residual that may hold 1 / RESIDUAL_FULL_SHARE of the activation or more is multiplied as a dense matrix.
+bool heavy_residual(const fp4_qtensor* a, int64_t M, int64_t K) {
+  return a->csr_rowptr && a->csc_colptr && a->sparse_cap * RESIDUAL_FULL_SHARE > M * K && M >= 512;
+}
+
 int check_qtensor_dense(const fp4_qtensor* q) {
   if (!q || !q->amax) return FP4_ERR_NULL;
   if (!q->codes && !q->codes_t) return FP4_ERR_NULL;
@@ -75,11 +95,7 @@ const char* fp4_status_string(int code) {
 
 size_t fp4_workspace_bytes(int64_t M, int64_t K, int64_t N) {
   if (M <= 0 || K <= 0 || N <= 0) return 0;
-  // forward: A and W are quantised concurrently, each in its own scratch; backward: dY alone
-  size_t q = quantize_scratch_bytes(M, K) + quantize_scratch_bytes(K, N);
-  const size_t qg = quantize_scratch_bytes(M, N);
-  if (qg > q) q = qg;
-  return q + linear_scratch_bytes(M, K, N) + 4096;
+  return least_workspace_bytes(M, K, N) + full_scratch_bytes(M, K);
 }
 
 int fp4_create(fp4_ctx** out, int device, size_t workspace_bytes) {
@@ -275,7 +291,7 @@ int fp4_linear_fwd(fp4_ctx* ctx, void* stream, const void* A_bf16, const void* W
     int rc = check_qtensor_sparse(savedA, n_tail);
     if (rc != FP4_OK) return rc;
   }
-  if (fp4_workspace_bytes(M, K, N) > ctx->workspace_bytes) return FP4_ERR_WORKSPACE;
+  if (least_workspace_bytes(M, K, N) > ctx->workspace_bytes) return FP4_ERR_WORKSPACE;
   // (linear_fwd_impl sets these too, but does not run when the call is replayed)
   if (!(reuse & FP4_REUSE_A)) { savedA->rows = M; savedA->cols = K; }
   if (!(reuse & FP4_REUSE_W)) { savedW->rows = K; savedW->cols = N; }
@@ -315,9 +331,14 @@ int linear_fwd_impl(fp4_ctx* ctx, cudaStream_t st, Arena arena, const void* A_bf
   float* y1 = occ ? arena.take<float>(size_t(M) * size_t(N)) : nullptr;
   char* scratch_a = reuse_a ? nullptr : arena.take<char>(quantize_scratch_bytes(M, K));
   char* scratch_w = reuse_w ? nullptr : arena.take<char>(quantize_scratch_bytes(K, N));
-  // A heavy residual (the caller's capacity says it may hold at least 1 % of the activation, alpha <=
-  // 0.995) sends its hot columns through the GEMM as a dense tail instead of per-entry gathers.
-  const bool tail_on = occ && savedA->csr_rowptr && savedA->csc_colptr &&
+  // A residual that fills a few per cent of the activation or more is multiplied as a dense matrix, ahead of the
+  // GEMM, whose epilogue adds the product.  A lighter one that still may hold 1 % (by the caller's capacity: alpha
+  // <= 0.995) sends its hot columns through the GEMM as a dense tail instead of per-entry gathers.
+  const size_t full_bytes = residual_full_scratch_bytes(M, K);
+  char* scratch_full = occ && heavy_residual(savedA, M, K) && full_bytes && arena.ok && arena.size - arena.off >= full_bytes
+                           ? arena.take<char>(full_bytes) : nullptr;
+  const bool full_on = scratch_full != nullptr;
+  const bool tail_on = occ && !full_on && savedA->csr_rowptr && savedA->csc_colptr && !heavy_residual(savedA, M, K) &&
                        savedA->sparse_cap * 100 >= M * K && M >= 512;   // a hot column holds at least 512 entries
   char* scratch_tail = tail_on ? arena.take<char>(fwd_tail_scratch_bytes(M, K, N)) : nullptr;
   if (!arena.ok) return FP4_ERR_WORKSPACE;
@@ -346,10 +367,11 @@ int linear_fwd_impl(fp4_ctx* ctx, cudaStream_t st, Arena arena, const void* A_bf
     savedA->rows = M;
     savedA->cols = K;
     // CSR on side stream 1, CSC on side stream 0 (behind W's short chain, which has ended by then)
-    // (with a dense tail: once the tail's operands are there, beside the GEMM; earlier it would hold up the
+    // (with a dense tail: once the tail's operands are there, beside the GEMM; with a heavy residual beside its
+    // product; earlier it would hold up the
     // CSR's fill, which the tail waits for: 8192 x 11008, 1 % per tail, CSR ready after 33 instead of 67 us)
     const SparseOverlap so = {ctx->side[1], ctx->ev[2], ctx->ev[3], ctx->side[0], ctx->ev[7], ctx->ev[4],
-                              tail_on ? &csc_fill : nullptr};
+                              tail_on || full_on ? &csc_fill : nullptr};
     rc = launch_quantize(ctx, st, a, A_bf16, M, K, /*scale_axis=*/0, alpha, nullptr, 0.0f, savedA, status,
                          occ && ov ? &so : nullptr);
     if (rc != FP4_OK) return rc;
@@ -369,7 +391,33 @@ int linear_fwd_impl(fp4_ctx* ctx, cudaStream_t st, Arena arena, const void* A_bf
                            gemm_kind, status, nullptr, a8, w8);
   }
   GemmTail tail = {nullptr, nullptr, nullptr};
-  const int* hot_slot_of_col = nullptr;
+  auto fill_csc_beside = [&]() {
+    FP4_CUDA_TRY(cudaEventRecord(ctx->ev[8], st));
+    FP4_CUDA_TRY(cudaStreamWaitEvent(ctx->side[0], ctx->ev[8], 0));
+    const int r = launch_csc_fill(ctx, ctx->side[0], csc_fill);
+    if (r != FP4_OK) return r;
+    FP4_CUDA_TRY(cudaEventRecord(ctx->ev[7], ctx->side[0]));
+    return FP4_OK;
+  };
+  if (full_on) {
+    if (!reuse_a && ov) {
+      FP4_CUDA_TRY(cudaStreamWaitEvent(st, ctx->ev[3], 0));
+      rc = fill_csc_beside();
+      if (rc != FP4_OK) return rc;
+    }
+    Arena fa(scratch_full, full_bytes);
+    rc = launch_residual_full(ctx, st, savedA->csr_rowptr, savedA->csr_col, savedA->csr_val, M, K, W_bf16, N, fa, y1, KC_COMP_FWD,
+                              status);
+    if (rc != FP4_OK) return rc;
+    GemmEpilogue epi = {};
+    epi.addend = y1;
+    epi.slot_of_row = savedA->csr_rowptr;              // every row has one: any vector of non-negative numbers
+    rc = launch_gemm_fp4(ctx, st, savedA->codes, savedW->codes_t, M, N, K, savedA->amax, savedW->amax, Y, out_f32, gemm_kind,
+                         status, &epi, a8, w8);
+    if (rc != FP4_OK) return rc;
+    if (!reuse_a && ov) FP4_CUDA_TRY(cudaStreamWaitEvent(st, ctx->ev[7], 0));  // savedA is complete on return
+    return FP4_OK;
+  }
   const void* kept = nullptr;
   const int* kept_end = nullptr;
   if (tail_on) {
@@ -380,15 +428,11 @@ int linear_fwd_impl(fp4_ctx* ctx, cudaStream_t st, Arena arena, const void* A_bf
       FP4_CUDA_TRY(cudaStreamWaitEvent(st, ctx->ev[4], 0));
     }
     Arena ta(scratch_tail, fwd_tail_scratch_bytes(M, K, N));
-    rc = launch_fwd_tail(ctx, st, savedA, W_bf16, savedW->amax, fp8_max(w8), ta, M, K, N, &tail, &hot_slot_of_col, &kept,
-                         &kept_end);
+    rc = launch_fwd_tail(ctx, st, savedA, W_bf16, savedW->amax, fp8_max(w8), ta, M, K, N, &tail, &kept, &kept_end);
     if (rc != FP4_OK) return rc;
     if (!reuse_a && ov) {
-      FP4_CUDA_TRY(cudaEventRecord(ctx->ev[8], st));
-      FP4_CUDA_TRY(cudaStreamWaitEvent(ctx->side[0], ctx->ev[8], 0));
-      rc = launch_csc_fill(ctx, ctx->side[0], csc_fill);
+      rc = fill_csc_beside();
       if (rc != FP4_OK) return rc;
-      FP4_CUDA_TRY(cudaEventRecord(ctx->ev[7], ctx->side[0]));
     }
   }
   rc = launch_gemm_fp4(ctx, st, savedA->codes, savedW->codes_t, M, N, K, savedA->amax, savedW->amax, y1, 1, gemm_kind,
@@ -397,7 +441,7 @@ int linear_fwd_impl(fp4_ctx* ctx, cudaStream_t st, Arena arena, const void* A_bf
   // Y = store(Y1 + (A - A_c) W): one rounding of the fp32 sum.  Needs the CSR.
   if (!reuse_a && ov) FP4_CUDA_TRY(cudaStreamWaitEvent(st, ctx->ev[3], 0));
   rc = launch_comp_fwd(ctx, st, y1, savedA->csr_rowptr, savedA->csr_col, savedA->csr_val, W_bf16, M, K, N, Y, out_f32,
-                       hot_slot_of_col, tail.count, kept, kept_end);
+                       tail.count, kept, kept_end);
   if (rc != FP4_OK) return rc;
   if (!reuse_a && ov) FP4_CUDA_TRY(cudaStreamWaitEvent(st, ctx->ev[7], 0));  // the CSC too: savedA is complete on return
   return FP4_OK;
@@ -426,7 +470,7 @@ int fp4_linear_bwd(fp4_ctx* ctx, void* stream, const void* dY_bf16, const void* 
   if (dge_on && !(dge_k > 1.0f && dge_clip > 0.0f)) return FP4_ERR_ARG;
   if (!savedA->codes_t || !savedA->amax || !savedW->codes || !savedW->amax) return FP4_ERR_NULL;
   if (!aligned16(dY_bf16) || !aligned16(W_bf16) || !aligned16(dA) || !aligned16(dW)) return FP4_ERR_ALIGN;
-  if (fp4_workspace_bytes(M, K, N) > ctx->workspace_bytes) return FP4_ERR_WORKSPACE;
+  if (least_workspace_bytes(M, K, N) > ctx->workspace_bytes) return FP4_ERR_WORKSPACE;
   CallKey key;
   std::memset(&key, 0, sizeof(key));
   key.kind = CALL_BWD;
@@ -473,8 +517,12 @@ int linear_bwd_impl(fp4_ctx* ctx, cudaStream_t st, Arena arena, const void* dY_b
   float* g2_amax = arena.take<float>(size_t(N));
   Arena comp_arena(arena.base + arena.off, comp_wgrad_scratch_bytes(M, K, N));
   arena.take<char>(comp_wgrad_scratch_bytes(M, K, N));
-  int* slot_of_col = nullptr;
+  const int* slot_of_col = nullptr;
   if (!arena.ok) return FP4_ERR_WORKSPACE;
+  const size_t full_bytes = residual_full_scratch_bytes(K, M);
+  char* scratch_full = has_comp && heavy_residual(savedA, M, K) && full_bytes &&
+                               arena.size - arena.off >= full_bytes + quantize_scratch_bytes(M, N)
+                           ? arena.take<char>(full_bytes) : nullptr;
   Arena q_arena(arena.base + arena.off, arena.size - arena.off);
   int rc;
 
@@ -486,7 +534,13 @@ int linear_bwd_impl(fp4_ctx* ctx, cudaStream_t st, Arena arena, const void* dY_b
     FP4_CUDA_TRY(cudaEventRecord(ctx->ev[5], st));
     FP4_CUDA_TRY(cudaStreamWaitEvent(sw, ctx->ev[5], 0));
   }
-  if (has_comp) {
+  if (scratch_full) {
+    Arena fa(scratch_full, full_bytes);
+    rc = launch_residual_full(ctx, sw, savedA->csc_colptr, savedA->csc_row, savedA->csc_val, K, M, dY_bf16, N, fa, comp,
+                              KC_COMP_WGRAD, status);
+    if (rc != FP4_OK) return rc;
+    slot_of_col = savedA->csc_colptr;                  // every row has one: any vector of non-negative numbers
+  } else if (has_comp) {
     const CompOverlap beside = {ctx->side[1], ctx->ev[8], ctx->ev[9]};
     rc = launch_comp_wgrad(ctx, sw, savedA, dY_bf16, comp_arena, &slot_of_col, comp, M, K, N, status,
                            ctx->overlap ? &beside : nullptr);
@@ -601,7 +655,7 @@ size_t step_host_shared_bytes(int64_t M, int64_t K, int64_t N, double alpha) {
   b += 4 * round256(cap * 4) + round256((size_t(M) + 1) * 4) + round256((size_t(K) + 1) * 4) + 3 * 256;   // sparse
   b += round256(2 * size_t(M) * 4);                                                                      // thresholds
   b += 256;                                                                                              // status
-  return b + fp4_workspace_bytes(M, K, N);
+  return b + least_workspace_bytes(M, K, N);
 }
 
 }  // namespace
@@ -612,7 +666,9 @@ size_t fp4_step_host_workspace_bytes(int64_t M, int64_t K, int64_t N, double alp
   if (M <= 0 || K <= 0 || N <= 0) return 0;
   // Sized so that the pipelined layout fits: 2 HOST_STEP_SETS slots (input sets, then output sets)
   // in the first half, everything else in the second half.
-  const size_t io = step_host_io_bytes(M, K, N), shared = step_host_shared_bytes(M, K, N, alpha);
+  const size_t io = step_host_io_bytes(M, K, N);
+  const size_t shared = step_host_shared_bytes(M, K, N, alpha) +
+                        (step_capacity(M, K, alpha) * RESIDUAL_FULL_SHARE > M * K ? full_scratch_bytes(M, K) : 0);
   const size_t slots = 4 * HOST_STEP_SETS * io;
   return (slots > 2 * shared ? slots : 2 * shared) + 1024;
 }

@@ -247,14 +247,14 @@ int launch_quantize_dual(fp4_ctx* ctx, cudaStream_t stream, Arena& arena, const 
 // y[m,:] = store( y1[m,:] + sum_{entries of row m} val * dense[col,:] )
 int launch_comp_fwd(fp4_ctx* ctx, cudaStream_t stream, const float* y1, const int32_t* rowptr,
                     const int32_t* col, const float* val, const void* w_bf16, int64_t M, int64_t K,
-                    int64_t N, void* y, int out_f32, const int* slot_of_col = nullptr,
-                    const int* tail_count = nullptr, const void* kept = nullptr, const int* kept_end = nullptr);
+                    int64_t N, void* y, int out_f32, const int* tail_count = nullptr, const void* kept = nullptr,
+                    const int* kept_end = nullptr);
 // The forward GEMM's dense tail (see GemmTail): operands built from the saved activation and the weights.
 size_t fwd_tail_scratch_bytes(int64_t M, int64_t K, int64_t N);
-// `kept_out` / `kept_end_out`: per token, the entries the tail does not cover (null for residuals too heavy to list).
+// `kept_out` / `kept_end_out`: per token, the entries the tail does not cover.
 int launch_fwd_tail(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, const void* w_bf16, const float* w_amax,
                     float w_div, Arena& scratch, int64_t M, int64_t K, int64_t N, GemmTail* tail,
-                    const int** slot_of_col_out, const void** kept_out, const int** kept_end_out);
+                    const void** kept_out, const int** kept_end_out);
 // Weight-gradient compensation: for every column k of the residual that holds entries (slot_of_col[k] >= 0),
 // comp[k, :] = sum_{entries of column k} val * dy[row, :]; the other rows of `comp` are not written.
 // Lists, slots and the dense path's buffers are carved from `scratch` (comp_wgrad_scratch_bytes); the slot
@@ -265,9 +265,21 @@ struct CompOverlap {
   cudaEvent_t classified, long_done;
 };
 int launch_comp_wgrad(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, const void* dy_bf16, Arena& scratch,
-                      int** slot_of_col_out, float* comp, int64_t M, int64_t K, int64_t N, int32_t* status,
+                      const int** slot_of_col_out, float* comp, int64_t M, int64_t K, int64_t N, int32_t* status,
                       const CompOverlap* overlap = nullptr);
 size_t comp_wgrad_scratch_bytes(int64_t M, int64_t K, int64_t N);
+
+// out[r, :] = sum_c V[r, c] dense[c, :] for a whole sparse matrix V [R x C] (CSR: ptr, idx, val), as a dense product
+// on the tensor cores (wgrad_dense_tc.cu): the residual's rows times the weights, or its columns times dY.
+// What a gather costs grows with the entries, what this costs does not: two exact BF16 terms of V at about 1.2 PFLOP/s
+// against 13 TB/s of gathered rows meet at an entry share of 2 to 3 %; from RESIDUAL_FULL_SHARE on the dense
+// product is taken (alpha <= 0.98).  `scratch` holds a slab of V's terms.
+constexpr int RESIDUAL_FULL_SHARE = 25;              // entries: at least 1 / 25 of the matrix
+constexpr int64_t FULL_SLAB_BYTES = 128 << 20;       // about what L2 holds
+size_t residual_full_scratch_bytes(int64_t R, int64_t C);
+int launch_residual_full(fp4_ctx* ctx, cudaStream_t stream, const int32_t* ptr, const int32_t* idx, const float* val, int64_t R,
+                         int64_t C, const void* dense_bf16, int64_t N, Arena& scratch, float* out, int kernel_class,
+                         int32_t* status);
 
 // Dense columns of the residual in the weight gradient, on the tensor cores (wgrad_dense_tc.cu):
 // C[s, :] = sum_m V[m, s] dY[m, :] for the s < counts[0] <= DENSE_TC_MAX dense columns, as `splits`

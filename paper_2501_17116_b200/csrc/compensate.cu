@@ -88,66 +88,6 @@ comp_fwd_kernel(const float* __restrict__ y1, const int* __restrict__ rowptr, co
   store8(y, out_f32, off, y8);
 }
 
-// The same with the entries of the hot columns left out (the GEMM's dense tail has added them):
-// slot_of_col[k] in [0, *tail_count) marks a hot column.  The lanes of a warp share the token, so
-// they read 32 entries at a time, drop the hot ones and hand the others round by shuffle, four
-// weight-row loads in flight as above; the order of the additions stays ascending.
-__global__ void __launch_bounds__(COMP_THREADS)
-comp_fwd_skip_kernel(const float* __restrict__ y1, const int* __restrict__ rowptr, const int* __restrict__ col,
-                     const float* __restrict__ val, const uint4* __restrict__ w, int M, int N, void* y, int out_f32,
-                     const int* __restrict__ slot_of_col, const int* __restrict__ tail_count) {
-  const int m = blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  const int n0 = blockIdx.y * COMP_COLS + 8 * lane;
-  if (m >= M) return;                                   // whole warps only: the shuffles below need every lane
-  const bool live = n0 < N;
-  const long long off = (long long)m * N + (live ? n0 : 0);
-  float4 a = make_float4(0, 0, 0, 0), b = a;
-  if (live) {
-    a = __ldg(reinterpret_cast<const float4*>(y1 + off));
-    b = __ldg(reinterpret_cast<const float4*>(y1 + off + 4));
-  }
-  const unsigned hot = unsigned(__ldg(tail_count));
-  const int vec_per_row = N >> 3, vcol = (live ? n0 : 0) >> 3;
-  float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  const int e1 = __ldg(&rowptr[m + 1]);
-  for (int base = __ldg(&rowptr[m]); base < e1; base += 32) {
-    const int e = base + lane;
-    int k = 0;
-    float v = 0.0f;
-    bool keep = false;
-    if (e < e1) {
-      k = __ldg(&col[e]);
-      v = __ldg(&val[e]);
-      keep = unsigned(__ldg(&slot_of_col[k])) >= hot;   // -1 (no slot) compares as a large number
-    }
-    unsigned mask = __ballot_sync(0xFFFFFFFFu, keep);
-    while (mask) {
-      int r[4];
-      float vv[4];
-      uint4 d[4];
-      int cnt = 0;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int src = mask ? __ffs(mask) - 1 : 0;
-        r[u] = __shfl_sync(0xFFFFFFFFu, k, src);
-        vv[u] = __shfl_sync(0xFFFFFFFFu, v, src);
-        if (mask) { ++cnt; mask &= mask - 1; } else vv[u] = 0.0f;
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (u < cnt) d[u] = __ldg(&w[(long long)r[u] * vec_per_row + vcol]);
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (u < cnt) fma8(acc, vv[u], d[u]);
-    }
-  }
-  if (!live) return;
-  const float y8[8] = {a.x + acc[0], a.y + acc[1], a.z + acc[2], a.w + acc[3],
-                       b.x + acc[4], b.y + acc[5], b.z + acc[6], b.w + acc[7]};
-  store8(y, out_f32, off, y8);
-}
-
 // The forward compensation when the dense tail is in use: tail_a has listed, per token, the entries
 // the tail does not cover (`kept`: column and value bits, at the token's own range of the CSR, ending
 // at kept_end[m]), so this kernel walks a plain list: one 8-byte broadcast load per entry, eight
@@ -347,7 +287,7 @@ tail_a_kernel(const int* __restrict__ rowptr, const int* __restrict__ col, const
     }
     const bool is_hot = e < e1 && unsigned(slot) < unsigned(hot);
     const bool keep = e < e1 && !is_hot;
-    if (kept) {                                          // entries the tail does not cover, in column order
+    {                                                    // entries the tail does not cover, in column order
       const unsigned km = __ballot_sync(0xFFFFFFFFu, keep);
       if (keep) kept[n_kept + __popc(km & ((1u << lane) - 1u))] = make_uint2(uint32_t(k), __float_as_uint(v));
       n_kept += __popc(km);
@@ -362,7 +302,7 @@ tail_a_kernel(const int* __restrict__ rowptr, const int* __restrict__ col, const
     row[at + 64] = hi_small;
     row[at + 128] = lo_big;
   }
-  if (kept && lane == 0) kept_end[m] = n_kept;
+  if (lane == 0) kept_end[m] = n_kept;
   if (bad) atomicExch(count, 0);
 }
 
@@ -579,16 +519,13 @@ extern "C" int fp4_l2_read_probe(void* stream, const void* buf, size_t bytes, in
 
 int launch_comp_fwd(fp4_ctx* ctx, cudaStream_t stream, const float* y1, const int32_t* rowptr, const int32_t* col,
                     const float* val, const void* w_bf16, int64_t M, int64_t, int64_t N, void* y, int out_f32,
-                    const int* slot_of_col, const int* tail_count, const void* kept, const int* kept_end) {
+                    const int* tail_count, const void* kept, const int* kept_end) {
   const dim3 grid(unsigned((M + 7) / 8), unsigned((N + COMP_COLS - 1) / COMP_COLS));
   KernelScope scope(ctx, stream, KC_COMP_FWD, 1);
   if (kept && kept_end && tail_count)
     comp_fwd_kept_kernel<<<grid, COMP_THREADS, 0, stream>>>(y1, rowptr, col, val, static_cast<const uint2*>(kept),
                                                             kept_end, static_cast<const uint4*>(w_bf16), int(M), int(N),
                                                             y, out_f32, tail_count);
-  else if (slot_of_col && tail_count)
-    comp_fwd_skip_kernel<<<grid, COMP_THREADS, 0, stream>>>(y1, rowptr, col, val, static_cast<const uint4*>(w_bf16),
-                                                            int(M), int(N), y, out_f32, slot_of_col, tail_count);
   else
     comp_fwd_kernel<<<grid, COMP_THREADS, 0, stream>>>(y1, rowptr, col, val, static_cast<const uint4*>(w_bf16), int(M),
                                                        int(N), y, out_f32);
@@ -603,9 +540,8 @@ size_t comp_wgrad_scratch_bytes(int64_t M, int64_t K, int64_t N) {
   return b;
 }
 
-// Residual entries up to which the forward lists the entries its dense tail does not cover
-// (4 % of the activation: alpha >= 0.98); heavier residuals filter inside the per-entry kernel.
-static int64_t kept_list_capacity(int64_t M, int64_t K) { return M * K / 25; }
+// Residual entries the forward with a dense tail may have to list (heavier residuals take no tail).
+static int64_t kept_list_capacity(int64_t M, int64_t K) { return M * K / RESIDUAL_FULL_SHARE; }
 
 size_t fwd_tail_scratch_bytes(int64_t M, int64_t K, int64_t N) {
   auto r256 = [](size_t b) { return (b + 255) & ~size_t(255); };
@@ -614,19 +550,18 @@ size_t fwd_tail_scratch_bytes(int64_t M, int64_t K, int64_t N) {
 }
 
 // Prepares the dense tail of the forward GEMM from the saved activation `a` (CSR, CSC column
-// pointers, row amax) and the weights; fills `tail` and hands back the slot vector and the count
+// pointers, row amax) and the weights; fills `tail` and hands back the list
 // for the per-entry kernel.  Buffers come from `scratch` (fwd_tail_scratch_bytes).
 int launch_fwd_tail(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, const void* w_bf16, const float* w_amax,
                     float w_div, Arena& scratch, int64_t M, int64_t K, int64_t N, GemmTail* tail,
-                    const int** slot_of_col_out, const void** kept_out, const int** kept_end_out) {
+                    const void** kept_out, const int** kept_end_out) {
   __half* ta = scratch.take<__half>(size_t(M) * TAIL_WIDTH);
   __half* tb = scratch.take<__half>(size_t(N) * TAIL_WIDTH);
   int* slot_of_col = scratch.take<int>(size_t(K));
   int* list_hot = scratch.take<int>(TAIL_MAX_COLS);
   int* count = scratch.take<int>(1);
-  const bool list_kept = a->sparse_cap <= kept_list_capacity(M, K);
-  uint2* kept = list_kept ? scratch.take<uint2>(size_t(kept_list_capacity(M, K))) : nullptr;
-  int* kept_end = list_kept ? scratch.take<int>(size_t(M)) : nullptr;
+  uint2* kept = scratch.take<uint2>(size_t(kept_list_capacity(M, K)));
+  int* kept_end = scratch.take<int>(size_t(M));
   if (!scratch.ok) return FP4_ERR_WORKSPACE;
   *kept_out = kept;
   *kept_end_out = kept_end;
@@ -643,12 +578,11 @@ int launch_fwd_tail(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, con
   tail->a = ta;
   tail->b = tb;
   tail->count = count;
-  *slot_of_col_out = slot_of_col;
   return FP4_OK;
 }
 
 int launch_comp_wgrad(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, const void* dy_bf16, Arena& scratch,
-                      int** slot_of_col_out, float* comp, int64_t M, int64_t K, int64_t N, int32_t* status,
+                      const int** slot_of_col_out, float* comp, int64_t M, int64_t K, int64_t N, int32_t* status,
                       const CompOverlap* overlap) {
   // lists: [K] long columns, [K] short columns, the dense columns, three counters
   int* lists = scratch.take<int>(2 * size_t(K) + DENSE_TC_MAX + 4);

@@ -1473,7 +1473,6 @@ int launch_quantize(fp4_ctx* ctx, cudaStream_t stream, Arena& arena, const void*
     }
     const uint32_t* mask32 = reinterpret_cast<const uint32_t*>(sc.mask);
     const __nv_bfloat16* xb = static_cast<const __nv_bfloat16*>(x_bf16);
-    const int strips = rows / ENC_TM;
     // The CSC's fill takes a stream of its own where the caller offers one.
     cudaStream_t sc2 = sp;
     {

@@ -33,7 +33,8 @@ constexpr int DT_NT = 256;                       // output columns per CTA
 constexpr int DT_BOX = 64 * 64 * 2;              // one 64 x 64 BF16 box: 8 KB
 constexpr int DT_DY_BYTES = (DT_NT / 64) * DT_BOX;      // 32 KB of dY per stage
 constexpr int DT_THREADS = 64 + 8 * 32;
-constexpr int DT_SMEM = 1024 + 3 * (DT_DY_BYTES + 3 * DT_BOX) + 256;   // fits 3 stages (one V box per term) or 2 (two)
+constexpr int DT_RING = 3 * (DT_DY_BYTES + 4 * DT_BOX);      // 3 stages of up to four V boxes or 2 of six
+constexpr int DT_SMEM = 1024 + DT_RING + 256;
 
 // Shared-memory matrix descriptor of an MN-major operand tile made of 64 x 64 BF16 boxes (128-byte
 // rows = 64 consecutive MN elements of one contraction index, 128-byte swizzle): groups of 8
@@ -97,27 +98,77 @@ dense_split_kernel(const int* __restrict__ colptr, const int* __restrict__ row, 
   }
 }
 
+// The whole residual (or its transpose) as a dense operand, for residuals so heavy that gathering costs more:
+// row r of Vt[term][r][c] holds the terms of the residual's row r, zeros elsewhere.  A block writes one row, in
+// segments of ROW_SEG contraction indices.  Terms 1 and 2 are written always; term 3 is zero unless a value spans
+// more than 16 bits (500 times the threshold): *third says so, and a second launch (THIRD) then writes it.
+constexpr int ROW_SEG = 8192;
+template <bool THIRD>
+__global__ void __launch_bounds__(256)
+dense_rows_kernel(const int* __restrict__ ptr, const int* __restrict__ idx, const float* __restrict__ val, int row0, int rows,
+                  int C, __nv_bfloat16* __restrict__ vt, int* __restrict__ third) {
+  __shared__ __align__(16) __nv_bfloat16 tile[THIRD ? 1 : 2][ROW_SEG];
+  if (THIRD && *third == 0) return;
+  const int r = blockIdx.x, t = threadIdx.x;
+  const int e0 = ptr[row0 + r], e1 = ptr[row0 + r + 1];
+  uint4* t4 = reinterpret_cast<uint4*>(&tile[0][0]);
+  bool any = false;
+  for (int c0 = 0; c0 < C; c0 += ROW_SEG) {
+    const int c1 = min(C, c0 + ROW_SEG);
+    for (int i = t; i < (THIRD ? 1 : 2) * ROW_SEG / 8; i += 256) t4[i] = make_uint4(0, 0, 0, 0);
+    __syncthreads();
+    for (int e = e0 + t; e < e1; e += 256) {
+      const int c = idx[e];
+      if (c < c0 || c >= c1) continue;
+      const float v = val[e];
+      const __nv_bfloat16 b1 = __float2bfloat16_rn(v);
+      const float r1 = v - __bfloat162float(b1);                 // exact
+      const __nv_bfloat16 b2 = __float2bfloat16_rn(r1);
+      const float r2 = r1 - __bfloat162float(b2);                // exact
+      if (THIRD) {
+        tile[0][c - c0] = __float2bfloat16_rn(r2);               // exact
+      } else {
+        tile[0][c - c0] = b1;
+        tile[THIRD ? 0 : 1][c - c0] = b2;
+        any |= r2 != 0.0f;
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int term = 0; term < (THIRD ? 1 : 2); ++term)
+      for (int i = t; i < (c1 - c0) / 8; i += 256)
+        *reinterpret_cast<uint4*>(vt + (size_t(THIRD ? 2 : term) * rows + r) * size_t(C) + c0 + 8 * i) =
+            *reinterpret_cast<const uint4*>(&tile[term][8 * i]);
+    __syncthreads();
+  }
+  if (!THIRD && any) *third = 1;                     // (any number of threads writes the same)
+}
+
 struct DenseTcArgs {
-  int M, N;
+  int M, N;                  // length of the contraction, output columns
   int tiles;                 // blocks of DT_NT output columns
-  int splits;                // ranges of chunks per tile
-  const int* counts;         // counts[0] = number of dense columns (device)
-  float* partial;            // [splits][DENSE_TC_MAX][N]
+  int splits;                // ranges of chunks per tile; FULL: blocks of 128 rows
+  int vt_rows;               // rows of a term of Vt
+  const int* counts;         // counts[0] = number of dense columns (device); FULL: whether the third term is needed
+  float* partial;            // [splits][DENSE_TC_MAX][N]; FULL: [vt_rows][N]
   int32_t* status;
 };
 
+// FULL: every row of the result, in blocks of 128; else the dense columns' rows, in ranges of the contraction.
+template <bool FULL>
 __global__ void __launch_bounds__(DT_THREADS, 1)
 comp_wgrad_dense_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CUtensorMap map_vt,
                            const __grid_constant__ DenseTcArgs args) {
   extern __shared__ uint8_t smem_raw[];
-  const int n_dense = min(__ldg(args.counts), DENSE_TC_MAX);
+  const int n_dense = FULL ? DENSE_TC_MAX : min(__ldg(args.counts), DENSE_TC_MAX);
   if (n_dense == 0) return;                               // uniform: nothing allocated yet
+  const int terms = FULL && *args.counts == 0 ? 2 : 3;
   const int nb = (n_dense + 63) / 64;                     // 64-row boxes of V per term
-  const int stages = nb == 1 ? 3 : 2;
-  const uint32_t v_bytes = uint32_t(3 * nb * DT_BOX);
+  const int stages = nb == 1 || terms == 2 ? 3 : 2;
+  const uint32_t v_bytes = uint32_t(terms * nb * DT_BOX);
   const uint32_t stage_bytes = uint32_t(DT_DY_BYTES) + v_bytes;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* smem_misc = smem + 3 * (DT_DY_BYTES + 3 * DT_BOX);
+  uint8_t* smem_misc = smem + DT_RING;
   uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem_misc);
   uint64_t* empty_bar = full_bar + 3;
   uint64_t* acc_full = empty_bar + 3;
@@ -129,8 +180,9 @@ comp_wgrad_dense_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __g
   const int warp = __shfl_sync(0xFFFFFFFFu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int tile = blockIdx.x % args.tiles, split = blockIdx.x / args.tiles;
   const int chunks_total = (args.M + DT_CHUNK - 1) / DT_CHUNK;
-  const int c_begin = int((long long)chunks_total * split / args.splits);
-  const int c_end = int((long long)chunks_total * (split + 1) / args.splits);
+  const int c_begin = FULL ? 0 : int((long long)chunks_total * split / args.splits);
+  const int c_end = FULL ? chunks_total : int((long long)chunks_total * (split + 1) / args.splits);
+  const int s0 = FULL ? split * DENSE_TC_MAX : 0;         // first row of Vt
   const int n_chunks = c_end - c_begin;
   const int n0 = tile * DT_NT;
 
@@ -174,10 +226,10 @@ comp_wgrad_dense_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __g
         mbar_arrive_expect_tx(&full_bar[stage], stage_bytes);
         for (int j = 0; j < DT_NT / 64; ++j)                    // dY: box j = columns n0 + 64 j .. + 63, 64 tokens
           tma_load_2d(dst + j * DT_BOX, &map_dy, &full_bar[stage], n0 + 64 * j, m0);
-        for (int t = 0; t < 3; ++t)                             // V terms: 64 tokens x 64 rows per box
+        for (int t = 0; t < terms; ++t)                         // V terms: 64 tokens x 64 rows per box
           for (int b = 0; b < nb; ++b)
             tma_load_2d(dst + DT_DY_BYTES + (t * nb + b) * DT_BOX, &map_vt, &full_bar[stage], m0,
-                        t * DENSE_TC_MAX + 64 * b);
+                        t * args.vt_rows + s0 + 64 * b);
         ++fills;
         if (++stage == stages) { stage = 0; phase ^= 1u; }
       }
@@ -220,6 +272,7 @@ comp_wgrad_dense_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __g
               const uint64_t a_desc = make_smem_desc_mn(dy_addr + uint32_t(2 * h * DT_BOX + k * 2048), DT_BOX);
 #pragma unroll
               for (int t = 0; t < 3; ++t) {
+                if (FULL && t >= terms) break;
                 const uint64_t b_desc = make_smem_desc(v_addr + uint32_t(t * nb * DT_BOX + k * 32));
                 mma_f16(d_tmem, a_desc, b_desc, idesc, (half | k | t) != 0 ? 1u : 0u);
               }
@@ -274,7 +327,7 @@ comp_wgrad_dense_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __g
     }
     const int n = n0 + 128 * h + 32 * quarter + lane;
     if (!gave_up && n < args.N) {
-      float* dst = args.partial + size_t(split) * DENSE_TC_MAX * size_t(args.N) + n;
+      float* dst = args.partial + size_t(split) * DENSE_TC_MAX * size_t(args.N) + n;     // FULL: rows s0 ..
 #pragma unroll
       for (int s = 0; s < DENSE_TC_MAX; ++s)
         if (s < n_dense) dst[size_t(s) * size_t(args.N)] = run[s];
@@ -350,11 +403,57 @@ int launch_comp_wgrad_dense_tc(fp4_ctx* ctx, cudaStream_t stream, const fp4_qten
   args.N = int(N);
   args.tiles = int((N + DT_NT - 1) / DT_NT);
   args.splits = splits;
+  args.vt_rows = DENSE_TC_MAX;
   args.counts = counts;
   args.partial = partial;
   args.status = status;
-  FP4_CUDA_TRY(cudaFuncSetAttribute(comp_wgrad_dense_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DT_SMEM));
-  comp_wgrad_dense_tc_kernel<<<unsigned(args.tiles * splits), DT_THREADS, DT_SMEM, stream>>>(map_dy, map_vt, args);
+  FP4_CUDA_TRY(cudaFuncSetAttribute(comp_wgrad_dense_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, DT_SMEM));
+  comp_wgrad_dense_tc_kernel<false><<<unsigned(args.tiles * splits), DT_THREADS, DT_SMEM, stream>>>(map_dy, map_vt, args);
+  FP4_CUDA_TRY(cudaGetLastError());
+  return FP4_OK;
+}
+
+// Rows of the result that one slab of Vt holds (a multiple of 128).
+static int64_t full_slab_rows(int64_t R, int64_t C) {
+  const int64_t fit = FULL_SLAB_BYTES / (6 * C) / 128 * 128;
+  return fit >= R ? R : fit;
+}
+
+size_t residual_full_scratch_bytes(int64_t R, int64_t C) {
+  const int64_t rows = full_slab_rows(R, C);
+  return rows < 128 ? 0 : ((size_t(6) * size_t(rows) * size_t(C) + 255) & ~size_t(255)) + 256;
+}
+
+int launch_residual_full(fp4_ctx* ctx, cudaStream_t stream, const int32_t* ptr, const int32_t* idx, const float* val, int64_t R,
+                         int64_t C, const void* dense_bf16, int64_t N, Arena& scratch, float* out, int kernel_class,
+                         int32_t* status) {
+  const int64_t slab = full_slab_rows(R, C);
+  __nv_bfloat16* vt = scratch.take<__nv_bfloat16>(size_t(3) * size_t(slab) * size_t(C));
+  int* third = scratch.take<int>(1);
+  if (!scratch.ok) return FP4_ERR_WORKSPACE;
+  CUtensorMap map_dense, map_vt;
+  int rc = make_bf16_map(ctx, &map_dense, dense_bf16, C, N);
+  if (rc != FP4_OK) return rc;
+  FP4_CUDA_TRY(cudaFuncSetAttribute(comp_wgrad_dense_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, DT_SMEM));
+  FP4_CUDA_TRY(cudaMemsetAsync(third, 0, 4, stream));
+  KernelScope scope(ctx, stream, kernel_class, 3 * int((R + slab - 1) / slab));
+  for (int64_t r0 = 0; r0 < R; r0 += slab) {
+    const int64_t rows = R - r0 < slab ? R - r0 : slab;
+    rc = make_bf16_map(ctx, &map_vt, vt, 3 * rows, C);
+    if (rc != FP4_OK) return rc;
+    dense_rows_kernel<false><<<unsigned(rows), 256, 0, stream>>>(ptr, idx, val, int(r0), int(rows), int(C), vt, third);
+    dense_rows_kernel<true><<<unsigned(rows), 256, 0, stream>>>(ptr, idx, val, int(r0), int(rows), int(C), vt, third);
+    DenseTcArgs args;
+    args.M = int(C);
+    args.N = int(N);
+    args.tiles = int((N + DT_NT - 1) / DT_NT);
+    args.splits = int(rows / DENSE_TC_MAX);
+    args.vt_rows = int(rows);
+    args.counts = third;
+    args.partial = out + size_t(r0) * size_t(N);
+    args.status = status;
+    comp_wgrad_dense_tc_kernel<true><<<unsigned(args.tiles * args.splits), DT_THREADS, DT_SMEM, stream>>>(map_dense, map_vt, args);
+  }
   FP4_CUDA_TRY(cudaGetLastError());
   return FP4_OK;
 }

@@ -417,3 +417,38 @@ def test_weights_on_a_16_byte_boundary(lib, M, K, N):
     assert ctx.read_status() == 0
     assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
     ctx.close()
+
+
+@pytest.mark.parametrize("M,K,N,alpha,wide", [(512, 640, 384, 0.97, False), (512, 256, 128, 0.9, True), (640, 8320, 256, 0.95, True),
+                                              (16384, 1408, 384, 0.97, False), (1408, 16384, 128, 0.97, True)])
+def test_heavy_residual_as_a_dense_product(lib, M, K, N, alpha, wide):
+    """More than 4 % of the activation in the residual: the tensor cores multiply it whole (several slabs of rows,
+    rows longer than a segment, values that need a third BF16 term).  Against the per-entry kernels, which a
+    context without room for the dense operand uses; either differs from the exact sum by at most
+    4e-6 sum |residual| |dense|."""
+    gen = torch.Generator("cuda").manual_seed(M + K)
+    A = torch.randn((M, K), device="cuda", generator=gen)
+    if wide:
+        A *= torch.where(torch.rand((M, K), device="cuda", generator=gen) < 0.001, 3000.0, 1.0)
+    A = A.to(torch.bfloat16)
+    W = (torch.randn((K, N), device="cuda", generator=gen) * 0.02).to(torch.bfloat16)
+    dY = (torch.randn((M, N), device="cuda", generator=gen) * 1e-3).to(torch.bfloat16)
+    size = int(lib.load_library().fp4_workspace_bytes(M, K, N))
+    room, tight = lib.Context(0, size), lib.Context(0, size - 4096)
+    out = []
+    for c in (room, tight):
+        y, sa, sw = lib.fp4_linear_fwd(c, A, W, alpha, out_f32=True)
+        da, dw = lib.fp4_linear_bwd(c, dY, W, sa, sw, out_f32=True, dge_on=False)
+        torch.cuda.synchronize()
+        assert c.read_status() == 0
+        out.append((y, da, dw, sa))
+    lo, hi = out[0][3].thresholds.tolist()
+    res = (A.float() - A.float().clamp(lo, hi)).abs().double()
+    assert float((res > 0).double().mean()) > 0.04
+    (y, da, dw, _), (y1, da1, dw1, _) = out
+    assert torch.equal(da, da1)
+    # the two sums of the outputs' branches are fp32: 2^-23 of the larger value on top
+    assert bool(((y - y1).abs().double() <= 2 * 4e-6 * (res @ W.double().abs()) + 2.4e-7 * y.abs() + 1e-30).all())
+    assert bool(((dw - dw1).abs().double() <= 2 * 4e-6 * (res.T @ dY.double().abs()) + 2.4e-7 * dw.abs() + 1e-30).all())
+    room.close()
+    tight.close()
