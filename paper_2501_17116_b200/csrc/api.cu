@@ -47,9 +47,16 @@ size_t least_workspace_bytes(int64_t M, int64_t K, int64_t N) {
   return q + linear_scratch_bytes(M, K, N) + 4096;
 }
 
-// A residual that may hold 1 / RESIDUAL_FULL_SHARE of the activation or more is multiplied as a dense matrix.
+// A residual that may hold 1 / RESIDUAL_FULL_SHARE of the activation or more takes no dense tail ...
 bool heavy_residual(const fp4_qtensor* a, int64_t M, int64_t K) {
   return a->csr_rowptr && a->csc_colptr && a->sparse_cap * RESIDUAL_FULL_SHARE > M * K && M >= 512;
+}
+// ... and is multiplied as a dense matrix [R x C] (times [C x N]) unless the gathers take less time: small
+// products do not fill the chip (512 x 1024 x 1024 at 6 %: 11 us of gathers, 25 us).  In ns: 13 TB/s of gathered
+// rows; 1.9 us per 128 contraction indices of a 128 x 256 tile, one tile per SM at a time.
+bool full_product_pays(const fp4_ctx* ctx, const fp4_qtensor* a, int64_t R, int64_t C, int64_t N) {
+  const int64_t tiles = (R / 128) * ((N + 255) / 256), rounds = (tiles + ctx->num_sms - 1) / ctx->num_sms;
+  return rounds * (C / 128 * 1900 + 4000) + 6000 < a->sparse_cap * N / 6500 + 5000;
 }
 
 int check_qtensor_dense(const fp4_qtensor* q) {
@@ -335,7 +342,7 @@ int linear_fwd_impl(fp4_ctx* ctx, cudaStream_t st, Arena arena, const void* A_bf
   // GEMM, whose epilogue adds the product.  A lighter one that still may hold 1 % (by the caller's capacity: alpha
   // <= 0.995) sends its hot columns through the GEMM as a dense tail instead of per-entry gathers.
   const size_t full_bytes = residual_full_scratch_bytes(M, K);
-  char* scratch_full = occ && heavy_residual(savedA, M, K) && full_bytes && arena.ok && arena.size - arena.off >= full_bytes
+  char* scratch_full = occ && heavy_residual(savedA, M, K) && full_product_pays(ctx, savedA, M, K, N) && full_bytes && arena.ok && arena.size - arena.off >= full_bytes
                            ? arena.take<char>(full_bytes) : nullptr;
   const bool full_on = scratch_full != nullptr;
   const bool tail_on = occ && !full_on && savedA->csr_rowptr && savedA->csc_colptr && !heavy_residual(savedA, M, K) &&
@@ -520,7 +527,7 @@ int linear_bwd_impl(fp4_ctx* ctx, cudaStream_t st, Arena arena, const void* dY_b
   const int* slot_of_col = nullptr;
   if (!arena.ok) return FP4_ERR_WORKSPACE;
   const size_t full_bytes = residual_full_scratch_bytes(K, M);
-  char* scratch_full = has_comp && heavy_residual(savedA, M, K) && full_bytes &&
+  char* scratch_full = has_comp && heavy_residual(savedA, M, K) && full_product_pays(ctx, savedA, K, M, N) && full_bytes &&
                                arena.size - arena.off >= full_bytes + quantize_scratch_bytes(M, N)
                            ? arena.take<char>(full_bytes) : nullptr;
   Arena q_arena(arena.base + arena.off, arena.size - arena.off);

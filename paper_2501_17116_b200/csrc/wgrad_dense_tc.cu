@@ -55,6 +55,13 @@ __device__ __forceinline__ uint32_t idesc_dense(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (uint32_t(n >> 3) << 17) | (uint32_t(128 >> 4) << 24);
 }
 
+// The same product with the operands in the other places, for whole residuals: A = Vt (K-major, M = 128 rows of the
+// result), B = the dense matrix (MN-major, N = 256).  An instruction of 128 x 256 x 16 reads 12 KB of shared memory in
+// the 131 cycles it takes, one of 128 x 128 x 16 8 KB in 65: more than the port gives beside the copies.
+__device__ __forceinline__ uint32_t idesc_full() {
+  return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | (uint32_t(DT_NT >> 3) << 17) | (uint32_t(128 >> 4) << 24);
+}
+
 // Vt[term][s][m]: the three BF16 terms of the dense columns' residual values, zero where a token has
 // no entry.  A block owns SPLIT_TOK tokens of one column: it finds their entries in the column's list (one
 // sample per thread brackets the first one), scatters them into a shared tile and writes that out as whole
@@ -253,7 +260,7 @@ comp_wgrad_dense_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __g
       int acc = 0;
       uint32_t acc_phase = 0;
       bool ok = true;
-      const uint32_t idesc = idesc_dense(64 * nb);
+      const uint32_t idesc = FULL ? idesc_full() : idesc_dense(64 * nb);
       for (int c = 0; c < n_chunks && ok; ++c) {
         ok = mbar_wait(&acc_empty[acc], acc_phase ^ 1u, abort_flag, args.status);
         if (!ok) break;
@@ -264,6 +271,18 @@ comp_wgrad_dense_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __g
           tc_fence_after();
           const uint32_t dy_addr = smem_u32(smem + stage * stage_bytes);
           const uint32_t v_addr = dy_addr + DT_DY_BYTES;
+          if (FULL) {
+            const uint32_t d_tmem = tmem_base + uint32_t(acc * 256);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {                       // 16 contraction indices per instruction
+              const uint64_t b_desc = make_smem_desc_mn(dy_addr + uint32_t(k * 2048), DT_BOX);
+#pragma unroll
+              for (int t = 0; t < 3; ++t)
+                if (t < terms)
+                  mma_f16(d_tmem, make_smem_desc(v_addr + uint32_t(t * 2 * DT_BOX + k * 32)), b_desc, idesc,
+                          (half | k | t) != 0 ? 1u : 0u);
+            }
+          } else
 #pragma unroll
           for (int h = 0; h < 2; ++h) {                         // output columns n0 + 128 h .. + 127
             const uint32_t d_tmem = tmem_base + uint32_t(acc * 256 + h * 128);
@@ -272,7 +291,6 @@ comp_wgrad_dense_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __g
               const uint64_t a_desc = make_smem_desc_mn(dy_addr + uint32_t(2 * h * DT_BOX + k * 2048), DT_BOX);
 #pragma unroll
               for (int t = 0; t < 3; ++t) {
-                if (FULL && t >= terms) break;
                 const uint64_t b_desc = make_smem_desc(v_addr + uint32_t(t * nb * DT_BOX + k * 32));
                 mma_f16(d_tmem, a_desc, b_desc, idesc, (half | k | t) != 0 ? 1u : 0u);
               }
@@ -296,7 +314,8 @@ comp_wgrad_dense_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __g
     }
   } else {
     // ------------------------------------------------------------------ epilogue -----------
-    // Warp (h, q) owns output columns n0 + 128 h + 32 q .. + 31 (one per lane) and all dense rows.
+    // Warp (h, q) owns output columns n0 + 128 h + 32 q .. + 31 (one per lane) and all dense rows; FULL: rows
+    // s0 + 32 q .. + 31 (one per lane) and output columns n0 + 128 h .. + 127.
     const int quarter = warp & 3;
     const int h = (warp - 2) >> 2;
     float run[DENSE_TC_MAX];
@@ -325,9 +344,16 @@ comp_wgrad_dense_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __g
       if (lane == 0) mbar_arrive(&acc_empty[acc]);
       if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
-    const int n = n0 + 128 * h + 32 * quarter + lane;
-    if (!gave_up && n < args.N) {
-      float* dst = args.partial + size_t(split) * DENSE_TC_MAX * size_t(args.N) + n;     // FULL: rows s0 ..
+    const int n = FULL ? n0 + 128 * h : n0 + 128 * h + 32 * quarter + lane;
+    if (FULL) {
+      if (!gave_up && n < args.N) {                       // (N is a multiple of 128)
+        float4* dst = reinterpret_cast<float4*>(args.partial + size_t(s0 + 32 * quarter + lane) * size_t(args.N) + n);
+#pragma unroll
+        for (int j = 0; j < DENSE_TC_MAX / 4; ++j)
+          dst[j] = make_float4(run[4 * j], run[4 * j + 1], run[4 * j + 2], run[4 * j + 3]);
+      }
+    } else if (!gave_up && n < args.N) {
+      float* dst = args.partial + size_t(split) * DENSE_TC_MAX * size_t(args.N) + n;
 #pragma unroll
       for (int s = 0; s < DENSE_TC_MAX; ++s)
         if (s < n_dense) dst[size_t(s) * size_t(args.N)] = run[s];

@@ -419,8 +419,8 @@ def test_weights_on_a_16_byte_boundary(lib, M, K, N):
     ctx.close()
 
 
-@pytest.mark.parametrize("M,K,N,alpha,wide", [(512, 640, 384, 0.97, False), (512, 256, 128, 0.9, True), (640, 8320, 256, 0.95, True),
-                                              (16384, 1408, 384, 0.97, False), (1408, 16384, 128, 0.97, True)])
+@pytest.mark.parametrize("M,K,N,alpha,wide", [(1024, 1280, 2176, 0.97, False), (512, 256, 2176, 0.9, True), (640, 8320, 1152, 0.95, True),
+                                              (16384, 1408, 1152, 0.97, False), (1408, 16384, 1152, 0.97, True)])
 def test_heavy_residual_as_a_dense_product(lib, M, K, N, alpha, wide):
     """More than 4 % of the activation in the residual: the tensor cores multiply it whole (several slabs of rows,
     rows longer than a segment, values that need a third BF16 term).  Against the per-entry kernels, which a
