@@ -37,6 +37,30 @@ __device__ __forceinline__ int float_to_ordered(float f) {
 __device__ __forceinline__ float ordered_to_float(int k) {
   return __int_as_float(k ^ ((k >> 31) & 0x7FFFFFFF));
 }
+// Two fp32 numbers in a register pair: one instruction multiplies or fuses both (each rounded as usual).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// max(|m|, |a|, |b|); a NaN wins
+__device__ __forceinline__ float absmax3(float m, float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(m), "f"(fabsf(a)), "f"(fabsf(b)));
+  return r;
+}
 __device__ __forceinline__ float bf16_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
 
@@ -640,8 +664,8 @@ __global__ void descale_kernel(const float* __restrict__ amax, int n, float div,
 struct AbsmaxArgs {
   const uint4* x;
   int rows, cols;
-  const float* pre_col;         // multiplies along columns before the row-wise maximum (or null)
-  const float* pre_row;         // multiplies along rows before the column-wise maximum (or null)
+  const float* pre_col;         // PRE: multiplies along columns before the row-wise maximum
+  const float* pre_row;         // PRE: multiplies along rows before the column-wise maximum
   float pre_col_div, pre_row_div;   // > 0: the vector holds amax values: use amax / div (6 or 448) and store it
   float* d_col_out;             // dual mode: the de-scale vectors actually used, for the encoder
   float* d_row_out;
@@ -650,74 +674,191 @@ struct AbsmaxArgs {
   int32_t* status;              // FP4_DEV_NONFINITE is raised when a maximum is infinite or NaN
 };
 
-// Tile of 64 rows x 256 columns per block, same thread mapping as the encoder: warp w owns rows
-// 8w..8w+7, lane l the 8 columns 8l..8l+7.
+// Without a prescale: maxima of packed BF16 magnitudes (a NaN wins and is seen).  Tile of 64 rows x 256 columns per
+// block, same thread mapping as the encoder: warp w owns rows 8w..8w+7, lane l the 8 columns 8l..8l+7.  It needs no
+// scales and few registers, and many short blocks keep HBM busy (13824 x 13824, columns: 53 us, 7.1 TB/s).
 template <int MODE>
 __global__ void __launch_bounds__(ENC_THREADS)
 absmax_tile_kernel(const AbsmaxArgs a) {
-  __shared__ float s_pcol[ENC_TK];
-  __shared__ float s_prow[ENC_TM];
   __shared__ uint32_t s_cmax[8][ENC_TK];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int row0 = blockIdx.y * ENC_TM, col0 = blockIdx.x * ENC_TK;
+  const int row0 = blockIdx.y * ENC_TM + 8 * warp, col = blockIdx.x * ENC_TK + 8 * lane;
   const int vec_per_row = a.cols >> 3;
   constexpr bool want_rows = MODE != MODE_COLS, want_cols = MODE != MODE_ROWS;
-  if (want_rows && a.pre_col) {
-    const int c = col0 + tid;
-    if (c < a.cols) {
-      const float v = __ldg(&a.pre_col[c]);
-      s_pcol[tid] = a.pre_col_div > 0.0f ? __fdiv_rn(v, a.pre_col_div) : v;
-      if (a.d_col_out && blockIdx.y == 0) a.d_col_out[c] = s_pcol[tid];
-    }
-  }
-  if (want_cols && a.pre_row && tid < ENC_TM) {
-    const float v = __ldg(&a.pre_row[row0 + tid]);
-    s_prow[tid] = a.pre_row_div > 0.0f ? __fdiv_rn(v, a.pre_row_div) : v;
-    if (a.d_row_out && blockIdx.x == 0) a.d_row_out[row0 + tid] = s_prow[tid];
-  }
-  __syncthreads();
-  const int col = col0 + 8 * lane;
-  const bool in_cols = col < a.cols;
   uint4 v[8];
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
     v[r] = make_uint4(0, 0, 0, 0);
-    if (in_cols) v[r] = __ldg(&a.x[(long long)(row0 + 8 * warp + r) * vec_per_row + (col >> 3)]);
+    if (col < a.cols) v[r] = __ldg(&a.x[(long long)(row0 + r) * vec_per_row + (col >> 3)]);
   }
-  float pc[8];
+  __nv_bfloat162 cmax[4];
 #pragma unroll
-  for (int c = 0; c < 8; ++c) pc[c] = (want_rows && a.pre_col && in_cols) ? s_pcol[8 * lane + c] : 1.0f;
-  // maxima as unsigned bit patterns of |x|: they order like the numbers, and a NaN (which fmaxf
-  // would drop) ends up above infinity and is seen
-  uint32_t cm[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  for (int q = 0; q < 4; ++q) cmax[q] = __float2bfloat162_rn(0.0f);
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
     const uint32_t w[4] = {v[r].x, v[r].y, v[r].z, v[r].w};
-    const float pr = (want_cols && a.pre_row) ? s_prow[8 * warp + r] : 1.0f;
-    uint32_t rm = 0;
+    __nv_bfloat162 m[4];
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const float f = (c & 1) ? bf16_hi(w[c >> 1]) : bf16_lo(w[c >> 1]);
-      if (want_rows) rm = max(rm, __float_as_uint(fabsf(a.pre_col ? __fmul_rn(f, pc[c]) : f)));
-      if (want_cols) cm[c] = max(cm[c], __float_as_uint(fabsf(a.pre_row ? __fmul_rn(f, pr) : f)));
+    for (int q = 0; q < 4; ++q) m[q] = __habs2(*reinterpret_cast<const __nv_bfloat162*>(&w[q]));
+    if (want_cols) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) cmax[q] = __hmax2_nan(cmax[q], m[q]);
     }
     if (want_rows) {
-      const uint32_t g = __reduce_max_sync(0xFFFFFFFFu, rm);
+      const __nv_bfloat162 t = __hmax2_nan(__hmax2_nan(m[0], m[1]), __hmax2_nan(m[2], m[3]));
+      const uint32_t bits = *reinterpret_cast<const uint32_t*>(&t);
+      const uint32_t g = __reduce_max_sync(0xFFFFFFFFu, max(bits << 16, bits & 0x7FFF0000u));
       if (lane == 0) {
-        atomicMax(&a.amax_rows[row0 + 8 * warp + r], g);
+        atomicMax(&a.amax_rows[row0 + r], g);
         if (g >= 0x7F800000u && a.status) atomicOr(a.status, FP4_DEV_NONFINITE);
       }
     }
   }
   if (want_cols) {
 #pragma unroll
-    for (int c = 0; c < 8; ++c) s_cmax[warp][8 * lane + c] = cm[c];
+    for (int q = 0; q < 4; ++q) {
+      const uint32_t bits = *reinterpret_cast<const uint32_t*>(&cmax[q]);
+      s_cmax[warp][8 * lane + 2 * q] = bits << 16;
+      s_cmax[warp][8 * lane + 2 * q + 1] = bits & 0xFFFF0000u;
+    }
     __syncthreads();
     uint32_t m = 0;
 #pragma unroll
     for (int w8 = 0; w8 < 8; ++w8) m = max(m, s_cmax[w8][tid]);
-    if (col0 + tid < a.cols) {
-      atomicMax(&a.amax_cols[col0 + tid], m);
+    const int c = blockIdx.x * ENC_TK + tid;
+    if (c < a.cols) {
+      atomicMax(&a.amax_cols[c], m);
+      if (m >= 0x7F800000u && a.status) atomicOr(a.status, FP4_DEV_NONFINITE);
+    }
+  }
+}
+
+// With a prescale: a block walks down a strip of 256 columns, 32 rows per step: warp w owns rows 4w..4w+3 of a step, lane l the 8
+// columns 8l..8l+7.  Steps travel to shared memory (cp.async), two in flight while one is looked at; every lane reads
+// only what it copied itself.  The grid is one wave of blocks, four per SM.  (Blocks that loaded one tile each, scales
+// first, spent two thirds of their time waiting for it: dY of 8192 x 5120, both axes, 25 us, 18 now; 13824 x 5120
+// 45 -> 30.)  Maxima of three, products two at a time; a NaN wins and is seen.
+constexpr int AB_ROWS = 32, AB_STAGES = 3;
+template <int MODE>
+__global__ void __launch_bounds__(ENC_THREADS, 4)
+absmax_strip_kernel(const AbsmaxArgs a) {
+  __shared__ __align__(16) uint4 s_buf[AB_STAGES][4][ENC_THREADS];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int col = blockIdx.x * ENC_TK + 8 * lane;
+  const bool in_cols = col < a.cols;
+  const int vec_per_row = a.cols >> 3;
+  constexpr bool want_rows = MODE != MODE_COLS, want_cols = MODE != MODE_ROWS;
+  const int steps = a.rows / AB_ROWS;
+  const int st0 = int((long long)steps * blockIdx.y / gridDim.y), st1 = int((long long)steps * (blockIdx.y + 1) / gridDim.y);
+  auto request = [&](int st) {
+    if (in_cols && st < st1) {
+      const uint4* px = a.x + (long long)(AB_ROWS * st + 4 * warp) * vec_per_row + (col >> 3);
+      const uint32_t slot = uint32_t(__cvta_generic_to_shared(&s_buf[(st - st0) % AB_STAGES][0][tid]));
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(slot + uint32_t(r * ENC_THREADS * 16)),
+                     "l"(px + (long long)r * vec_per_row)
+                     : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  request(st0);
+  request(st0 + 1);
+  f32x2 pc[4];
+  if (want_rows) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float p[2] = {0.0f, 0.0f};
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        if (in_cols) {
+          const float v = __ldg(&a.pre_col[col + 2 * q + h]);
+          p[h] = a.pre_col_div > 0.0f ? __fdiv_rn(v, a.pre_col_div) : v;
+          if (a.d_col_out && blockIdx.y == 0 && warp == 0) a.d_col_out[col + 2 * q + h] = p[h];
+        }
+      pc[q] = pack2(p[0], p[1]);
+    }
+  }
+  float cmax[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  float prow = 0.0f;                                  // lane r: prescale of the step's row r (r = lane mod 4)
+  auto fetch_prow = [&](int st) {
+    if (want_cols && st < st1) prow = __ldg(&a.pre_row[AB_ROWS * st + 4 * warp + (lane & 3)]);
+  };
+  fetch_prow(st0);
+  for (int st = st0; st < st1; ++st) {
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    const int row = AB_ROWS * st + 4 * warp;
+    const uint4* slot = &s_buf[(st - st0) % AB_STAGES][0][tid];
+    uint4 v[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) v[r] = in_cols ? slot[r * ENC_THREADS] : make_uint4(0, 0, 0, 0);
+    request(st + 2);
+    float pr = prow;
+    if (want_cols) {
+      if (a.pre_row_div > 0.0f) pr = __fdiv_rn(pr, a.pre_row_div);
+      if (a.d_row_out && blockIdx.x == 0 && lane < 4) a.d_row_out[row + lane] = pr;
+      fetch_prow(st + 1);
+    }
+    uint32_t rm[4];                                   // bits of the maxima: they order like the numbers
+#pragma unroll
+    for (int r = 0; r < 4; r += 2) {                // two rows at a time
+      const uint32_t w[2][4] = {{v[r].x, v[r].y, v[r].z, v[r].w}, {v[r + 1].x, v[r + 1].y, v[r + 1].z, v[r + 1].w}};
+      float rmax[2] = {0.0f, 0.0f};
+      f32x2 p[2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+        if (want_cols) {
+          const float t = __shfl_sync(0xFFFFFFFFu, pr, r + i);
+          p[i] = pack2(t, t);
+        }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        float lo[2], hi[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const f32x2 x = pack2(bf16_lo(w[i][q]), bf16_hi(w[i][q]));
+          if (want_rows) {
+            float f, g;
+            unpack2(mul2(x, pc[q]), f, g);
+            rmax[i] = absmax3(rmax[i], f, g);
+          }
+          if (want_cols) unpack2(mul2(x, p[i]), lo[i], hi[i]);
+        }
+        if (want_cols) {
+          cmax[2 * q] = absmax3(cmax[2 * q], lo[0], lo[1]);
+          cmax[2 * q + 1] = absmax3(cmax[2 * q + 1], hi[0], hi[1]);
+        }
+      }
+      rm[r] = __float_as_uint(rmax[0]);
+      rm[r + 1] = __float_as_uint(rmax[1]);
+    }
+    if (want_rows) {
+      // four reductions over the warp; lane r keeps row r's
+      uint32_t g = 0;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const uint32_t t = __reduce_max_sync(0xFFFFFFFFu, rm[r]);
+        if (lane == r) g = t;
+      }
+      if (lane < 4) {
+        atomicMax(&a.amax_rows[row + lane], g);
+        if (g >= 0x7F800000u && a.status) atomicOr(a.status, FP4_DEV_NONFINITE);
+      }
+    }
+  }
+  if (want_cols) {
+    uint32_t* s_cmax = reinterpret_cast<uint32_t*>(&s_buf[0][0][0]);      // [8][ENC_TK]
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < 8; ++c) s_cmax[warp * ENC_TK + 8 * lane + c] = __float_as_uint(cmax[c]);
+    __syncthreads();
+    uint32_t m = 0;
+#pragma unroll
+    for (int w8 = 0; w8 < 8; ++w8) m = max(m, s_cmax[w8 * ENC_TK + tid]);
+    const int c = blockIdx.x * ENC_TK + tid;
+    if (c < a.cols) {
+      atomicMax(&a.amax_cols[c], m);
       if (m >= 0x7F800000u && a.status) atomicOr(a.status, FP4_DEV_NONFINITE);
     }
   }
@@ -733,7 +874,7 @@ absmax_tile_kernel(const AbsmaxArgs a) {
 // have a zero last bit, so no other value crosses one.  The conversion's "-0" nibble is cleared.
 __device__ __forceinline__ float nudge(float v) {
   const uint32_t u = __float_as_uint(v);
-  return __uint_as_float((u - (u >> 31)) | 1u);
+  return __uint_as_float((u + uint32_t(int(u) >> 31)) | 1u);
 }
 __device__ __forceinline__ uint32_t encode8(const float (&v)[8]) {
   uint32_t w;
@@ -804,7 +945,7 @@ struct EncodeArgs {
 template <int MODE, bool OCC, bool PRESCALE, bool PER_TOKEN = false>
 __global__ void __launch_bounds__(ENC_THREADS, 4)
 encode_kernel(const EncodeArgs a) {
-  __shared__ float s_gcol[ENC_TK];
+  __shared__ __align__(16) float s_gcol[ENC_TK];
   __shared__ float s_grow[ENC_TM];
   __shared__ float s_prow[ENC_TM];
   __shared__ uint32_t tile_t[8 * 8 * 32];
@@ -862,49 +1003,56 @@ encode_kernel(const EncodeArgs a) {
     v[r] = make_uint4(0, 0, 0, 0);
     if (in_cols) v[r] = __ldg(&a.x[(long long)(row0 + 8 * warp + r) * vec_per_row + (col >> 3)]);
   }
-  float gc[8], pc[8];
-  if (COL_SCALED) {
+  f32x2 gc[4], pc[4];
 #pragma unroll
-    for (int c = 0; c < 8; ++c) gc[c] = in_cols ? s_gcol[8 * lane + c] : 0.0f;
-  }
-  if (ROW_SCALED && PRESCALE) {
-#pragma unroll
-    for (int c = 0; c < 8; ++c) pc[c] = in_cols ? __ldg(&a.pre_col[col + c]) : 0.0f;
+  for (int q = 0; q < 4; ++q) {
+    if (COL_SCALED) gc[q] = in_cols ? *reinterpret_cast<const f32x2*>(&s_gcol[8 * lane + 2 * q]) : 0ull;
+    if (ROW_SCALED && PRESCALE) {
+      const int c = in_cols ? col + 2 * q : 0;
+      const float2 p = make_float2(__ldg(&a.pre_col[c]), __ldg(&a.pre_col[c + 1]));
+      pc[q] = in_cols ? pack2(p.x, p.y) : 0ull;
+    }
   }
 
   uint32_t word[8];                                   // codes of the row-major output
   uint32_t word_t[MODE == MODE_DUAL ? 8 : 1];         // dual: codes of the column-scaled tensor
   uint32_t any_bits = 0, lo4 = 0, hi4 = 0;            // clamp: mask bytes of rows 0..3 / 4..7
+  __nv_bfloat162 lo2, hi2;                            // the thresholds are BF16 numbers: the clamp needs no unpacking
+  if (OCC && !PER_TOKEN) { lo2 = __float2bfloat162_rn(lo); hi2 = __float2bfloat162_rn(hi); }
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
     const uint32_t w[4] = {v[r].x, v[r].y, v[r].z, v[r].w};
     float f[8], f2[8];
     uint32_t obits = 0;
-    const float grow = ROW_SCALED ? s_grow[8 * warp + r] : 0.0f;
-    const float prow = (COL_SCALED && PRESCALE) ? s_prow[8 * warp + r] : 1.0f;
+    const float grow1 = ROW_SCALED ? s_grow[8 * warp + r] : 0.0f;
+    const float prow1 = (COL_SCALED && PRESCALE) ? s_prow[8 * warp + r] : 1.0f;
+    const f32x2 grow = pack2(grow1, grow1), prow = pack2(prow1, prow1);
     if constexpr (PER_TOKEN) {
-      lo = s_thr[2 * (8 * warp + r)];
-      hi = s_thr[2 * (8 * warp + r) + 1];
+      lo2 = __float2bfloat162_rn(s_thr[2 * (8 * warp + r)]);
+      hi2 = __float2bfloat162_rn(s_thr[2 * (8 * warp + r) + 1]);
     }
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      float xv = (c & 1) ? bf16_hi(w[c >> 1]) : bf16_lo(w[c >> 1]);
+    for (int q = 0; q < 4; ++q) {
+      uint32_t x = w[q];
       if (OCC) {
-        const float xc = fminf(fmaxf(xv, lo), hi);
-        obits |= (xc != xv ? 1u : 0u) << c;
-        xv = xc;
+        const __nv_bfloat162 xb = *reinterpret_cast<const __nv_bfloat162*>(&w[q]);
+        const __nv_bfloat162 xc = __hmin2(__hmax2(xb, lo2), hi2);
+        // bit 2 q for the lower element, 17 + 2 q for the upper one
+        obits |= __hne2_mask(xc, xb) & (0x00020001u << (2 * q));
+        x = *reinterpret_cast<const uint32_t*>(&xc);
       }
-      // "+ 0.0f" turns a -0 product into +0 (the nudge needs a non-negative zero)
+      const f32x2 xv = pack2(bf16_lo(x), bf16_hi(x));
+      // "+ 0" turns a -0 product into +0 (the nudge needs a non-negative zero)
       if constexpr (MODE == MODE_ROWS) {
-        f[c] = __fmaf_rn(PRESCALE ? __fmul_rn(xv, pc[c]) : xv, grow, 0.0f);
+        unpack2(fma2(PRESCALE ? mul2(xv, pc[q]) : xv, grow, 0ull), f[2 * q], f[2 * q + 1]);
       } else if constexpr (MODE == MODE_COLS) {
-        f[c] = __fmaf_rn(PRESCALE ? __fmul_rn(xv, prow) : xv, gc[c], 0.0f);
+        unpack2(fma2(PRESCALE ? mul2(xv, prow) : xv, gc[q], 0ull), f[2 * q], f[2 * q + 1]);
       } else {
-        f[c] = __fmaf_rn(__fmul_rn(xv, pc[c]), grow, 0.0f);
-        f2[c] = __fmaf_rn(__fmul_rn(xv, prow), gc[c], 0.0f);
+        unpack2(fma2(mul2(xv, pc[q]), grow, 0ull), f[2 * q], f[2 * q + 1]);
+        unpack2(fma2(mul2(xv, prow), gc[q], 0ull), f2[2 * q], f2[2 * q + 1]);
       }
     }
-    if (OCC && !in_cols) obits = 0;                   // beyond the tensor: its zeros may lie outside [lo, hi]
+    if (OCC) obits = in_cols ? (obits | (obits >> 16)) & 0xFFu : 0u;   // beyond the tensor: its zeros may lie outside [lo, hi]
     word[r] = encode8(f);
     if constexpr (MODE == MODE_DUAL) word_t[r] = encode8(f2);
     if (in_cols) {
@@ -989,7 +1137,7 @@ __device__ __forceinline__ void transpose4x4_bytes(uint32_t a0, uint32_t a1, uin
 template <int MODE, bool PRESCALE>
 __global__ void __launch_bounds__(ENC_THREADS)
 encode_fp8_kernel(const EncodeArgs a) {
-  __shared__ float s_gcol[ENC_TK];
+  __shared__ __align__(16) float s_gcol[ENC_TK];
   __shared__ float s_grow[ENC_TM];
   __shared__ float s_prow[ENC_TM];
   __shared__ uint2 tile_t[8 * 8 * 32];
@@ -1321,6 +1469,14 @@ void launch_select(SelectArgs& a, int num_sms, cudaStream_t stream) {
   tail_select_kernel<<<(a.rows + per - 1) / per, SEL_THREADS, SEL_DYN_SMEM, stream>>>(a);
 }
 
+// One wave of blocks, four per SM, each with at least one step of rows.
+dim3 absmax_grid(int rows, int cols, int num_sms) {
+  const int strips = (cols + ENC_TK - 1) / ENC_TK, steps = rows / AB_ROWS;
+  int groups = 4 * num_sms / strips;
+  groups = groups < 1 ? 1 : groups > steps ? steps : groups;
+  return dim3(strips, groups);
+}
+
 size_t r256(size_t b) { return (b + 255) & ~size_t(255); }
 
 struct Scratch {
@@ -1518,7 +1674,10 @@ int launch_quantize(fp4_ctx* ctx, cudaStream_t stream, Arena& arena, const void*
       FP4_CUDA_TRY(cudaMemsetAsync(sc.amax_rows, 0, size_t(rows) * 4, stream));
       {
         KernelScope scope(ctx, stream, KC_ABSMAX, 1);
-        absmax_tile_kernel<MODE_ROWS><<<tile_grid, ENC_THREADS, 0, stream>>>(aa);
+        if (prescale)
+          absmax_strip_kernel<MODE_ROWS><<<absmax_grid(rows, cols, ctx->num_sms), ENC_THREADS, 0, stream>>>(aa);
+        else
+          absmax_tile_kernel<MODE_ROWS><<<tile_grid, ENC_THREADS, 0, stream>>>(aa);
       }
       KernelScope scope(ctx, stream, KC_ENCODE, 1);
       if (e4m3 && prescale)
@@ -1535,7 +1694,10 @@ int launch_quantize(fp4_ctx* ctx, cudaStream_t stream, Arena& arena, const void*
       FP4_CUDA_TRY(cudaMemsetAsync(sc.amax_cols, 0, size_t(cols) * 4, stream));
       {
         KernelScope scope(ctx, stream, KC_ABSMAX, 1);
-        absmax_tile_kernel<MODE_COLS><<<tile_grid, ENC_THREADS, 0, stream>>>(aa);
+        if (prescale)
+          absmax_strip_kernel<MODE_COLS><<<absmax_grid(rows, cols, ctx->num_sms), ENC_THREADS, 0, stream>>>(aa);
+        else
+          absmax_tile_kernel<MODE_COLS><<<tile_grid, ENC_THREADS, 0, stream>>>(aa);
       }
       KernelScope scope(ctx, stream, KC_ENCODE, 1);
       if (e4m3 && prescale)
@@ -1582,7 +1744,7 @@ int launch_quantize_dual(fp4_ctx* ctx, cudaStream_t stream, Arena& arena, const 
                                stream));
   {
     KernelScope scope(ctx, stream, KC_ABSMAX, 1);
-    absmax_tile_kernel<MODE_DUAL><<<tile_grid, ENC_THREADS, 0, stream>>>(aa);
+    absmax_strip_kernel<MODE_DUAL><<<absmax_grid(rows, cols, ctx->num_sms), ENC_THREADS, 0, stream>>>(aa);
   }
   EncodeArgs ea = {};
   ea.x = aa.x;
