@@ -12,8 +12,11 @@
  * ---------------------------------------
  *  - Every tensor pointer is a DEVICE pointer unless the parameter is documented as host.
  *    Tensors are dense, row-major and 16-byte aligned.  The caller owns every tensor; the
- *    context owns only its workspace.  Nothing is allocated after fp4_create() (outside profiling
- *    mode, fp4_profile_enable, which creates a pair of CUDA events per kernel class and call).
+ *    context owns only its workspace.  After fp4_create() no device buffer is allocated; the
+ *    third fp4_quantize / fp4_linear_fwd / fp4_linear_bwd with the same arguments on a context
+ *    instantiates its launches as a CUDA graph that later calls replay (at most 512 are kept,
+ *    released by fp4_destroy; not while the caller's stream is being captured), and profiling mode,
+ *    fp4_profile_enable, creates a pair of CUDA events per kernel class and call.
  *  - Notation: A[M x K] activations, W[K x N] weights (input channels x output channels),
  *    Y[M x N] = A W.  M, K and N must be multiples of 128.
  *  - E2M1 codes are sign-magnitude nibbles (bit 3 sign; 0..7 -> 0, .5, 1, 1.5, 2, 3, 4, 6),
@@ -22,7 +25,8 @@
  *    a negative FP4_ERR_* code for errors found on the host before anything is enqueued.
  *  - A context holds one workspace and a few counters that its calls share: the work of two calls
  *    on the same context must not overlap on the GPU (issue them on one stream, or order the
- *    streams); use one context per concurrent stream.
+ *    streams); use one context per concurrent stream.  Host threads that call into one context
+ *    take turns.
  *  - Conditions found on the device are OR-ed into the caller's device word `*status`
  *    (FP4_DEV_* bits).  When a bit is set the outputs are unspecified but every write stayed
  *    inside the caller's buffers.  Every device-side wait is bounded: a stalled pipeline
@@ -113,7 +117,9 @@ typedef struct fp4_qtensor {
 int fp4_create(fp4_ctx** out, int device, size_t workspace_bytes);
 int fp4_destroy(fp4_ctx* ctx);
 
-/* Workspace that fp4_quantize / fp4_linear_fwd / fp4_linear_bwd need for these sizes.      */
+/* Workspace that fp4_quantize / fp4_linear_fwd / fp4_linear_bwd need for these sizes.  It includes
+ * up to 128 MB for the dense form of a heavy residual (see fp4_linear_fwd); a workspace that is
+ * smaller by that much is accepted too, and the residual's entries are then added one by one.  */
 size_t fp4_workspace_bytes(int64_t M, int64_t K, int64_t N);
 
 /* Residual entries that clamping at `alpha` can produce at most (Section 3.2: two tails of
@@ -197,6 +203,9 @@ int fp4_gemm(fp4_ctx* ctx, void* stream, const uint8_t* a_codes, const uint8_t* 
  *   A residual value
  *   beyond 43 000 times its token's clamped absmax does not fit the FP16 operand: the call
  *   then adds every entry per entry.
+ *   A residual that may fill more than 4 % of the activation (sparse_cap, M >= 512) is multiplied
+ *   as a dense matrix where that takes less time: exact three-term BF16 split, chunks of 128 input
+ *   channels added in fp32 in order.  Same bound, without the second term.
  */
 #define FP4_REUSE_W 1
 #define FP4_REUSE_A 2
@@ -219,7 +228,8 @@ int fp4_linear_fwd(fp4_ctx* ctx, void* stream, const void* A_bf16, const void* W
  *   With a heavy residual (same condition as in fp4_linear_fwd, and at least 512 tokens) the
  *   residual's dense columns -- the same outlier channels -- are multiplied with dY on the tensor
  *   cores (exact three-term BF16 split of the residual, chunks of 128 tokens added in fp32 in token
- *   order); the other entries are added per entry in fp32.  That part of dW differs from the
+ *   order); the other entries are added per entry in fp32.  A residual above 4 % is multiplied
+ *   whole in that way, where that takes less time.  That part of dW differs from the
  *   per-entry sum by at most 4e-6 * sum_m |A - A_c|[m,k] |dY|[m,n] (times the DGE factor).
  *   gemm_kind | FP4_BWD_DY_E4M3 (or FP4_BWD_DY_E5M2) quantises both copies of dY to E4M3 (E5M2)
  *   bytes; the saved operands keep the formats the forward gave them; with an 8-bit weight Q' = 1
@@ -333,8 +343,8 @@ int64_t fp4_launch_count(fp4_ctx* ctx);
  * are then unspecified.
  * The work is enqueued on `stream` for the current device.  The first call on each device also
  * looks up the device address of the scratch array and sets a kernel attribute (once per device,
- * safe to race between host threads); make that first call before any stream capture begins.  All calls on a device share the one scratch array
- * (it is cleared at the start of each call): two calls whose work overlaps on the GPU -- issued
+ * safe to race between host threads); make that first call before any stream capture begins.
+ * All calls on a device share the one scratch array (it is cleared at the start of each call): two calls whose work overlaps on the GPU -- issued
  * to different streams without ordering between them -- race and give wrong thresholds.
  */
 #define FP4_STATIC_MAX_ROWS 65536

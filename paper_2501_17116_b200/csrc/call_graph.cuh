@@ -10,10 +10,11 @@
 // What is compared is every argument that reaches a kernel or decides which kernels run (CallKey).
 // Calls made while the caller's stream is being captured, with profiling on or with a debug setting are
 // enqueued as they are.  At most GRAPH_MAX calls are remembered per context, the least recently used one
-// leaves first; all are released with the context.
+// leaves first; all are released with the context.  One host thread at a time enqueues a call of a context.
 #pragma once
 
 #include <cstring>
+#include <mutex>
 #include <unordered_map>
 #include <vector>
 
@@ -36,6 +37,7 @@ static_assert(sizeof(CallKey) % 8 == 0 && sizeof(CallKey) == 8 * 4 + 2 * 4 + 8 +
 class CallGraphs {
  public:
   static constexpr size_t GRAPH_MAX = 512;
+  static constexpr size_t GRAVEYARD_MAX = 64;
   static constexpr int CAPTURE_AT = 3;               // which call with the same arguments is captured
 
   bool init() {
@@ -57,6 +59,7 @@ class CallGraphs {
   // Runs `enqueue(stream)` (an FP4_* code) or its graph on `st`.
   template <class F>
   int run(fp4_ctx* ctx, cudaStream_t st, const CallKey& key, F&& enqueue) {
+    std::lock_guard<std::mutex> lock(mutex_);
     if (ctx->profile || ctx->debug_wait_limit_ns || ctx->debug_skip_fill >= 0) return enqueue(st);
     cudaStreamCaptureStatus capturing;
     if (cudaStreamIsCapturing(st, &capturing) != cudaSuccess) {
@@ -134,6 +137,7 @@ class CallGraphs {
   // recorded behind its last launch has passed (calls of one context are ordered on the GPU).
   void make_room(cudaStream_t st) {
     if (entries_.size() < GRAPH_MAX) return;
+    if (graveyard_.size() >= GRAVEYARD_MAX) cudaEventSynchronize(retired_);
     if (!graveyard_.empty() && cudaEventQuery(retired_) == cudaSuccess) {
       for (cudaGraphExec_t e : graveyard_) cudaGraphExecDestroy(e);
       graveyard_.clear();
@@ -149,6 +153,7 @@ class CallGraphs {
     entries_.erase(oldest);
   }
 
+  std::mutex mutex_;
   cudaStream_t stream_ = nullptr;                    // calls are captured from here
   cudaEvent_t retired_ = nullptr, in_ = nullptr, out_ = nullptr;
   std::unordered_map<uint64_t, Entry> entries_;

@@ -1,5 +1,5 @@
 // Outlier compensation (Section 3.2: the sparse residual times a dense high-precision matrix):
-// forward fused with the final store, weight gradient (Eq. 6) as compact rows for the GEMM's epilogue.
+// forward fused with the final store, weight gradient (Eq. 6) as rows for the GEMM's epilogue.
 //
 //   forward   Y[m, :]  = store( Y1[m, :] + sum_{(m,k) in dA} dA[m,k] * W[k, :] )
 //   wgrad     C[k, :] = sum_{(m,k) in dA} dA[m,k] * dY[m, :]   for the columns k that hold entries;
@@ -74,8 +74,9 @@ comp_fwd_kernel(const float* __restrict__ y1, const int* __restrict__ rowptr, co
                 const float* __restrict__ val, const uint4* __restrict__ w, int M, int N, void* y, int out_f32) {
   // blocks that follow one another share the 256 output columns, i.e. the same slab of the weight
   // rows (K x 512 bytes): it stays in L2 while the tokens stream past
-  const int m = blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int n0 = blockIdx.y * COMP_COLS + 8 * (threadIdx.x & 31);
+  // (from the end: what the GEMM wrote last is still in L2)
+  const int m = (gridDim.x - 1 - blockIdx.x) * 8 + (threadIdx.x >> 5);
+  const int n0 = (gridDim.y - 1 - blockIdx.y) * COMP_COLS + 8 * (threadIdx.x & 31);
   if (m >= M || n0 >= N) return;
   // Y1 is requested first: its latency runs under the dependent chain row pointer -> entry -> weight row
   const long long off = (long long)m * N + n0;
@@ -100,8 +101,8 @@ comp_fwd_kept_kernel(const float* __restrict__ y1, const int* __restrict__ rowpt
                      const float* __restrict__ val, const uint2* __restrict__ kept, const int* __restrict__ kept_end,
                      const uint4* __restrict__ w, int M, int N, void* y, int out_f32,
                      const int* __restrict__ tail_count) {
-  const int m = blockIdx.x * 8 + (threadIdx.x >> 5);
-  const int n0 = blockIdx.y * COMP_COLS + 8 * (threadIdx.x & 31);
+  const int m = (gridDim.x - 1 - blockIdx.x) * 8 + (threadIdx.x >> 5);
+  const int n0 = (gridDim.y - 1 - blockIdx.y) * COMP_COLS + 8 * (threadIdx.x & 31);
   if (m >= M || n0 >= N) return;
   const long long off = (long long)m * N + n0;
   const float4 a = __ldg(reinterpret_cast<const float4*>(y1 + off));

@@ -749,11 +749,11 @@ absmax_strip_kernel(const AbsmaxArgs a) {
   const int vec_per_row = a.cols >> 3;
   constexpr bool want_rows = MODE != MODE_COLS, want_cols = MODE != MODE_ROWS;
   const int steps = a.rows / AB_ROWS;
-  const int st0 = int((long long)steps * blockIdx.y / gridDim.y), st1 = int((long long)steps * (blockIdx.y + 1) / gridDim.y);
-  auto request = [&](int st) {
-    if (in_cols && st < st1) {
+  const int st0 = blockIdx.y, stride = gridDim.y;     // all blocks go down the tensor together
+  auto request = [&](int st, int stage) {
+    if (in_cols && st < steps) {
       const uint4* px = a.x + (long long)(AB_ROWS * st + 4 * warp) * vec_per_row + (col >> 3);
-      const uint32_t slot = uint32_t(__cvta_generic_to_shared(&s_buf[(st - st0) % AB_STAGES][0][tid]));
+      const uint32_t slot = uint32_t(__cvta_generic_to_shared(&s_buf[stage][0][tid]));
 #pragma unroll
       for (int r = 0; r < 4; ++r)
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(slot + uint32_t(r * ENC_THREADS * 16)),
@@ -762,8 +762,8 @@ absmax_strip_kernel(const AbsmaxArgs a) {
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  request(st0);
-  request(st0 + 1);
+  request(st0, 0);
+  request(st0 + stride, 1);
   f32x2 pc[4];
   if (want_rows) {
 #pragma unroll
@@ -782,22 +782,24 @@ absmax_strip_kernel(const AbsmaxArgs a) {
   float cmax[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   float prow = 0.0f;                                  // lane r: prescale of the step's row r (r = lane mod 4)
   auto fetch_prow = [&](int st) {
-    if (want_cols && st < st1) prow = __ldg(&a.pre_row[AB_ROWS * st + 4 * warp + (lane & 3)]);
+    if (want_cols && st < steps) prow = __ldg(&a.pre_row[AB_ROWS * st + 4 * warp + (lane & 3)]);
   };
   fetch_prow(st0);
-  for (int st = st0; st < st1; ++st) {
+  int stage = 0;
+  for (int st = st0; st < steps; st += stride) {
     asm volatile("cp.async.wait_group 1;" ::: "memory");
     const int row = AB_ROWS * st + 4 * warp;
-    const uint4* slot = &s_buf[(st - st0) % AB_STAGES][0][tid];
+    const uint4* slot = &s_buf[stage][0][tid];
     uint4 v[4];
 #pragma unroll
     for (int r = 0; r < 4; ++r) v[r] = in_cols ? slot[r * ENC_THREADS] : make_uint4(0, 0, 0, 0);
-    request(st + 2);
+    request(st + 2 * stride, stage == 0 ? 2 : stage - 1);       // the stage before this one
+    stage = stage == AB_STAGES - 1 ? 0 : stage + 1;
     float pr = prow;
     if (want_cols) {
       if (a.pre_row_div > 0.0f) pr = __fdiv_rn(pr, a.pre_row_div);
       if (a.d_row_out && blockIdx.x == 0 && lane < 4) a.d_row_out[row + lane] = pr;
-      fetch_prow(st + 1);
+      fetch_prow(st + stride);
     }
     uint32_t rm[4];                                   // bits of the maxima: they order like the numbers
 #pragma unroll
@@ -953,7 +955,8 @@ encode_kernel(const EncodeArgs a) {
   __shared__ float s_thr[PER_TOKEN ? 2 * ENC_TM : 1];      // per-token clamp: lo, hi of the tile's rows
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
-  const int row0 = blockIdx.y * ENC_TM;
+  const int strip = gridDim.y - 1 - blockIdx.y;       // from the end: what the pass before read last is still in L2
+  const int row0 = strip * ENC_TM;
   const int col0 = blockIdx.x * ENC_TK;
   const int vec_per_row = a.cols >> 3;
   constexpr bool ROW_SCALED = MODE != MODE_COLS;      // a row-scaled output exists
@@ -1088,10 +1091,10 @@ encode_kernel(const EncodeArgs a) {
   }
   __syncthreads();
   if (OCC && col0 + tid < a.cols) {
-    a.strip_cnt[(long long)blockIdx.y * a.cols + col0 + tid] = uint8_t(s_colcnt[tid]);
+    a.strip_cnt[(long long)strip * a.cols + col0 + tid] = uint8_t(s_colcnt[tid]);
     if (s_colcnt[tid]) {                              // integer sums: order-independent
       atomicAdd(&a.col_cnt[col0 + tid], s_colcnt[tid]);
-      atomicAdd(&a.super_cnt[(long long)(blockIdx.y / SUPER) * a.cols + col0 + tid], s_colcnt[tid]);
+      atomicAdd(&a.super_cnt[(long long)(strip / SUPER) * a.cols + col0 + tid], s_colcnt[tid]);
     }
   }
   if (a.codes_t) {
@@ -1143,7 +1146,8 @@ encode_fp8_kernel(const EncodeArgs a) {
   __shared__ uint2 tile_t[8 * 8 * 32];
   const int tid = threadIdx.x;
   const int warp = tid >> 5, lane = tid & 31;
-  const int row0 = blockIdx.y * ENC_TM;
+  const int strip = gridDim.y - 1 - blockIdx.y;       // from the end: what the pass before read last is still in L2
+  const int row0 = strip * ENC_TM;
   const int col0 = blockIdx.x * ENC_TK;
   const int vec_per_row = a.cols >> 3;
   constexpr bool ROW_SCALED = MODE != MODE_COLS;
