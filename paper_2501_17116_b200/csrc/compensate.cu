@@ -44,35 +44,47 @@ __device__ __forceinline__ void store8(void* out, int out_f32, long long off, co
   }
 }
 
+// acc += n entries, gathered together
+template <int n>
+__device__ __forceinline__ void add_entries(float (&acc)[8], const int* __restrict__ idx, const float* __restrict__ val,
+                                            const uint4* __restrict__ dense, int vec_per_row, int vcol) {
+  int r[n];
+  float v[n];
+  uint4 d[n];
+#pragma unroll
+  for (int u = 0; u < n; ++u) {
+    r[u] = __ldg(&idx[u]);
+    v[u] = __ldg(&val[u]);
+  }
+#pragma unroll
+  for (int u = 0; u < n; ++u) d[u] = __ldg(&dense[(long long)r[u] * vec_per_row + vcol]);
+#pragma unroll
+  for (int u = 0; u < n; ++u) fma8(acc, v[u], d[u]);
+}
+template <int n>
+__device__ __forceinline__ void add_kept(float (&acc)[8], const uint2* __restrict__ kept, const uint4* __restrict__ dense,
+                                         int vec_per_row, int vcol) {
+  uint2 t[n];
+  uint4 d[n];
+#pragma unroll
+  for (int u = 0; u < n; ++u) t[u] = __ldg(&kept[u]);
+#pragma unroll
+  for (int u = 0; u < n; ++u) d[u] = __ldg(&dense[(long long)t[u].x * vec_per_row + vcol]);
+#pragma unroll
+  for (int u = 0; u < n; ++u) fma8(acc, __uint_as_float(t[u].y), d[u]);
+}
+
 // acc[0..7] += sum over the entries [e0, e1) of val[e] * dense[idx[e], col .. col+7]
 __device__ __forceinline__ void sparse_row_times_dense(float (&acc)[8], const int* __restrict__ idx,
                                                        const float* __restrict__ val, int e0, int e1,
                                                        const uint4* __restrict__ dense, int vec_per_row, int vcol) {
   int e = e0;
-  for (; e + 4 <= e1; e += 4) {                 // four independent loads in flight
-    int r[4];
-    float v[4];
-    uint4 d[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      r[u] = __ldg(&idx[e + u]);
-      v[u] = __ldg(&val[e + u]);
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) d[u] = __ldg(&dense[(long long)r[u] * vec_per_row + vcol]);
-#pragma unroll
-    for (int u = 0; u < 4; ++u) fma8(acc, v[u], d[u]);
-  }
+  for (; e + 4 <= e1; e += 4) add_entries<4>(acc, idx + e, val + e, dense, vec_per_row, vcol);   // four loads in flight
   if (e + 2 <= e1) {
-    const int r0 = __ldg(&idx[e]), r1 = __ldg(&idx[e + 1]);
-    const float v0 = __ldg(&val[e]), v1 = __ldg(&val[e + 1]);
-    const uint4 d0 = __ldg(&dense[(long long)r0 * vec_per_row + vcol]);
-    const uint4 d1 = __ldg(&dense[(long long)r1 * vec_per_row + vcol]);
-    fma8(acc, v0, d0);
-    fma8(acc, v1, d1);
+    add_entries<2>(acc, idx + e, val + e, dense, vec_per_row, vcol);
     e += 2;
   }
-  if (e < e1) fma8(acc, __ldg(&val[e]), __ldg(&dense[(long long)__ldg(&idx[e]) * vec_per_row + vcol]));
+  if (e < e1) add_entries<1>(acc, idx + e, val + e, dense, vec_per_row, vcol);
 }
 
 // Y1 is read for the last time and Y leaves with streaming stores, so that neither pushes the rest of Y1 and the slab
@@ -123,30 +135,17 @@ comp_fwd_kept_kernel(const float* __restrict__ y1, const int* __restrict__ rowpt
   if (__ldg(tail_count) > 0) {
     int e = __ldg(&rowptr[m]);
     const int e1 = __ldg(&kept_end[m]);
-    for (; e + FWD_FLY <= e1; e += FWD_FLY) {
-      uint2 t[FWD_FLY];
-      uint4 d[FWD_FLY];
-#pragma unroll
-      for (int u = 0; u < FWD_FLY; ++u) t[u] = __ldg(&kept[e + u]);
-#pragma unroll
-      for (int u = 0; u < FWD_FLY; ++u) d[u] = __ldg(&w[(long long)t[u].x * vec_per_row + vcol]);
-#pragma unroll
-      for (int u = 0; u < FWD_FLY; ++u) fma8(acc, __uint_as_float(t[u].y), d[u]);
+    for (; e + FWD_FLY <= e1; e += FWD_FLY) add_kept<FWD_FLY>(acc, kept + e, w, vec_per_row, vcol);
+    // the last one to seven: four, two, one
+    if (e + 4 <= e1) {
+      add_kept<4>(acc, kept + e, w, vec_per_row, vcol);
+      e += 4;
     }
-    for (; e + 4 <= e1; e += 4) {
-      uint2 t[4];
-      uint4 d[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) t[u] = __ldg(&kept[e + u]);
-#pragma unroll
-      for (int u = 0; u < 4; ++u) d[u] = __ldg(&w[(long long)t[u].x * vec_per_row + vcol]);
-#pragma unroll
-      for (int u = 0; u < 4; ++u) fma8(acc, __uint_as_float(t[u].y), d[u]);
+    if (e + 2 <= e1) {
+      add_kept<2>(acc, kept + e, w, vec_per_row, vcol);
+      e += 2;
     }
-    for (; e < e1; ++e) {
-      const uint2 t = __ldg(&kept[e]);
-      fma8(acc, __uint_as_float(t.y), __ldg(&w[(long long)t.x * vec_per_row + vcol]));
-    }
+    if (e < e1) add_kept<1>(acc, kept + e, w, vec_per_row, vcol);
   } else {
     sparse_row_times_dense(acc, col, val, __ldg(&rowptr[m]), __ldg(&rowptr[m + 1]), w, vec_per_row, vcol);
   }
@@ -168,7 +167,7 @@ constexpr int LONG_FEW = 64, LONG_FEW_MAX = 256;
 struct ColumnClasses {
   int* list_dense;             // [DENSE_TC_MAX] dense columns, ascending
   int* list_long;              // [K]
-  int* list_short;             // [K]
+  int4* list_short;            // [K] column, its entries' range
   int* counts;                 // numbers of dense, long and short columns
   int* slot_of_col;            // [K] position among the dense columns; DENSE_TC_MAX for a long or short one; -1: empty
 };
@@ -248,7 +247,10 @@ classify_columns_kernel(const int* __restrict__ colptr, int K, int dense_from, c
   const int at_long = large_b + block_exclusive_scan_1024(is_long, warp_tot);
   const int at_short = any_b - large_b - min(cand_b, DENSE_TC_MAX) + block_exclusive_scan_1024(is_short, warp_tot);
   if (is_long) out.list_long[at_long] = k;
-  if (is_short) out.list_short[at_short] = k;
+  if (is_short) {
+    const int e0 = __ldg(&colptr[k]);
+    out.list_short[at_short] = make_int4(k, e0, e0 + n, 0);
+  }
   if (k < K) out.slot_of_col[k] = dense ? rank : n > 0 ? DENSE_TC_MAX : -1;
   if (k == 0) {
     out.counts[0] = n_dense;
@@ -401,11 +403,6 @@ __device__ __forceinline__ void strided_entries_times_dense(float (&acc)[8], con
   }
 }
 
-__device__ __forceinline__ void store8_f32(float* dst, const float (&t)[8]) {
-  *reinterpret_cast<float4*>(dst) = make_float4(t[0], t[1], t[2], t[3]);
-  *reinterpret_cast<float4*>(dst + 4) = make_float4(t[4], t[5], t[6], t[7]);
-}
-
 // Weight-gradient compensation of the columns that are not dense:
 //   comp[k, :] = sum over the entries of column k of dA[m,k] * dY[m, :].
 // Long columns: a cluster of four blocks per (column, 256 outputs).  Its 32 warps take the entries
@@ -454,40 +451,52 @@ comp_wgrad_long_kernel(float* __restrict__ comp, const int* __restrict__ colptr,
 // in that order, so that the blocks in flight at any time read one or two 512-byte-wide slabs of dY
 // (tokens x 512 bytes: a few MB, which stay in L2) instead of all of it: every token's piece of a
 // slab is gathered by about 1 % of the columns, and those re-reads then hit L2.
+// Heavy residuals are bound by L2; light ones (one or two entries per column) by the chain of loads per kilobyte of
+// output: the list holds the column's range of entries, the next item's is fetched beside this one, and the last one
+// to seven entries travel four, two and one at a time.  8192 x 5120 x 5120 at 0.01 %: 51 -> 43 us.
 __global__ void __launch_bounds__(COMP_THREADS, 4)
-comp_wgrad_short_kernel(float* __restrict__ comp, const int* __restrict__ colptr, const int* __restrict__ row,
-                        const float* __restrict__ val, const uint4* __restrict__ dy, const int* __restrict__ list,
-                        const int* __restrict__ counts, int N) {
+comp_wgrad_short_kernel(float* __restrict__ comp, const int* __restrict__ row, const float* __restrict__ val,
+                        const uint4* __restrict__ dy, const int4* __restrict__ list, const int* __restrict__ counts, int N) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_cols = counts[2];
-  const int groups = (n_cols + 7) >> 3;
-  const int n_blocks = (N + COMP_COLS - 1) / COMP_COLS;
-  const long long items = (long long)groups * n_blocks;
-  for (long long it = blockIdx.x; it < items; it += gridDim.x) {
-    const int nb = int(it / groups);
-    const int slot = int(it - (long long)nb * groups) * 8 + warp;
-    const int n0 = nb * COMP_COLS + 8 * lane;
-    if (slot >= n_cols || n0 >= N) continue;
-    const int k = list[slot];
+  const unsigned groups = unsigned(n_cols + 7) >> 3;
+  const unsigned items = groups * unsigned((N + COMP_COLS - 1) / COMP_COLS);
+  int4 next = make_int4(-1, 0, 0, 0);                 // the warp's column of the item after this one
+  int next_n0 = 0;
+  auto fetch = [&](unsigned it) {
+    const unsigned nb = it / groups;
+    const int slot = int(it - nb * groups) * 8 + warp;
+    next_n0 = int(nb) * COMP_COLS + 8 * lane;
+    next.x = -1;
+    if (slot < n_cols && next_n0 < N) next = __ldg(&list[slot]);
+  };
+  if (blockIdx.x < items) fetch(blockIdx.x);
+  for (unsigned it = blockIdx.x; it < items; it += gridDim.x) {
+    const int4 c = next;
+    const int k = c.x, n0 = next_n0;
+    if (it + gridDim.x < items) fetch(it + gridDim.x);
+    if (k < 0) continue;
     float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     {
       const int vec_per_row = N >> 3, vcol = n0 >> 3;
-      int e = colptr[k];
-      const int e1 = colptr[k + 1];
-      for (; e + 8 <= e1; e += 8) {                 // eight gathers in flight, entries in order
-        int r[8];
-        float v[8];
-        uint4 d[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) { r[u] = __ldg(&row[e + u]); v[u] = __ldg(&val[e + u]); }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) d[u] = __ldg(&dy[(long long)r[u] * vec_per_row + vcol]);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) fma8(acc, v[u], d[u]);
+      int e = c.y;
+      const int e1 = c.z;
+      for (; e + 8 <= e1; e += 8)                   // eight gathers in flight, entries in order
+        add_entries<8>(acc, row + e, val + e, dy, vec_per_row, vcol);
+      // the last one to seven: four, two, one
+      if (e + 4 <= e1) {
+        add_entries<4>(acc, row + e, val + e, dy, vec_per_row, vcol);
+        e += 4;
       }
-      for (; e < e1; ++e) fma8(acc, __ldg(&val[e]), __ldg(&dy[(long long)__ldg(&row[e]) * vec_per_row + vcol]));
+      if (e + 2 <= e1) {
+        add_entries<2>(acc, row + e, val + e, dy, vec_per_row, vcol);
+        e += 2;
+      }
+      if (e < e1) add_entries<1>(acc, row + e, val + e, dy, vec_per_row, vcol);
     }
-    store8_f32(comp + (long long)k * N + n0, acc);
+    float4* dst = reinterpret_cast<float4*>(comp + (long long)k * N + n0);   // streaming: dY stays in L2
+    __stcs(dst, make_float4(acc[0], acc[1], acc[2], acc[3]));
+    __stcs(dst + 1, make_float4(acc[4], acc[5], acc[6], acc[7]));
   }
 }
 
@@ -547,7 +556,7 @@ int launch_comp_fwd(fp4_ctx* ctx, cudaStream_t stream, const float* y1, const in
 
 size_t comp_wgrad_scratch_bytes(int64_t M, int64_t K, int64_t N) {
   auto r256 = [](size_t b) { return (b + 255) & ~size_t(255); };
-  size_t b = r256((2 * size_t(K) + DENSE_TC_MAX + 4) * 4) + r256(size_t(K) * 4);                     // lists + counters, slots
+  size_t b = r256((size_t(K) + DENSE_TC_MAX + 4) * 4) + r256(size_t(K) * 16) + r256(size_t(K) * 4);      // lists + counters, slots
   b += dense_tc_scratch_bytes(M, N);                                                  // BF16 terms, partial sums
   return b;
 }
@@ -596,15 +605,16 @@ int launch_fwd_tail(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, con
 int launch_comp_wgrad(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, const void* dy_bf16, Arena& scratch,
                       const int** slot_of_col_out, float* comp, int64_t M, int64_t K, int64_t N, int32_t* status,
                       const CompOverlap* overlap) {
-  // lists: [K] long columns, [K] short columns, the dense columns, three counters
-  int* lists = scratch.take<int>(2 * size_t(K) + DENSE_TC_MAX + 4);
+  // lists: [K] long columns, the dense columns, three counters
+  int* lists = scratch.take<int>(size_t(K) + DENSE_TC_MAX + 4);
+  int4* list_short = scratch.take<int4>(size_t(K));
   int* slot_of_col = scratch.take<int>(size_t(K));
   const int splits = dense_tc_splits(ctx, M, N);
   void* vt = scratch.take<uint16_t>(size_t(3) * DENSE_TC_MAX * size_t(M));
   float* partial = scratch.take<float>(size_t(splits) * DENSE_TC_MAX * size_t(N));
   if (!scratch.ok) return FP4_ERR_WORKSPACE;
   *slot_of_col_out = slot_of_col;
-  const ColumnClasses classes = {lists + 2 * K, lists, lists + K, lists + 2 * K + DENSE_TC_MAX, slot_of_col};
+  const ColumnClasses classes = {lists + K, lists, list_short, lists + K + DENSE_TC_MAX, slot_of_col};
   // Columns that at least a quarter of the tokens hit (the outlier channels) form the dense class,
   // whose product runs on the tensor cores.  It costs three launches, which pay
   // when the residual is heavy: when it may hold at least 1 % of the activation (alpha <= 0.995).
@@ -638,8 +648,8 @@ int launch_comp_wgrad(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, c
     const long long max_items = (long long)((K + 7) / 8) * n_blocks;
     long long g = 32LL * ctx->num_sms;
     g = g > max_items ? max_items : g;
-    comp_wgrad_short_kernel<<<unsigned(g), COMP_THREADS, 0, stream>>>(comp, a->csc_colptr, a->csc_row, a->csc_val, dy,
-                                                                     classes.list_short, classes.counts, int(N));
+    comp_wgrad_short_kernel<<<unsigned(g), COMP_THREADS, 0, stream>>>(comp, a->csc_row, a->csc_val, dy, classes.list_short,
+                                                                     classes.counts, int(N));
   }
   if (sl != stream) {
     FP4_CUDA_TRY(cudaEventRecord(overlap->long_done, sl));
