@@ -91,14 +91,17 @@ __device__ __forceinline__ void sparse_row_times_dense(float (&acc)[8], const in
 // of weight rows out of L2; two or three last entries of a token travel together.  One token per warp and 40
 // registers: the chain row pointer -> entry -> weight row is hidden by the other warps (walking tokens with the next
 // Y1 in flight took 17 us of 4096 x 2048 x 2048 instead of 11).  8192 x 5120 x 5120 at 0.01 %: 65 -> 52.5 us, 4096 x
-// 2048 x 5504 at 0.1 %: 37 -> 28, with the walk from the end below.
-__global__ void __launch_bounds__(COMP_THREADS)
+// 2048 x 5504 at 0.1 %: 37 -> 28, with the walk from the end below.  Blocks of four warps: with eight, a block's
+// slots waited for its slowest warp (51 % of the warps active; 51.8 -> 49.6, 28.1 -> 26.9; blocks of two are slower;
+// comp_fwd_kept, 2048 x 512 x 2048 at 1 %: 9.4 -> 8.9).
+constexpr int FWD_THREADS = 128;
+__global__ void __launch_bounds__(FWD_THREADS)
 comp_fwd_kernel(const float* __restrict__ y1, const int* __restrict__ rowptr, const int* __restrict__ col,
                 const float* __restrict__ val, const uint4* __restrict__ w, int M, int N, void* y, int out_f32) {
   // blocks that follow one another share the 256 output columns, i.e. the same slab of the weight
   // rows (K x 512 bytes): it stays in L2 while the tokens stream past
   // (from the end: what the GEMM wrote last is still in L2)
-  const int m = (gridDim.x - 1 - blockIdx.x) * 8 + (threadIdx.x >> 5);
+  const int m = (gridDim.x - 1 - blockIdx.x) * (FWD_THREADS / 32) + (threadIdx.x >> 5);
   const int n0 = (gridDim.y - 1 - blockIdx.y) * COMP_COLS + 8 * (threadIdx.x & 31);
   if (m >= M || n0 >= N) return;
   // Y1 is requested first: its latency runs under the dependent chain row pointer -> entry -> weight row
@@ -119,12 +122,12 @@ comp_fwd_kernel(const float* __restrict__ y1, const int* __restrict__ rowptr, co
 // flight 9.3 ms per step, eight 7.7 ms, twelve at three blocks 8.0 ms, sixteen at two blocks 10.2 ms).  If the tail was switched off on the device (*tail_count == 0: a value
 // FP16 cannot hold) the list is not valid and the whole CSR row is added instead.
 constexpr int FWD_FLY = 8;                 // weight-row gathers a lane keeps in flight
-__global__ void __launch_bounds__(COMP_THREADS, 4)
+__global__ void __launch_bounds__(FWD_THREADS, 8)
 comp_fwd_kept_kernel(const float* __restrict__ y1, const int* __restrict__ rowptr, const int* __restrict__ col,
                      const float* __restrict__ val, const uint2* __restrict__ kept, const int* __restrict__ kept_end,
                      const uint4* __restrict__ w, int M, int N, void* y, int out_f32,
                      const int* __restrict__ tail_count) {
-  const int m = (gridDim.x - 1 - blockIdx.x) * 8 + (threadIdx.x >> 5);
+  const int m = (gridDim.x - 1 - blockIdx.x) * (FWD_THREADS / 32) + (threadIdx.x >> 5);
   const int n0 = (gridDim.y - 1 - blockIdx.y) * COMP_COLS + 8 * (threadIdx.x & 31);
   if (m >= M || n0 >= N) return;
   const long long off = (long long)m * N + n0;
@@ -541,14 +544,15 @@ extern "C" int fp4_l2_read_probe(void* stream, const void* buf, size_t bytes, in
 int launch_comp_fwd(fp4_ctx* ctx, cudaStream_t stream, const float* y1, const int32_t* rowptr, const int32_t* col,
                     const float* val, const void* w_bf16, int64_t M, int64_t, int64_t N, void* y, int out_f32,
                     const int* tail_count, const void* kept, const int* kept_end) {
-  const dim3 grid(unsigned((M + 7) / 8), unsigned((N + COMP_COLS - 1) / COMP_COLS));
+  const unsigned rows = FWD_THREADS / 32;             // a warp each
+  const dim3 grid(unsigned((M + rows - 1) / rows), unsigned((N + COMP_COLS - 1) / COMP_COLS));
   KernelScope scope(ctx, stream, KC_COMP_FWD, 1);
   if (kept && kept_end && tail_count)
-    comp_fwd_kept_kernel<<<grid, COMP_THREADS, 0, stream>>>(y1, rowptr, col, val, static_cast<const uint2*>(kept),
+    comp_fwd_kept_kernel<<<grid, FWD_THREADS, 0, stream>>>(y1, rowptr, col, val, static_cast<const uint2*>(kept),
                                                             kept_end, static_cast<const uint4*>(w_bf16), int(M), int(N),
                                                             y, out_f32, tail_count);
   else
-    comp_fwd_kernel<<<grid, COMP_THREADS, 0, stream>>>(y1, rowptr, col, val, static_cast<const uint4*>(w_bf16), int(M),
+    comp_fwd_kernel<<<grid, FWD_THREADS, 0, stream>>>(y1, rowptr, col, val, static_cast<const uint4*>(w_bf16), int(M),
                                                        int(N), y, out_f32);
   FP4_CUDA_TRY(cudaGetLastError());
   return FP4_OK;
