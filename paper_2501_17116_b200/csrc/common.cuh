@@ -113,11 +113,12 @@ struct Arena {
 // below 2, 1 on [2, 4) and 2 from 4 up, i.e. delta = 2^(max(e, 0) - 1) with e the binary exponent
 // of |w| (capped at the last interval, whose formula continues past 6).  With g the interval's lower
 // end, the position inside it, mapped to [-1, 1], is u = (|w| - g) 2 / delta - 1, and the factor is
-// |u|^(1/k - 1) / k = 2^(expo log2 |u| + log2(1/k)).
-// Branch-free, 17 instructions (a fused epilogue evaluates it for every weight): delta and 2 / delta are
+// |u|^(1/k - 1) / k = 2^(expo log2 |u|) / k.  (1 / k multiplies last: as a summand of the exponent it would
+// save an instruction, but the rounded log2(1/k) and the larger exponent cost precision.)
+// Branch-free, 18 instructions (a fused epilogue evaluates it for every weight): delta and 2 / delta are
 // put together from the exponent bits; g comes from an addition of 2^23 delta rounded down (exact; floorf
 // would go to the pipe that also serves the two special functions).
-__device__ __forceinline__ float dge_factor(float ws, float expo, float log2_inv_k, float clip) {
+__device__ __forceinline__ float dge_factor(float ws, float expo, float inv_k, float clip) {
   const float a = fabsf(ws);
   const uint32_t eb = min(max(__float_as_uint(a) & 0x7F800000u, 0x3F800000u), 0x40800000u);   // 1, 2 or 4
   const float big = __uint_as_float(eb + (22u << 23));           // 2^23 delta
@@ -127,8 +128,8 @@ __device__ __forceinline__ float dge_factor(float ws, float expo, float log2_inv
   // weight gradient): log2(0) = -inf, times the negative exponent +inf, 2^+inf = +inf, capped below
   float l, p;
   asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l) : "f"(u));
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(p) : "f"(fmaf(expo, l, log2_inv_k)));
-  return fminf(p, clip);
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(p) : "f"(expo * l));
+  return fminf(inv_k * p, clip);
 }
 
 // Work fused into the epilogue of the weight-gradient GEMM (all null / zero: plain epilogue):

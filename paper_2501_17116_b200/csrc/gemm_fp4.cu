@@ -26,8 +26,6 @@
 // frees its tensor memory and returns.
 #include <cuda.h>
 
-#include <cmath>
-
 #include "common.cuh"
 #include "tc_ptx.cuh"
 
@@ -94,7 +92,7 @@ struct GemmArgs {
   const int* slot_of_row;      // rows with a compensation row: not negative (null: none)
   bool has_w;                  // the DGE factor applies
   const float* w_amax;
-  float log2_inv_k, expo, clip;
+  float inv_k, expo, clip;
   // dense tail (single-problem launches only): after the FP4 k-blocks of a tile, 3 * ceil(*tail_count / 64)
   // k-blocks of 64 FP16 columns each from the maps that otherwise describe a second problem are
   // accumulated into the same tile with kind::f16 (null: no tail)
@@ -324,7 +322,7 @@ __device__ __forceinline__ bool epilogue_tile_wgrad(const GemmArgs& args, int ro
         for (int e = 0; e < 4; ++e) {
           const int c = 4 * q + e;
           const float wf = __uint_as_float((c & 1) ? (w[c >> 1] & 0xFFFF0000u) : (w[c >> 1] << 16));
-          y[c] *= dge_factor(__fmul_rn(wf, g[e]), args.expo, args.log2_inv_k, args.clip);
+          y[c] *= dge_factor(__fmul_rn(wf, g[e]), args.expo, args.inv_k, args.clip);
         }
       }
     }
@@ -846,9 +844,8 @@ int make_problem(fp4_ctx* ctx, Problem* p, const Fp4GemmDesc& d, int gemm_kind, 
   if (args.has_w && (rc = make_in_map(ctx, &p->map_w, epi->w_bf16, d.I, d.J, false)) != FP4_OK) return rc;
   if (args.slot_of_row && (rc = make_in_map(ctx, &p->map_add, epi->addend, d.I, d.J, true)) != FP4_OK) return rc;
   args.w_amax = fused ? epi->w_amax : nullptr;
-  const float inv_k = fused && epi->w_bf16 ? 1.0f / epi->dge_k : 1.0f;
-  args.log2_inv_k = std::log2(inv_k);
-  args.expo = inv_k - 1.0f;
+  args.inv_k = fused && epi->w_bf16 ? 1.0f / epi->dge_k : 1.0f;
+  args.expo = args.inv_k - 1.0f;
   args.clip = fused ? epi->dge_clip : 0.0f;
   args.wait_limit_ns = ctx->debug_wait_limit_ns ? ctx->debug_wait_limit_ns : WAIT_LIMIT_NS;
   args.skip_fill = ctx->debug_skip_fill;

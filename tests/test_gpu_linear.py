@@ -354,6 +354,22 @@ def test_dge_factor_alone_on_every_scaled_weight(lib, ctx):
     assert np.array_equal(got[b.dge == 3.0], b.dge[b.dge == 3.0])      # the cap is exact
 
 
+@pytest.mark.parametrize("k", [3.0, 5.0, 6.0, 7.0, 9.0])
+def test_dge_factor_on_the_grid_is_one_over_k(lib, ctx, k):
+    """On the grid |u| = 1, where the power is exactly 1: the factor is RN32(1 / k) to the last bit, not one that
+    went through a rounded logarithm of it.  (Weights +-0.5 ... +-6 with column maximum 6, S = 4.5 as above.)"""
+    M, K, N = 128, 128, 128
+    grid = torch.tensor([6.0, 0.5, 1.0, 1.5, 2.0, 3.0, 4.0, -0.5, -1.0, -1.5, -2.0, -3.0, -4.0, -6.0, 6.0, 6.0])
+    W = grid.repeat(K // 16)[:, None].expand(K, N).to(torch.bfloat16).cuda().contiguous()
+    A = torch.zeros((M, K), dtype=torch.bfloat16, device="cuda")
+    dY = torch.zeros((M, N), dtype=torch.bfloat16, device="cuda")
+    A[0], dY[0] = 6.0, 0.75
+    _, sa, sw = lib.fp4_linear_fwd(ctx, A, W, 1.0)
+    _, dw = lib.fp4_linear_bwd(ctx, dY, W, sa, sw, dge_k=k, out_f32=True, want_da=False)
+    want = np.float32(4.5) * (np.float32(1.0) / np.float32(k))
+    assert bool((dw == float(want)).all()), (dw.unique().tolist(), float(want))
+
+
 def test_tensor_core_accumulation_stays_inside_its_floor(lib, ctx):
     """Measures what TAIL_FLOOR allows for.  120 hot columns whose residual entries alternate in
     sign against weights of one sign make the compensation branch cancel (sums of ~120 terms far
