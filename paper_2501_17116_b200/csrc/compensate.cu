@@ -409,17 +409,15 @@ __device__ __forceinline__ void strided_entries_times_dense(float (&acc)[8], con
 // Weight-gradient compensation of the columns that are not dense:
 //   comp[k, :] = sum over the entries of column k of dA[m,k] * dY[m, :].
 // Long columns: a cluster of four blocks per (column, 256 outputs).  Its 32 warps take the entries
-// round-robin inside the block's quarter of them; partial sums are added in warp order, then in block order
-// (distributed shared memory), so the result does not depend on scheduling.  (One block of 32 warps
-// per item left ten outlier channels x 8 blocks of outputs with 80 blocks for 148 SMs.)
+// round-robin; every block adds a quarter of the outputs, all 32 partial sums of each in warp order
+// (distributed shared memory), so the result does not depend on scheduling nor on the cluster's size.
+// (One block of 32 warps per item left ten outlier channels x 8 blocks of outputs with 80 blocks for 148 SMs.)
 constexpr int LONG_CLUSTER = 4, LONG_WARPS = 8;
 __global__ void __cluster_dims__(LONG_CLUSTER, 1, 1) __launch_bounds__(32 * LONG_WARPS, 4)
 comp_wgrad_long_kernel(float* __restrict__ comp, const int* __restrict__ colptr, const int* __restrict__ row,
                        const float* __restrict__ val, const uint4* __restrict__ dy, const int* __restrict__ list,
                        const int* __restrict__ counts, int N) {
-  static_assert(32 * LONG_WARPS == COMP_COLS, "one thread per output of the block sums");
   __shared__ float part[LONG_WARPS][32][9];         // [warp][lane][8 (+1 pad)]
-  __shared__ float block_sum[COMP_COLS];
   cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n_long = counts[1], n_blocks = (N + COMP_COLS - 1) / COMP_COLS;
@@ -427,23 +425,29 @@ comp_wgrad_long_kernel(float* __restrict__ comp, const int* __restrict__ colptr,
   for (int it = blockIdx.x / LONG_CLUSTER; it < n_long * n_blocks; it += clusters) {
     const int nb = it / n_long, k = list[it - nb * n_long];
     const int n0 = nb * COMP_COLS + 8 * lane;
-    const int e0 = colptr[k], n = colptr[k + 1] - e0;
-    const int ea = e0 + int((long long)n * rank / LONG_CLUSTER), eb = e0 + int((long long)n * (rank + 1) / LONG_CLUSTER);
     float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    if (n0 < N) strided_entries_times_dense(acc, row, val, ea + warp, eb, LONG_WARPS, dy, N >> 3, n0 >> 3);
+    if (n0 < N)
+      strided_entries_times_dense(acc, row, val, colptr[k] + rank * LONG_WARPS + warp, colptr[k + 1], LONG_CLUSTER * LONG_WARPS,
+                                  dy, N >> 3, n0 >> 3);
 #pragma unroll
     for (int c = 0; c < 8; ++c) part[warp][lane][c] = acc[c];
-    __syncthreads();
-    float t = 0.0f;
-#pragma unroll
-    for (int w = 0; w < LONG_WARPS; ++w) t += part[w][tid >> 3][tid & 7];
-    block_sum[tid] = t;
     cluster.sync();
-    if (rank == 0 && nb * COMP_COLS + tid < N) {
-      t = 0.0f;
+    constexpr int OWN = COMP_COLS / LONG_CLUSTER;   // outputs that this block adds, one per thread
+    const int o = rank * OWN + tid;
+    if (tid < OWN && nb * COMP_COLS + o < N) {
+      float p[LONG_CLUSTER][LONG_WARPS];
 #pragma unroll
-      for (int r = 0; r < LONG_CLUSTER; ++r) t += cluster.map_shared_rank(block_sum, r)[tid];
-      comp[(long long)k * N + nb * COMP_COLS + tid] = t;
+      for (int r = 0; r < LONG_CLUSTER; ++r) {
+        const float* from = cluster.map_shared_rank(&part[0][o >> 3][o & 7], r);
+#pragma unroll
+        for (int w = 0; w < LONG_WARPS; ++w) p[r][w] = from[w * 32 * 9];
+      }
+      float t = 0.0f;
+#pragma unroll
+      for (int r = 0; r < LONG_CLUSTER; ++r)
+#pragma unroll
+        for (int w = 0; w < LONG_WARPS; ++w) t += p[r][w];
+      comp[(long long)k * N + nb * COMP_COLS + o] = t;
     }
     cluster.sync();                                 // the sums have been read
   }

@@ -468,3 +468,38 @@ def test_heavy_residual_as_a_dense_product(lib, M, K, N, alpha, wide):
     assert bool(((dw - dw1).abs().double() <= 2 * 4e-6 * (res.T @ dY.double().abs()) + 2.4e-7 * dw.abs() + 1e-30).all())
     room.close()
     tight.close()
+
+
+def test_long_columns_are_added_in_32_interleaved_chains(lib):
+    """The order of the weight gradient's per-entry sums, bit for bit: a column with many entries is added as 32
+    chains of fused multiply-adds (entries i, i + 32, ...) whose results are added in order, a column with few as
+    one chain.  Positive and negative entries number less than n_tail and everything else is zero, so the
+    thresholds are 0, the codes are 0 and dW is the compensation alone.  (Entries and dY are BF16 numbers of
+    similar magnitude: a float64 holds product plus sum exactly, so each step is rounded once, as on the GPU.)"""
+    M, K, N, alpha = 1024, 256, 384, 0.996
+    sizes = {3: 700, 70: 600, 128: 100, 200: 65, 255: 513, 10: 40, 11: 7, 12: 1}     # column: entries
+    rng = np.random.default_rng(5)
+    a = np.zeros((M, K), dtype=np.float32)
+    for k, n in sizes.items():
+        a[rng.choice(M, n, replace=False), k] = rng.standard_normal(n) + 0.01
+    a_bits, dy_bits = WL.to_bf16_bits(a), WL.to_bf16_bits(rng.standard_normal((M, N)).astype(np.float32))
+    w_bits = WL.small_case(M, K, N, seed=3)[1]
+    a, dy = O.bf16_bits_to_f64(a_bits), O.bf16_bits_to_f64(dy_bits)
+    assert max((a > 0).sum(), (a < 0).sum()) < round((1 - alpha) * M * K)
+    want = np.zeros((K, N), dtype=np.float32)
+    for k in sizes:
+        rows = np.flatnonzero(a[:, k])
+        chains = 32 if rows.size >= 64 else 1
+        for c in range(chains):
+            part = np.zeros(N, dtype=np.float32)
+            for m in rows[c::chains]:
+                part = (a[m, k] * dy[m] + part).astype(np.float32)
+            want[k] = want[k] + part
+    ctx = lib.Context.for_shape(M, K, N)
+    W, dY = _dev(w_bits), _dev(dy_bits)
+    _, sa, sw = lib.fp4_linear_fwd(ctx, _dev(a_bits), W, alpha)
+    _, dw = lib.fp4_linear_bwd(ctx, dY, W, sa, sw, out_f32=True, want_da=False, dge_on=False)
+    torch.cuda.synchronize()
+    assert ctx.read_status() == 0 and not sa.codes.any()
+    np.testing.assert_array_equal(dw.cpu().numpy(), want)
+    ctx.close()
