@@ -118,8 +118,9 @@ int fp4_create(fp4_ctx** out, int device, size_t workspace_bytes);
 int fp4_destroy(fp4_ctx* ctx);
 
 /* Workspace that fp4_quantize / fp4_linear_fwd / fp4_linear_bwd need for these sizes.  It includes
- * up to 128 MB for the dense form of a heavy residual (see fp4_linear_fwd); a workspace that is
- * smaller by that much is accepted too, and the residual's entries are then added one by one.  */
+ * up to 128 MB for the dense form of a heavy residual (see fp4_linear_fwd); a workspace smaller
+ * than this by up to that much is accepted too, and the residual's entries are then added one by
+ * one.  */
 size_t fp4_workspace_bytes(int64_t M, int64_t K, int64_t N);
 
 /* Residual entries that clamping at `alpha` can produce at most (Section 3.2: two tails of

@@ -32,7 +32,7 @@ size_t linear_scratch_bytes(int64_t M, int64_t K, int64_t N) {
   return b;
 }
 
-// Scratch of the heavy residual's dense product, forward or backward: used where the workspace has room for it.
+// Scratch of the heavy residual's dense product, forward or backward.
 size_t full_scratch_bytes(int64_t M, int64_t K) {
   const size_t f = residual_full_scratch_bytes(M, K), b = residual_full_scratch_bytes(K, M);
   return f > b ? f : b;
@@ -57,6 +57,12 @@ bool heavy_residual(const fp4_qtensor* a, int64_t M, int64_t K) {
 bool full_product_pays(const fp4_ctx* ctx, const fp4_qtensor* a, int64_t R, int64_t C, int64_t N) {
   const int64_t tiles = (R / 128) * ((N + 255) / 256), rounds = (tiles + ctx->num_sms - 1) / ctx->num_sms;
   return rounds * (C / 128 * 1900 + 4000) + 6000 < a->sparse_cap * N / 6500 + 5000;
+}
+
+// A workspace of fp4_workspace_bytes holds the dense operand, a smaller one is not searched for spare room: which
+// form a residual takes depends on the sizes alone.
+bool full_product_fits(const Arena& whole, int64_t M, int64_t K, int64_t N) {
+  return whole.size >= least_workspace_bytes(M, K, N) + full_scratch_bytes(M, K);
 }
 
 int check_qtensor_dense(const fp4_qtensor* q) {
@@ -342,7 +348,8 @@ int linear_fwd_impl(fp4_ctx* ctx, cudaStream_t st, Arena arena, const void* A_bf
   // GEMM, whose epilogue adds the product.  A lighter one that still may hold 1 % (by the caller's capacity: alpha
   // <= 0.995) sends its hot columns through the GEMM as a dense tail instead of per-entry gathers.
   const size_t full_bytes = residual_full_scratch_bytes(M, K);
-  char* scratch_full = occ && heavy_residual(savedA, M, K) && full_product_pays(ctx, savedA, M, K, N) && full_bytes && arena.ok && arena.size - arena.off >= full_bytes
+  const bool full_room = full_bytes && full_product_fits(arena, M, K, N);
+  char* scratch_full = occ && full_room && heavy_residual(savedA, M, K) && full_product_pays(ctx, savedA, M, K, N)
                            ? arena.take<char>(full_bytes) : nullptr;
   const bool full_on = scratch_full != nullptr;
   const bool tail_on = occ && !full_on && savedA->csr_rowptr && savedA->csc_colptr && !heavy_residual(savedA, M, K) &&
@@ -527,9 +534,10 @@ int linear_bwd_impl(fp4_ctx* ctx, cudaStream_t st, Arena arena, const void* dY_b
   const int* slot_of_col = nullptr;
   if (!arena.ok) return FP4_ERR_WORKSPACE;
   const size_t full_bytes = residual_full_scratch_bytes(K, M);
-  char* scratch_full = has_comp && heavy_residual(savedA, M, K) && full_product_pays(ctx, savedA, K, M, N) && full_bytes &&
-                               arena.size - arena.off >= full_bytes + quantize_scratch_bytes(M, N)
+  const bool full_room = full_bytes && full_product_fits(arena, M, K, N);
+  char* scratch_full = has_comp && full_room && heavy_residual(savedA, M, K) && full_product_pays(ctx, savedA, K, M, N)
                            ? arena.take<char>(full_bytes) : nullptr;
+  if (!arena.ok) return FP4_ERR_WORKSPACE;
   Arena q_arena(arena.base + arena.off, arena.size - arena.off);
   int rc;
 

@@ -420,7 +420,7 @@ def test_tensor_core_accumulation_stays_inside_its_floor(lib, ctx):
 
 @pytest.mark.parametrize("M,K,N", [(128, 128, 128), (256, 1024, 1024), (640, 512, 1408)])
 def test_weights_on_a_16_byte_boundary(lib, M, K, N):
-    """The ABI asks for 16-byte alignment; the fused epilogue reads weights on a 32-byte boundary with wider loads."""
+    """The ABI asks for 16-byte alignment: weights half-way between two 32-byte sectors give the same gradients."""
     a, w, dy = (torch.from_numpy(b.view(np.int16)).cuda().view(torch.bfloat16) for b in WL.small_case(M, K, N, seed=9))
     moved = torch.empty(K * N + 8, dtype=torch.bfloat16, device="cuda")[8:].view(K, N)
     moved.copy_(w)
@@ -435,13 +435,19 @@ def test_weights_on_a_16_byte_boundary(lib, M, K, N):
     ctx.close()
 
 
-@pytest.mark.parametrize("M,K,N,alpha,wide", [(1024, 1280, 2176, 0.97, False), (512, 256, 2176, 0.9, True), (640, 8320, 1152, 0.95, True),
-                                              (16384, 1408, 1152, 0.97, False), (1408, 16384, 1152, 0.97, True)])
-def test_heavy_residual_as_a_dense_product(lib, M, K, N, alpha, wide):
+@pytest.mark.parametrize("M,K,N,alpha,wide,fwd,bwd", [
+    (1024, 1280, 2176, 0.97, False, True, True),
+    (512, 256, 2176, 0.9, True, True, False),
+    (640, 8320, 1152, 0.95, True, False, True),
+    (16384, 1408, 1152, 0.96, False, True, True),      # backward: rows of 16384, two segments
+    (1408, 16384, 1152, 0.96, True, True, True),       # forward: rows of 16384; backward: several slabs of rows
+])
+def test_heavy_residual_as_a_dense_product(lib, M, K, N, alpha, wide, fwd, bwd):
     """More than 4 % of the activation in the residual: the tensor cores multiply it whole (several slabs of rows,
-    rows longer than a segment, values that need a third BF16 term).  Against the per-entry kernels, which a
-    context without room for the dense operand uses; either differs from the exact sum by at most
-    4e-6 sum |residual| |dense|."""
+    rows longer than a segment, values that need a third BF16 term), where that takes less time (`fwd`, `bwd`).
+    Against the per-entry kernels, which a context takes whose workspace is smaller than fp4_workspace_bytes;
+    either differs from the exact sum by at most 4e-6 sum |residual| |dense|.  The two add in different orders, so
+    outputs that agree in every bit would mean that both contexts took the same path."""
     gen = torch.Generator("cuda").manual_seed(M + K)
     A = torch.randn((M, K), device="cuda", generator=gen)
     if wide:
@@ -450,7 +456,7 @@ def test_heavy_residual_as_a_dense_product(lib, M, K, N, alpha, wide):
     W = (torch.randn((K, N), device="cuda", generator=gen) * 0.02).to(torch.bfloat16)
     dY = (torch.randn((M, N), device="cuda", generator=gen) * 1e-3).to(torch.bfloat16)
     size = int(lib.load_library().fp4_workspace_bytes(M, K, N))
-    room, tight = lib.Context(0, size), lib.Context(0, size - 4096)
+    room, tight = lib.Context(0, size), lib.Context(0, size - 256)
     out = []
     for c in (room, tight):
         y, sa, sw = lib.fp4_linear_fwd(c, A, W, alpha, out_f32=True)
@@ -463,6 +469,7 @@ def test_heavy_residual_as_a_dense_product(lib, M, K, N, alpha, wide):
     assert float((res > 0).double().mean()) > 0.04
     (y, da, dw, _), (y1, da1, dw1, _) = out
     assert torch.equal(da, da1)
+    assert torch.equal(y, y1) != fwd and torch.equal(dw, dw1) != bwd
     # the two sums of the outputs' branches are fp32: 2^-23 of the larger value on top
     assert bool(((y - y1).abs().double() <= 2 * 4e-6 * (res @ W.double().abs()) + 2.4e-7 * y.abs() + 1e-30).all())
     assert bool(((dw - dw1).abs().double() <= 2 * 4e-6 * (res.T @ dY.double().abs()) + 2.4e-7 * dw.abs() + 1e-30).all())
