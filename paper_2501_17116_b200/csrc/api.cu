@@ -47,16 +47,14 @@ size_t least_workspace_bytes(int64_t M, int64_t K, int64_t N) {
   return q + linear_scratch_bytes(M, K, N) + 4096;
 }
 
-// A residual that may hold 1 / RESIDUAL_FULL_SHARE of the activation or more takes no dense tail ...
+// A residual that may fill more than 1 / RESIDUAL_FULL_SHARE of the activation takes no dense tail ...
 bool heavy_residual(const fp4_qtensor* a, int64_t M, int64_t K) {
   return a->csr_rowptr && a->csc_colptr && a->sparse_cap * RESIDUAL_FULL_SHARE > M * K && M >= 512;
 }
-// ... and is multiplied as a dense matrix [R x C] (times [C x N]) unless the gathers take less time: small
-// products do not fill the chip (512 x 1024 x 1024 at 6 %: 11 us of gathers, 25 us).  In ns: 13 TB/s of gathered
-// rows; 1.9 us per 128 contraction indices of a 128 x 256 tile, one tile per SM at a time.
+// ... and is multiplied as a dense matrix [R x C] (times [C x N]) unless the gathers take less time: small products
+// do not fill the chip.
 bool full_product_pays(const fp4_ctx* ctx, const fp4_qtensor* a, int64_t R, int64_t C, int64_t N) {
-  const int64_t tiles = (R / 128) * ((N + 255) / 256), rounds = (tiles + ctx->num_sms - 1) / ctx->num_sms;
-  return rounds * (C / 128 * 1900 + 4000) + 6000 < a->sparse_cap * N / 6500 + 5000;
+  return residual_full_from(ctx, R, C, N) <= a->sparse_cap;
 }
 
 // A workspace of fp4_workspace_bytes holds the dense operand, a smaller one is not searched for spare room: which

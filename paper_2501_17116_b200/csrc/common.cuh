@@ -272,12 +272,14 @@ size_t comp_wgrad_scratch_bytes(int64_t M, int64_t K, int64_t N);
 
 // out[r, :] = sum_c V[r, c] dense[c, :] for a whole sparse matrix V [R x C] (CSR: ptr, idx, val), as a dense product
 // on the tensor cores (wgrad_dense_tc.cu): the residual's rows times the weights, or its columns times dY.
-// What a gather costs grows with the entries, what this costs does not: two exact BF16 terms of V at about 1.2 PFLOP/s
-// against 13 TB/s of gathered rows meet at an entry share of 2 to 3 %; from RESIDUAL_FULL_SHARE on the dense
-// product is taken (alpha <= 0.98).  `scratch` holds a slab of V's terms.
-constexpr int RESIDUAL_FULL_SHARE = 25;              // entries: at least 1 / 25 of the matrix
+// What a gather costs grows with the entries, what this costs does not: residual_full_from is the number of entries
+// from which it takes less time.  It is offered residuals that may fill more than 1 / RESIDUAL_FULL_SHARE of the
+// matrix; the number of entries that are there, known on the device, decides (dense_rows_kernel).  `scratch`
+// holds a slab of V's terms.
+constexpr int RESIDUAL_FULL_SHARE = 25;
 constexpr int64_t FULL_SLAB_BYTES = 128 << 20;       // about what L2 holds
 size_t residual_full_scratch_bytes(int64_t R, int64_t C);
+int64_t residual_full_from(const fp4_ctx* ctx, int64_t R, int64_t C, int64_t N);
 int launch_residual_full(fp4_ctx* ctx, cudaStream_t stream, const int32_t* ptr, const int32_t* idx, const float* val, int64_t R,
                          int64_t C, const void* dense_bf16, int64_t N, Arena& scratch, float* out, int kernel_class,
                          int32_t* status);

@@ -13,20 +13,12 @@
 #include <cuda_fp16.h>
 
 #include "common.cuh"
+#include "gather.cuh"
 
 namespace {
 
 constexpr int COMP_THREADS = 256;          // 8 warps = 8 output rows per block
 constexpr int COMP_COLS = 256;             // columns per block (8 per lane)
-
-__device__ __forceinline__ void fma8(float (&acc)[8], float v, const uint4& d) {
-  const uint32_t w[4] = {d.x, d.y, d.z, d.w};
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    acc[2 * q] = fmaf(v, __uint_as_float(w[q] << 16), acc[2 * q]);
-    acc[2 * q + 1] = fmaf(v, __uint_as_float(w[q] & 0xFFFF0000u), acc[2 * q + 1]);
-  }
-}
 
 __device__ __forceinline__ void store8(void* out, int out_f32, long long off, const float (&y)[8]) {
   if (out_f32) {
@@ -44,23 +36,6 @@ __device__ __forceinline__ void store8(void* out, int out_f32, long long off, co
   }
 }
 
-// acc += n entries, gathered together
-template <int n>
-__device__ __forceinline__ void add_entries(float (&acc)[8], const int* __restrict__ idx, const float* __restrict__ val,
-                                            const uint4* __restrict__ dense, int vec_per_row, int vcol) {
-  int r[n];
-  float v[n];
-  uint4 d[n];
-#pragma unroll
-  for (int u = 0; u < n; ++u) {
-    r[u] = __ldg(&idx[u]);
-    v[u] = __ldg(&val[u]);
-  }
-#pragma unroll
-  for (int u = 0; u < n; ++u) d[u] = __ldg(&dense[(long long)r[u] * vec_per_row + vcol]);
-#pragma unroll
-  for (int u = 0; u < n; ++u) fma8(acc, v[u], d[u]);
-}
 template <int n>
 __device__ __forceinline__ void add_kept(float (&acc)[8], const uint2* __restrict__ kept, const uint4* __restrict__ dense,
                                          int vec_per_row, int vcol) {
@@ -72,19 +47,6 @@ __device__ __forceinline__ void add_kept(float (&acc)[8], const uint2* __restric
   for (int u = 0; u < n; ++u) d[u] = __ldg(&dense[(long long)t[u].x * vec_per_row + vcol]);
 #pragma unroll
   for (int u = 0; u < n; ++u) fma8(acc, __uint_as_float(t[u].y), d[u]);
-}
-
-// acc[0..7] += sum over the entries [e0, e1) of val[e] * dense[idx[e], col .. col+7]
-__device__ __forceinline__ void sparse_row_times_dense(float (&acc)[8], const int* __restrict__ idx,
-                                                       const float* __restrict__ val, int e0, int e1,
-                                                       const uint4* __restrict__ dense, int vec_per_row, int vcol) {
-  int e = e0;
-  for (; e + 4 <= e1; e += 4) add_entries<4>(acc, idx + e, val + e, dense, vec_per_row, vcol);   // four loads in flight
-  if (e + 2 <= e1) {
-    add_entries<2>(acc, idx + e, val + e, dense, vec_per_row, vcol);
-    e += 2;
-  }
-  if (e < e1) add_entries<1>(acc, idx + e, val + e, dense, vec_per_row, vcol);
 }
 
 // Y1 is read for the last time and Y leaves with streaming stores, so that neither pushes the rest of Y1 and the slab

@@ -23,6 +23,7 @@
 #include <cuda.h>
 
 #include "common.cuh"
+#include "gather.cuh"
 #include "tc_ptx.cuh"
 
 namespace {
@@ -108,47 +109,80 @@ dense_split_kernel(const int* __restrict__ colptr, const int* __restrict__ row, 
 // The whole residual (or its transpose) as a dense operand, for residuals so heavy that gathering costs more:
 // row r of Vt[term][r][c] holds the terms of the residual's row r, zeros elsewhere.  A block writes one row, in
 // segments of ROW_SEG contraction indices.  Terms 1 and 2 are written always; term 3 is zero unless a value spans
-// more than 16 bits (500 times the threshold): *third says so, and a second launch (THIRD) then writes it.
+// more than 16 bits (500 times the threshold): *third says so, and a second launch (SECOND) then writes it.
+// How many entries there are is known on the device only (ties at the thresholds leave fewer than alpha allows,
+// an activation of three values none): below `dense_from` of them this operand and the product are left out, and
+// the second launch adds the entries one by one instead, a warp per row and 256 outputs.
 constexpr int ROW_SEG = 8192;
-template <bool THIRD>
-__global__ void __launch_bounds__(256)
-dense_rows_kernel(const int* __restrict__ ptr, const int* __restrict__ idx, const float* __restrict__ val, int row0, int rows,
-                  int C, __nv_bfloat16* __restrict__ vt, int* __restrict__ third) {
-  __shared__ __align__(16) __nv_bfloat16 tile[THIRD ? 1 : 2][ROW_SEG];
-  if (THIRD && *third == 0) return;
-  const int r = blockIdx.x, t = threadIdx.x;
-  const int e0 = ptr[row0 + r], e1 = ptr[row0 + r + 1];
+struct DenseRowsArgs {
+  const int* ptr;              // the whole matrix: R rows
+  const int* idx;
+  const float* val;
+  int R, C, row0, rows;        // the slab: rows row0 ..
+  int dense_from;
+  __nv_bfloat16* vt;
+  int* third;
+  const uint4* dense;          // [C x N]
+  int N;
+  float* out;                  // [R x N]
+};
+template <bool SECOND>
+__global__ void __launch_bounds__(256, 6)
+dense_rows_kernel(const __grid_constant__ DenseRowsArgs a) {
+  __shared__ __align__(16) __nv_bfloat16 tile[SECOND ? 1 : 2][ROW_SEG];
+  const int* __restrict__ ptr = a.ptr;
+  const int* __restrict__ idx = a.idx;
+  const float* __restrict__ val = a.val;
+  const int t = threadIdx.x;
+  if (__ldg(&ptr[a.R]) < a.dense_from) {
+    if (!SECOND) return;
+    // (outputs the slow index: the rows of the dense matrix that are in use at a time stay in L2)
+    const int groups = a.rows >> 3, items = groups * ((a.N + 255) >> 8);
+    for (int it = blockIdx.x; it < items; it += a.rows) {
+      const int nb = it / groups, row = a.row0 + (it - nb * groups) * 8 + (t >> 5), n0 = 256 * nb + 8 * (t & 31);
+      if (n0 >= a.N) continue;
+      float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+      sparse_row_times_dense(acc, idx, val, __ldg(&ptr[row]), __ldg(&ptr[row + 1]), a.dense, a.N >> 3, n0 >> 3);
+      float4* dst = reinterpret_cast<float4*>(a.out + (long long)row * a.N + n0);
+      dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
+      dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+    }
+    return;
+  }
+  if (SECOND && *a.third == 0) return;
+  const int r = blockIdx.x;
+  const int e0 = __ldg(&ptr[a.row0 + r]), e1 = __ldg(&ptr[a.row0 + r + 1]);
   uint4* t4 = reinterpret_cast<uint4*>(&tile[0][0]);
   bool any = false;
-  for (int c0 = 0; c0 < C; c0 += ROW_SEG) {
-    const int c1 = min(C, c0 + ROW_SEG);
-    for (int i = t; i < (THIRD ? 1 : 2) * ROW_SEG / 8; i += 256) t4[i] = make_uint4(0, 0, 0, 0);
+  for (int c0 = 0; c0 < a.C; c0 += ROW_SEG) {
+    const int c1 = min(a.C, c0 + ROW_SEG);
+    for (int i = t; i < (SECOND ? 1 : 2) * ROW_SEG / 8; i += 256) t4[i] = make_uint4(0, 0, 0, 0);
     __syncthreads();
     for (int e = e0 + t; e < e1; e += 256) {
-      const int c = idx[e];
+      const int c = __ldg(&idx[e]);
       if (c < c0 || c >= c1) continue;
-      const float v = val[e];
+      const float v = __ldg(&val[e]);
       const __nv_bfloat16 b1 = __float2bfloat16_rn(v);
       const float r1 = v - __bfloat162float(b1);                 // exact
       const __nv_bfloat16 b2 = __float2bfloat16_rn(r1);
       const float r2 = r1 - __bfloat162float(b2);                // exact
-      if (THIRD) {
+      if (SECOND) {
         tile[0][c - c0] = __float2bfloat16_rn(r2);               // exact
       } else {
         tile[0][c - c0] = b1;
-        tile[THIRD ? 0 : 1][c - c0] = b2;
+        tile[1 - SECOND][c - c0] = b2;
         any |= r2 != 0.0f;
       }
     }
     __syncthreads();
 #pragma unroll
-    for (int term = 0; term < (THIRD ? 1 : 2); ++term)
+    for (int term = 0; term < 2 - SECOND; ++term)
       for (int i = t; i < (c1 - c0) / 8; i += 256)
-        *reinterpret_cast<uint4*>(vt + (size_t(THIRD ? 2 : term) * rows + r) * size_t(C) + c0 + 8 * i) =
+        *reinterpret_cast<uint4*>(a.vt + (size_t(SECOND ? 2 : term) * a.rows + r) * size_t(a.C) + c0 + 8 * i) =
             *reinterpret_cast<const uint4*>(&tile[term][8 * i]);
     __syncthreads();
   }
-  if (!THIRD && any) *third = 1;                     // (any number of threads writes the same)
+  if (!SECOND && any) *a.third = 1;                  // (any number of threads writes the same)
 }
 
 struct DenseTcArgs {
@@ -158,6 +192,8 @@ struct DenseTcArgs {
   int vt_rows;               // rows of a term of Vt
   const int* counts;         // counts[0] = number of dense columns (device); FULL: whether the third term is needed
   float* partial;            // [splits][DENSE_TC_MAX][N]; FULL: [vt_rows][N]
+  const int* entries;        // FULL: number of entries (device); fewer than dense_from: nothing to do
+  int dense_from;
   int32_t* status;
 };
 
@@ -168,7 +204,7 @@ comp_wgrad_dense_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __g
                            const __grid_constant__ DenseTcArgs args) {
   extern __shared__ uint8_t smem_raw[];
   const int n_dense = FULL ? DENSE_TC_MAX : min(__ldg(args.counts), DENSE_TC_MAX);
-  if (n_dense == 0) return;                               // uniform: nothing allocated yet
+  if (n_dense == 0 || (FULL && __ldg(args.entries) < args.dense_from)) return;      // uniform: nothing allocated yet
   const int terms = FULL && *args.counts == 0 ? 2 : 3;
   const int nb = (n_dense + 63) / 64;                     // 64-row boxes of V per term
   const int stages = nb == 1 || terms == 2 ? 3 : 2;
@@ -433,6 +469,8 @@ int launch_comp_wgrad_dense_tc(fp4_ctx* ctx, cudaStream_t stream, const fp4_qten
   args.counts = counts;
   args.partial = partial;
   args.status = status;
+  args.entries = nullptr;
+  args.dense_from = 0;
   FP4_CUDA_TRY(cudaFuncSetAttribute(comp_wgrad_dense_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, DT_SMEM));
   comp_wgrad_dense_tc_kernel<false><<<unsigned(args.tiles * splits), DT_THREADS, DT_SMEM, stream>>>(map_dy, map_vt, args);
   FP4_CUDA_TRY(cudaGetLastError());
@@ -450,6 +488,21 @@ size_t residual_full_scratch_bytes(int64_t R, int64_t C) {
   return rows < 128 ? 0 : ((size_t(6) * size_t(rows) * size_t(C) + 255) & ~size_t(255)) + 256;
 }
 
+// In ns: 15 TB/s of gathered rows (2 N bytes an entry) against 1.9 us per 128 contraction indices of a 128 x 256 tile,
+// one tile per SM at a time, slab after slab (4096 x 11008 x 512: three slabs of 30 tiles, 480 us; the gathers 220),
+// and the operand's 4 bytes per element.
+int64_t residual_full_from(const fp4_ctx* ctx, int64_t R, int64_t C, int64_t N) {
+  const int64_t slab = full_slab_rows(R, C);
+  if (slab < 128) return INT64_MAX;
+  int64_t ns = 0;
+  for (int64_t r0 = 0; r0 < R; r0 += slab) {
+    const int64_t rows = R - r0 < slab ? R - r0 : slab;
+    const int64_t tiles = rows / 128 * ((N + DT_NT - 1) / DT_NT), rounds = (tiles + ctx->num_sms - 1) / ctx->num_sms;
+    ns += rounds * (C / 128 * 1900 + 4000) + 6000 + rows * C / 1200;
+  }
+  return (ns > 5000 ? ns - 5000 : 0) * 7500 / N + 1;
+}
+
 int launch_residual_full(fp4_ctx* ctx, cudaStream_t stream, const int32_t* ptr, const int32_t* idx, const float* val, int64_t R,
                          int64_t C, const void* dense_bf16, int64_t N, Arena& scratch, float* out, int kernel_class,
                          int32_t* status) {
@@ -463,12 +516,26 @@ int launch_residual_full(fp4_ctx* ctx, cudaStream_t stream, const int32_t* ptr, 
   FP4_CUDA_TRY(cudaFuncSetAttribute(comp_wgrad_dense_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, DT_SMEM));
   FP4_CUDA_TRY(cudaMemsetAsync(third, 0, 4, stream));
   KernelScope scope(ctx, stream, kernel_class, 3 * int((R + slab - 1) / slab));
+  DenseRowsArgs ra;
+  ra.ptr = ptr;
+  ra.idx = idx;
+  ra.val = val;
+  ra.R = int(R);
+  ra.C = int(C);
+  ra.dense_from = int(residual_full_from(ctx, R, C, N));          // (the caller has compared it with a bound below 2^31)
+  ra.vt = vt;
+  ra.third = third;
+  ra.dense = static_cast<const uint4*>(dense_bf16);
+  ra.N = int(N);
+  ra.out = out;
   for (int64_t r0 = 0; r0 < R; r0 += slab) {
     const int64_t rows = R - r0 < slab ? R - r0 : slab;
     rc = make_bf16_map(ctx, &map_vt, vt, 3 * rows, C);
     if (rc != FP4_OK) return rc;
-    dense_rows_kernel<false><<<unsigned(rows), 256, 0, stream>>>(ptr, idx, val, int(r0), int(rows), int(C), vt, third);
-    dense_rows_kernel<true><<<unsigned(rows), 256, 0, stream>>>(ptr, idx, val, int(r0), int(rows), int(C), vt, third);
+    ra.row0 = int(r0);
+    ra.rows = int(rows);
+    dense_rows_kernel<false><<<unsigned(rows), 256, 0, stream>>>(ra);
+    dense_rows_kernel<true><<<unsigned(rows), 256, 0, stream>>>(ra);
     DenseTcArgs args;
     args.M = int(C);
     args.N = int(N);
@@ -478,6 +545,8 @@ int launch_residual_full(fp4_ctx* ctx, cudaStream_t stream, const int32_t* ptr, 
     args.counts = third;
     args.partial = out + size_t(r0) * size_t(N);
     args.status = status;
+    args.entries = ptr + R;
+    args.dense_from = ra.dense_from;
     comp_wgrad_dense_tc_kernel<true><<<unsigned(args.tiles * args.splits), DT_THREADS, DT_SMEM, stream>>>(map_dense, map_vt, args);
   }
   FP4_CUDA_TRY(cudaGetLastError());

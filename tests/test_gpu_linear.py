@@ -436,11 +436,11 @@ def test_weights_on_a_16_byte_boundary(lib, M, K, N):
 
 
 @pytest.mark.parametrize("M,K,N,alpha,wide,fwd,bwd", [
-    (1024, 1280, 2176, 0.97, False, True, True),
-    (512, 256, 2176, 0.9, True, True, False),
+    (1024, 1280, 2176, 0.95, False, True, True),
+    (2048, 512, 2048, 0.97, True, True, False),
     (640, 8320, 1152, 0.95, True, False, True),
-    (16384, 1408, 1152, 0.96, False, True, True),      # backward: rows of 16384, two segments
-    (1408, 16384, 1152, 0.96, True, True, True),       # forward: rows of 16384; backward: several slabs of rows
+    (16384, 1408, 2176, 0.95, False, True, True),      # backward: rows of 16384, two segments
+    (1408, 16384, 2176, 0.95, True, True, True),       # forward: rows of 16384; backward: several slabs of rows
 ])
 def test_heavy_residual_as_a_dense_product(lib, M, K, N, alpha, wide, fwd, bwd):
     """More than 4 % of the activation in the residual: the tensor cores multiply it whole (several slabs of rows,
@@ -510,3 +510,30 @@ def test_long_columns_are_added_in_32_interleaved_chains(lib):
     assert ctx.read_status() == 0 and not sa.codes.any()
     np.testing.assert_array_equal(dw.cpu().numpy(), want)
     ctx.close()
+
+
+@pytest.mark.parametrize("M,K,N", [(1024, 1280, 2176), (1920, 5504, 2048), (2048, 640, 4992)])
+@pytest.mark.parametrize("kind", ["empty", "one-sided"])
+def test_residual_with_fewer_entries_than_alpha_allows(lib, M, K, N, kind):
+    """alpha = 0.95 allows 10 %, but ties at the thresholds leave none (three values) or one tail (rectified): the
+    device counts the entries and adds them one by one where that is the shorter way, in the per-entry kernels'
+    order.  A third of a percent in all is far below where a dense product starts to pay."""
+    gen = torch.Generator("cuda").manual_seed(M + K)
+    A = torch.randn((M, K), device="cuda", generator=gen)
+    if kind == "empty":
+        A = A.round().clamp(-1, 1)
+    else:                                   # 0.3 % positive values, the rest zero: both thresholds are 0
+        A = torch.where(torch.rand((M, K), device="cuda", generator=gen) < 0.003, A.abs(), 0.0)
+    A = A.to(torch.bfloat16)
+    W = (torch.randn((K, N), device="cuda", generator=gen) * 0.02).to(torch.bfloat16)
+    dY = (torch.randn((M, N), device="cuda", generator=gen) * 1e-3).to(torch.bfloat16)
+    size = int(lib.load_library().fp4_workspace_bytes(M, K, N))
+    out = []
+    for c in (lib.Context(0, size), lib.Context(0, size - 256)):
+        y, sa, sw = lib.fp4_linear_fwd(c, A, W, 0.95, out_f32=True)
+        _, dw = lib.fp4_linear_bwd(c, dY, W, sa, sw, out_f32=True, dge_on=False, want_da=False)
+        torch.cuda.synchronize()
+        assert c.read_status() == 0 and (int(sa.nnz) == 0) == (kind == "empty") and int(sa.nnz) < 0.004 * M * K
+        out.append((y, dw))
+        c.close()
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
