@@ -205,7 +205,7 @@ int fp4_gemm(fp4_ctx* ctx, void* stream, const uint8_t* a_codes, const uint8_t* 
  *   beyond 43 000 times its token's clamped absmax does not fit the FP16 operand: the call
  *   then adds every entry per entry.
  *   A residual that may fill more than 4 % of the activation (sparse_cap, M >= 512) is multiplied
- *   as a dense matrix where that takes less time: exact three-term BF16 split, chunks of 128 input
+ *   as a dense matrix where that takes less time for the entries that are there: exact three-term BF16 split, chunks of 64 input
  *   channels added in fp32 in order.  Same bound, without the second term.
  */
 #define FP4_REUSE_W 1

@@ -198,6 +198,10 @@ struct DenseTcArgs {
 };
 
 // FULL: every row of the result, in blocks of 128; else the dense columns' rows, in ranges of the contraction.
+// FULL drains tensor memory every 64 contraction indices: of the 8 or 12 truncating additions behind a drained sum four
+// bring its leading term.  (Chunks of 128, terms interleaved: 7 % further from the exact sum than the gathers' fused
+// multiply-adds at a contraction of 512 without hot columns, now 3 % nearer; and slower, 1920 x 5504 x 2048 at alpha
+// 0.97 forward 167 us, 158 now: a stage is freed and a drain begins twice as often.)
 template <bool FULL>
 __global__ void __launch_bounds__(DT_THREADS, 1)
 comp_wgrad_dense_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __grid_constant__ CUtensorMap map_vt,
@@ -222,7 +226,8 @@ comp_wgrad_dense_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __g
 
   const int warp = __shfl_sync(0xFFFFFFFFu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const int tile = blockIdx.x % args.tiles, split = blockIdx.x / args.tiles;
-  const int chunks_total = (args.M + DT_CHUNK - 1) / DT_CHUNK;
+  constexpr int HALVES = FULL ? 1 : 2, CHUNK = HALVES * DT_TOK;      // stages and contraction indices per chunk
+  const int chunks_total = (args.M + CHUNK - 1) / CHUNK;
   const int c_begin = FULL ? 0 : int((long long)chunks_total * split / args.splits);
   const int c_end = FULL ? chunks_total : int((long long)chunks_total * (split + 1) / args.splits);
   const int s0 = FULL ? split * DENSE_TC_MAX : 0;         // first row of Vt
@@ -261,8 +266,8 @@ comp_wgrad_dense_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __g
       int stage = 0;
       uint32_t phase = 0, fills = 0;
       bool ok = true;
-      for (int c = 0; c < 2 * n_chunks && ok; ++c) {            // one stage = 64 tokens
-        const int m0 = c_begin * DT_CHUNK + c * DT_TOK;
+      for (int c = 0; c < HALVES * n_chunks && ok; ++c) {       // one stage = 64 tokens
+        const int m0 = c_begin * CHUNK + c * DT_TOK;
         ok = mbar_wait(&empty_bar[stage], phase ^ 1u, abort_flag, args.status);
         if (!ok) break;
         uint8_t* dst = smem + stage * stage_bytes;
@@ -301,23 +306,26 @@ comp_wgrad_dense_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __g
         ok = mbar_wait(&acc_empty[acc], acc_phase ^ 1u, abort_flag, args.status);
         if (!ok) break;
         tc_fence_after();
-        for (int half = 0; half < 2 && ok; ++half) {            // the two stages of this chunk
+        for (int half = 0; half < HALVES && ok; ++half) {       // the stages of this chunk
           ok = mbar_wait(&full_bar[stage], phase, abort_flag, args.status);
           if (!ok) break;
           tc_fence_after();
           const uint32_t dy_addr = smem_u32(smem + stage * stage_bytes);
           const uint32_t v_addr = dy_addr + DT_DY_BYTES;
           if (FULL) {
+            // The small terms first: what an addition loses grows with the running sum, which the last term brings.
             const uint32_t d_tmem = tmem_base + uint32_t(acc * 256);
+            uint32_t accumulate = 0u;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {                       // 16 contraction indices per instruction
-              const uint64_t b_desc = make_smem_desc_mn(dy_addr + uint32_t(k * 2048), DT_BOX);
+            for (int t = 2; t >= 0; --t)
+              if (t < terms) {
 #pragma unroll
-              for (int t = 0; t < 3; ++t)
-                if (t < terms)
-                  mma_f16(d_tmem, make_smem_desc(v_addr + uint32_t(t * 2 * DT_BOX + k * 32)), b_desc, idesc,
-                          (half | k | t) != 0 ? 1u : 0u);
-            }
+                for (int k = 0; k < 4; ++k) {                   // 16 contraction indices per instruction
+                  mma_f16(d_tmem, make_smem_desc(v_addr + uint32_t(t * 2 * DT_BOX + k * 32)),
+                          make_smem_desc_mn(dy_addr + uint32_t(k * 2048), DT_BOX), idesc, accumulate);
+                  accumulate = 1u;
+                }
+              }
           } else
 #pragma unroll
           for (int h = 0; h < 2; ++h) {                         // output columns n0 + 128 h .. + 127

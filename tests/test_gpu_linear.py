@@ -537,3 +537,28 @@ def test_residual_with_fewer_entries_than_alpha_allows(lib, M, K, N, kind):
         out.append((y, dw))
         c.close()
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("M,K,N", [(2048, 512, 2048), (8192, 512, 1024), (1920, 5504, 2048)])
+def test_dense_product_of_a_heavy_residual_is_no_less_precise_than_its_gathers(lib, M, K, N):
+    """Laplace activations with outliers in single elements: no hot column, every entry is one fused multiply-add in
+    the per-entry kernel.  Y of the dense form must not be further from the float64 sum (2-norm; 2 % for which
+    roundings happen to fall where) than Y of the per-entry form."""
+    gen = torch.Generator("cuda").manual_seed(K)
+    A = torch.empty((M, K), device="cuda").exponential_(generator=gen) * torch.randn((M, K), device="cuda", generator=gen).sign()
+    A = torch.where(torch.rand((M, K), device="cuda", generator=gen) < 0.002, A * 100.0, A).to(torch.bfloat16)
+    W = (torch.randn((K, N), device="cuda", generator=gen) * 0.02).to(torch.bfloat16)
+    size = int(lib.load_library().fp4_workspace_bytes(M, K, N))
+    values = torch.tensor([0, 0.5, 1, 1.5, 2, 3, 4, 6, 0, -0.5, -1, -1.5, -2, -3, -4, -6], dtype=torch.float64, device="cuda")
+    decode = lambda c: torch.stack([values[(c & 15).long()], values[(c >> 4).long()]], -1).flatten(1)     # noqa: E731
+    err = []
+    for c in (lib.Context(0, size), lib.Context(0, size - 256)):
+        y, sa, sw = lib.fp4_linear_fwd(c, A, W, 0.97, out_f32=True)
+        torch.cuda.synchronize()
+        assert c.read_status() == 0
+        lo, hi = sa.thresholds.double().tolist()
+        exact = (decode(sa.codes) @ decode(sw.codes_t).T) * (sa.amax / 6).double()[:, None] * (sw.amax / 6).double()
+        exact += (A.double() - A.double().clamp(lo, hi)) @ W.double()
+        err.append(float((y.double() - exact).norm() / exact.norm()))
+        c.close()
+    assert err[0] != err[1] and err[0] <= 1.02 * err[1], err
