@@ -50,14 +50,22 @@ __device__ __forceinline__ void add_kept(float (&acc)[8], const uint2* __restric
 }
 
 // Y1 is read for the last time and Y leaves with streaming stores, so that neither pushes the rest of Y1 and the slab
-// of weight rows out of L2; two or three last entries of a token travel together.  One token per warp and 40
-// registers: the chain row pointer -> entry -> weight row is hidden by the other warps (walking tokens with the next
+// of weight rows out of L2; two or three last entries of a token travel together.  One token per
+// warp and few registers: the chain row pointer -> entry -> weight row is hidden by the other warps (walking tokens with the next
 // Y1 in flight took 17 us of 4096 x 2048 x 2048 instead of 11).  8192 x 5120 x 5120 at 0.01 %: 65 -> 52.5 us, 4096 x
 // 2048 x 5504 at 0.1 %: 37 -> 28, with the walk from the end below.  Blocks of four warps: with eight, a block's
 // slots waited for its slowest warp (51 % of the warps active; 51.8 -> 49.6, 28.1 -> 26.9; blocks of two are slower;
 // comp_fwd_kept, 2048 x 512 x 2048 at 1 %: 9.4 -> 8.9).
+// Long rows, 32 entries at a time: forward 128 x 4096 x 4096 with every hundredth token beyond the thresholds 682 -> 450
+// us.  Ten blocks of 48 registers per SM instead of twelve of 40 cost light residuals 1 to 3 % of their forward; 52
+// registers without a bound gain the long rows little (618).
 constexpr int FWD_THREADS = 128;
-__global__ void __launch_bounds__(FWD_THREADS)
+__device__ __forceinline__ float4 load_y1(const float* p) {
+  float4 v;
+  asm volatile("ld.global.cs.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+__global__ void __launch_bounds__(FWD_THREADS, 10)
 comp_fwd_kernel(const float* __restrict__ y1, const int* __restrict__ rowptr, const int* __restrict__ col,
                 const float* __restrict__ val, const uint4* __restrict__ w, int M, int N, void* y, int out_f32) {
   // blocks that follow one another share the 256 output columns, i.e. the same slab of the weight
@@ -65,13 +73,22 @@ comp_fwd_kernel(const float* __restrict__ y1, const int* __restrict__ rowptr, co
   // (from the end: what the GEMM wrote last is still in L2)
   const int m = (gridDim.x - 1 - blockIdx.x) * (FWD_THREADS / 32) + (threadIdx.x >> 5);
   const int n0 = (gridDim.y - 1 - blockIdx.y) * COMP_COLS + 8 * (threadIdx.x & 31);
-  if (m >= M || n0 >= N) return;
+  if (m >= M) return;
+  const bool live = n0 < N;                           // (every lane takes part in the walk over a long row)
   // Y1 is requested first: its latency runs under the dependent chain row pointer -> entry -> weight row
-  const long long off = (long long)m * N + n0;
-  const float4 a = __ldcs(reinterpret_cast<const float4*>(y1 + off));
-  const float4 b = __ldcs(reinterpret_cast<const float4*>(y1 + off + 4));
+  const long long off = (long long)m * N + (live ? n0 : 0);
+  float4 a = load_y1(y1 + off), b = load_y1(y1 + off + 4);
   float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  sparse_row_times_dense(acc, col, val, __ldg(&rowptr[m]), __ldg(&rowptr[m + 1]), w, N >> 3, n0 >> 3);
+  const int vcol = live ? n0 >> 3 : 0, e1 = __ldg(&rowptr[m + 1]);
+  int e = __ldg(&rowptr[m]);
+  if (e + 32 <= e1) {
+    add_groups_of_32(acc, col, val, e, e1, w, N >> 3, vcol);
+    e += (e1 - e) & ~31;
+    a = load_y1(y1 + off);                            // (not kept over the walk: registers)
+    b = load_y1(y1 + off + 4);
+  }
+  sparse_row_times_dense(acc, col, val, e, e1, w, N >> 3, vcol);
+  if (!live) return;
   const float y8[8] = {a.x + acc[0], a.y + acc[1], a.z + acc[2], a.w + acc[3],
                        b.x + acc[4], b.y + acc[5], b.z + acc[6], b.w + acc[7]};
   store8(y, out_f32, off, y8);

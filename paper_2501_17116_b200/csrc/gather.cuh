@@ -33,6 +33,27 @@ __device__ __forceinline__ void add_entries(float (&acc)[8], const int* __restri
 #pragma unroll
   for (int u = 0; u < n; ++u) fma8(acc, v[u], d[u]);
 }
+// The entries of a row in whole groups of 32 (those behind them are the caller's), by all lanes of the warp together.
+// A row that holds many (a token that lies beyond the thresholds as a whole) is one chain that nothing hides: the
+// lanes fetch 32 entries at once and hand them round, which leaves one round trip to L2 per four entries, not two.
+__device__ __forceinline__ void add_groups_of_32(float (&acc)[8], const int* __restrict__ idx, const float* __restrict__ val,
+                                                 int e, int e1, const uint4* __restrict__ dense, int vec_per_row, int vcol) {
+#pragma unroll 1
+  for (; e + 32 <= e1; e += 32) {
+    const int r = __ldg(&idx[e + (threadIdx.x & 31)]);
+    const float v = __ldg(&val[e + (threadIdx.x & 31)]);
+#pragma unroll 1
+    for (int u0 = 0; u0 < 32; u0 += 4) {
+      uint4 d[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        d[u] = __ldg(&dense[(long long)__shfl_sync(0xFFFFFFFFu, r, u0 + u) * vec_per_row + vcol]);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) fma8(acc, __shfl_sync(0xFFFFFFFFu, v, u0 + u), d[u]);
+    }
+  }
+}
+
 // acc[0..7] += sum over the entries [e0, e1) of val[e] * dense[idx[e], col .. col+7]
 __device__ __forceinline__ void sparse_row_times_dense(float (&acc)[8], const int* __restrict__ idx,
                                                        const float* __restrict__ val, int e0, int e1,

@@ -127,7 +127,7 @@ struct DenseRowsArgs {
   float* out;                  // [R x N]
 };
 template <bool SECOND>
-__global__ void __launch_bounds__(256, 6)
+__global__ void __launch_bounds__(256, SECOND ? 5 : 6)
 dense_rows_kernel(const __grid_constant__ DenseRowsArgs a) {
   __shared__ __align__(16) __nv_bfloat16 tile[SECOND ? 1 : 2][ROW_SEG];
   const int* __restrict__ ptr = a.ptr;
@@ -140,9 +140,13 @@ dense_rows_kernel(const __grid_constant__ DenseRowsArgs a) {
     const int groups = a.rows >> 3, items = groups * ((a.N + 255) >> 8);
     for (int it = blockIdx.x; it < items; it += a.rows) {
       const int nb = it / groups, row = a.row0 + (it - nb * groups) * 8 + (t >> 5), n0 = 256 * nb + 8 * (t & 31);
-      if (n0 >= a.N) continue;
+      const int vcol = n0 < a.N ? n0 >> 3 : 0, e1 = __ldg(&ptr[row + 1]);      // (every lane takes part in the walk)
+      int e = __ldg(&ptr[row]);
       float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-      sparse_row_times_dense(acc, idx, val, __ldg(&ptr[row]), __ldg(&ptr[row + 1]), a.dense, a.N >> 3, n0 >> 3);
+      add_groups_of_32(acc, idx, val, e, e1, a.dense, a.N >> 3, vcol);
+      e += max(e1 - e, 0) & ~31;
+      sparse_row_times_dense(acc, idx, val, e, e1, a.dense, a.N >> 3, vcol);
+      if (n0 >= a.N) continue;
       float4* dst = reinterpret_cast<float4*>(a.out + (long long)row * a.N + n0);
       dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
       dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);

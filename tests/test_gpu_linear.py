@@ -562,3 +562,28 @@ def test_dense_product_of_a_heavy_residual_is_no_less_precise_than_its_gathers(l
         err.append(float((y.double() - exact).norm() / exact.norm()))
         c.close()
     assert err[0] != err[1] and err[0] <= 1.02 * err[1], err
+
+
+@pytest.mark.parametrize("M,K,N", [(128, 256, 384), (256, 1152, 128)])
+def test_tokens_beyond_the_thresholds_as_a_whole(lib, M, K, N):
+    """Rows of 32 entries and more, of every remainder modulo 32 in turn, beside empty ones: the entries are added as one
+    chain of fused multiply-adds in column order (thresholds 0, codes 0: Y is the compensation alone; see the test of the
+    long columns for the emulation)."""
+    rng = np.random.default_rng(N)
+    a = np.zeros((M, K), dtype=np.float32)
+    for m in range(0, M, 3):
+        n = min(m, K)
+        a[m, rng.choice(K, n, replace=False)] = rng.standard_normal(n) + 0.01
+    a_bits, w_bits = WL.to_bf16_bits(a), WL.to_bf16_bits(rng.standard_normal((K, N)).astype(np.float32))
+    a, w = O.bf16_bits_to_f64(a_bits), O.bf16_bits_to_f64(w_bits)
+    alpha = 1.0 - (max((a > 0).sum(), (a < 0).sum()) + 1) / (M * K)
+    want = np.zeros((M, N), dtype=np.float32)
+    for m in range(M):
+        for k in np.flatnonzero(a[m]):
+            want[m] = (a[m, k] * w[k] + want[m]).astype(np.float32)
+    ctx = lib.Context.for_shape(M, K, N)
+    y, sa, _ = lib.fp4_linear_fwd(ctx, _dev(a_bits), _dev(w_bits), alpha, out_f32=True)
+    torch.cuda.synchronize()
+    assert ctx.read_status() == 0 and not sa.codes.any() and int(sa.nnz) == (a != 0).sum()
+    np.testing.assert_array_equal(y.cpu().numpy(), want)
+    ctx.close()
