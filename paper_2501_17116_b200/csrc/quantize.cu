@@ -1326,6 +1326,10 @@ sparse_prefix_kernel(const int* __restrict__ row_cnt, int rows, int* __restrict_
 // us of 1920 x 5504 at 3 % per tail, 8 and 10 now.)  No shared memory: a GEMM that runs beside the fills
 // leaves none on its SM, and blocks that need some would wait for its end.
 constexpr int FILL_WARPS = 8;
+// Entries among 1024 columns from which a row's columns are taken one after another instead, all 32 words of them in
+// four rounds of loads: what ten rounds of the search take (from 256 on the two were equal at 128 x 65536).  Every
+// hundredth token beyond the thresholds as a whole, alpha 0.99: 2048 x 11008 186 -> 115 us, 128 x 65536 631 -> 261.
+constexpr int FILL_DENSE = 320;
 
 // Position of set bit number r (from 0, r < popc(m)) of m.
 __device__ __forceinline__ int nth_set_bit(uint32_t m, int r) {
@@ -1379,6 +1383,27 @@ csr_fill_kernel(const uint32_t* __restrict__ mask, const __nv_bfloat16* __restri
     next = w0 + 32 + lane < words ? mrow[w0 + 32 + lane] : 0u;
     const int c = __popc(m);
     const int incl = warp_inclusive_scan(c), total = __shfl_sync(0xFFFFFFFFu, incl, 31);
+    if (total >= FILL_DENSE) {
+      // word by word, a lane per column: the row's own order, eight coalesced loads in flight
+#pragma unroll 1
+      for (int j0 = 0; j0 < 32 && w0 + j0 < words; j0 += 8) {
+        __nv_bfloat16 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = xrow[32 * min(w0 + j0 + u, words - 1) + lane];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {                   // (words beyond the row are zero)
+          const uint32_t word = __shfl_sync(0xFFFFFFFFu, m, j0 + u);
+          const int at = base + __shfl_sync(0xFFFFFFFFu, incl - c, j0 + u) + __popc(word & ((1u << lane) - 1u));
+          if (((word >> lane) & 1u) && at < cap) {
+            const float f = __bfloat162float(v[u]);
+            csr_col[at] = 32 * (w0 + j0 + u) + lane;
+            csr_val[at] = __fsub_rn(f, f > hi ? hi : lo);
+          }
+        }
+      }
+      base += total;
+      continue;
+    }
     for (int i0 = 0; i0 < total; i0 += 32) {
       const int i = min(i0 + lane, total - 1);
       const int src = lane_of_entry(i, incl);

@@ -454,3 +454,26 @@ def test_per_token_thresholds_through_the_layer(lib):
     assert_close_f32(da32.cpu().numpy(), b.da, b.da, None, "dA")
     assert_close_f32(dw32.cpu().numpy(), b.dw, b.s_fp4 * b.dge, b.s_comp * b.dge, "dW")
     c.close()
+
+
+@pytest.mark.parametrize("M,K,share", [(128, 128, 1.0), (256, 1152, 0.9), (128, 2176, 0.3), (128, 3200, 1.0)])
+def test_rows_that_lie_beyond_the_thresholds(lib, M, K, share):
+    """Every fourth row far out in `share` of its columns, on either side of where a row's entries are listed column by
+    column: both forms of the residual, in order, values exact."""
+    gen = torch.Generator("cuda").manual_seed(K)
+    x = torch.randn((M, K), device="cuda", generator=gen)
+    x[::4] = torch.where(torch.rand((M // 4, K), device="cuda", generator=gen) < share, x[::4] * 64.0, x[::4])
+    x = x.to(torch.bfloat16)
+    ctx = lib.Context.for_shape(M, K, 128)
+    q = lib.fp4_quantize(ctx, x, 0, alpha=0.87)
+    torch.cuda.synchronize()
+    assert ctx.read_status() == 0
+    lo, hi = q.thresholds.tolist()
+    r = x.float() - x.float().clamp(lo, hi)
+    nnz = int(q.nnz)
+    for mat, ptr, idx, val in ((r, q.csr_rowptr, q.csr_col, q.csr_val), (r.T, q.csc_colptr, q.csc_row, q.csc_val)):
+        at = mat.nonzero()
+        assert nnz == at.shape[0] > 0.1 * M * K
+        assert torch.equal(ptr[1:].long(), (mat != 0).sum(1).cumsum(0)) and int(ptr[0]) == 0
+        assert torch.equal(idx[:nnz].long(), at[:, 1]) and torch.equal(val[:nnz], mat[at[:, 0], at[:, 1]])
+    ctx.close()
