@@ -140,11 +140,13 @@ comp_fwd_kept_kernel(const float* __restrict__ y1, const int* __restrict__ rowpt
 // candidate for the dense class: an outlier channel that most tokens hit (Appendix D).
 constexpr int LONG_COLUMN = 512;
 // From how many entries a column's gathers are spread over a whole cluster of blocks instead of one warp:
-// LONG_FEW entries as long as at most LONG_FEW_MAX columns reach that, else LONG_COLUMN.  A warp walks eight
-// entries per round trip to L2, so the few outlier channels of a small batch (256 entries: 32 round trips)
-// are what everything waits for; thousands of columns with a hundred-odd entries each, as in the heavy
-// residuals of the 7B and 13B shapes, keep all warps busy as they are.
-constexpr int LONG_FEW = 64, LONG_FEW_MAX = 256;
+// LONG_FEW entries as long as those columns keep a cluster per SM busy for LONG_FEW_ROUNDS items at most, else
+// LONG_COLUMN.  A warp walks eight entries per round trip to L2, so the few outlier channels of a small batch (256
+// entries: 32 round trips) are what everything waits for (256 x 4096 x 4096 with 40 of them, four rounds: backward 91
+// us by clusters, 99 by warps).  An item of a cluster takes about 4 us however short its column is: a hundred channels
+// with 400 entries each (512 x 11008 x 4096, 16 items a channel: 150 us by warps, 176 by clusters) or a few hundred
+// columns with 64 (2048 x 512 x 2048 at 4 %: 72 and 92) stay with the warps.
+constexpr int LONG_FEW = 64, LONG_FEW_ROUNDS = 5;
 
 struct ColumnClasses {
   int* list_dense;             // [DENSE_TC_MAX] dense columns, ascending
@@ -185,7 +187,7 @@ __device__ __forceinline__ int block_exclusive_scan_1024(int c, int* warp_tot) {
 // block waits for another: one block walking all columns in stretches took 4.5 us of 2048 and 17.5 of 11008.
 template <bool ALL>
 __global__ void __launch_bounds__(1024, 1)
-classify_columns_kernel(const int* __restrict__ colptr, int K, int dense_from, const ColumnClasses out) {
+classify_columns_kernel(const int* __restrict__ colptr, int K, int dense_from, int few_max, const ColumnClasses out) {
   __shared__ int warp_tot[32];
   const int t = threadIdx.x, c0 = blockIdx.x * 1024;
   int cand_b = 0, cand = 0, few = 0, few_b = 0, large = 0, large_b = 0, any = 0, any_b = 0;   // _b: before c0
@@ -218,7 +220,7 @@ classify_columns_kernel(const int* __restrict__ colptr, int K, int dense_from, c
     return;
   }
   few = block_sum_1024(few, warp_tot);
-  const bool use_few = few <= LONG_FEW_MAX;
+  const bool use_few = few <= few_max;
   const int long_from = use_few ? LONG_FEW : LONG_COLUMN;
   // (candidates beyond DENSE_TC_MAX hold LONG_COLUMN entries or more: they are long)
   large = (use_few ? few : block_sum_1024(large, warp_tot)) + cand - n_dense;
@@ -576,7 +578,7 @@ int launch_fwd_tail(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, con
   const int hot_from = int(M / 4 > LONG_COLUMN ? M / 4 : LONG_COLUMN);
   KernelScope scope(ctx, stream, KC_COMP_FWD, 3);
   const ColumnClasses classes = {list_hot, nullptr, nullptr, count, slot_of_col};
-  classify_columns_kernel<false><<<unsigned((K + 1023) / 1024), 1024, 0, stream>>>(a->csc_colptr, int(K), hot_from, classes);
+  classify_columns_kernel<false><<<unsigned((K + 1023) / 1024), 1024, 0, stream>>>(a->csc_colptr, int(K), hot_from, 0, classes);
   FP4_CUDA_TRY(cudaMemsetAsync(tb, 0, size_t(N) * TAIL_WIDTH * 2, stream));
   tail_a_kernel<<<unsigned((M + 7) / 8), COMP_THREADS, 0, stream>>>(a->csr_rowptr, a->csr_col, a->csr_val, slot_of_col,
                                                                    count, a->amax, 6.0f, ta, int(M), kept, kept_end);
@@ -609,7 +611,9 @@ int launch_comp_wgrad(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, c
   const bool dense = a->csr_rowptr != nullptr && a->sparse_cap * 100 >= M * K && M >= LONG_COLUMN;
   const int dense_from = dense ? int(M / 4 > LONG_COLUMN ? M / 4 : LONG_COLUMN) : INT_MAX;
   KernelScope scope(ctx, stream, KC_COMP_WGRAD, 3 + (dense ? 3 : 0));
-  classify_columns_kernel<true><<<unsigned((K + 1023) / 1024), 1024, 0, stream>>>(a->csc_colptr, int(K), dense_from, classes);
+  const unsigned n_blocks = unsigned((N + COMP_COLS - 1) / COMP_COLS);
+  const int few_max = int(LONG_FEW_ROUNDS * unsigned(ctx->num_sms) / n_blocks);
+  classify_columns_kernel<true><<<unsigned((K + 1023) / 1024), 1024, 0, stream>>>(a->csc_colptr, int(K), dense_from, few_max, classes);
   const uint4* dy = static_cast<const uint4*>(dy_bf16);
   // The long columns (a few blocks, latency) run beside the others.
   cudaStream_t sl = stream;
@@ -625,7 +629,6 @@ int launch_comp_wgrad(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, c
     dense_reduce_kernel<<<unsigned(2 * ctx->num_sms), 256, 0, stream>>>(comp, partial, classes.list_dense, classes.counts,
                                                                        int(N), splits, (long long)DENSE_TC_MAX * N);
   }
-  const unsigned n_blocks = unsigned((N + COMP_COLS - 1) / COMP_COLS);
   // long columns: up to four blocks per SM
   const unsigned clusters = unsigned(4 * ctx->num_sms / LONG_CLUSTER);
   comp_wgrad_long_kernel<<<clusters * LONG_CLUSTER, 32 * LONG_WARPS, 0, sl>>>(comp, a->csc_colptr, a->csc_row, a->csc_val, dy,
