@@ -109,7 +109,9 @@ typedef struct fp4_qtensor {
                               operand of the W4A8 / W8A4 settings of Section 4.3; or
                               FP4_FORMAT_E5M2: OCP E5M2 bytes in the same layouts, MAX = 57344,
                               saturation to the largest finite value (never an infinity)    */
-  int32_t  reserved;       /* 0                                                               */
+  int32_t  reserved;       /* set to 0 by the caller; a call that clamps the operand (or a forward
+                              that quantises it) notes there what alpha allows, for the calls that
+                              use it later                                                    */
 } fp4_qtensor;
 
 /* Create a context on `device` with a workspace of `workspace_bytes` (cudaMalloc'ed here,
@@ -204,9 +206,9 @@ int fp4_gemm(fp4_ctx* ctx, void* stream, const uint8_t* a_codes, const uint8_t* 
  *   A residual value
  *   beyond 43 000 times its token's clamped absmax does not fit the FP16 operand: the call
  *   then adds every entry per entry.
- *   A residual that may fill more than 4 % of the activation (sparse_cap, M >= 512) is multiplied
- *   as a dense matrix where that takes less time for the entries that are there: exact three-term BF16 split, chunks of 64 input
- *   channels added in fp32 in order.  Same bound, without the second term.
+ *   A residual that may fill more than 4 % of the activation (by alpha; M >= 512) is
+ *   multiplied as a dense matrix where that takes less time for the entries that are there: exact
+ *   three-term BF16 split, chunks of 64 input channels added in fp32 in order.  Same bound, without the second term.
  */
 #define FP4_REUSE_W 1
 #define FP4_REUSE_A 2

@@ -47,14 +47,17 @@ size_t least_workspace_bytes(int64_t M, int64_t K, int64_t N) {
   return q + linear_scratch_bytes(M, K, N) + 4096;
 }
 
+// Residual entries that clamping at `alpha` can leave, in the context's form of the clamp (n_tail: of one tail).
+void note_residual(fp4_qtensor* q, int64_t n_tail) { q->reserved = int32_t(2 * n_tail + 1); }
+
 // A residual that may fill more than 1 / RESIDUAL_FULL_SHARE of the activation takes no dense tail ...
 bool heavy_residual(const fp4_qtensor* a, int64_t M, int64_t K) {
-  return a->csr_rowptr && a->csc_colptr && a->sparse_cap * RESIDUAL_FULL_SHARE > M * K && M >= 512;
+  return a->csr_rowptr && a->csc_colptr && residual_entries(a) * RESIDUAL_FULL_SHARE > M * K && M >= 512;
 }
 // ... and is multiplied as a dense matrix [R x C] (times [C x N]) unless the gathers take less time: small products
 // do not fill the chip.
 bool full_product_pays(const fp4_ctx* ctx, const fp4_qtensor* a, int64_t R, int64_t C, int64_t N) {
-  return residual_full_from(ctx, R, C, N) <= a->sparse_cap;
+  return residual_full_from(ctx, R, C, N) <= residual_entries(a);
 }
 
 // A workspace of fp4_workspace_bytes holds the dense operand, a smaller one is not searched for spare room: which
@@ -219,10 +222,11 @@ int fp4_quantize(fp4_ctx* ctx, void* stream, const void* x_bf16, int64_t rows, i
   if (!known_format(out->format)) return FP4_ERR_ARG;
   if (!aligned16(x_bf16) || !aligned16(out->codes) || !aligned16(out->codes_t) || !aligned16(out->amax))
     return FP4_ERR_ALIGN;
+  int64_t n_tail = 0;
   if (alpha < 1.0) {
     if (scale_axis != 0 || prescale || out->format != FP4_FORMAT_E2M1) return FP4_ERR_ARG;
     const int64_t n = rows * cols;
-    int64_t n_tail = llround((1.0 - alpha) * double(n));
+    n_tail = llround((1.0 - alpha) * double(n));
     if (2 * n_tail >= n) return FP4_ERR_ALPHA;
     if (ctx->quantile_mode == FP4_QUANTILE_TOKEN) {       // per token: every row has its own two tails
       const int64_t per_row = llround((1.0 - alpha) * double(cols));
@@ -233,6 +237,7 @@ int fp4_quantize(fp4_ctx* ctx, void* stream, const void* x_bf16, int64_t rows, i
     if (rc != FP4_OK) return rc;
   }
   if (quantize_scratch_bytes(rows, cols) > ctx->workspace_bytes) return FP4_ERR_WORKSPACE;
+  if (alpha < 1.0) note_residual(out, n_tail);
   out->rows = rows;
   out->cols = cols;
   CallKey key;
@@ -285,6 +290,7 @@ int fp4_linear_fwd(fp4_ctx* ctx, void* stream, const void* A_bf16, const void* W
   if (!savedW->codes || !savedW->codes_t || !savedW->amax) return FP4_ERR_NULL;
   if (!aligned16(A_bf16) || !aligned16(W_bf16) || !aligned16(Y)) return FP4_ERR_ALIGN;
   const bool occ = alpha < 1.0;
+  int64_t n_tail = 0;
   {
     const bool a8 = is_fp8(savedA->format), w8 = is_fp8(savedW->format);
     if (!known_format(savedA->format) || !known_format(savedW->format)) return FP4_ERR_ARG;
@@ -292,7 +298,7 @@ int fp4_linear_fwd(fp4_ctx* ctx, void* stream, const void* A_bf16, const void* W
     if (a8 && occ) return FP4_ERR_ARG;                                    // clamping belongs to 4-bit activations
   }
   if (occ) {
-    int64_t n_tail = llround((1.0 - alpha) * double(M * K));
+    n_tail = llround((1.0 - alpha) * double(M * K));
     if (2 * n_tail >= M * K) return FP4_ERR_ALPHA;
     if (ctx->quantile_mode == FP4_QUANTILE_TOKEN) {       // per token: every row has its own two tails
       const int64_t per_row = llround((1.0 - alpha) * double(K));
@@ -304,7 +310,7 @@ int fp4_linear_fwd(fp4_ctx* ctx, void* stream, const void* A_bf16, const void* W
   }
   if (least_workspace_bytes(M, K, N) > ctx->workspace_bytes) return FP4_ERR_WORKSPACE;
   // (linear_fwd_impl sets these too, but does not run when the call is replayed)
-  if (!(reuse & FP4_REUSE_A)) { savedA->rows = M; savedA->cols = K; }
+  if (!(reuse & FP4_REUSE_A)) { savedA->rows = M; savedA->cols = K; note_residual(savedA, n_tail); }
   if (!(reuse & FP4_REUSE_W)) { savedW->rows = K; savedW->cols = N; }
   CallKey key;
   std::memset(&key, 0, sizeof(key));
@@ -351,7 +357,7 @@ int linear_fwd_impl(fp4_ctx* ctx, cudaStream_t st, Arena arena, const void* A_bf
                            ? arena.take<char>(full_bytes) : nullptr;
   const bool full_on = scratch_full != nullptr;
   const bool tail_on = occ && !full_on && savedA->csr_rowptr && savedA->csc_colptr && !heavy_residual(savedA, M, K) &&
-                       savedA->sparse_cap * 100 >= M * K && M >= 512;   // a hot column holds at least 512 entries
+                       residual_entries(savedA) * 100 >= M * K && M >= 512;   // a hot column holds at least 512 entries
   char* scratch_tail = tail_on ? arena.take<char>(fwd_tail_scratch_bytes(M, K, N)) : nullptr;
   if (!arena.ok) return FP4_ERR_WORKSPACE;
   int rc;
@@ -726,6 +732,9 @@ int fp4_linear_step_host(fp4_ctx* ctx, void* stream, const void* A_host, const v
   int32_t* status = arena.take<int32_t>(1);
   fp4_qtensor qa, qw;
   carve_qtensor(arena, &qa, M, K, 0, step_capacity(M, K, alpha));
+  if (alpha < 1.0)
+    note_residual(&qa, ctx->quantile_mode == FP4_QUANTILE_TOKEN ? M * llround((1.0 - alpha) * double(K))
+                                                                : llround((1.0 - alpha) * double(M * K)));
   carve_qtensor(arena, &qw, K, N, 1, 0);
   if (!arena.ok || !in_arena.ok || !out_arena.ok) return FP4_ERR_WORKSPACE;
   Arena rest(arena.base + arena.off, arena.size - arena.off);

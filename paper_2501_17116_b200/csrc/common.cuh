@@ -142,6 +142,12 @@ struct GemmEpilogue {
   float dge_k, dge_clip;
 };
 
+// Residual entries that a clamped operand can hold.  The call that clamps it knows them from alpha and notes them
+// (plus one) in `reserved` for the later calls that do not: sparse_cap may be sized for another alpha.  0: not noted.
+inline int64_t residual_entries(const fp4_qtensor* q) {
+  return q->reserved > 0 && q->reserved - 1 < q->sparse_cap ? q->reserved - 1 : q->sparse_cap;
+}
+
 // Largest value of an operand format: what an absmax scale maps the vector's maximum to.
 inline float fp8_max(int format) {
   return format == FP4_FORMAT_E5M2 ? 57344.0f : (format == FP4_FORMAT_E4M3 ? 448.0f : 6.0f);

@@ -255,12 +255,12 @@ __device__ __forceinline__ void split_half(float x, __half& hi, __half& hi_small
 // A operand of the dense tail: row m holds, for hot column s = 64 j + c, the value
 // x = residual[m, k_s] / (d_A[m] * TAIL_SCALE) as x_hi at column 192 j + c, x_hi / TAIL_BALANCE at
 // 192 j + 64 + c and TAIL_BALANCE x_lo at 192 j + 128 + c; zero elsewhere.  One warp per token walks the token's CSR row.  A value
-// that FP16 cannot hold (or a token whose de-scale is zero) switches the tail off for this call:
+// that FP16 cannot hold (or a token whose de-scale is zero, or a list that is too short) switches the tail off for this call:
 // *count becomes 0 and the per-entry kernel keeps every entry.
 __global__ void __launch_bounds__(COMP_THREADS)
 tail_a_kernel(const int* __restrict__ rowptr, const int* __restrict__ col, const float* __restrict__ val,
               const int* __restrict__ slot_of_col, int* __restrict__ count, const float* __restrict__ amax_row,
-              float row_div, __half* __restrict__ ta, int M, uint2* __restrict__ kept, int* __restrict__ kept_end) {
+              float row_div, __half* __restrict__ ta, int M, uint2* __restrict__ kept, int kept_cap, int* __restrict__ kept_end) {
   const int hot = *count;
   if (hot == 0) return;
   const int lane = threadIdx.x & 31;
@@ -287,7 +287,9 @@ tail_a_kernel(const int* __restrict__ rowptr, const int* __restrict__ col, const
     const bool keep = e < e1 && !is_hot;
     {                                                    // entries the tail does not cover, in column order
       const unsigned km = __ballot_sync(0xFFFFFFFFu, keep);
-      if (keep) kept[n_kept + __popc(km & ((1u << lane) - 1u))] = make_uint2(uint32_t(k), __float_as_uint(v));
+      const int at = n_kept + __popc(km & ((1u << lane) - 1u));
+      if (keep && at < kept_cap) kept[at] = make_uint2(uint32_t(k), __float_as_uint(v));
+      bad |= keep && at >= kept_cap;                     // (more entries than were noted beside the operand)
       n_kept += __popc(km);
     }
     if (!is_hot) continue;
@@ -581,7 +583,8 @@ int launch_fwd_tail(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, con
   classify_columns_kernel<false><<<unsigned((K + 1023) / 1024), 1024, 0, stream>>>(a->csc_colptr, int(K), hot_from, 0, classes);
   FP4_CUDA_TRY(cudaMemsetAsync(tb, 0, size_t(N) * TAIL_WIDTH * 2, stream));
   tail_a_kernel<<<unsigned((M + 7) / 8), COMP_THREADS, 0, stream>>>(a->csr_rowptr, a->csr_col, a->csr_val, slot_of_col,
-                                                                   count, a->amax, 6.0f, ta, int(M), kept, kept_end);
+                                                                   count, a->amax, 6.0f, ta, int(M), kept,
+                                                                   int(kept_list_capacity(M, K)), kept_end);
   tail_b_kernel<<<dim3(unsigned((N + 255) / 256), 16), 256, 0, stream>>>(static_cast<const __nv_bfloat16*>(w_bf16),
                                                                         list_hot, count, w_amax, w_div, tb, int(N));
   FP4_CUDA_TRY(cudaGetLastError());
@@ -608,7 +611,7 @@ int launch_comp_wgrad(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, c
   // whose product runs on the tensor cores.  It costs three launches, which pay
   // when the residual is heavy: when it may hold at least 1 % of the activation (alpha <= 0.995).
   // (No column can reach LONG_COLUMN entries with fewer tokens than that.)
-  const bool dense = a->csr_rowptr != nullptr && a->sparse_cap * 100 >= M * K && M >= LONG_COLUMN;
+  const bool dense = a->csr_rowptr != nullptr && residual_entries(a) * 100 >= M * K && M >= LONG_COLUMN;
   const int dense_from = dense ? int(M / 4 > LONG_COLUMN ? M / 4 : LONG_COLUMN) : INT_MAX;
   KernelScope scope(ctx, stream, KC_COMP_WGRAD, 3 + (dense ? 3 : 0));
   const unsigned n_blocks = unsigned((N + COMP_COLS - 1) / COMP_COLS);

@@ -587,3 +587,26 @@ def test_tokens_beyond_the_thresholds_as_a_whole(lib, M, K, N):
     assert ctx.read_status() == 0 and not sa.codes.any() and int(sa.nnz) == (a != 0).sum()
     np.testing.assert_array_equal(y.cpu().numpy(), want)
     ctx.close()
+
+
+@pytest.mark.parametrize("alpha", [0.999, 0.99, 0.97, 1.0])
+def test_the_capacity_of_the_residual_decides_nothing(lib, alpha):
+    """A saved operand with room for a tenth of the activation beyond either threshold, used at a lighter clamp: the
+    same kernels as with the capacity that alpha asks for, i.e. the same bits, in both directions and with the
+    activation reused."""
+    M, K, N = 1024, 1280, 2176
+    a_bits, w_bits, dy_bits = WL.small_case(M, K, N, seed=8, alpha_outliers=12)
+    A, W, dY = _dev(a_bits), _dev(w_bits), _dev(dy_bits)
+    ctx = lib.Context.for_shape(M, K, N)
+    out = []
+    for cap in (lib.tail_capacity(M, K, alpha) or lib.tail_capacity(M, K, 0.999), lib.tail_capacity(M, K, 0.9)):
+        sa = lib.QTensor(M, K, 0, "cuda", cap)
+        y, _, sw = lib.fp4_linear_fwd(ctx, A, W, alpha, saved_a=sa, out_f32=True)
+        before = ctx.launch_count()
+        _, dw = lib.fp4_linear_bwd(ctx, dY, W, sa, sw, out_f32=True, want_da=False)
+        y2, _, _ = lib.fp4_linear_fwd(ctx, A, W, alpha, saved_a=sa, saved_w=sw, reuse_a=True, reuse_w=True, out_f32=True)
+        out.append((y, dw, y2, ctx.launch_count() - before))
+    torch.cuda.synchronize()
+    assert ctx.read_status() == 0
+    assert all(torch.equal(a, b) for a, b in zip(out[0][:3], out[1][:3])) and out[0][3] == out[1][3]
+    ctx.close()
