@@ -214,6 +214,7 @@ int fp4_destroy(fp4_ctx* ctx) {
 int fp4_quantize(fp4_ctx* ctx, void* stream, const void* x_bf16, int64_t rows, int64_t cols, int scale_axis,
                  double alpha, const float* prescale, fp4_qtensor* out, int32_t* status) {
   if (!ctx || !x_bf16 || !out || !status) return FP4_ERR_NULL;
+  std::lock_guard<std::mutex> turn(ctx->mutex);
   if (!mult128(rows) || !mult128(cols) || rows * cols >= (int64_t(1) << 31)) return FP4_ERR_SHAPE;
   if (scale_axis != 0 && scale_axis != 1) return FP4_ERR_ARG;
   if (!(alpha > 0.5 && alpha <= 1.0)) return FP4_ERR_ALPHA;
@@ -262,6 +263,7 @@ int fp4_gemm(fp4_ctx* ctx, void* stream, const uint8_t* a_codes, const uint8_t* 
              int64_t C, const float* row_amax, const float* col_amax, void* out, int out_f32, int gemm_kind,
              int32_t* status) {
   if (!ctx || !a_codes || !b_codes || !out || !status) return FP4_ERR_NULL;
+  std::lock_guard<std::mutex> turn(ctx->mutex);
   if (!mult128(I) || !mult128(J) || !mult128(C)) return FP4_ERR_SHAPE;
   if (!aligned16(out)) return FP4_ERR_ALIGN;
   const int e5m2_flags = gemm_kind & (FP4_GEMM_A_E5M2 | FP4_GEMM_B_E5M2);
@@ -282,6 +284,7 @@ int fp4_linear_fwd(fp4_ctx* ctx, void* stream, const void* A_bf16, const void* W
                    int64_t N, double alpha, int reuse, int gemm_kind, void* Y, int out_f32, fp4_qtensor* savedA,
                    fp4_qtensor* savedW, int32_t* status) {
   if (!ctx || !A_bf16 || !W_bf16 || !Y || !savedA || !savedW || !status) return FP4_ERR_NULL;
+  std::lock_guard<std::mutex> turn(ctx->mutex);
   if (!mult128(M) || !mult128(K) || !mult128(N)) return FP4_ERR_SHAPE;
   if (M * K >= (int64_t(1) << 31) || K * N >= (int64_t(1) << 31) || M * N >= (int64_t(1) << 31)) return FP4_ERR_SHAPE;
   if (!(alpha > 0.5 && alpha <= 1.0)) return FP4_ERR_ALPHA;
@@ -474,6 +477,7 @@ int fp4_linear_bwd(fp4_ctx* ctx, void* stream, const void* dY_bf16, const void* 
                    float dge_clip, int gemm_kind, void* dA, void* dW, int out_f32, int32_t* status) {
   if (!ctx || !dY_bf16 || !W_bf16 || !savedA || !savedW || !status) return FP4_ERR_NULL;
   if (!dA && !dW) return FP4_ERR_NULL;
+  std::lock_guard<std::mutex> turn(ctx->mutex);
   if (!mult128(M) || !mult128(K) || !mult128(N)) return FP4_ERR_SHAPE;
   if (M * K >= (int64_t(1) << 31) || K * N >= (int64_t(1) << 31) || M * N >= (int64_t(1) << 31)) return FP4_ERR_SHAPE;
   {
@@ -696,6 +700,7 @@ int fp4_linear_step_host(fp4_ctx* ctx, void* stream, const void* A_host, const v
                          int64_t M, int64_t K, int64_t N, double alpha, int dge_on, float dge_k, float dge_clip,
                          int gemm_kind, void* Y_host, void* dA_host, void* dW_host, int32_t* status_host) {
   if (!ctx || !A_host || !W_host || !dY_host || !Y_host || !dA_host || !dW_host) return FP4_ERR_NULL;
+  std::unique_lock<std::mutex> turn(ctx->mutex);
   if (!mult128(M) || !mult128(K) || !mult128(N)) return FP4_ERR_SHAPE;
   if (M * K >= (int64_t(1) << 31) || K * N >= (int64_t(1) << 31) || M * N >= (int64_t(1) << 31)) return FP4_ERR_SHAPE;
   if (!(alpha > 0.5 && alpha <= 1.0)) return FP4_ERR_ALPHA;
@@ -787,12 +792,14 @@ int fp4_linear_step_host(fp4_ctx* ctx, void* stream, const void* A_host, const v
       FP4_CUDA_TRY(cudaEventRecord(ctx->host_step_computed[i], st));
     }
   }
+  turn.unlock();                                     // others may enqueue while this one waits
   if (status_host) FP4_CUDA_TRY(cudaStreamSynchronize(st));
   return FP4_OK;
 }
 
 int fp4_set_overlap(fp4_ctx* ctx, int on) {
   if (!ctx) return FP4_ERR_NULL;
+  std::lock_guard<std::mutex> turn(ctx->mutex);
   ctx->overlap = on ? 1 : 0;
   return FP4_OK;
 }
@@ -800,12 +807,14 @@ int fp4_set_overlap(fp4_ctx* ctx, int on) {
 int fp4_set_quantile_mode(fp4_ctx* ctx, int mode) {
   if (!ctx) return FP4_ERR_NULL;
   if (mode != FP4_QUANTILE_SIGNED && mode != FP4_QUANTILE_ABS && mode != FP4_QUANTILE_TOKEN) return FP4_ERR_ARG;
+  std::lock_guard<std::mutex> turn(ctx->mutex);
   ctx->quantile_mode = mode;
   return FP4_OK;
 }
 
 int fp4_debug_set(fp4_ctx* ctx, int key, int64_t value) {
   if (!ctx) return FP4_ERR_NULL;
+  std::lock_guard<std::mutex> turn(ctx->mutex);
   if (key == FP4_DEBUG_WAIT_LIMIT_US) {
     if (value < 0 || value > 10000000) return FP4_ERR_ARG;
     ctx->debug_wait_limit_ns = uint64_t(value) * 1000u;
@@ -829,12 +838,14 @@ int64_t fp4_sparse_capacity(int64_t rows, int64_t cols, double alpha, int quanti
 
 int fp4_profile_enable(fp4_ctx* ctx, int on) {
   if (!ctx) return FP4_ERR_NULL;
+  std::lock_guard<std::mutex> turn(ctx->mutex);
   ctx->profile = on ? 1 : 0;
   return FP4_OK;
 }
 
 int fp4_profile_reset(fp4_ctx* ctx) {
   if (!ctx) return FP4_ERR_NULL;
+  std::lock_guard<std::mutex> turn(ctx->mutex);
   for (ProfRecord& r : *ctx->records) {
     cudaEventDestroy(r.start);
     cudaEventDestroy(r.stop);
@@ -847,6 +858,7 @@ int fp4_profile_reset(fp4_ctx* ctx) {
 int fp4_profile_read(fp4_ctx* ctx, int kernel_class, double* total_ms, int64_t* launches) {
   if (!ctx || !total_ms || !launches) return FP4_ERR_NULL;
   if (kernel_class < 0 || kernel_class >= FP4_KC_COUNT) return FP4_ERR_ARG;
+  std::lock_guard<std::mutex> turn(ctx->mutex);
   double ms = 0.0;
   int64_t n = 0;
   for (ProfRecord& r : *ctx->records) {
@@ -862,6 +874,10 @@ int fp4_profile_read(fp4_ctx* ctx, int kernel_class, double* total_ms, int64_t* 
   return FP4_OK;
 }
 
-int64_t fp4_launch_count(fp4_ctx* ctx) { return ctx ? ctx->launch_count : -1; }
+int64_t fp4_launch_count(fp4_ctx* ctx) {
+  if (!ctx) return -1;
+  std::lock_guard<std::mutex> turn(ctx->mutex);
+  return ctx->launch_count;
+}
 
 }  // extern "C"

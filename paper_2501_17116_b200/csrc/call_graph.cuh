@@ -10,11 +10,10 @@
 // What is compared is every argument that reaches a kernel or decides which kernels run (CallKey).
 // Calls made while the caller's stream is being captured, with profiling on or with a debug setting are
 // enqueued as they are.  At most GRAPH_MAX calls are remembered per context, the least recently used one
-// leaves first; all are released with the context.  One host thread at a time enqueues a call of a context.
+// leaves first; all are released with the context.  The caller holds the context's mutex.
 #pragma once
 
 #include <cstring>
-#include <mutex>
 #include <unordered_map>
 #include <vector>
 
@@ -59,7 +58,6 @@ class CallGraphs {
   // Runs `enqueue(stream)` (an FP4_* code) or its graph on `st`.
   template <class F>
   int run(fp4_ctx* ctx, cudaStream_t st, const CallKey& key, F&& enqueue) {
-    std::lock_guard<std::mutex> lock(mutex_);
     if (ctx->profile || ctx->debug_wait_limit_ns || ctx->debug_skip_fill >= 0) return enqueue(st);
     cudaStreamCaptureStatus capturing;
     if (cudaStreamIsCapturing(st, &capturing) != cudaSuccess) {
@@ -153,7 +151,6 @@ class CallGraphs {
     entries_.erase(oldest);
   }
 
-  std::mutex mutex_;
   cudaStream_t stream_ = nullptr;                    // calls are captured from here
   cudaEvent_t retired_ = nullptr, in_ = nullptr, out_ = nullptr;
   std::unordered_map<uint64_t, Entry> entries_;

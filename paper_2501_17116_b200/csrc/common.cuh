@@ -6,6 +6,7 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <mutex>
 #include <vector>
 
 #include "fp4_linear.h"
@@ -36,6 +37,7 @@ constexpr int HOST_STEP_SETS = 2;
 class CallGraphs;                     // call_graph.cuh
 
 struct fp4_ctx {
+  std::mutex mutex;            // held while a call reads the settings below and enqueues: host threads take turns
   int      device;
   int      num_sms;
   char*    workspace;
