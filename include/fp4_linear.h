@@ -12,11 +12,12 @@
  * ---------------------------------------
  *  - Every tensor pointer is a DEVICE pointer unless the parameter is documented as host.
  *    Tensors are dense, row-major and 16-byte aligned.  The caller owns every tensor; the
- *    context owns only its workspace.  After fp4_create() no device buffer is allocated; the
+ *    context owns only its workspace.  After fp4_create() the library allocates no buffer; the
  *    third fp4_quantize / fp4_linear_fwd / fp4_linear_bwd with the same arguments on a context
- *    instantiates its launches as a CUDA graph that later calls replay (at most 512 are kept,
- *    released by fp4_destroy; not while the caller's stream is being captured), and profiling mode,
- *    fp4_profile_enable, creates a pair of CUDA events per kernel class and call.
+ *    instantiates its launches as a CUDA graph that later calls replay, for which the driver takes
+ *    about 0.5 MB of device memory (at most 1024 are kept per context, released by fp4_destroy;
+ *    none while the caller's stream is being captured), and profiling mode, fp4_profile_enable,
+ *    creates a pair of CUDA events per kernel class and call.
  *  - Notation: A[M x K] activations, W[K x N] weights (input channels x output channels),
  *    Y[M x N] = A W.  M, K and N must be multiples of 128.
  *  - E2M1 codes are sign-magnitude nibbles (bit 3 sign; 0..7 -> 0, .5, 1, 1.5, 2, 3, 4, 6),
