@@ -68,16 +68,19 @@ __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w 
 // 1. + 2. row extremes, histogram of the tails, order statistics -- one kernel
 // ------------------------------------------------------------------------------------------
 // The two thresholds are order statistics far out in the tails, so only the tails are counted value by
-// value.  Every block draws the same SEL_SAMPLES elements (stratified over the tensor, jittered by a hash
-// of the stratum) and takes from them a bracket Q < P that leaves slightly more than n_tail elements on
-// either side: the k-th smallest / largest sample, k six and a half standard deviations (plus eight)
-// above the expected n_tail * SEL_SAMPLES / n.  Elements strictly between Q and P are the bulk: a vector
-// of eight costs the packed maxima and minima that the row extremes need anyway and two packed
-// comparisons.  The others (2 to 6 % of the elements) are counted by pattern.  The number of bulk
+// value.  Every block draws the same SEL_SAMPLES elements (SEL_GROUPS groups of neighbours, stratified over
+// the tensor, jittered by a hash of the stratum) and takes from them a bracket Q < P that leaves more than
+// n_tail elements on either side: the k-th smallest / largest sample.  Elements strictly between Q and P are
+// the bulk: a vector of eight costs the packed maxima and minima that the row extremes need anyway and two
+// packed comparisons.  The others are counted by pattern.  The number of bulk
 // elements B is n minus what was counted, so the rank r of the whole tensor is rank r of the counters
 // below the bulk and rank r - B above it.  The result is exact whatever the sample was: a rank that does
-// not fall into its tail (a sample that misleads, about one in 10^9) makes the last block count the whole
-// tensor by itself.
+// not fall into its tail makes the last block count the whole tensor by itself, which takes a hundred times
+// as long.  k is chosen for that to happen to one tensor in 10^8 at most, also where the tail consists of
+// whole tokens, so that neighbours lie in it together: the groups, not the elements, are the independent
+// draws then.  (A margin for 2048 independent ones is half as wide: 8192 x 4096, clamped and encoded, 76.4
+// us instead of 78 at 0.1 % per tail, 105 instead of 109 at 3 %.  But it misses one layout of outlier
+// tokens in 3000, and on every call where they stay in place, because the positions depend on the size alone.)
 //
 // What bounds it: a fixed chain of about 8 us (sample -> bracket, and flush -> ticket -> selection), then
 // HBM for light clamps and the counting loop for heavy ones.  A histogram of every element needed 180 KB
@@ -105,7 +108,8 @@ __device__ __forceinline__ float bf16_hi(uint32_t w) { return __uint_as_float(w 
 constexpr int SEL_THREADS = 512;
 constexpr int SEL_WARPS = SEL_THREADS / 32;
 constexpr int SEL_BLOCKS_PER_SM = 2;
-constexpr int SEL_SAMPLES = 4 * SEL_THREADS;        // one 8-byte load per thread
+constexpr int SEL_GROUP = 4, SEL_GROUPS = SEL_THREADS;        // one 8-byte load per thread
+constexpr int SEL_SAMPLES = SEL_GROUP * SEL_GROUPS;
 constexpr int SEL_EXPS = 24;
 constexpr int SEL_WINDOW = SEL_EXPS * 128;         // 3072 magnitudes in the window, per sign
 constexpr int SEL_ALL = 8192;                       // elements per SM below which everything is counted
@@ -538,10 +542,14 @@ tail_select_kernel(const __grid_constant__ SelectArgs a) {
   }
 }
 
-// Sample rank of the bracket (see above): six and a half standard deviations of the sample count, plus eight.
+// Sample rank of the bracket (see above): four times the number of groups that a tail of whole groups is hit by with a
+// probability of 1e-8 at most, by Chernoff's bound for a binomial (Poisson) variable of mean m:
+// P(X >= g) <= exp(-(g ln(g / m) - g + m)).
 int select_sample_rank(long long n, long long n_tail) {
-  const double mean = double(n_tail) / double(n) * SEL_SAMPLES;
-  return int(mean + 6.5 * std::sqrt(mean) + 8.0);
+  const double m = double(n_tail) / double(n) * SEL_GROUPS;
+  int g = int(m) + 1;
+  while (m > 0.0 && g * std::log(g / m) - g + m < 18.42) ++g;
+  return (g - 1) * SEL_GROUP;
 }
 
 // ------------------------------------------------------------------------------------------

@@ -477,3 +477,51 @@ def test_rows_that_lie_beyond_the_thresholds(lib, M, K, share):
         assert torch.equal(ptr[1:].long(), (mat != 0).sum(1).cumsum(0)) and int(ptr[0]) == 0
         assert torch.equal(idx[:nnz].long(), at[:, 1]) and torch.equal(val[:nnz], mat[at[:, 0], at[:, 1]])
     ctx.close()
+
+
+def _sampled_rows(M, K):
+    """Rows from which the selection draws its groups of four neighbours: one group per 512th of the tensor, at a place
+    inside it that a hash of its number gives."""
+    q, rows = M * K // 4, []
+    for i in range(512):
+        b, e = q * i // 512, q * (i + 1) // 512
+        h = (i * 2654435761 + 0x9E3779B9) & 0xFFFFFFFF
+        h ^= h >> 15
+        h = h * 0x2C1B3C6D & 0xFFFFFFFF
+        h ^= h >> 13
+        rows.append(4 * (b + h % (e - b)) // K)
+    return rows
+
+
+@pytest.mark.parametrize("alpha,hit", [(0.999, 6), (0.99, 18), (0.97, 36)])
+def test_selection_where_the_tail_is_whole_tokens(lib, alpha, hit):
+    """The upper tail is made of whole rows, `hit` of which hold a group of the selection's sample: far above the mean
+    (0.5, 5 and 15) and what one layout in 10^5 to 10^6 has.  The bracket must still hold both thresholds: where it does
+    not, one block counts the whole tensor, which shows as a hundred times the time (and would on every call of this
+    size, since the positions are fixed).  Beside it the same rows in a layout that none of the sample hits."""
+    M, K = 4096, 2048
+    sampled = sorted(set(_sampled_rows(M, K)))
+    others = sorted(set(range(M)) - set(sampled))
+    gen = torch.Generator("cuda").manual_seed(2)
+    x = torch.randn((M, K), device="cuda", generator=gen)
+    n_rows = int(round((1 - alpha) * M)) + 2
+    ctx = lib.Context.for_shape(M, K, 128)
+    ctx.profile_enable()
+    took = []
+    for hits in (0, min(hit, n_rows)):
+        rows = torch.tensor(sampled[:hits] + others[:n_rows - hits], device="cuda")
+        y = x.clone()
+        y[rows] = y[rows].abs() * 64.0 + 64.0
+        y = y.to(torch.bfloat16)
+        q = lib.fp4_quantize(ctx, y, 0, alpha=alpha)
+        ctx.profile_reset()
+        for _ in range(3):
+            lib.fp4_quantize(ctx, y, 0, alpha=alpha, out=q)
+        torch.cuda.synchronize()
+        took.append(ctx.profile_read()["select"][0])
+        n_tail = round((1 - alpha) * M * K)
+        order = y.float().flatten().sort().values
+        assert q.thresholds.tolist() == [float(order[n_tail]), float(order[-1 - n_tail])]
+    assert ctx.read_status() == 0
+    assert took[1] < 10 * took[0], took
+    ctx.close()
