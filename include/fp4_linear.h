@@ -197,7 +197,7 @@ int fp4_gemm(fp4_ctx* ctx, void* stream, const uint8_t* a_codes, const uint8_t* 
  *   change once per optimizer step) and is not recomputed; FP4_REUSE_A -- savedA already holds
  *   this activation quantised with the same alpha (the q/k/v projections of a layer, or its
  *   gate/up projections, read the same activation) and is not recomputed.
- *   With a heavy residual (savedA->sparse_cap at least 1 % of M * K, i.e. alpha <= 0.995) the
+ *   With a heavy residual (alpha allows at least 1 % of M * K entries: alpha <= 0.995) the
  *   residual's columns that at least max(M / 4, 512) tokens hit -- the outlier channels of
  *   Appendix D, up to 128 of them -- are multiplied on the tensor cores inside the GEMM (two-term
  *   FP16 splits of residual and weight); the other entries are added per entry in fp32.  The
@@ -207,9 +207,9 @@ int fp4_gemm(fp4_ctx* ctx, void* stream, const uint8_t* a_codes, const uint8_t* 
  *   A residual value
  *   beyond 43 000 times its token's clamped absmax does not fit the FP16 operand: the call
  *   then adds every entry per entry.
- *   A residual that may fill more than 4 % of the activation (by alpha; M >= 512) is
- *   multiplied as a dense matrix where that takes less time for the entries that are there: exact
- *   three-term BF16 split, chunks of 64 input channels added in fp32 in order.  Same bound, without the second term.
+ *   A residual that may fill more than 4 % of the activation (by alpha; M >= 512) is multiplied as a
+ *   dense matrix where that takes less time for the entries that are there: exact three-term BF16
+ *   split, chunks of 64 input channels added in fp32 in order.  Same bound, without the second term.
  */
 #define FP4_REUSE_W 1
 #define FP4_REUSE_A 2

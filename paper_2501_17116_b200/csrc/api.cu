@@ -387,10 +387,10 @@ int linear_fwd_impl(fp4_ctx* ctx, cudaStream_t st, Arena arena, const void* A_bf
     Arena a(scratch_a, quantize_scratch_bytes(M, K));
     savedA->rows = M;
     savedA->cols = K;
-    // CSR on side stream 1, CSC on side stream 0 (behind W's short chain, which has ended by then)
-    // (with a dense tail: once the tail's operands are there, beside the GEMM; with a heavy residual beside its
-    // product; earlier it would hold up the
-    // CSR's fill, which the tail waits for: 8192 x 11008, 1 % per tail, CSR ready after 33 instead of 67 us)
+    // CSR on side stream 1, CSC on side stream 0 (behind W's short chain, which has ended by then).  With a dense tail
+    // or a dense product the CSC's fill waits until their operands are there and runs beside the GEMM or the
+    // product: earlier it would hold up the CSR's fill, which those operands wait for (8192 x 11008, 1 % per tail:
+    // CSR ready after 33 instead of 67 us).
     const SparseOverlap so = {ctx->side[1], ctx->ev[2], ctx->ev[3], ctx->side[0], ctx->ev[7], ctx->ev[4],
                               tail_on || full_on ? &csc_fill : nullptr};
     rc = launch_quantize(ctx, st, a, A_bf16, M, K, /*scale_axis=*/0, alpha, nullptr, 0.0f, savedA, status,

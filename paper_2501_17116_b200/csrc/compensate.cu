@@ -97,9 +97,9 @@ comp_fwd_kernel(const float* __restrict__ y1, const int* __restrict__ rowptr, co
 // The forward compensation when the dense tail is in use: tail_a has listed, per token, the entries
 // the tail does not cover (`kept`: column and value bits, at the token's own range of the CSR, ending
 // at kept_end[m]), so this kernel walks a plain list: one 8-byte broadcast load per entry, eight
-// weight-row gathers in flight per lane at four blocks per SM (measured on the 13B layer: four in
-// flight 9.3 ms per step, eight 7.7 ms, twelve at three blocks 8.0 ms, sixteen at two blocks 10.2 ms).  If the tail was switched off on the device (*tail_count == 0: a value
-// FP16 cannot hold) the list is not valid and the whole CSR row is added instead.
+// weight-row gathers in flight per lane at 32 warps per SM (measured on the 13B layer: four in flight 9.3 ms per
+// step, eight 7.7 ms, twelve at 24 warps 8.0 ms, sixteen at 16 warps 10.2 ms).  If the tail was switched off on the
+// device (*tail_count == 0: a value FP16 cannot hold) the list is not valid and the whole CSR row is added instead.
 constexpr int FWD_FLY = 8;                 // weight-row gathers a lane keeps in flight
 __global__ void __launch_bounds__(FWD_THREADS, 8)
 comp_fwd_kept_kernel(const float* __restrict__ y1, const int* __restrict__ rowptr, const int* __restrict__ col,
