@@ -48,10 +48,6 @@ NCU_TRAFFIC_PER_LAUNCH = {
     "llama-1.3b-layer": {
         "gemm": 17.4e6,        # profiles/gemm_fp4_llama1p3b.md: forward 6.4 MB, backward (two GEMMs per launch) 28.3 MB
         "encode": 14.0e6,      # profiles/quantizer_encode_llama1p3b.md (writes still in L2 at kernel end)
-        "select": 16.9e6,      # profiles/quantizer_select_absmax_llama1p3b.md
-        "absmax": 12.6e6,
-        "comp_fwd": 36.1e6,    # profiles/compensation_llama1p3b.md
-        "comp_wgrad_dge": 6.5e6,
     },
     # profiles/compensation_gather_llama7b_mlp.md: captured on the 7B MLP block (same kernels, same
     # residual density; the 13B layer is too large for a multi-pass capture) and scaled to the mean
