@@ -250,6 +250,8 @@ constexpr uint32_t IN_PHASE = 1, IN_PENDING = 2;     // parity of the next wait;
 __device__ __forceinline__ void wgrad_request(WgradInput& in, int w_bytes, int row0, int col) {
   const uint32_t bytes = in.state & (IN_W_BYTES | IN_ADD_BYTES);
   if (!bytes) return;
+  fence_async_smem();                                  // the lanes' reads of the chunk before, then the copy over it
+  __syncwarp();
   if (elect_one()) {
     mbar_arrive_expect_tx(in.bar, bytes);
     if (bytes & IN_W_BYTES) tma_load_2d(in.buf, in.map_w, in.bar, col, row0);
@@ -280,15 +282,15 @@ __device__ __forceinline__ bool epilogue_tile_wgrad(const GemmArgs& args, int ro
   const uint8_t* add_smem = in.buf + w_bytes + lane * 64;
   const int w_fx = (lane >> 2) & 1, add_fx = (lane >> 1) & 3;
   uint32_t v[32];
-  tmem_ld_32x16(t_base + uint32_t(c0), v);
 #pragma unroll 1
   for (; c0 < n_valid; c0 += 16 * G) {
     const int next = c0 + 16 * G;
+    // (loaded and waited for in one iteration: no load into registers stays in flight over the waits below)
+    tmem_ld_32x16(t_base + uint32_t(c0), v);
     tmem_ld_wait();
     float y[16];
     uint32_t w[8];
     descale_chunk<16>(v, d_row, dcol + c0, y);
-    if (next < n_valid) tmem_ld_32x16(t_base + uint32_t(next), v);
     if (in.state & IN_PENDING) {
       const bool ok = mbar_wait(in.bar, in.state & IN_PHASE, abort_flag, args.status, wait_limit_ns);
       if (!__all_sync(0xFFFFFFFFu, ok)) return false;
