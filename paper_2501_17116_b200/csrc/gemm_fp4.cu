@@ -250,7 +250,9 @@ constexpr uint32_t IN_PHASE = 1, IN_PENDING = 2;     // parity of the next wait;
 __device__ __forceinline__ void wgrad_request(WgradInput& in, int w_bytes, int row0, int col) {
   const uint32_t bytes = in.state & (IN_W_BYTES | IN_ADD_BYTES);
   if (!bytes) return;
-  fence_async_smem();                                  // the lanes' reads of the chunk before, then the copy over it
+  // The copy goes over what the lanes have read of the chunk before.  Their loads are of another proxy than the copy and
+  // may be carried out behind it without this fence: half rows of weights then came from the chunk after theirs.
+  fence_async_smem();
   __syncwarp();
   if (elect_one()) {
     mbar_arrive_expect_tx(in.bar, bytes);

@@ -218,7 +218,7 @@ def test_weight_gradient_of_wide_tiles_without_clamp_is_the_same_every_time(lib,
     """No clamp, DGE on, tiles of 240 columns: the fused epilogue's four chunks per warp.  Thirty passes give the same
     BF16 dW, and it is the rounding of the fp32 dW (the same sums through another staging of the outputs)."""
     g = torch.Generator("cuda").manual_seed(K)
-    A = (torch.randn((M, K), device="cuda", generator=g) / torch.rand((M, K), device="cuda", generator=g).sqrt()).bfloat16()
+    A = (torch.randn((M, K), device="cuda", generator=g) / (torch.rand((M, K), device="cuda", generator=g) + 1e-3).sqrt()).bfloat16()
     W = (torch.randn((K, N), device="cuda", generator=g) * 0.02).bfloat16()
     dY = (torch.randn((M, N), device="cuda", generator=g) * 1e-3).bfloat16()
     ctx = lib.Context.for_shape(M, K, N)
