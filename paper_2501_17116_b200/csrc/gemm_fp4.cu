@@ -6,9 +6,12 @@
 // form of all three GEMMs of the layer (Fig. 2; Eq. 3; Appendix C.2).  The two de-scales are
 // applied to the accumulators in the epilogue, after the GEMM, as Appendix C.2 prescribes.
 //
-// Structure: persistent CTAs (one per SM), 128 x BN output tile per CTA:
+// Structure: persistent CTAs (one per SM), 128 x BN output tile per CTA, or 256 x BN per pair of CTAs
+// (cta_group::2: each CTA holds its 128 rows of A, half of B's rows and the accumulators of its rows; the even one
+// issues the MMAs of both):
 //   warp 0      TMA producer: cp.async.bulk.tensor loads into 128-byte-swizzled shared memory,
-//               a ring of 3 or 4 stages guarded by full/empty mbarriers;
+//               a ring of 3 to 6 stages guarded by full/empty mbarriers (of a pair: the copies of both
+//               complete on the even CTA's full barrier, its commits free the stage in both);
 //   warp 1      allocates tensor memory and issues tcgen05.mma from one thread, fp32
 //               accumulators in tensor memory; tcgen05.commit releases stages and publishes tiles;
 //   warps 2..   epilogue (8 warps; 16 with the fused weight-gradient epilogue): tcgen05.ld the
@@ -51,17 +54,17 @@ __host__ __device__ constexpr int tile_n(int kind, int epi) {
   return kind == FP4_GEMM_F8F6F4 && epi == EPI_PLAIN ? 256 : 240;
 }
 // Shared memory: operand ring, epilogue buffers, barriers, column de-scales [2][256], DGE column scales [2][256].
-// The ring has MAX_STAGES stages (A and B tile of one k-block) where they fit, else three.
-constexpr int MAX_STAGES = 4;
+// The ring has MAX_STAGES stages (A and B tile of one k-block; of a pair half of the B tile) where they fit, else fewer.
+constexpr int MAX_STAGES = 4, MAX_STAGES_PAIR = 6;
 constexpr int MISC_BYTES = 512;
 constexpr int FIXED_SMEM = 1024 + MISC_BYTES + 2 * 256 * 4 + 2 * 256 * 4;
 constexpr int MOST_SMEM = 227 * 1024;
 struct SmemPlan {
   int stages, stage_bytes, out_bytes, in_bytes;      // out_bytes, in_bytes: per epilogue warp
 };
-SmemPlan plan_smem(int epi, int bn, bool has_w, bool has_add, bool f32) {
-  const int avail = MOST_SMEM - FIXED_SMEM, stage = A_STAGE_BYTES + 128 * bn, warps = epi_warps(epi);
-  SmemPlan p = {MAX_STAGES, stage, STAGE_OUT_BYTES, 0};
+SmemPlan plan_smem(int epi, bool pair, int bn, bool has_w, bool has_add, bool f32) {
+  const int avail = MOST_SMEM - FIXED_SMEM, stage = A_STAGE_BYTES + (pair ? 64 : 128) * bn, warps = epi_warps(epi);
+  SmemPlan p = {pair ? MAX_STAGES_PAIR : MAX_STAGES, stage, STAGE_OUT_BYTES, 0};
   if (epi == EPI_WGRAD) {
     p.out_bytes = FUSED_OUT_BYTES;
     p.in_bytes = (has_w ? IN_W_BYTES : 0) + (has_add ? IN_ADD_BYTES : 0);
@@ -105,20 +108,20 @@ struct GemmArgs {
   int skip_fill;
 };
 
-// Instruction descriptors: M = 128, N = bn, both operands K-major, E2M1 x E2M1 -> fp32.
+// Instruction descriptors: M = 128 (a pair of CTAs: 256), N = bn, both operands K-major, E2M1 x E2M1 -> fp32.
 // kind::f8f6f4 format fields: E4M3 = 0, E2M1 = 5
 // format field of the byte-container kind for an operand format of the C interface
 __host__ __device__ constexpr uint32_t f8f6f4_code(int format) {
   return format == FP4_FORMAT_E4M3 ? 0u : (format == FP4_FORMAT_E5M2 ? 1u : 5u);
 }
-constexpr uint32_t idesc_f8f6f4(int bn, int a_format, int b_format) {
+constexpr uint32_t idesc_f8f6f4(int m, int bn, int a_format, int b_format) {
   return (1u << 4) | (f8f6f4_code(a_format) << 7) | (f8f6f4_code(b_format) << 10) | (uint32_t(bn >> 3) << 17) |
-         (uint32_t(BM >> 4) << 24);
+         (uint32_t(m >> 4) << 24);
 }
 // kind::f16 with FP16 operands (format 0) and fp32 accumulators
-constexpr uint32_t idesc_f16(int bn) { return (1u << 4) | (uint32_t(bn >> 3) << 17) | (uint32_t(BM >> 4) << 24); }
-constexpr uint32_t idesc_mxf4(int bn) {
-  return (1u << 7) | (1u << 10) | (uint32_t(bn >> 3) << 17) | (1u << 23) | (uint32_t(BM >> 4) << 24);
+constexpr uint32_t idesc_f16(int m, int bn) { return (1u << 4) | (uint32_t(bn >> 3) << 17) | (uint32_t(m >> 4) << 24); }
+constexpr uint32_t idesc_mxf4(int m, int bn) {
+  return (1u << 7) | (1u << 10) | (uint32_t(bn >> 3) << 17) | (1u << 23) | (uint32_t(m >> 4) << 24);
 }
 
 // Where the bulk stores of the epilogue take their boxes from and how they are described.
@@ -335,7 +338,7 @@ __device__ __forceinline__ bool epilogue_tile_wgrad(const GemmArgs& args, int ro
   return true;
 }
 
-template <int KIND, int EPI>
+template <int KIND, int EPI, bool PAIR>
 __global__ void __launch_bounds__(num_threads(EPI), 1)
 gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                 const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_out_aux,
@@ -351,8 +354,8 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   uint8_t* s_out = s_in + epi_warps(EPI) * args.smem.in_bytes;         // staging of each epilogue warp
   uint8_t* smem_misc = s_out + epi_warps(EPI) * args.smem.out_bytes;
   uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem_misc);
-  uint64_t* empty_bar = full_bar + MAX_STAGES;
-  uint64_t* acc_full = empty_bar + MAX_STAGES;
+  uint64_t* empty_bar = full_bar + MAX_STAGES_PAIR;
+  uint64_t* acc_full = empty_bar + MAX_STAGES_PAIR;
   uint64_t* acc_empty = acc_full + 2;
   uint64_t* in_bar = acc_empty + 2;                    // [16]
   uint64_t* final_bar = in_bar + 16;
@@ -368,10 +371,14 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   // under the MMAs of the other's first.
   const int tiles_first = args.num_m_blocks * args.num_n_blocks;
   const int num_tiles = tiles_first + args2.num_m_blocks * args2.num_n_blocks;
+  // A worker is a CTA, or a pair of them: the even one issues the MMAs of both.
+  constexpr int CTAS = PAIR ? 2 : 1;
+  const int rank = PAIR ? int(cluster_ctarank()) : 0;
+  const int worker = int(blockIdx.x) / CTAS, workers = int(gridDim.x) / CTAS;
 
   int pre = 0;          // k-blocks of the first tile that thread 0 has requested already (see below)
-  if (int(blockIdx.x) < num_tiles) {
-    const int kbs = int(blockIdx.x) >= tiles_first ? args2.num_k_blocks : args.num_k_blocks;
+  if (!PAIR && worker < num_tiles) {
+    const int kbs = worker >= tiles_first ? args2.num_k_blocks : args.num_k_blocks;
     pre = kbs < STAGES ? kbs : STAGES;
   }
   if (threadIdx.x == 0) {
@@ -381,7 +388,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     }
     for (int a = 0; a < 2; ++a) {
       mbar_init(&acc_full[a], 1);
-      mbar_init(&acc_empty[a], epi_warps(EPI));
+      mbar_init(&acc_empty[a], CTAS * epi_warps(EPI));
     }
     if (EPI == EPI_WGRAD)
       for (int w = 0; w < epi_warps(EPI); ++w) mbar_init(&in_bar[w], 1);
@@ -392,12 +399,12 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     // This thread is the producer.  The stages are empty and the barriers are its own work, so it
     // requests the first k-blocks of its first tile now: they travel while tensor memory is
     // allocated and the block synchronises.
-    if (int(blockIdx.x) < num_tiles) {
-      const bool second = int(blockIdx.x) >= tiles_first;
+    if (!PAIR && worker < num_tiles) {
+      const bool second = worker >= tiles_first;
       const GemmArgs& pa = second ? args2 : args;
       const CUtensorMap* ma = second ? &map_a2 : &map_a;
       const CUtensorMap* mb = second ? &map_b2 : &map_b;
-      const int tt = second ? int(blockIdx.x) - tiles_first : int(blockIdx.x);
+      const int tt = second ? worker - tiles_first : worker;
       const int m_blk = tt % pa.num_m_blocks, n_blk = tt / pa.num_m_blocks;
       for (int kb = 0; kb < pre; ++kb) {
         mbar_arrive_expect_tx(&full_bar[kb], pa.tx_bytes);
@@ -420,12 +427,7 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       asm volatile("prefetch.tensormap [%0];" ::"l"(&map_out2) : "memory");
     }
   }
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(TMEM_COLS)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
+  if (warp == 1) tmem_alloc<CTAS>(tmem_slot, TMEM_COLS);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -440,7 +442,13 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     }
     tc_fence_before();
-    __syncthreads();
+    if (!PAIR) __syncthreads();
+    tc_fence_after();
+  }
+  if (PAIR) {
+    // the peer's barriers exist, and both tensor memories hold their scales
+    tc_fence_before();
+    cluster_sync_all();
     tc_fence_after();
   }
 
@@ -455,21 +463,23 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       uint32_t fills = uint32_t(pre);
       bool ok = true;
       const int tail_kb = args.tail_count ? 3 * ((min(*args.tail_count, TAIL_MAX_COLS) + 63) / 64) : 0;
-      for (int t = blockIdx.x; t < num_tiles && ok; t += gridDim.x) {
+      // (in a pair the copies of both CTAs complete on the even one's barriers)
+      const uint32_t full0 = PAIR ? cluster_address(full_bar, 0) : smem_u32(full_bar);
+      for (int t = worker; t < num_tiles && ok; t += workers) {
         const bool second = t >= tiles_first;
         const GemmArgs& pa = second ? args2 : args;
         const CUtensorMap* ma = second ? &map_a2 : &map_a;
         const CUtensorMap* mb = second ? &map_b2 : &map_b;
         const int tt = second ? t - tiles_first : t;
-        const int m_blk = tt % pa.num_m_blocks;
-        const int n_blk = tt / pa.num_m_blocks;
-        for (int kb = (t == int(blockIdx.x) ? pre : 0); kb < pa.num_k_blocks; ++kb) {
+        const int a_row = (CTAS * (tt % pa.num_m_blocks) + rank) * BM;
+        const int b_row = (tt / pa.num_m_blocks) * pa.bn + rank * (pa.bn / 2);
+        for (int kb = (t == worker ? pre : 0); kb < pa.num_k_blocks; ++kb) {
           ok = mbar_wait(&empty_bar[stage], phase ^ 1u, abort_flag, args.status, args.wait_limit_ns);
           if (!ok) break;
           if (blockIdx.x != 0 || int(fills) != args.skip_fill) {      // a left-out fill: no copy, no arrival
-            mbar_arrive_expect_tx(&full_bar[stage], pa.tx_bytes);
-            tma_load_2d(smem + stage * STAGE_BYTES, ma, &full_bar[stage], kb * 128, m_blk * BM);
-            tma_load_2d(smem + stage * STAGE_BYTES + A_STAGE_BYTES, mb, &full_bar[stage], kb * 128, n_blk * pa.bn);
+            if (rank == 0) mbar_arrive_expect_tx(&full_bar[stage], CTAS * pa.tx_bytes);
+            tma_load_2d_group<CTAS>(smem + stage * STAGE_BYTES, ma, full0 + 8 * stage, kb * 128, a_row);
+            tma_load_2d_group<CTAS>(smem + stage * STAGE_BYTES + A_STAGE_BYTES, mb, full0 + 8 * stage, kb * 128, b_row);
           }
           ++fills;
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
@@ -477,14 +487,18 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         for (int kb = 0; kb < tail_kb && ok; ++kb) {      // dense tail: FP16 columns 64 kb .. 64 kb + 63
           ok = mbar_wait(&empty_bar[stage], phase ^ 1u, abort_flag, args.status, args.wait_limit_ns);
           if (!ok) break;
-          mbar_arrive_expect_tx(&full_bar[stage], args.tail_tx_bytes);
-          tma_load_2d(smem + stage * STAGE_BYTES, &map_a2, &full_bar[stage], kb * 64, m_blk * BM);
-          tma_load_2d(smem + stage * STAGE_BYTES + A_STAGE_BYTES, &map_b2, &full_bar[stage], kb * 64, n_blk * args.bn);
+          if (rank == 0) mbar_arrive_expect_tx(&full_bar[stage], CTAS * args.tail_tx_bytes);
+          tma_load_2d_group<CTAS>(smem + stage * STAGE_BYTES, &map_a2, full0 + 8 * stage, kb * 64, a_row);
+          tma_load_2d_group<CTAS>(smem + stage * STAGE_BYTES + A_STAGE_BYTES, &map_b2, full0 + 8 * stage, kb * 64, b_row);
           ++fills;
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
       }
-      if (!ok) {
+      if (!ok && PAIR) {
+        // Gave up: the peer's copies complete on the even CTA's barriers too, so the copies in flight are given time to land.
+        const uint64_t t0 = global_timer_ns();
+        while (global_timer_ns() - t0 < 1000000ull) {}
+      } else if (!ok) {
         // Gave up: let the copies already in flight land before shared memory is released.
         const uint32_t last = fills < uint32_t(STAGES) ? fills : uint32_t(STAGES);
         for (uint32_t back = 1; back <= last; ++back) {
@@ -498,14 +512,14 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer ---------
-    if (elect_one()) {
+    if (rank == 0 && elect_one()) {
       int stage = 0;
       uint32_t phase = 0;
       int acc = 0;
       uint32_t acc_phase = 0;
       bool ok = true;
       const int tail_kb = args.tail_count ? 3 * ((min(*args.tail_count, TAIL_MAX_COLS) + 63) / 64) : 0;
-      for (int t = blockIdx.x; t < num_tiles && ok; t += gridDim.x) {
+      for (int t = worker; t < num_tiles && ok; t += workers) {
         ok = mbar_wait(&acc_empty[acc], acc_phase ^ 1u, abort_flag, args.status, args.wait_limit_ns);
         if (!ok) break;
         tc_fence_after();
@@ -523,13 +537,13 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
             // 32 bytes of the swizzled 128-byte row per instruction: +2 in the (>>4) address field
             const uint32_t accumulate = (kb | k) != 0 ? 1u : 0u;
             if (KIND == FP4_GEMM_F8F6F4) {
-              mma_f8f6f4(d_tmem, a_desc + uint64_t(2 * k), b_desc + uint64_t(2 * k), idesc, accumulate);
+              mma_f8f6f4<CTAS>(d_tmem, a_desc + uint64_t(2 * k), b_desc + uint64_t(2 * k), idesc, accumulate);
             } else {
-              mma_mxf4(d_tmem, a_desc + uint64_t(2 * k), b_desc + uint64_t(2 * k), idesc, tmem_base + SF_COL_A,
+              mma_mxf4<CTAS>(d_tmem, a_desc + uint64_t(2 * k), b_desc + uint64_t(2 * k), idesc, tmem_base + SF_COL_A,
                        tmem_base + SF_COL_B, accumulate);
             }
           }
-          tc_commit(&empty_bar[stage]);       // frees the stage once these MMAs have read it
+          tc_commit_all<CTAS>(&empty_bar[stage]);       // frees the stage once these MMAs have read it
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
         for (int kb = 0; kb < tail_kb && ok; ++kb) {
@@ -540,16 +554,16 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           const uint64_t b_desc = make_smem_desc(smem_u32(smem + stage * STAGE_BYTES + A_STAGE_BYTES));
 #pragma unroll
           for (int k = 0; k < 4; ++k)          // 16 FP16 columns = 32 bytes of the 128-byte row per instruction
-            mma_f16(d_tmem, a_desc + uint64_t(2 * k), b_desc + uint64_t(2 * k), args.tail_idesc, 1u);
-          tc_commit(&empty_bar[stage]);
+            mma_f16<CTAS>(d_tmem, a_desc + uint64_t(2 * k), b_desc + uint64_t(2 * k), args.tail_idesc, 1u);
+          tc_commit_all<CTAS>(&empty_bar[stage]);
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
-        tc_commit(&acc_full[acc]);            // accumulators of this tile are complete
+        tc_commit_all<CTAS>(&acc_full[acc]);            // accumulators of this tile are complete
         if (++acc == NACC) { acc = 0; acc_phase ^= 1u; }
       }
       // All MMAs issued by this thread must have retired before tensor memory is freed.
-      tc_commit(final_bar);
+      tc_commit<CTAS>(final_bar);
       const uint64_t t0 = global_timer_ns();
       while (!mbar_try_wait(final_bar, 0)) {
         if (global_timer_ns() - t0 > args.wait_limit_ns) {
@@ -572,16 +586,18 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     uint32_t store_seq = 0;
     WgradInput in = {&map_w, &map_add, s_in + (warp - 2) * args.smem.in_bytes, &in_bar[warp - 2], 0u};
     bool dead = false;
-    for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
+    const uint32_t acc_empty0 = PAIR ? cluster_address(acc_empty, 0) : smem_u32(acc_empty);   // the issuer's
+    for (int t = worker; t < num_tiles; t += workers) {
       const bool second = t >= tiles_first;
       const GemmArgs& pa = second ? args2 : args;
       const OutMaps out_maps = {second ? &map_out2 : &map_out, second ? &map_out_aux2 : &map_out_aux};
       const int tt = second ? t - tiles_first : t;
-      const int m_blk = tt % pa.num_m_blocks;
+      const int m_blk = CTAS * (tt % pa.num_m_blocks) + rank;        // this CTA's 128 rows
       const int n_blk = tt / pa.num_m_blocks;
+      const bool rows_valid = !PAIR || m_blk * BM < pa.I;            // an odd number of them: the last one is missing
       // De-scales of this tile are fetched before the accumulators are awaited, under the MMAs.
       const int row = m_blk * BM + quarter * 32 + lane;
-      const float d_row = pa.row_amax ? __fdiv_rn(__ldg(&pa.row_amax[row]), pa.row_div) : 1.0f;
+      const float d_row = pa.row_amax && rows_valid ? __fdiv_rn(__ldg(&pa.row_amax[row]), pa.row_div) : 1.0f;
       float* dcol = s_dcol + tile_parity * 256;
       float* gcol = s_gcol + tile_parity * 256;
       for (int c = et; c < pa.bn; c += 32 * EW) {
@@ -594,17 +610,19 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       }
       bool add_row = false;
       if (EPI == EPI_WGRAD) {
-        add_row = pa.slot_of_row && __ldg(&pa.slot_of_row[row]) >= 0;
+        add_row = pa.slot_of_row && rows_valid && __ldg(&pa.slot_of_row[row]) >= 0;
         in.state = (in.state & (IN_PHASE | IN_PENDING)) | (pa.has_w ? IN_W_BYTES : 0u) |
                    (__any_sync(0xFFFFFFFFu, add_row) ? IN_ADD_BYTES : 0u);
-        if (!dead && 16 * group < min(pa.bn, pa.J - n_blk * pa.bn))
+        if (!dead && rows_valid && 16 * group < min(pa.bn, pa.J - n_blk * pa.bn))
           wgrad_request(in, pa.has_w ? IN_W_BYTES : 0, m_blk * BM + quarter * 32, n_blk * pa.bn + 16 * group);
       }
       const bool ok = mbar_wait(&acc_full[acc], acc_phase, abort_flag, args.status, args.wait_limit_ns);
       if (epilogue_bar_any(!ok, 32 * EW)) break;   // also publishes dcol to the other warps
       tc_fence_after();
       const uint32_t t_base = tmem_base + (uint32_t(quarter * 32) << 16) + uint32_t(acc * ACC_STRIDE);
-      if (EPI == EPI_WGRAD)
+      if (!rows_valid) {
+        // nothing to store
+      } else if (EPI == EPI_WGRAD)
         dead = !epilogue_tile_wgrad<G>(pa, m_blk, n_blk, t_base, d_row, dcol, gcol, add_row, in, abort_flag,
                                        args.wait_limit_ns, stage, quarter, group, lane, out_maps, store_seq,
                                        args.smem.out_bytes == FUSED_OUT_BYTES);
@@ -613,7 +631,9 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
                                    store_seq);
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&acc_empty[acc]);
+      if (lane == 0) {
+        if (PAIR) mbar_arrive_cluster(acc_empty0 + 8 * acc); else mbar_arrive(&acc_empty[acc]);
+      }
       if (++acc == NACC) { acc = 0; acc_phase ^= 1u; }
       tile_parity ^= 1u;
     }
@@ -626,9 +646,8 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
 
   tc_fence_before();
   __syncthreads();
-  if (warp == 1) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
-  }
+  if (PAIR) cluster_sync_all();               // neither CTA leaves while the other's MMAs or arrivals may touch it
+  if (warp == 1) tmem_dealloc<CTAS>(tmem_base, TMEM_COLS);
 }
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -726,81 +745,117 @@ struct Problem {
   bool fused;
 };
 
-template <int KIND, int EPI>
-int launch_kernel(int grid, cudaStream_t stream, const Problem& p, const Problem* second = nullptr) {
-  FP4_CUDA_TRY(cudaFuncSetAttribute(gemm_fp4_kernel<KIND, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, MOST_SMEM));
+template <int KIND, int EPI, bool PAIR>
+int launch_kernel(int workers, cudaStream_t stream, const Problem& p, const Problem* second) {
+  const auto kernel = gemm_fp4_kernel<KIND, EPI, PAIR>;
+  FP4_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MOST_SMEM));
   Problem none = p;
   none.args.num_m_blocks = none.args.num_n_blocks = 0;          // a second problem without tiles
   const Problem& q = second ? *second : none;
   GemmArgs args = p.args;
-  args.smem = plan_smem(EPI, p.args.bn > q.args.bn ? p.args.bn : q.args.bn, args.has_w, args.slot_of_row != nullptr,
+  args.smem = plan_smem(EPI, PAIR, p.args.bn > q.args.bn ? p.args.bn : q.args.bn, args.has_w, args.slot_of_row != nullptr,
                         args.out_f32 != 0);
   const int smem = FIXED_SMEM + args.smem.stages * args.smem.stage_bytes +
                    epi_warps(EPI) * (args.smem.out_bytes + args.smem.in_bytes);
-  gemm_fp4_kernel<KIND, EPI><<<grid, num_threads(EPI), smem, stream>>>(p.map_a, p.map_b, p.map_out, p.map_out_aux, args,
-                                                                       q.map_a, q.map_b, q.map_out, q.map_out_aux,
-                                                                       q.args, p.map_w, p.map_add);
+  cudaLaunchAttribute cluster = {};
+  cluster.id = cudaLaunchAttributeClusterDimension;
+  cluster.val.clusterDim.x = 2;
+  cluster.val.clusterDim.y = cluster.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(unsigned(PAIR ? 2 * workers : workers));
+  cfg.blockDim = dim3(unsigned(num_threads(EPI)));
+  cfg.dynamicSmemBytes = size_t(smem);
+  cfg.stream = stream;
+  cfg.attrs = &cluster;
+  cfg.numAttrs = PAIR ? 1 : 0;
+  FP4_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, p.map_a, p.map_b, p.map_out, p.map_out_aux, args, q.map_a, q.map_b, q.map_out,
+                                  q.map_out_aux, q.args, p.map_w, p.map_add));
   return FP4_OK;
 }
+int launch_problems(int gemm_kind, bool fused, bool pair, int workers, cudaStream_t stream, const Problem& p, const Problem* second) {
+  const bool f8 = gemm_kind == FP4_GEMM_F8F6F4;
+  if (pair) {
+    if (f8) return fused ? launch_kernel<FP4_GEMM_F8F6F4, EPI_WGRAD, true>(workers, stream, p, second)
+                         : launch_kernel<FP4_GEMM_F8F6F4, EPI_PLAIN, true>(workers, stream, p, second);
+    return fused ? launch_kernel<FP4_GEMM_MXF4, EPI_WGRAD, true>(workers, stream, p, second)
+                 : launch_kernel<FP4_GEMM_MXF4, EPI_PLAIN, true>(workers, stream, p, second);
+  }
+  if (f8) return fused ? launch_kernel<FP4_GEMM_F8F6F4, EPI_WGRAD, false>(workers, stream, p, second)
+                       : launch_kernel<FP4_GEMM_F8F6F4, EPI_PLAIN, false>(workers, stream, p, second);
+  return fused ? launch_kernel<FP4_GEMM_MXF4, EPI_WGRAD, false>(workers, stream, p, second)
+               : launch_kernel<FP4_GEMM_MXF4, EPI_PLAIN, false>(workers, stream, p, second);
+}
 
-// Tile widths of a launch's problems (each a multiple of 16): the ones for which the CTA with the most work
-// ends soonest, under a model of the kernel.  Narrow tiles spread a small GEMM over all SMs and shorten the
-// epilogue that nothing hides; wide ones move fewer operand bytes per flop, so that they win as soon as
-// there are a few rounds.  The constants (ns) were fitted to sweeps of the width over 29 launches, in 27 of
-// which the choice is within 1.5 % of the best width: a tile costs 800, a k-block 170 + 0.85 per column, an
-// epilogue 10 per column (12 with fp32 outputs), with the fused weight gradient 500 + 40 per column.
+// Form of a launch and tile widths of its problems (each a multiple of 16): the ones for which the CTA or pair with
+// the most work ends soonest, under a model of the kernel.  Narrow tiles spread a small GEMM over all SMs and shorten
+// the epilogue that nothing hides; wide ones move fewer operand bytes per flop, so that they win as soon as there are
+// a few rounds.  Pairs fetch half of B per SM, which shortens a k-block of 240 columns from 0.40 to 0.35 us (MMAs on
+// operands that are never loaded: 0.33), but a tile's hand-over between two CTAs and a pair's start cost more: long
+// contractions and large GEMMs take them (8192 x 5120 x 5120 82 -> 74.5 us, 8192^3 196 -> 178, back to back under
+// the power cap 238 -> 223; byte containers 359 -> 310), 4096 x 5504 x 2048 does not (22.0 by CTAs, 25.5 by pairs).
+// The constants (ns) were fitted to sweeps of the width over 40 launches in either form; the choice is within 2 %
+// of the best of them in all but two (byte containers, 4096 x 5504 x 2048: 6 %; backward of 256 x 1024 x 1024: 3 %).
+// By CTAs a tile costs 800, a k-block 170 (byte containers 130) + 0.85 per column, an epilogue 10 per column (12 with
+// fp32 outputs), with the fused weight gradient 500 + 40 per column; by pairs a tile 1300, a k-block 105 + 0.83 per
+// column, an epilogue 900 more, the launch 1000 more, of two problems 2000.
 // Measured: 128 x 11008 x 4096 (width 80 instead of 240) 9.5 -> 7.1 us, 1024^3 (64) 6.2 -> 4.9, backward of
 // 256 x 1024 x 1024 (64 and 144) 12.0 -> 6.2.
 struct TileWidths {
   int first, second;
+  bool pair;
 };
 struct TileCost {
   long long tiles;
   int steady, alone;           // time per tile in a row of tiles; what the last one adds
 };
-TileCost tile_cost(const Fp4GemmDesc& d, int gemm_kind, int bn) {
+TileCost tile_cost(const Fp4GemmDesc& d, int gemm_kind, bool pair, int bn) {
   const int per_stage = gemm_kind == FP4_GEMM_F8F6F4 ? 128 : 256;
-  const int kbs = int((d.C + per_stage - 1) / per_stage);
-  const int mma = 800 + kbs * (170 + (17 * bn) / 20);
+  const int kbs = int((d.C + per_stage - 1) / per_stage), rows = pair ? 2 * BM : BM;
+  const int mma = pair ? 1300 + kbs * (105 + (83 * bn) / 100)
+                       : 800 + kbs * ((gemm_kind == FP4_GEMM_F8F6F4 ? 130 : 170) + (17 * bn) / 20);
   const bool dge = d.epilogue && d.epilogue->w_bf16;
-  const int epi = dge ? 500 + 40 * bn : (d.out_f32 ? 12 : 10) * bn;
-  return {(d.I / BM) * ((d.J + bn - 1) / bn), mma > epi ? mma : epi, mma > epi ? epi : mma};
+  const int epi = (dge ? 500 + 40 * bn : (d.out_f32 ? 12 : 10) * bn) + (pair ? 900 : 0);
+  return {((d.I + rows - 1) / rows) * ((d.J + bn - 1) / bn), mma > epi ? mma : epi, mma > epi ? epi : mma};
 }
-TileWidths choose_bn(const fp4_ctx* ctx, const Fp4GemmDesc& p, const Fp4GemmDesc* q, int gemm_kind) {
+TileWidths choose_widths(const fp4_ctx* ctx, const Fp4GemmDesc& p, const Fp4GemmDesc* q, int gemm_kind) {
   constexpr int LEAST = 32, WIDTHS = 15;
   const bool fused = q || (p.epilogue && (p.epilogue->addend || p.epilogue->w_bf16));
   const int most = tile_n(gemm_kind, fused ? EPI_WGRAD : EPI_PLAIN);
-  TileCost costs[2][WIDTHS];
-  int n = 0;
-  for (int bn = most; bn >= LEAST; bn -= 16, ++n) {
-    costs[0][n] = tile_cost(p, gemm_kind, bn);
-    costs[1][n] = q ? tile_cost(*q, gemm_kind, bn) : TileCost{0, 0, 0};
-  }
-  TileWidths best = {most, most};
+  TileWidths best = {most, most, false};
   long long best_cost = -1;
-  const long long G = ctx->num_sms;
-  for (int i = 0; i < n; ++i)
-    for (int j = 0; j < (q ? n : 1); ++j) {
-      const TileCost &c = costs[0][i], &d = costs[1][j];
-      // CTA r takes tiles r, r + G, ...: the counts change at r = tiles mod G of the first problem and of both
-      const long long all = c.tiles + d.tiles;
-      const long long at[3] = {0, c.tiles % G, all % G};
-      long long cost = 0;
-      for (const long long r : at) {
-        const long long n1 = (c.tiles - r + G - 1) / G, n2 = (all - r + G - 1) / G - n1;
-        const long long t = n1 * c.steady + n2 * d.steady + (n2 ? d.alone : n1 ? c.alone : 0);
-        if (t > cost) cost = t;
-      }
-      if (best_cost < 0 || cost < best_cost) {
-        best_cost = cost;
-        best = {most - 16 * i, q ? most - 16 * j : most};
-      }
+  for (const bool pair : {false, true}) {
+    const long long G = pair ? ctx->num_sms / 2 : ctx->num_sms;
+    if (!G) continue;
+    TileCost costs[2][WIDTHS];
+    int n = 0;
+    for (int bn = most; bn >= LEAST; bn -= 16, ++n) {
+      costs[0][n] = tile_cost(p, gemm_kind, pair, bn);
+      costs[1][n] = q ? tile_cost(*q, gemm_kind, pair, bn) : TileCost{0, 0, 0};
     }
+    for (int i = 0; i < n; ++i)
+      for (int j = 0; j < (q ? n : 1); ++j) {
+        const TileCost &c = costs[0][i], &d = costs[1][j];
+        // worker r takes tiles r, r + G, ...: the counts change at r = tiles mod G of the first problem and of both
+        const long long all = c.tiles + d.tiles;
+        const long long at[3] = {0, c.tiles % G, all % G};
+        long long cost = 0;
+        for (const long long r : at) {
+          const long long n1 = (c.tiles - r + G - 1) / G, n2 = (all - r + G - 1) / G - n1;
+          const long long t = n1 * c.steady + n2 * d.steady + (n2 ? d.alone : n1 ? c.alone : 0);
+          if (t > cost) cost = t;
+        }
+        if (pair) cost += q ? 2000 : 1000;
+        if (best_cost < 0 || cost < best_cost) {
+          best_cost = cost;
+          best = {most - 16 * i, q ? most - 16 * j : most, pair};
+        }
+      }
+  }
   return best;
 }
 
 // Tensor maps and arguments of one GEMM.
-int make_problem(fp4_ctx* ctx, Problem* p, const Fp4GemmDesc& d, int gemm_kind, int bn, int32_t* status) {
+int make_problem(fp4_ctx* ctx, Problem* p, const Fp4GemmDesc& d, int gemm_kind, bool pair, int bn, int32_t* status) {
   if (gemm_kind != FP4_GEMM_MXF4 && gemm_kind != FP4_GEMM_F8F6F4) return FP4_ERR_ARG;
   const bool a8 = d.a_format != FP4_FORMAT_E2M1, b8 = d.b_format != FP4_FORMAT_E2M1;   // FP8 bytes
   if ((a8 || b8) && gemm_kind != FP4_GEMM_F8F6F4) return FP4_ERR_ARG;   // FP8 operands need the byte-container kind
@@ -811,7 +866,7 @@ int make_problem(fp4_ctx* ctx, Problem* p, const Fp4GemmDesc& d, int gemm_kind, 
     return FP4_ERR_ALIGN;
   int rc = make_codes_map(ctx, &p->map_a, d.a_codes, d.I, d.C, BM, gemm_kind, a8);
   if (rc != FP4_OK) return rc;
-  rc = make_codes_map(ctx, &p->map_b, d.b_codes, d.J, d.C, bn, gemm_kind, b8);
+  rc = make_codes_map(ctx, &p->map_b, d.b_codes, d.J, d.C, pair ? bn / 2 : bn, gemm_kind, b8);
   if (rc != FP4_OK) return rc;
   if (reinterpret_cast<uintptr_t>(d.out) & 15) return FP4_ERR_ALIGN;
   rc = make_out_maps(ctx, &p->map_out, &p->map_out_aux, d.out, d.I, d.J, d.out_f32);
@@ -822,16 +877,17 @@ int make_problem(fp4_ctx* ctx, Problem* p, const Fp4GemmDesc& d, int gemm_kind, 
   args.J = int(d.J);
   const int k_per_stage = gemm_kind == FP4_GEMM_F8F6F4 ? 128 : 256;   // elements per 128-byte row
   args.num_k_blocks = int((d.C + k_per_stage - 1) / k_per_stage);
-  args.num_m_blocks = int(d.I / BM);
+  const int rows = pair ? 2 * BM : BM, b_bytes = (pair ? 64 : 128) * bn;       // of a tile; of a CTA's part of B
+  args.num_m_blocks = int((d.I + rows - 1) / rows);
   args.bn = bn;
   args.num_n_blocks = int((d.J + bn - 1) / bn);
   // The transaction count of a copy is in bytes read from global memory: the byte-container form
   // fills a stage's 128-byte rows from 64 bytes of packed nibbles (E2M1) or from 128 bytes (E4M3).
   if (gemm_kind == FP4_GEMM_F8F6F4)
-    args.tx_bytes = uint32_t(A_STAGE_BYTES / (a8 ? 1 : 2) + 128 * bn / (b8 ? 1 : 2));
+    args.tx_bytes = uint32_t(A_STAGE_BYTES / (a8 ? 1 : 2) + b_bytes / (b8 ? 1 : 2));
   else
-    args.tx_bytes = uint32_t(A_STAGE_BYTES + 128 * bn);
-  args.idesc = gemm_kind == FP4_GEMM_F8F6F4 ? idesc_f8f6f4(bn, d.a_format, d.b_format) : idesc_mxf4(bn);
+    args.tx_bytes = uint32_t(A_STAGE_BYTES + b_bytes);
+  args.idesc = gemm_kind == FP4_GEMM_F8F6F4 ? idesc_f8f6f4(rows, bn, d.a_format, d.b_format) : idesc_mxf4(rows, bn);
   args.row_div = fp8_max(d.a_format);
   args.col_div = fp8_max(d.b_format);
   args.row_amax = d.row_amax;
@@ -854,8 +910,8 @@ int make_problem(fp4_ctx* ctx, Problem* p, const Fp4GemmDesc& d, int gemm_kind, 
   args.wait_limit_ns = ctx->debug_wait_limit_ns ? ctx->debug_wait_limit_ns : WAIT_LIMIT_NS;
   args.skip_fill = ctx->debug_skip_fill;
   args.tail_count = nullptr;
-  args.tail_tx_bytes = uint32_t(A_STAGE_BYTES + 128 * bn);
-  args.tail_idesc = idesc_f16(bn);
+  args.tail_tx_bytes = uint32_t(A_STAGE_BYTES + b_bytes);
+  args.tail_idesc = idesc_f16(rows, bn);
   return FP4_OK;
 }
 
@@ -869,8 +925,9 @@ int launch_gemm_fp4(fp4_ctx* ctx, cudaStream_t stream, const uint8_t* a_codes, c
   d.a_format = a_format;
   d.b_format = b_format;
   Problem p;
-  const int bn = choose_bn(ctx, d, nullptr, gemm_kind).first;
-  int rc = make_problem(ctx, &p, d, gemm_kind, bn, status);
+  const TileWidths widths = choose_widths(ctx, d, nullptr, gemm_kind);
+  const int bn = widths.first;
+  int rc = make_problem(ctx, &p, d, gemm_kind, widths.pair, bn, status);
   if (rc != FP4_OK) return rc;
   // The dense tail's operands travel in the slots of a second problem that has no tiles.
   Problem with_tail;
@@ -879,23 +936,15 @@ int launch_gemm_fp4(fp4_ctx* ctx, cudaStream_t stream, const uint8_t* a_codes, c
     with_tail.args.num_m_blocks = with_tail.args.num_n_blocks = 0;
     rc = make_tail_map(ctx, &with_tail.map_a, tail->a, I, BM);
     if (rc != FP4_OK) return rc;
-    rc = make_tail_map(ctx, &with_tail.map_b, tail->b, J, bn);
+    rc = make_tail_map(ctx, &with_tail.map_b, tail->b, J, widths.pair ? bn / 2 : bn);
     if (rc != FP4_OK) return rc;
     p.args.tail_count = tail->count;
   }
   const Problem* second = tail ? &with_tail : nullptr;
-  const GemmArgs& args = p.args;
-  const int tiles = args.num_m_blocks * args.num_n_blocks;
-  const int grid = tiles < ctx->num_sms ? tiles : ctx->num_sms;
+  const int tiles = p.args.num_m_blocks * p.args.num_n_blocks, most = widths.pair ? ctx->num_sms / 2 : ctx->num_sms;
   KernelScope scope(ctx, stream, KC_GEMM, 1);
-  int rc2;
-  if (gemm_kind == FP4_GEMM_F8F6F4)
-    rc2 = p.fused ? launch_kernel<FP4_GEMM_F8F6F4, EPI_WGRAD>(grid, stream, p, second)
-                  : launch_kernel<FP4_GEMM_F8F6F4, EPI_PLAIN>(grid, stream, p, second);
-  else
-    rc2 = p.fused ? launch_kernel<FP4_GEMM_MXF4, EPI_WGRAD>(grid, stream, p, second)
-                  : launch_kernel<FP4_GEMM_MXF4, EPI_PLAIN>(grid, stream, p, second);
-  if (rc2 != FP4_OK) return rc2;
+  rc = launch_problems(gemm_kind, p.fused, widths.pair, tiles < most ? tiles : most, stream, p, second);
+  if (rc != FP4_OK) return rc;
   FP4_CUDA_TRY(cudaGetLastError());
   return FP4_OK;
 }
@@ -905,17 +954,16 @@ int launch_gemm_fp4(fp4_ctx* ctx, cudaStream_t stream, const uint8_t* a_codes, c
 int launch_gemm_fp4_two(fp4_ctx* ctx, cudaStream_t stream, const Fp4GemmDesc& first, const Fp4GemmDesc& second,
                         int gemm_kind, int32_t* status) {
   Problem p, q;
-  const TileWidths bn = choose_bn(ctx, first, &second, gemm_kind);
-  int rc = make_problem(ctx, &p, first, gemm_kind, bn.first, status);
+  const TileWidths bn = choose_widths(ctx, first, &second, gemm_kind);
+  int rc = make_problem(ctx, &p, first, gemm_kind, bn.pair, bn.first, status);
   if (rc != FP4_OK) return rc;
-  rc = make_problem(ctx, &q, second, gemm_kind, bn.second, status);
+  rc = make_problem(ctx, &q, second, gemm_kind, bn.pair, bn.second, status);
   if (rc != FP4_OK) return rc;
   const int tiles = p.args.num_m_blocks * p.args.num_n_blocks + q.args.num_m_blocks * q.args.num_n_blocks;
-  const int grid = tiles < ctx->num_sms ? tiles : ctx->num_sms;
+  const int most = bn.pair ? ctx->num_sms / 2 : ctx->num_sms;
   KernelScope scope(ctx, stream, KC_GEMM, 1);
-  const int rc2 = gemm_kind == FP4_GEMM_F8F6F4 ? launch_kernel<FP4_GEMM_F8F6F4, EPI_WGRAD>(grid, stream, p, &q)
-                                                : launch_kernel<FP4_GEMM_MXF4, EPI_WGRAD>(grid, stream, p, &q);
-  if (rc2 != FP4_OK) return rc2;
+  rc = launch_problems(gemm_kind, true, bn.pair, tiles < most ? tiles : most, stream, p, &q);
+  if (rc != FP4_OK) return rc;
   FP4_CUDA_TRY(cudaGetLastError());
   return FP4_OK;
 }

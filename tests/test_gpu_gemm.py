@@ -64,6 +64,62 @@ def test_tile_widths(lib, ctx, kind, shape, f32):
 
 
 @pytest.mark.parametrize("kind", KINDS)
+@pytest.mark.parametrize("shape", [(4224, 4096, 4224), (3200, 2944, 6144)])
+@pytest.mark.parametrize("f32", [True, False])
+def test_pairs_of_ctas(lib, ctx, kind, shape, f32):
+    """Sizes that are computed by pairs of CTAs, with an odd number of 128-row blocks (the last pair's second half is
+    missing) and a ragged last tile: exact; and a wait that runs out in a pair ends both CTAs."""
+    I, J, C = shape
+    rng = np.random.default_rng(I + J + C)
+    ca, cb = _codes(rng, I, C), _codes(rng, J, C)
+    got = _run(lib, ctx, ca, cb, kind, out_f32=f32)
+    val = torch.tensor([0, .5, 1, 1.5, 2, 3, 4, 6, 0, -.5, -1, -1.5, -2, -3, -4, -6], dtype=torch.float64, device="cuda")
+    dec = lambda c: val[torch.from_numpy(c).cuda().long()]                                     # noqa: E731
+    want = (dec(ca) @ dec(cb).T).to(got.dtype)                                                 # exact in double
+    assert torch.equal(got, want)
+    c = lib.Context(0, 1 << 20)
+    a, b = torch.from_numpy(O.pack_nibbles(ca)).cuda(), torch.from_numpy(O.pack_nibbles(cb)).cuda()
+    c.debug_set(lib.binding.FP4_DEBUG_WAIT_LIMIT_US, 1000)
+    c.debug_set(lib.binding.FP4_DEBUG_SKIP_FILL, 7)
+    lib.fp4_gemm(c, a, b, gemm_kind=kind, out_f32=f32)
+    torch.cuda.synchronize()
+    assert c.read_status() & lib.FP4_DEV_TIMEOUT
+    c.debug_set(lib.binding.FP4_DEBUG_SKIP_FILL, -1)
+    c.debug_set(lib.binding.FP4_DEBUG_WAIT_LIMIT_US, 0)
+    c.status.zero_()
+    again = lib.fp4_gemm(c, a, b, gemm_kind=kind, out_f32=f32)
+    torch.cuda.synchronize()
+    assert c.read_status() == 0 and torch.equal(again, want)
+    c.close()
+
+
+def test_both_gradients_by_pairs_of_ctas(lib):
+    """The two backward GEMMs of a layer of 63 x 25 row blocks share a launch of pairs; slices of the layer, too small for
+    pairs, give the same bits (every sum is exact; the scales are pinned by a large value in each slice)."""
+    M, K, N = 8064, 3200, 4096
+    g = torch.Generator(device="cuda").manual_seed(3)
+    A = torch.randn((M, K), device="cuda", generator=g).bfloat16()
+    W = (torch.randn((K, N), device="cuda", generator=g) * 0.02).bfloat16()
+    dY = (torch.randn((M, N), device="cuda", generator=g) * 1e-3).bfloat16()
+    A[:, 0] = A[:, K - 256] = 8.0
+    W[0] = W[K - 256] = 0.25
+    c = lib.Context.for_shape(M, K, N)
+    _, sa, sw = lib.fp4_linear_fwd(c, A, W, 1.0)
+    dA, dW = lib.fp4_linear_bwd(c, dY, W, sa, sw)
+    for k0 in (0, K - 256):
+        As, Ws = A[:, k0:k0 + 256].contiguous(), W[k0:k0 + 256].contiguous()
+        _, sas, sws = lib.fp4_linear_fwd(c, As, Ws, 1.0)
+        _, dWs = lib.fp4_linear_bwd(c, dY, Ws, sas, sws)
+        assert torch.equal(dW[k0:k0 + 256], dWs)
+    for m0 in (0, M - 256):
+        _, sas, _ = lib.fp4_linear_fwd(c, A[m0:m0 + 256].contiguous(), W, 1.0)
+        dAs, _ = lib.fp4_linear_bwd(c, dY[m0:m0 + 256].contiguous(), W, sas, sw)
+        assert torch.equal(dA[m0:m0 + 256], dAs)
+    assert c.read_status() == 0
+    c.close()
+
+
+@pytest.mark.parametrize("kind", KINDS)
 def test_extreme_codes_long_contraction(lib, ctx, kind):
     """All +-6 operands over the longest contraction of the workloads (16384): |acc| up to 589824."""
     rng = np.random.default_rng(5)
