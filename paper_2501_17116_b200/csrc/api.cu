@@ -351,8 +351,8 @@ int linear_fwd_impl(fp4_ctx* ctx, cudaStream_t st, Arena arena, const void* A_bf
   float* y1 = occ ? arena.take<float>(size_t(M) * size_t(N)) : nullptr;
   char* scratch_a = reuse_a ? nullptr : arena.take<char>(quantize_scratch_bytes(M, K));
   char* scratch_w = reuse_w ? nullptr : arena.take<char>(quantize_scratch_bytes(K, N));
-  // A residual that fills a few per cent of the activation or more is multiplied as a dense matrix, ahead of the
-  // GEMM, whose epilogue adds the product.  A lighter one that still may hold 1 % (by the caller's capacity: alpha
+  // A residual that fills a few per cent of the activation or more is multiplied as a dense matrix, behind the
+  // GEMM, whose product it adds.  A lighter one that still may hold 1 % (by the caller's capacity: alpha
   // <= 0.995) sends its hot columns through the GEMM as a dense tail instead of per-entry gathers.
   const size_t full_bytes = residual_full_scratch_bytes(M, K);
   const bool full_room = full_bytes && full_product_fits(arena, M, K, N);
@@ -421,20 +421,43 @@ int linear_fwd_impl(fp4_ctx* ctx, cudaStream_t st, Arena arena, const void* A_bf
     return FP4_OK;
   };
   if (full_on) {
+    // The FP4 GEMM runs beside the making of the product's operand (side stream 0, behind W's chain, which the GEMM waits
+    // for too) and beside the CSR's chain; the product's epilogue adds Y1 and stores Y.
+    ResidualFull f = {};
+    f.ptr = savedA->csr_rowptr;
+    f.idx = savedA->csr_col;
+    f.val = savedA->csr_val;
+    f.R = M;
+    f.C = K;
+    f.act_bf16 = reuse_a ? nullptr : A_bf16;           // (with a reused operand the activation need not be there)
+    f.thresholds = savedA->thresholds;
+    f.thr_per_row = ctx->quantile_mode == FP4_QUANTILE_TOKEN;
+    f.dense_bf16 = W_bf16;
+    f.N = N;
+    f.out = {y1, Y, out_f32};
+    f.kernel_class = KC_COMP_FWD;
+    f.status = status;
+    Arena fa(scratch_full, full_bytes);
+    rc = residual_full_begin(ctx, f, fa);
+    if (rc != FP4_OK) return rc;
+    cudaStream_t so = ov ? ctx->side[0] : st;
+    if (ov) {
+      FP4_CUDA_TRY(cudaEventRecord(ctx->ev[5], st));
+      FP4_CUDA_TRY(cudaStreamWaitEvent(so, ctx->ev[5], 0));
+    }
+    rc = launch_residual_operand(ctx, so, f, 0);
+    if (rc != FP4_OK) return rc;
+    if (ov) FP4_CUDA_TRY(cudaEventRecord(ctx->ev[6], so));
+    rc = launch_gemm_fp4(ctx, st, savedA->codes, savedW->codes_t, M, N, K, savedA->amax, savedW->amax, y1, 1, gemm_kind, status,
+                         nullptr, a8, w8);
+    if (rc != FP4_OK) return rc;
+    if (ov) FP4_CUDA_TRY(cudaStreamWaitEvent(st, ctx->ev[6], 0));
     if (!reuse_a && ov) {
-      FP4_CUDA_TRY(cudaStreamWaitEvent(st, ctx->ev[3], 0));
+      FP4_CUDA_TRY(cudaStreamWaitEvent(st, ctx->ev[4], 0));      // the number of entries
       rc = fill_csc_beside();
       if (rc != FP4_OK) return rc;
     }
-    Arena fa(scratch_full, full_bytes);
-    rc = launch_residual_full(ctx, st, savedA->csr_rowptr, savedA->csr_col, savedA->csr_val, M, K, W_bf16, N, fa, y1, KC_COMP_FWD,
-                              status);
-    if (rc != FP4_OK) return rc;
-    GemmEpilogue epi = {};
-    epi.addend = y1;
-    epi.slot_of_row = savedA->csr_rowptr;              // every row has one: any vector of non-negative numbers
-    rc = launch_gemm_fp4(ctx, st, savedA->codes, savedW->codes_t, M, N, K, savedA->amax, savedW->amax, Y, out_f32, gemm_kind,
-                         status, &epi, a8, w8);
+    rc = launch_residual_full(ctx, st, f, true, !reuse_a && ov ? ctx->ev[3] : nullptr);
     if (rc != FP4_OK) return rc;
     if (!reuse_a && ov) FP4_CUDA_TRY(cudaStreamWaitEvent(st, ctx->ev[7], 0));  // savedA is complete on return
     return FP4_OK;
@@ -558,9 +581,20 @@ int linear_bwd_impl(fp4_ctx* ctx, cudaStream_t st, Arena arena, const void* dY_b
     FP4_CUDA_TRY(cudaStreamWaitEvent(sw, ctx->ev[5], 0));
   }
   if (scratch_full) {
+    ResidualFull f = {};
+    f.ptr = savedA->csc_colptr;
+    f.idx = savedA->csc_row;
+    f.val = savedA->csc_val;
+    f.R = K;
+    f.C = M;
+    f.dense_bf16 = dY_bf16;
+    f.N = N;
+    f.out = {nullptr, comp, 1};
+    f.kernel_class = KC_COMP_WGRAD;
+    f.status = status;
     Arena fa(scratch_full, full_bytes);
-    rc = launch_residual_full(ctx, sw, savedA->csc_colptr, savedA->csc_row, savedA->csc_val, K, M, dY_bf16, N, fa, comp,
-                              KC_COMP_WGRAD, status);
+    rc = residual_full_begin(ctx, f, fa);
+    if (rc == FP4_OK) rc = launch_residual_full(ctx, sw, f, false, nullptr);
     if (rc != FP4_OK) return rc;
     slot_of_col = savedA->csc_colptr;                  // every row has one: any vector of non-negative numbers
   } else if (has_comp) {

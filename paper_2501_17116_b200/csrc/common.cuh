@@ -288,9 +288,35 @@ constexpr int RESIDUAL_FULL_SHARE = 25;
 constexpr int64_t FULL_SLAB_BYTES = 128 << 20;       // about what L2 holds
 size_t residual_full_scratch_bytes(int64_t R, int64_t C);
 int64_t residual_full_from(const fp4_ctx* ctx, int64_t R, int64_t C, int64_t N);
-int launch_residual_full(fp4_ctx* ctx, cudaStream_t stream, const int32_t* ptr, const int32_t* idx, const float* val, int64_t R,
-                         int64_t C, const void* dense_bf16, int64_t N, Arena& scratch, float* out, int kernel_class,
-                         int32_t* status);
+// Where the product goes: y = y1 + product, rounded once, or (y1 null) the product itself in fp32.
+struct ResidualOut {
+  const float* y1;
+  void* y;
+  int f32;
+};
+struct ResidualFull {
+  const int32_t *ptr, *idx;    // CSR of V [R x C]
+  const float* val;
+  int64_t R, C;
+  const void* act_bf16;        // the matrix V was taken from, with its thresholds, where it is at hand: the operand is made of
+  const float* thresholds;     // it and does not wait for the CSR
+  int thr_per_row;
+  const void* dense_bf16;      // [C x N]
+  int64_t N;
+  ResidualOut out;
+  int kernel_class;
+  int32_t* status;
+  // set by residual_full_begin
+  int64_t slab;                // rows of V whose terms the scratch holds
+  void* vt;
+  int* third;
+  int dense_from;
+};
+int residual_full_begin(const fp4_ctx* ctx, ResidualFull& f, Arena& scratch);
+// Slab after slab, operand and product; the first slab's operand may have been made before.  An operand made of `act_bf16`
+// needs the number of entries (ptr[R]) only for the product; `entries_ready` (may be null) says when the rest is there.
+int launch_residual_operand(fp4_ctx* ctx, cudaStream_t stream, const ResidualFull& f, int64_t r0);
+int launch_residual_full(fp4_ctx* ctx, cudaStream_t stream, const ResidualFull& f, bool first_operand_ready, cudaEvent_t entries_ready);
 
 // Dense columns of the residual in the weight gradient, on the tensor cores (wgrad_dense_tc.cu):
 // C[s, :] = sum_m V[m, s] dY[m, :] for the s < counts[0] <= DENSE_TC_MAX dense columns, as `splits`

@@ -16,6 +16,23 @@ __device__ __forceinline__ void fma8(float (&acc)[8], float v, const uint4& d) {
   }
 }
 
+// eight consecutive outputs, in fp32 or rounded to BF16 once; streaming
+__device__ __forceinline__ void store8(void* out, int out_f32, long long off, const float (&y)[8]) {
+  if (out_f32) {
+    float4* dst = reinterpret_cast<float4*>(static_cast<float*>(out) + off);
+    __stcs(dst, make_float4(y[0], y[1], y[2], y[3]));
+    __stcs(dst + 1, make_float4(y[4], y[5], y[6], y[7]));
+  } else {
+    uint32_t w[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      __nv_bfloat162 h = __floats2bfloat162_rn(y[2 * q], y[2 * q + 1]);
+      w[q] = *reinterpret_cast<uint32_t*>(&h);
+    }
+    __stcs(reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(out) + off), make_uint4(w[0], w[1], w[2], w[3]));
+  }
+}
+
 // acc += n entries, gathered together
 template <int n>
 __device__ __forceinline__ void add_entries(float (&acc)[8], const int* __restrict__ idx, const float* __restrict__ val,

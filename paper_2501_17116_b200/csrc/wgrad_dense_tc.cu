@@ -107,12 +107,80 @@ dense_split_kernel(const int* __restrict__ colptr, const int* __restrict__ row, 
 }
 
 // The whole residual (or its transpose) as a dense operand, for residuals so heavy that gathering costs more:
-// row r of Vt[term][r][c] holds the terms of the residual's row r, zeros elsewhere.  A block writes one row, in
-// segments of ROW_SEG contraction indices.  Terms 1 and 2 are written always; term 3 is zero unless a value spans
-// more than 16 bits (500 times the threshold): *third says so, and a second launch (SECOND) then writes it.
+// row r of Vt[term][r][c] holds the terms of the residual's row r, zeros elsewhere.  Terms 1 and 2 are written always;
+// term 3 is zero unless a value spans more than 16 bits (500 times the threshold): *third says so, and a second launch
+// then writes it.
+//
+// dense_act_kernel writes it from the activation itself, eight elements per thread: it needs the thresholds only, so it
+// runs beside the FP4 GEMM and the CSR's chain (1920 x 5504 at alpha 0.97: both were ahead of it on the one path).
+// The number of entries is not known to it: where they turn out too few for the product its work is not used.
+struct DenseActArgs {
+  const uint4* x;              // rows row0 .. of the activation
+  long long n_vec;             // of the slab
+  int vec_per_row, row0;
+  const float* thresholds;
+  int thr_per_row;
+  uint4* vt;                   // [term][rows][C]
+  int* third;
+};
+template <bool THIRD>
+__global__ void __launch_bounds__(256)
+dense_act_kernel(const __grid_constant__ DenseActArgs a) {
+  if (THIRD && *a.third == 0) return;
+  constexpr int FLY = 4;
+  const long long i0 = (long long)blockIdx.x * (256 * FLY) + threadIdx.x;
+  uint4 v[FLY];
+#pragma unroll
+  for (int u = 0; u < FLY; ++u)
+    if (i0 + 256 * u < a.n_vec) v[u] = __ldg(&a.x[i0 + 256 * u]);
+  float lo = a.thresholds[0], hi = a.thresholds[1];
+  bool any = false;
+#pragma unroll
+  for (int u = 0; u < FLY; ++u) {
+    const long long i = i0 + 256 * u;
+    if (i >= a.n_vec) break;
+    if (a.thr_per_row) {
+      const int row = a.row0 + int(i / a.vec_per_row);
+      lo = a.thresholds[2 * row];
+      hi = a.thresholds[2 * row + 1];
+    }
+    const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+    uint32_t o1[4], o2[4], o3[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float r[2], b1[2], b2[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float x = __uint_as_float(h ? w[q] & 0xFFFF0000u : w[q] << 16);
+        r[h] = x > hi ? __fsub_rn(x, hi) : x < lo ? __fsub_rn(x, lo) : 0.0f;
+      }
+      const __nv_bfloat162 t1 = __floats2bfloat162_rn(r[0], r[1]);
+      b1[0] = __low2float(t1); b1[1] = __high2float(t1);
+      const float s0 = r[0] - b1[0], s1 = r[1] - b1[1];            // exact
+      const __nv_bfloat162 t2 = __floats2bfloat162_rn(s0, s1);
+      b2[0] = __low2float(t2); b2[1] = __high2float(t2);
+      any |= s0 != b2[0] || s1 != b2[1];
+      const __nv_bfloat162 t3 = __floats2bfloat162_rn(s0 - b2[0], s1 - b2[1]);          // exact
+      o3[q] = *reinterpret_cast<const uint32_t*>(&t3);
+      o1[q] = *reinterpret_cast<const uint32_t*>(&t1);
+      o2[q] = *reinterpret_cast<const uint32_t*>(&t2);
+    }
+    if (THIRD) {
+      a.vt[2 * a.n_vec + i] = make_uint4(o3[0], o3[1], o3[2], o3[3]);
+    } else {
+      a.vt[i] = make_uint4(o1[0], o1[1], o1[2], o1[3]);
+      a.vt[a.n_vec + i] = make_uint4(o2[0], o2[1], o2[2], o2[3]);
+    }
+  }
+  if (!THIRD && any) *a.third = 1;                             // (any number of threads writes the same)
+}
+
+// The same from the sparse form (the transpose, or an activation that was quantised by an earlier call): a block
+// writes one row, in segments of ROW_SEG contraction indices.
 // How many entries there are is known on the device only (ties at the thresholds leave fewer than alpha allows,
-// an activation of three values none): below `dense_from` of them this operand and the product are left out, and
-// the second launch adds the entries one by one instead, a warp per row and 256 outputs.
+// an activation of three values none): below `dense_from` of them the product is left out, and
+// dense_rows_kernel<true> adds the entries one by one instead, a warp per row and 256 outputs.  Its other task is the
+// third term (write_third).
 constexpr int ROW_SEG = 8192;
 struct DenseRowsArgs {
   const int* ptr;              // the whole matrix: R rows
@@ -120,11 +188,12 @@ struct DenseRowsArgs {
   const float* val;
   int R, C, row0, rows;        // the slab: rows row0 ..
   int dense_from;
+  bool write_third;
   __nv_bfloat16* vt;
   int* third;
   const uint4* dense;          // [C x N]
   int N;
-  float* out;                  // [R x N]
+  ResidualOut out;
 };
 template <bool SECOND>
 __global__ void __launch_bounds__(256, SECOND ? 5 : 6)
@@ -138,7 +207,7 @@ dense_rows_kernel(const __grid_constant__ DenseRowsArgs a) {
     if (!SECOND) return;
     // (outputs the slow index: the rows of the dense matrix that are in use at a time stay in L2)
     const int groups = a.rows >> 3, items = groups * ((a.N + 255) >> 8);
-    for (int it = blockIdx.x; it < items; it += a.rows) {
+    for (int it = blockIdx.x; it < items; it += gridDim.x) {
       const int nb = it / groups, row = a.row0 + (it - nb * groups) * 8 + (t >> 5), n0 = 256 * nb + 8 * (t & 31);
       const int vcol = n0 < a.N ? n0 >> 3 : 0, e1 = __ldg(&ptr[row + 1]);      // (every lane takes part in the walk)
       int e = __ldg(&ptr[row]);
@@ -147,46 +216,52 @@ dense_rows_kernel(const __grid_constant__ DenseRowsArgs a) {
       e += max(e1 - e, 0) & ~31;
       sparse_row_times_dense(acc, idx, val, e, e1, a.dense, a.N >> 3, vcol);
       if (n0 >= a.N) continue;
-      float4* dst = reinterpret_cast<float4*>(a.out + (long long)row * a.N + n0);
-      dst[0] = make_float4(acc[0], acc[1], acc[2], acc[3]);
-      dst[1] = make_float4(acc[4], acc[5], acc[6], acc[7]);
+      const long long off = (long long)row * a.N + n0;
+      if (a.out.y1) {
+        const float4 p = *reinterpret_cast<const float4*>(a.out.y1 + off), q = *reinterpret_cast<const float4*>(a.out.y1 + off + 4);
+        const float y1[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int c = 0; c < 8; ++c) acc[c] = y1[c] + acc[c];
+      }
+      store8(a.out.y, a.out.f32, off, acc);
     }
     return;
   }
-  if (SECOND && *a.third == 0) return;
-  const int r = blockIdx.x;
-  const int e0 = __ldg(&ptr[a.row0 + r]), e1 = __ldg(&ptr[a.row0 + r + 1]);
-  uint4* t4 = reinterpret_cast<uint4*>(&tile[0][0]);
-  bool any = false;
-  for (int c0 = 0; c0 < a.C; c0 += ROW_SEG) {
-    const int c1 = min(a.C, c0 + ROW_SEG);
-    for (int i = t; i < (SECOND ? 1 : 2) * ROW_SEG / 8; i += 256) t4[i] = make_uint4(0, 0, 0, 0);
-    __syncthreads();
-    for (int e = e0 + t; e < e1; e += 256) {
-      const int c = __ldg(&idx[e]);
-      if (c < c0 || c >= c1) continue;
-      const float v = __ldg(&val[e]);
-      const __nv_bfloat16 b1 = __float2bfloat16_rn(v);
-      const float r1 = v - __bfloat162float(b1);                 // exact
-      const __nv_bfloat16 b2 = __float2bfloat16_rn(r1);
-      const float r2 = r1 - __bfloat162float(b2);                // exact
-      if (SECOND) {
-        tile[0][c - c0] = __float2bfloat16_rn(r2);               // exact
-      } else {
-        tile[0][c - c0] = b1;
-        tile[1 - SECOND][c - c0] = b2;
-        any |= r2 != 0.0f;
+  if (SECOND && (!a.write_third || *a.third == 0)) return;
+  for (int r = blockIdx.x; r < a.rows; r += gridDim.x) {
+    const int e0 = __ldg(&ptr[a.row0 + r]), e1 = __ldg(&ptr[a.row0 + r + 1]);
+    uint4* t4 = reinterpret_cast<uint4*>(&tile[0][0]);
+    bool any = false;
+    for (int c0 = 0; c0 < a.C; c0 += ROW_SEG) {
+      const int c1 = min(a.C, c0 + ROW_SEG);
+      for (int i = t; i < (SECOND ? 1 : 2) * ROW_SEG / 8; i += 256) t4[i] = make_uint4(0, 0, 0, 0);
+      __syncthreads();
+      for (int e = e0 + t; e < e1; e += 256) {
+        const int c = __ldg(&idx[e]);
+        if (c < c0 || c >= c1) continue;
+        const float v = __ldg(&val[e]);
+        const __nv_bfloat16 b1 = __float2bfloat16_rn(v);
+        const float r1 = v - __bfloat162float(b1);                 // exact
+        const __nv_bfloat16 b2 = __float2bfloat16_rn(r1);
+        const float r2 = r1 - __bfloat162float(b2);                // exact
+        if (SECOND) {
+          tile[0][c - c0] = __float2bfloat16_rn(r2);               // exact
+        } else {
+          tile[0][c - c0] = b1;
+          tile[1 - SECOND][c - c0] = b2;
+          any |= r2 != 0.0f;
+        }
       }
-    }
-    __syncthreads();
+      __syncthreads();
 #pragma unroll
-    for (int term = 0; term < 2 - SECOND; ++term)
-      for (int i = t; i < (c1 - c0) / 8; i += 256)
-        *reinterpret_cast<uint4*>(a.vt + (size_t(SECOND ? 2 : term) * a.rows + r) * size_t(a.C) + c0 + 8 * i) =
-            *reinterpret_cast<const uint4*>(&tile[term][8 * i]);
-    __syncthreads();
+      for (int term = 0; term < 2 - SECOND; ++term)
+        for (int i = t; i < (c1 - c0) / 8; i += 256)
+          *reinterpret_cast<uint4*>(a.vt + (size_t(SECOND ? 2 : term) * a.rows + r) * size_t(a.C) + c0 + 8 * i) =
+              *reinterpret_cast<const uint4*>(&tile[term][8 * i]);
+      __syncthreads();
+    }
+    if (!SECOND && any) *a.third = 1;                // (any number of threads writes the same)
   }
-  if (!SECOND && any) *a.third = 1;                  // (any number of threads writes the same)
 }
 
 struct DenseTcArgs {
@@ -195,7 +270,8 @@ struct DenseTcArgs {
   int splits;                // ranges of chunks per tile; FULL: blocks of 128 rows
   int vt_rows;               // rows of a term of Vt
   const int* counts;         // counts[0] = number of dense columns (device); FULL: whether the third term is needed
-  float* partial;            // [splits][DENSE_TC_MAX][N]; FULL: [vt_rows][N]
+  float* partial;            // [splits][DENSE_TC_MAX][N]
+  ResidualOut out;           // FULL: rows of the slab
   const int* entries;        // FULL: number of entries (device); fewer than dense_from: nothing to do
   int dense_from;
   int32_t* status;
@@ -372,6 +448,8 @@ comp_wgrad_dense_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __g
     int acc = 0;
     uint32_t acc_phase = 0;
     bool gave_up = false;
+    // The stage goes back as soon as its last columns are in registers, ahead of their additions.  (The warps stay together
+    // from chunk to chunk: left to drift apart they take longer, 1920 x 5504 x 2048 at alpha 0.97 142 us, 146 then.)
     for (int c = 0; c < n_chunks; ++c) {
       const bool ok = mbar_wait(&acc_full[acc], acc_phase, abort_flag, args.status);
       if (epilogue_bar_any(!ok, 8 * 32)) { gave_up = true; break; }
@@ -382,23 +460,52 @@ comp_wgrad_dense_tc_kernel(const __grid_constant__ CUtensorMap map_dy, const __g
         if (c0 < 64 * nb) {
           uint32_t v[32];
           tmem_ld_32x32(t_base + uint32_t(c0), v);
-          tmem_ld_wait();
+          tmem_ld_wait(v);
+          if (c0 + 32 == DENSE_TC_MAX || c0 + 32 == 64 * nb) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&acc_empty[acc]);
+          }
 #pragma unroll
           for (int i = 0; i < 32; ++i) run[c0 + i] += __uint_as_float(v[i]);
         }
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&acc_empty[acc]);
       if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
     const int n = FULL ? n0 + 128 * h : n0 + 128 * h + 32 * quarter + lane;
     if (FULL) {
-      if (!gave_up && n < args.N) {                       // (N is a multiple of 128)
-        float4* dst = reinterpret_cast<float4*>(args.partial + size_t(s0 + 32 * quarter + lane) * size_t(args.N) + n);
+      // Every MMA has retired, so the ring is free: a warp's 32 x 128 sums go through it, a row at a time to the
+      // output (a lane's own row piece by piece touched 32 lines with every store).
+      if (!gave_up && n < args.N) {         // (N is a multiple of 128)
+        constexpr int PITCH = 128 + 4;
+        float* mine = reinterpret_cast<float*>(smem) + (warp - 2) * 32 * PITCH;
 #pragma unroll
         for (int j = 0; j < DENSE_TC_MAX / 4; ++j)
-          dst[j] = make_float4(run[4 * j], run[4 * j + 1], run[4 * j + 2], run[4 * j + 3]);
+          *reinterpret_cast<float4*>(mine + lane * PITCH + 4 * j) =
+              make_float4(run[4 * j], run[4 * j + 1], run[4 * j + 2], run[4 * j + 3]);
+        __syncwarp();
+        const long long off = (long long)(s0 + 32 * quarter) * args.N + n + 4 * lane;
+#pragma unroll
+        for (int r0 = 0; r0 < 32; r0 += 8) {
+          float4 y1[8];
+#pragma unroll
+          for (int u = 0; u < 8; ++u)
+            y1[u] = args.out.y1 ? __ldcs(reinterpret_cast<const float4*>(args.out.y1 + off + (long long)(r0 + u) * args.N))
+                                : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const float4 v = *reinterpret_cast<const float4*>(mine + (r0 + u) * PITCH + 4 * lane);
+            const float4 y = args.out.y1 ? make_float4(y1[u].x + v.x, y1[u].y + v.y, y1[u].z + v.z, y1[u].w + v.w) : v;
+            const long long o = off + (long long)(r0 + u) * args.N;
+            if (args.out.f32) {
+              *reinterpret_cast<float4*>(static_cast<float*>(args.out.y) + o) = y;
+            } else {
+              const __nv_bfloat162 p = __floats2bfloat162_rn(y.x, y.y), q = __floats2bfloat162_rn(y.z, y.w);
+              *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(args.out.y) + o) =
+                  make_uint2(*reinterpret_cast<const uint32_t*>(&p), *reinterpret_cast<const uint32_t*>(&q));
+            }
+          }
+        }
       }
     } else if (!gave_up && n < args.N) {
       float* dst = args.partial + size_t(split) * DENSE_TC_MAX * size_t(args.N) + n;
@@ -480,6 +587,7 @@ int launch_comp_wgrad_dense_tc(fp4_ctx* ctx, cudaStream_t stream, const fp4_qten
   args.vt_rows = DENSE_TC_MAX;
   args.counts = counts;
   args.partial = partial;
+  args.out = ResidualOut{nullptr, nullptr, 1};
   args.status = status;
   args.entries = nullptr;
   args.dense_from = 0;
@@ -515,52 +623,106 @@ int64_t residual_full_from(const fp4_ctx* ctx, int64_t R, int64_t C, int64_t N) 
   return (ns > 5000 ? ns - 5000 : 0) * 7500 / N + 1;
 }
 
-int launch_residual_full(fp4_ctx* ctx, cudaStream_t stream, const int32_t* ptr, const int32_t* idx, const float* val, int64_t R,
-                         int64_t C, const void* dense_bf16, int64_t N, Arena& scratch, float* out, int kernel_class,
-                         int32_t* status) {
-  const int64_t slab = full_slab_rows(R, C);
-  __nv_bfloat16* vt = scratch.take<__nv_bfloat16>(size_t(3) * size_t(slab) * size_t(C));
-  int* third = scratch.take<int>(1);
-  if (!scratch.ok) return FP4_ERR_WORKSPACE;
-  CUtensorMap map_dense, map_vt;
-  int rc = make_bf16_map(ctx, &map_dense, dense_bf16, C, N);
-  if (rc != FP4_OK) return rc;
-  FP4_CUDA_TRY(cudaFuncSetAttribute(comp_wgrad_dense_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, DT_SMEM));
-  FP4_CUDA_TRY(cudaMemsetAsync(third, 0, 4, stream));
-  KernelScope scope(ctx, stream, kernel_class, 3 * int((R + slab - 1) / slab));
+int residual_full_begin(const fp4_ctx* ctx, ResidualFull& f, Arena& scratch) {
+  f.slab = full_slab_rows(f.R, f.C);
+  f.vt = scratch.take<__nv_bfloat16>(size_t(3) * size_t(f.slab) * size_t(f.C));
+  f.third = scratch.take<int>(1);
+  f.dense_from = int(residual_full_from(ctx, f.R, f.C, f.N));     // (the caller has compared it with a bound below 2^31)
+  return scratch.ok ? FP4_OK : FP4_ERR_WORKSPACE;
+}
+
+// The slab's rows of the result, or of what is to be stored.
+static ResidualOut slab_out(const ResidualFull& f, int64_t r0) {
+  const size_t at = size_t(r0) * size_t(f.N);
+  return {f.out.y1 ? f.out.y1 + at : nullptr, static_cast<char*>(f.out.y) + at * (f.out.f32 ? 4 : 2), f.out.f32};
+}
+static DenseRowsArgs dense_rows_args(const ResidualFull& f, int64_t r0, int64_t rows) {
   DenseRowsArgs ra;
-  ra.ptr = ptr;
-  ra.idx = idx;
-  ra.val = val;
-  ra.R = int(R);
-  ra.C = int(C);
-  ra.dense_from = int(residual_full_from(ctx, R, C, N));          // (the caller has compared it with a bound below 2^31)
-  ra.vt = vt;
-  ra.third = third;
-  ra.dense = static_cast<const uint4*>(dense_bf16);
-  ra.N = int(N);
-  ra.out = out;
-  for (int64_t r0 = 0; r0 < R; r0 += slab) {
-    const int64_t rows = R - r0 < slab ? R - r0 : slab;
-    rc = make_bf16_map(ctx, &map_vt, vt, 3 * rows, C);
-    if (rc != FP4_OK) return rc;
-    ra.row0 = int(r0);
-    ra.rows = int(rows);
-    dense_rows_kernel<false><<<unsigned(rows), 256, 0, stream>>>(ra);
-    dense_rows_kernel<true><<<unsigned(rows), 256, 0, stream>>>(ra);
-    DenseTcArgs args;
-    args.M = int(C);
-    args.N = int(N);
-    args.tiles = int((N + DT_NT - 1) / DT_NT);
-    args.splits = int(rows / DENSE_TC_MAX);
-    args.vt_rows = int(rows);
-    args.counts = third;
-    args.partial = out + size_t(r0) * size_t(N);
-    args.status = status;
-    args.entries = ptr + R;
-    args.dense_from = ra.dense_from;
-    comp_wgrad_dense_tc_kernel<true><<<unsigned(args.tiles * args.splits), DT_THREADS, DT_SMEM, stream>>>(map_dense, map_vt, args);
+  ra.ptr = f.ptr;
+  ra.idx = f.idx;
+  ra.val = f.val;
+  ra.R = int(f.R);
+  ra.C = int(f.C);
+  ra.row0 = int(r0);
+  ra.rows = int(rows);
+  ra.dense_from = f.dense_from;
+  ra.write_third = !f.act_bf16;
+  ra.vt = static_cast<__nv_bfloat16*>(f.vt);
+  ra.third = f.third;
+  ra.dense = static_cast<const uint4*>(f.dense_bf16);
+  ra.N = int(f.N);
+  ra.out = f.out;
+  return ra;
+}
+
+static void launch_dense_rows_second(const fp4_ctx* ctx, cudaStream_t stream, const DenseRowsArgs& a) {
+  const int some = 5 * ctx->num_sms;                   // (idle as a rule: one wave of blocks)
+  dense_rows_kernel<true><<<unsigned(a.rows < some ? a.rows : some), 256, 0, stream>>>(a);
+}
+
+int launch_residual_operand(fp4_ctx* ctx, cudaStream_t stream, const ResidualFull& f, int64_t r0) {
+  const int64_t rows = f.R - r0 < f.slab ? f.R - r0 : f.slab;
+  if (r0 == 0) FP4_CUDA_TRY(cudaMemsetAsync(f.third, 0, 4, stream));
+  KernelScope scope(ctx, stream, f.kernel_class, 2);
+  if (f.act_bf16) {
+    DenseActArgs a;
+    a.x = static_cast<const uint4*>(f.act_bf16) + r0 * f.C / 8;
+    a.n_vec = rows * f.C / 8;
+    a.vec_per_row = int(f.C / 8);
+    a.row0 = int(r0);
+    a.thresholds = f.thresholds;
+    a.thr_per_row = f.thr_per_row;
+    a.vt = static_cast<uint4*>(f.vt);
+    a.third = f.third;
+    const unsigned blocks = unsigned((a.n_vec + 1023) / 1024);
+    dense_act_kernel<false><<<blocks, 256, 0, stream>>>(a);
+    dense_act_kernel<true><<<blocks, 256, 0, stream>>>(a);
+  } else {
+    const DenseRowsArgs a = dense_rows_args(f, r0, rows);
+    dense_rows_kernel<false><<<unsigned(rows), 256, 0, stream>>>(a);
+    launch_dense_rows_second(ctx, stream, a);
   }
+  FP4_CUDA_TRY(cudaGetLastError());
+  return FP4_OK;
+}
+
+int launch_residual_product(fp4_ctx* ctx, cudaStream_t stream, const ResidualFull& f, int64_t r0) {
+  const int64_t rows = f.R - r0 < f.slab ? f.R - r0 : f.slab;
+  CUtensorMap map_dense, map_vt;
+  int rc = make_bf16_map(ctx, &map_dense, f.dense_bf16, f.C, f.N);
+  if (rc != FP4_OK) return rc;
+  rc = make_bf16_map(ctx, &map_vt, f.vt, 3 * rows, f.C);
+  if (rc != FP4_OK) return rc;
+  KernelScope scope(ctx, stream, f.kernel_class, 1);
+  DenseTcArgs args;
+  args.M = int(f.C);
+  args.N = int(f.N);
+  args.tiles = int((f.N + DT_NT - 1) / DT_NT);
+  args.splits = int(rows / DENSE_TC_MAX);
+  args.vt_rows = int(rows);
+  args.counts = f.third;
+  args.partial = nullptr;
+  args.out = slab_out(f, r0);
+  args.status = f.status;
+  args.entries = f.ptr + f.R;
+  args.dense_from = f.dense_from;
+  FP4_CUDA_TRY(cudaFuncSetAttribute(comp_wgrad_dense_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, DT_SMEM));
+  comp_wgrad_dense_tc_kernel<true><<<unsigned(args.tiles * args.splits), DT_THREADS, DT_SMEM, stream>>>(map_dense, map_vt, args);
+  FP4_CUDA_TRY(cudaGetLastError());
+  return FP4_OK;
+}
+
+int launch_residual_full(fp4_ctx* ctx, cudaStream_t stream, const ResidualFull& f, bool first_operand_ready, cudaEvent_t entries_ready) {
+  for (int64_t r0 = 0; r0 < f.R; r0 += f.slab) {
+    int rc = r0 == 0 && first_operand_ready ? FP4_OK : launch_residual_operand(ctx, stream, f, r0);
+    if (rc == FP4_OK) rc = launch_residual_product(ctx, stream, f, r0);
+    if (rc != FP4_OK) return rc;
+  }
+  if (!f.act_bf16) return FP4_OK;
+  // The operand was made without the entries: where they are too few for the product they are added now.
+  if (entries_ready) FP4_CUDA_TRY(cudaStreamWaitEvent(stream, entries_ready, 0));
+  KernelScope scope(ctx, stream, f.kernel_class, 1);
+  launch_dense_rows_second(ctx, stream, dense_rows_args(f, 0, f.R));
   FP4_CUDA_TRY(cudaGetLastError());
   return FP4_OK;
 }
