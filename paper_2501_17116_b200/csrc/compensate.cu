@@ -140,90 +140,78 @@ struct ColumnClasses {
   int* slot_of_col;            // [K] position among the dense columns; DENSE_TC_MAX for a long or short one; -1: empty
 };
 
-__device__ __forceinline__ int block_sum_1024(int v, int* warp_tot) {
-  v = __reduce_add_sync(0xFFFFFFFFu, v);
-  __syncthreads();                                   // warp_tot may still be read from the previous sum
-  if ((threadIdx.x & 31) == 0) warp_tot[threadIdx.x >> 5] = v;
-  __syncthreads();
-  return __reduce_add_sync(0xFFFFFFFFu, warp_tot[threadIdx.x & 31]);
-}
-
-// Exclusive scan of one int per thread over a 1024-thread block.
-__device__ __forceinline__ int block_exclusive_scan_1024(int c, int* warp_tot) {
+// Exclusive counts of a flag over a block of 1024 threads: how many threads before this one have it set.  Two flags travel
+// together (low and high half of a word).
+__device__ __forceinline__ int block_rank_1024(bool f, bool g, int* warp_tot) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int incl = c;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const int up = __shfl_up_sync(0xFFFFFFFFu, incl, off);
-    if (lane >= off) incl += up;
-  }
-  __syncthreads();                                   // warp_tot may still be read from the previous scan
-  if (lane == 31) warp_tot[warp] = incl;
+  const unsigned mf = __ballot_sync(0xFFFFFFFFu, f), mg = __ballot_sync(0xFFFFFFFFu, g), below = (1u << lane) - 1u;
+  if (lane == 0) warp_tot[warp] = __popc(mf) | (__popc(mg) << 16);
   __syncthreads();
-  int before = lane < warp ? warp_tot[lane] : 0;
-  before = __reduce_add_sync(0xFFFFFFFFu, before);
-  return before + incl - c;
+  const int before = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? warp_tot[lane] : 0);     // (at most 1024 each)
+  return before + (__popc(mf & below) | (__popc(mg & below) << 16));
 }
 
 // Dense columns: the first DENSE_TC_MAX, in ascending order, that hold at least `dense_from` entries (INT_MAX:
 // none).  With ALL the others are listed too, long and short ones, in ascending order.
 // A block owns 1024 columns and counts all earlier ones itself (coalesced reads of a few KB from L2), so no
-// block waits for another: one block walking all columns in stretches took 4.5 us of 2048 and 17.5 of 11008.
+// block waits for another: one block walking all columns in stretches took 4.5 us of 2048 and 17.5 of 11008.  The
+// sums meet behind one barrier and the ranks come from ballots (a barrier or two for every sum and scan: backward of 128 x 4096 x 11008 112.6 us, 111.1 now).
 template <bool ALL>
 __global__ void __launch_bounds__(1024, 1)
 classify_columns_kernel(const int* __restrict__ colptr, int K, int dense_from, int few_max, const ColumnClasses out) {
-  __shared__ int warp_tot[32];
-  const int t = threadIdx.x, c0 = blockIdx.x * 1024;
-  int cand_b = 0, cand = 0, few = 0, few_b = 0, large = 0, large_b = 0, any = 0, any_b = 0;   // _b: before c0
-  for (int k = t; k < K; k += 1024) {
-    const int n = __ldg(&colptr[k + 1]) - __ldg(&colptr[k]);
-    const bool b = k < c0, c = n >= dense_from;
-    cand += c;
-    cand_b += c && b;
-    if (ALL) {
-      few += n >= LONG_FEW && !c;
-      few_b += n >= LONG_FEW && !c && b;
-      large += n >= LONG_COLUMN && !c;
-      large_b += n >= LONG_COLUMN && !c && b;
-      any += n > 0;
-      any_b += n > 0 && b;
+  constexpr int SUMS = ALL ? 8 : 2;
+  __shared__ int part[SUMS][32], rank_tot[2][32];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, c0 = blockIdx.x * 1024, k = c0 + t;
+  const int e0 = k < K ? __ldg(&colptr[k]) : 0, n = k < K ? __ldg(&colptr[k + 1]) - e0 : 0;
+  // candidates, columns with LONG_FEW entries and more, with LONG_COLUMN and more (both without candidates), with any:
+  // in all, and before c0
+  int sum[SUMS] = {};
+  for (int j = t; j < K; j += 1024) {
+    const int m = __ldg(&colptr[j + 1]) - __ldg(&colptr[j]);
+    const bool b = j < c0, c = m >= dense_from;
+    sum[0] += c;
+    sum[1] += c && b;
+    if constexpr (ALL) {
+      sum[2] += m >= LONG_FEW && !c;
+      sum[3] += m >= LONG_FEW && !c && b;
+      sum[4] += m >= LONG_COLUMN && !c;
+      sum[5] += m >= LONG_COLUMN && !c && b;
+      sum[6] += m > 0;
+      sum[7] += m > 0 && b;
     }
   }
-  cand = block_sum_1024(cand, warp_tot);
-  cand_b = block_sum_1024(cand_b, warp_tot);
-  const int n_dense = min(cand, DENSE_TC_MAX);
-  const int k = c0 + t;
-  const int n = k < K ? __ldg(&colptr[k + 1]) - __ldg(&colptr[k]) : 0;
+#pragma unroll
+  for (int i = 0; i < SUMS; ++i) {
+    const int v = __reduce_add_sync(0xFFFFFFFFu, sum[i]);
+    if (lane == 0) part[i][warp] = v;
+  }
   const bool is_cand = n >= dense_from;
-  const int rank = cand_b + block_exclusive_scan_1024(is_cand, warp_tot);
+  const int cand_rank = block_rank_1024(is_cand, false, rank_tot[0]);       // (its barrier is the sums' too)
+#pragma unroll
+  for (int i = 0; i < SUMS; ++i) sum[i] = __reduce_add_sync(0xFFFFFFFFu, part[i][lane]);
+  const int cand = sum[0], cand_b = sum[1], n_dense = min(cand, DENSE_TC_MAX), rank = cand_b + cand_rank;
   const bool dense = is_cand && rank < DENSE_TC_MAX;
   if (dense) out.list_dense[rank] = k;
-  if (!ALL) {
+  if constexpr (!ALL) {
     if (k < K) out.slot_of_col[k] = dense ? rank : -1;
     if (k == 0) out.counts[0] = n_dense;
-    return;
-  }
-  few = block_sum_1024(few, warp_tot);
-  const bool use_few = few <= few_max;
-  const int long_from = use_few ? LONG_FEW : LONG_COLUMN;
-  // (candidates beyond DENSE_TC_MAX hold LONG_COLUMN entries or more: they are long)
-  large = (use_few ? few : block_sum_1024(large, warp_tot)) + cand - n_dense;
-  large_b = block_sum_1024(use_few ? few_b : large_b, warp_tot) + max(0, cand_b - DENSE_TC_MAX);
-  any = block_sum_1024(any, warp_tot);
-  any_b = block_sum_1024(any_b, warp_tot);
-  const bool is_long = !dense && n >= long_from, is_short = !dense && !is_long && n > 0;
-  const int at_long = large_b + block_exclusive_scan_1024(is_long, warp_tot);
-  const int at_short = any_b - large_b - min(cand_b, DENSE_TC_MAX) + block_exclusive_scan_1024(is_short, warp_tot);
-  if (is_long) out.list_long[at_long] = k;
-  if (is_short) {
-    const int e0 = __ldg(&colptr[k]);
-    out.list_short[at_short] = make_int4(k, e0, e0 + n, 0);
-  }
-  if (k < K) out.slot_of_col[k] = dense ? rank : n > 0 ? DENSE_TC_MAX : -1;
-  if (k == 0) {
-    out.counts[0] = n_dense;
-    out.counts[1] = large;
-    out.counts[2] = any - n_dense - large;
+  } else {
+    const bool use_few = sum[2] <= few_max;
+    const int long_from = use_few ? LONG_FEW : LONG_COLUMN;
+    // (candidates beyond DENSE_TC_MAX hold LONG_COLUMN entries or more: they are long)
+    const int large = (use_few ? sum[2] : sum[4]) + cand - n_dense;
+    const int large_b = (use_few ? sum[3] : sum[5]) + max(0, cand_b - DENSE_TC_MAX);
+    const int any = sum[6], any_b = sum[7];
+    const bool is_long = !dense && n >= long_from, is_short = !dense && !is_long && n > 0;
+    const int ranks = block_rank_1024(is_long, is_short, rank_tot[1]);
+    if (is_long) out.list_long[large_b + (ranks & 0xFFFF)] = k;
+    if (is_short) out.list_short[any_b - large_b - min(cand_b, DENSE_TC_MAX) + (ranks >> 16)] = make_int4(k, e0, e0 + n, 0);
+    if (k < K) out.slot_of_col[k] = dense ? rank : n > 0 ? DENSE_TC_MAX : -1;
+    if (k == 0) {
+      out.counts[0] = n_dense;
+      out.counts[1] = large;
+      out.counts[2] = any - n_dense - large;
+    }
   }
 }
 
