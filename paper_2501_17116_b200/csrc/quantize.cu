@@ -513,12 +513,15 @@ tail_select_kernel(const __grid_constant__ SelectArgs a) {
   __syncthreads();
   if (tid < HIST_COARSE && s.coarse[tid]) atomicAdd(&gcoarse[tid], s.coarse[tid]);
   // ---- the last block to get here selects -------------------------------------------------
-  __threadfence();
+  // (one thread's fences, behind and ahead of a barrier, order the whole block's counters)
   __syncthreads();
-  if (tid == 0) s.last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
+  if (tid == 0) {
+    __threadfence();
+    s.last = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
+    __threadfence();
+  }
   __syncthreads();
   if (!s.last) return;
-  __threadfence();
   select_ranks(a, s, ghist, gcoarse, false);
   if (s.fail) {
     // The bracket missed: count the whole tensor into the cleared set, nothing left out.
