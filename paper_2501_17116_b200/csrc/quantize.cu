@@ -411,8 +411,9 @@ tail_select_kernel(const __grid_constant__ SelectArgs a) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int r_begin = int((long long)a.rows * blockIdx.x / gridDim.x);
   const int r_end = int((long long)a.rows * (blockIdx.x + 1) / gridDim.x);
+  // loads issued first, so that their latency runs under the clearing below; the parity is not looked at before the
+  // sample has been (the clearing of the global counters, which needs it, waited a microsecond for it alone)
   const unsigned par = a.parity ? (*reinterpret_cast<volatile unsigned*>(a.parity) & 1u) : 0u;
-  // loads issued first, so that their latency runs under the clearing below
   const bool sampled = a.sample_rank >= 0;
   uint2 sample = make_uint2(0, 0);
   uint4 first = make_uint4(0, 0, 0, 0);
@@ -433,16 +434,6 @@ tail_select_kernel(const __grid_constant__ SelectArgs a) {
       select_request<1>(a, warp + SEL_WARPS, units, r_begin, 1);
     }
   }
-  uint32_t* ghist = a.sets + size_t(par) * HIST_SET_WORDS;
-  uint32_t* gcoarse = ghist + 65536;
-  if (a.parity) {
-    // this block's slice of the other set, for the next call
-    uint32_t* other = a.sets + size_t(par ^ 1u) * HIST_SET_WORDS;
-    const int per = (HIST_SET_WORDS + gridDim.x - 1) / gridDim.x;
-    const int w0 = blockIdx.x * per, w1 = min(HIST_SET_WORDS, w0 + per);
-    for (int i = w0 + tid; i < w1; i += SEL_THREADS) other[i] = 0;
-  }
-  for (int i = blockIdx.x * SEL_THREADS + tid; i < a.clear_words; i += gridDim.x * SEL_THREADS) a.clear[i] = 0;
   for (int i = tid; i < 2 * SEL_WINDOW / 4; i += SEL_THREADS) reinterpret_cast<uint4*>(s.window)[i] = make_uint4(0, 0, 0, 0);
   if (tid < HIST_COARSE) s.coarse[tid] = 0;
   if (tid == 0) { s.top = 0; s.fail = 0; }
@@ -499,6 +490,16 @@ tail_select_kernel(const __grid_constant__ SelectArgs a) {
     q_bits = pos_to_bits(q_pos);
   }
   __syncthreads();
+  uint32_t* ghist = a.sets + size_t(par) * HIST_SET_WORDS;
+  uint32_t* gcoarse = ghist + 65536;
+  if (a.parity) {
+    // this block's slice of the other set, for the next call
+    uint32_t* other = a.sets + size_t(par ^ 1u) * HIST_SET_WORDS;
+    const int per = (HIST_SET_WORDS + gridDim.x - 1) / gridDim.x;
+    const int w0 = blockIdx.x * per, w1 = min(HIST_SET_WORDS, w0 + per);
+    for (int i = w0 + tid; i < w1; i += SEL_THREADS) other[i] = 0;
+  }
+  for (int i = blockIdx.x * SEL_THREADS + tid; i < a.clear_words; i += gridDim.x * SEL_THREADS) a.clear[i] = 0;
   if (tid == 0) { s.p_pos = p_pos; s.q_pos = q_pos; }
   const int e_top = min(254, int(s.top >> 7) + SEL_HEADROOM);
   const uint32_t base = uint32_t(max(0, e_top - SEL_EXPS + 1)) << 7;
