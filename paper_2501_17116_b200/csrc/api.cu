@@ -245,6 +245,7 @@ int fp4_quantize(fp4_ctx* ctx, void* stream, const void* x_bf16, int64_t rows, i
   std::memset(&key, 0, sizeof(key));
   key.kind = CALL_QUANTIZE;
   key.quantile_mode = ctx->quantile_mode;
+  key.overlap = ctx->overlap;
   key.scale_axis = scale_axis;
   key.alpha = alpha;
   key.M = rows;
@@ -255,7 +256,10 @@ int fp4_quantize(fp4_ctx* ctx, void* stream, const void* x_bf16, int64_t rows, i
   key.a = *out;
   return ctx->graphs->run(ctx, static_cast<cudaStream_t>(stream), key, [&](cudaStream_t st) {
     Arena arena(ctx->workspace, ctx->workspace_bytes);
-    return launch_quantize(ctx, st, arena, x_bf16, rows, cols, scale_axis, alpha, prescale, 0.0f, out, status);
+    // the CSC's fill beside the CSR's
+    const SparseOverlap so = {nullptr, nullptr, nullptr, ctx->side[0], ctx->ev[7], ctx->ev[4], nullptr};
+    return launch_quantize(ctx, st, arena, x_bf16, rows, cols, scale_axis, alpha, prescale, 0.0f, out, status,
+                           ctx->overlap ? &so : nullptr);
   });
 }
 

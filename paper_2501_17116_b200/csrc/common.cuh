@@ -207,7 +207,8 @@ int launch_gemm_fp4_two(fp4_ctx* ctx, cudaStream_t stream, const Fp4GemmDesc& fi
 // starts after `encoded` (recorded on the main stream); the pointers kernel and the CSR fill run on
 // `stream`, which records `colptr_done` once row and column pointers are complete and `csr_done`
 // after the CSR fill; the CSC fill runs on `stream_csc` behind `colptr_done` and records `csc_done`
-// there (null: it follows the CSR fill on `stream`).  The caller joins the streams.
+// there (null: it follows the CSR fill on `stream`).  The caller joins the streams.  Without `stream` all but the CSC fill
+// stays on the caller's stream, which waits for `csc_done` at the end.
 struct SparseOverlap {
   cudaStream_t stream;
   cudaEvent_t encoded;

@@ -1367,10 +1367,11 @@ __device__ __forceinline__ int lane_of_entry(int i, int incl) {
 
 // CSR: one warp per row, 32 mask words (1024 columns) at a time.  A round's values are stored in the next
 // round, so that their latency runs under its search.
-__device__ __forceinline__ void csr_fill(const uint32_t* __restrict__ mask, const __nv_bfloat16* __restrict__ x, int rows, int cols,
-                                         const float* __restrict__ thresholds, int thr_per_row, const int* __restrict__ rowptr,
-                                         long long cap, int* __restrict__ csr_col, float* __restrict__ csr_val, int block) {
-  const int row = block * FILL_WARPS + (threadIdx.x >> 5);
+__global__ void __launch_bounds__(32 * FILL_WARPS)
+csr_fill_kernel(const uint32_t* __restrict__ mask, const __nv_bfloat16* __restrict__ x, int rows, int cols,
+                const float* __restrict__ thresholds, int thr_per_row, const int* __restrict__ rowptr, long long cap,
+                int* __restrict__ csr_col, float* __restrict__ csr_val) {
+  const int row = blockIdx.x * FILL_WARPS + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= rows) return;
   int base = rowptr[row];
@@ -1446,12 +1447,13 @@ __device__ __forceinline__ uint32_t transpose_bits(uint32_t v) {
 
 // CSC: one warp per (64-row strip, 32-column word of the mask).  The word's two 32 x 32 blocks are
 // transposed: lane c holds the marked rows of column c.
-__device__ __forceinline__ void csc_fill(const uint32_t* __restrict__ mask, const __nv_bfloat16* __restrict__ x, int cols,
-                                         const float* __restrict__ thresholds, int thr_per_row, const int* __restrict__ colptr,
-                                         const uint8_t* __restrict__ strip_cnt, const int* __restrict__ super_cnt, long long cap,
-                                         int* __restrict__ csc_row, float* __restrict__ csc_val, int block, int strip) {
+__global__ void __launch_bounds__(32 * FILL_WARPS)
+csc_fill_kernel(const uint32_t* __restrict__ mask, const __nv_bfloat16* __restrict__ x, int rows, int cols,
+                const float* __restrict__ thresholds, int thr_per_row, const int* __restrict__ colptr,
+                const uint8_t* __restrict__ strip_cnt, const int* __restrict__ super_cnt, long long cap,
+                int* __restrict__ csc_row, float* __restrict__ csc_val) {
   const int lane = threadIdx.x & 31;
-  const int q = block * FILL_WARPS + (threadIdx.x >> 5);
+  const int q = blockIdx.x * FILL_WARPS + (threadIdx.x >> 5), strip = blockIdx.y;
   const int words_per_row = cols >> 5;
   if (q >= words_per_row) return;
   const int r0 = strip * ENC_TM;
@@ -1496,48 +1498,6 @@ __device__ __forceinline__ void csc_fill(const uint32_t* __restrict__ mask, cons
     held = x[(long long)r * cols + 32 * q + src];
   }
   put();
-}
-
-struct CsrFill {
-  const uint32_t* mask;
-  const void* x_bf16;
-  int rows, cols;
-  const float* thresholds;
-  int thr_per_row;
-  const int* rowptr;
-  long long cap;
-  int* csr_col;
-  float* csr_val;
-};
-__global__ void __launch_bounds__(32 * FILL_WARPS)
-csr_fill_kernel(const uint32_t* __restrict__ mask, const __nv_bfloat16* __restrict__ x, int rows, int cols,
-                const float* __restrict__ thresholds, int thr_per_row, const int* __restrict__ rowptr, long long cap,
-                int* __restrict__ csr_col, float* __restrict__ csr_val) {
-  csr_fill(mask, x, rows, cols, thresholds, thr_per_row, rowptr, cap, csr_col, csr_val, blockIdx.x);
-}
-__global__ void __launch_bounds__(32 * FILL_WARPS)
-csc_fill_kernel(const uint32_t* __restrict__ mask, const __nv_bfloat16* __restrict__ x, int cols,
-                const float* __restrict__ thresholds, int thr_per_row, const int* __restrict__ colptr,
-                const uint8_t* __restrict__ strip_cnt, const int* __restrict__ super_cnt, long long cap,
-                int* __restrict__ csc_row, float* __restrict__ csc_val) {
-  csc_fill(mask, x, cols, thresholds, thr_per_row, colptr, strip_cnt, super_cnt, cap, csc_row, csc_val, blockIdx.x, blockIdx.y);
-}
-__device__ __forceinline__ void csc_fill_block(const CscFill& f, int block) {
-  const int per_strip = (f.cols / 32 + FILL_WARPS - 1) / FILL_WARPS;
-  csc_fill(f.mask, static_cast<const __nv_bfloat16*>(f.x_bf16), f.cols, f.thresholds, f.thr_per_row, f.colptr, f.strip_cnt,
-           f.super_cnt, f.cap, f.csc_row, f.csc_val, block % per_strip, block / per_strip);
-}
-int csc_fill_blocks(const CscFill& f) { return (f.cols / 32 + FILL_WARPS - 1) / FILL_WARPS * (f.rows / ENC_TM); }
-// Both on one stream: either is bound by the latency of its chain (mask -> bits -> value), which the other's warps
-// cover.  8192 x 4096 at 0.1 % per tail: 19.2 us one after the other, 15.6 together; 1920 x 5504 at 3 %, clamped and
-// encoded, 53.5 -> 47.6.
-__global__ void __launch_bounds__(32 * FILL_WARPS)
-both_fills_kernel(const __grid_constant__ CsrFill r, const __grid_constant__ CscFill c, int csc_blocks) {
-  if (int(blockIdx.x) < csc_blocks)
-    csc_fill_block(c, blockIdx.x);
-  else
-    csr_fill(r.mask, static_cast<const __nv_bfloat16*>(r.x_bf16), r.rows, r.cols, r.thresholds, r.thr_per_row, r.rowptr, r.cap,
-             r.csr_col, r.csr_val, blockIdx.x - csc_blocks);
 }
 
 // At most two blocks per SM, and as few as give no block more rows than that.  Small tensors (a block
@@ -1621,7 +1581,7 @@ size_t quantize_scratch_bytes(int64_t rows, int64_t cols) {
 int launch_csc_fill(fp4_ctx* ctx, cudaStream_t stream, const CscFill& f) {
   KernelScope scope(ctx, stream, KC_SPARSE, 1);
   const dim3 grid((f.cols / 32 + FILL_WARPS - 1) / FILL_WARPS, f.rows / ENC_TM);
-  csc_fill_kernel<<<grid, 32 * FILL_WARPS, 0, stream>>>(f.mask, static_cast<const __nv_bfloat16*>(f.x_bf16), f.cols,
+  csc_fill_kernel<<<grid, 32 * FILL_WARPS, 0, stream>>>(f.mask, static_cast<const __nv_bfloat16*>(f.x_bf16), f.rows, f.cols,
                                                        f.thresholds, f.thr_per_row, f.colptr, f.strip_cnt, f.super_cnt, f.cap,
                                                        f.csc_row, f.csc_val);
   FP4_CUDA_TRY(cudaGetLastError());
@@ -1710,39 +1670,35 @@ int launch_quantize(fp4_ctx* ctx, cudaStream_t stream, Arena& arena, const void*
     }
     const uint32_t* mask32 = reinterpret_cast<const uint32_t*>(sc.mask);
     const __nv_bfloat16* xb = static_cast<const __nv_bfloat16*>(x_bf16);
-    const CsrFill csr = {mask32, x_bf16, rows, cols, out->thresholds, per_token, out->csr_rowptr, out->sparse_cap, out->csr_col,
-                         out->csr_val};
-    const CscFill csc = {mask32, x_bf16, rows, cols, out->thresholds, per_token, out->csc_colptr,
-                         sc.strip_cnt, sc.super_cnt, out->sparse_cap, out->csc_row, out->csc_val};
-    const unsigned csr_blocks = unsigned((rows + FILL_WARPS - 1) / FILL_WARPS);
-    // The CSC's fill takes a stream of its own where the caller offers one.
+    // The CSC's fill takes a stream of its own where the caller offers one: either fill is bound by the latency of its
+    // chain (mask -> bits -> value), which the other's warps cover (8192 x 4096 at 0.1 %
+    // per tail, clamped and encoded: 77.8 us one after the other, 72.0 now; as one launch of both 74).
     cudaStream_t sc2 = sp;
     {
       KernelScope scope(ctx, sp, KC_SPARSE, 2);
       sparse_prefix_kernel<<<1 + (cols + 1023) / 1024, 1024, 0, sp>>>(sc.row_cnt, rows, out->csr_rowptr, out->nnz,
                                                                     sc.col_cnt, cols, out->csc_colptr);
-      if (sp == stream) {
-        const int csc_blocks = csc_fill_blocks(csc);
-        both_fills_kernel<<<csr_blocks + unsigned(csc_blocks), 32 * FILL_WARPS, 0, stream>>>(csr, csc, csc_blocks);
-        FP4_CUDA_TRY(cudaGetLastError());
-        return FP4_OK;
-      }
-      if (overlap->colptr_done) FP4_CUDA_TRY(cudaEventRecord(overlap->colptr_done, sp));
-      if (overlap->stream_csc && overlap->colptr_done) {
+      if (overlap && overlap->colptr_done) FP4_CUDA_TRY(cudaEventRecord(overlap->colptr_done, sp));
+      if (overlap && overlap->stream_csc && overlap->colptr_done) {
         sc2 = overlap->stream_csc;
         FP4_CUDA_TRY(cudaStreamWaitEvent(sc2, overlap->colptr_done, 0));
       }
-      csr_fill_kernel<<<csr_blocks, 32 * FILL_WARPS, 0, sp>>>(mask32, xb, rows, cols, out->thresholds, per_token, out->csr_rowptr,
-                                                              out->sparse_cap, out->csr_col, out->csr_val);
+      csr_fill_kernel<<<(rows + FILL_WARPS - 1) / FILL_WARPS, 32 * FILL_WARPS, 0, sp>>>(mask32, xb, rows, cols, out->thresholds, per_token, out->csr_rowptr,
+                                                      out->sparse_cap, out->csr_col, out->csr_val);
     }
-    FP4_CUDA_TRY(cudaEventRecord(overlap->csr_done, sp));
-    if (overlap->later) {
-      *overlap->later = csc;
+    if (sp != stream) FP4_CUDA_TRY(cudaEventRecord(overlap->csr_done, sp));
+    const CscFill fill = {mask32, x_bf16, rows, cols, out->thresholds, per_token, out->csc_colptr,
+                          sc.strip_cnt, sc.super_cnt, out->sparse_cap, out->csc_row, out->csc_val};
+    if (sp != stream && overlap->later) {
+      *overlap->later = fill;
       return FP4_OK;
     }
-    const int rc = launch_csc_fill(ctx, sc2, csc);
+    const int rc = launch_csc_fill(ctx, sc2, fill);
     if (rc != FP4_OK) return rc;
-    if (overlap->csc_done) FP4_CUDA_TRY(cudaEventRecord(overlap->csc_done, sc2));
+    if (sc2 != stream && overlap->csc_done) {
+      FP4_CUDA_TRY(cudaEventRecord(overlap->csc_done, sc2));
+      if (sp == stream) FP4_CUDA_TRY(cudaStreamWaitEvent(stream, overlap->csc_done, 0));   // nobody else waits for it
+    }
   } else {
     if (prescale && prescale_div > 0.0f) {
       float* d = scale_axis == 0 ? sc.pre_cols : sc.pre_rows;
