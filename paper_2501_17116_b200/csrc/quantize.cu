@@ -50,6 +50,11 @@ __device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
+__device__ __forceinline__ f32x2 add2_rm(f32x2 a, f32x2 b) {      // toward -infinity
+  f32x2 r;
+  asm("add.rm.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
 __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
   f32x2 r;
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
@@ -884,16 +889,19 @@ absmax_strip_kernel(const AbsmaxArgs a) {
 // Q of Appendix A for eight float32 values -> eight nibbles (element 0 in bits 3:0).
 // The chain sends a value that equals a threshold to the larger neighbour, i.e. it rounds to the
 // nearest grid value with ties toward +infinity.  The hardware conversion rounds ties to even, so
-// each input is first moved off the tie: its magnitude bits become (bits - sign) | 1.  Thresholds
-// have a zero last bit, so no other value crosses one.  The conversion's "-0" nibble is cleared.
-__device__ __forceinline__ float nudge(float v) {
-  const uint32_t u = __float_as_uint(v);
-  return __uint_as_float((u + uint32_t(int(u) >> 31)) | 1u);
-}
-// (ADD: the clearing in three instructions instead of seven.  The encoder of both axes, which the ALUs bound, takes it: 16384 x
-// 5120 absmax and codes 145 -> 143.6 us with two GEMMs; the clamping one is slower with it, 8192 x 5120 79.0 -> 80.3.)
-template <bool ADD>
-__device__ __forceinline__ uint32_t encode8(const float (&v)[8]) {
+// each input is first moved off the tie, to the inside of its cell of width 1/8: thresholds are multiples of 1/4, and a
+// value belongs to the cell it is the lower end of.  Added to TIE_C with rounding toward -infinity it becomes the cell's
+// lower end w (units of 1/8 are the last place there); w + TIE_C times 1 - 2^-24, minus TIE_C - 1/8, is w + 1/32 less
+// w 2^-24.  Two instructions for two values, where nudging the bit patterns took four on the unit that bounds the
+// encoders (8192 x 5120 clamped and encoded 78.8 -> 76.7 us, 8192 x 4096 71.4 -> 69.8; backward of 4096 x 2048 x 5504
+// 111.0 -> 109.1).  The conversion's "-0" nibble is cleared: a nibble's magnitude + 7 reaches bit 3 where it is not zero,
+// and never the next nibble.
+constexpr float TIE_C = 1572864.0f;                    // 1.5 * 2^20
+__device__ __forceinline__ uint32_t encode8(const f32x2 (&v)[4]) {
+  const f32x2 up = pack2(TIE_C, TIE_C), scale = pack2(0x0.FFFFFFp0f, 0x0.FFFFFFp0f), down = pack2(0.125f - TIE_C, 0.125f - TIE_C);
+  float f[8];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) unpack2(fma2(add2_rm(v[q], up), scale, down), f[2 * q], f[2 * q + 1]);
   uint32_t w;
   asm("{\n\t.reg .b8 b0, b1, b2, b3;\n\t"
       "cvt.rn.satfinite.e2m1x2.f32 b0, %2, %1;\n\t"
@@ -902,13 +910,8 @@ __device__ __forceinline__ uint32_t encode8(const float (&v)[8]) {
       "cvt.rn.satfinite.e2m1x2.f32 b3, %8, %7;\n\t"
       "mov.b32 %0, {b0, b1, b2, b3};\n\t}"
       : "=r"(w)
-      : "f"(nudge(v[0])), "f"(nudge(v[1])), "f"(nudge(v[2])), "f"(nudge(v[3])), "f"(nudge(v[4])),
-        "f"(nudge(v[5])), "f"(nudge(v[6])), "f"(nudge(v[7])));
-  // a nibble's magnitude + 7 reaches bit 3 where it is not zero, and never the next nibble
-  if (ADD) return w & (((w & 0x77777777u) + 0x77777777u) | 0x77777777u);
-  const uint32_t m = w & 0x77777777u;
-  const uint32_t nz = (m | (m >> 1) | (m >> 2)) & 0x11111111u;   // 1 where the magnitude is not zero
-  return w & ((nz << 3) | 0x77777777u);
+      : "f"(f[0]), "f"(f[1]), "f"(f[2]), "f"(f[3]), "f"(f[4]), "f"(f[5]), "f"(f[6]), "f"(f[7]));
+  return w & (((w & 0x77777777u) + 0x77777777u) | 0x77777777u);
 }
 
 // 8 x 8 nibble transpose: in[r] nibble c  ->  out[c] nibble r
@@ -1060,7 +1063,7 @@ encode_kernel(const EncodeArgs a) {
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
     const uint32_t w[4] = {v[r].x, v[r].y, v[r].z, v[r].w};
-    float f[8], f2[8];
+    f32x2 f[4], f2[4];
     uint32_t obits = 0;
     const float grow1 = ROW_SCALED ? s_grow[8 * warp + r] : 0.0f;
     const float prow1 = (COL_SCALED && PRESCALE) ? s_prow[8 * warp + r] : 1.0f;
@@ -1080,19 +1083,18 @@ encode_kernel(const EncodeArgs a) {
         x = *reinterpret_cast<const uint32_t*>(&xc);
       }
       const f32x2 xv = pack2(bf16_lo(x), bf16_hi(x));
-      // "+ 0" turns a -0 product into +0 (the nudge needs a non-negative zero)
       if constexpr (MODE == MODE_ROWS) {
-        unpack2(fma2(PRESCALE ? mul2(xv, pc[q]) : xv, grow, 0ull), f[2 * q], f[2 * q + 1]);
+        f[q] = mul2(PRESCALE ? mul2(xv, pc[q]) : xv, grow);
       } else if constexpr (MODE == MODE_COLS) {
-        unpack2(fma2(PRESCALE ? mul2(xv, prow) : xv, gc[q], 0ull), f[2 * q], f[2 * q + 1]);
+        f[q] = mul2(PRESCALE ? mul2(xv, prow) : xv, gc[q]);
       } else {
-        unpack2(fma2(mul2(xv, pc[q]), grow, 0ull), f[2 * q], f[2 * q + 1]);
-        unpack2(fma2(mul2(xv, prow), gc[q], 0ull), f2[2 * q], f2[2 * q + 1]);
+        f[q] = mul2(mul2(xv, pc[q]), grow);
+        f2[q] = mul2(mul2(xv, prow), gc[q]);
       }
     }
     if (OCC) obits = in_cols ? (obits | (obits >> 16)) & 0xFFu : 0u;   // beyond the tensor: its zeros may lie outside [lo, hi]
-    word[r] = encode8<MODE == MODE_DUAL>(f);
-    if constexpr (MODE == MODE_DUAL) word_t[r] = encode8<true>(f2);
+    word[r] = encode8(f);
+    if constexpr (MODE == MODE_DUAL) word_t[r] = encode8(f2);
     if (in_cols) {
       const long long o = (long long)(row0 + 8 * warp + r) * vec_per_row + (col >> 3);
       if (a.codes) a.codes[o] = word[r];
