@@ -1153,13 +1153,21 @@ encode_kernel(const EncodeArgs a) {
 // ------------------------------------------------------------------------------------------
 // Two floats -> two FP8 bytes (first value in the low byte), E4M3 or E5M2: nearest even, saturating
 // at the format's largest finite value (448 / 57344), the sign kept also on zero.
-__device__ __forceinline__ uint32_t fp8x2(float lo, float hi, int e5m2) {
+template <bool E5M2>
+__device__ __forceinline__ uint32_t fp8x2(f32x2 v) {
+  float lo, hi;
+  unpack2(v, lo, hi);
   uint16_t r;
-  if (e5m2)
+  if (E5M2)
     asm("cvt.rn.satfinite.e5m2x2.f32 %0, %1, %2;" : "=h"(r) : "f"(hi), "f"(lo));
   else
     asm("cvt.rn.satfinite.e4m3x2.f32 %0, %1, %2;" : "=h"(r) : "f"(hi), "f"(lo));
   return r;
+}
+// eight values -> eight bytes
+template <bool E5M2>
+__device__ __forceinline__ uint2 fp8x8(const f32x2 (&v)[4]) {
+  return make_uint2(fp8x2<E5M2>(v[0]) | (fp8x2<E5M2>(v[1]) << 16), fp8x2<E5M2>(v[2]) | (fp8x2<E5M2>(v[3]) << 16));
 }
 // 4 x 4 byte transpose: in[r] byte c -> out[c] byte r
 __device__ __forceinline__ void transpose4x4_bytes(uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t (&c)[4]) {
@@ -1174,8 +1182,11 @@ __device__ __forceinline__ void transpose4x4_bytes(uint32_t a0, uint32_t a1, uin
 // Same tile and thread mapping as encode_kernel, one byte per element: `codes` [rows x cols] bytes
 // (row-scaled in dual mode), `codes_t` [cols x rows] bytes (column-scaled in dual mode).  No
 // clamping: outlier clamping belongs to 4-bit activations.
-template <int MODE, bool PRESCALE>
-__global__ void __launch_bounds__(ENC_THREADS)
+// (Values in pairs and the format known when compiled: backward of 4096 x 2048 x 2048 with dY in E5M2 51.5 -> 49.5 us.  Columns'
+// tiles ahead of their scales: 5120 x 13824, absmax and codes, 88 -> 84.  Rows keep five blocks per SM: with four 8192 x 13824
+// took 131 us instead of 128.)
+template <int MODE, bool PRESCALE, bool E5M2>
+__global__ void __launch_bounds__(ENC_THREADS, MODE == MODE_DUAL ? 3 : MODE == MODE_ROWS && !PRESCALE ? 5 : 4)
 encode_fp8_kernel(const EncodeArgs a) {
   __shared__ __align__(16) float s_gcol[ENC_TK];
   __shared__ float s_grow[ENC_TM];
@@ -1189,6 +1200,14 @@ encode_fp8_kernel(const EncodeArgs a) {
   const int vec_per_row = a.cols >> 3;
   constexpr bool ROW_SCALED = MODE != MODE_COLS;
   constexpr bool COL_SCALED = MODE != MODE_ROWS;
+  uint4 v[8];
+  if (MODE == MODE_COLS) {                            // the tile is requested ahead of the scales (see the encoder)
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      v[r] = make_uint4(0, 0, 0, 0);
+      if (col0 + 8 * lane < a.cols) v[r] = load_now(&a.x[(long long)(row0 + 8 * warp + r) * vec_per_row + (col0 >> 3) + lane]);
+    }
+  }
   if (ROW_SCALED && tid < ENC_TM) {
     const int r = row0 + tid;
     const float amax = __uint_as_float(a.amax_rows[r]);
@@ -1208,52 +1227,49 @@ encode_fp8_kernel(const EncodeArgs a) {
 
   const int col = col0 + 8 * lane;
   const bool in_cols = col < a.cols;
-  uint4 v[8];
+  if (MODE != MODE_COLS) {
 #pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    v[r] = make_uint4(0, 0, 0, 0);
-    if (in_cols) v[r] = __ldg(&a.x[(long long)(row0 + 8 * warp + r) * vec_per_row + (col >> 3)]);
+    for (int r = 0; r < 8; ++r) {
+      v[r] = make_uint4(0, 0, 0, 0);
+      if (in_cols) v[r] = __ldg(&a.x[(long long)(row0 + 8 * warp + r) * vec_per_row + (col >> 3)]);
+    }
   }
-  float gc[8], pc[8];
-  if (COL_SCALED) {
+  f32x2 gc[4], pc[4];
 #pragma unroll
-    for (int c = 0; c < 8; ++c) gc[c] = in_cols ? s_gcol[8 * lane + c] : 0.0f;
-  }
-  if (ROW_SCALED && PRESCALE) {
-#pragma unroll
-    for (int c = 0; c < 8; ++c) pc[c] = in_cols ? __ldg(&a.pre_col[col + c]) : 0.0f;
+  for (int q = 0; q < 4; ++q) {
+    if (COL_SCALED) gc[q] = in_cols ? *reinterpret_cast<const f32x2*>(&s_gcol[8 * lane + 2 * q]) : 0ull;
+    if (ROW_SCALED && PRESCALE) {
+      const int c = in_cols ? col + 2 * q : 0;
+      const float2 p = make_float2(__ldg(&a.pre_col[c]), __ldg(&a.pre_col[c + 1]));
+      pc[q] = in_cols ? pack2(p.x, p.y) : 0ull;
+    }
   }
   uint32_t lo4[8], hi4[8];                            // bytes of columns 0..3 / 4..7 of each row (output for codes_t)
   uint8_t* codes8 = reinterpret_cast<uint8_t*>(a.codes);
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
     const uint32_t w[4] = {v[r].x, v[r].y, v[r].z, v[r].w};
-    float f[8], f2[8];
-    const float grow = ROW_SCALED ? s_grow[8 * warp + r] : 0.0f;
-    const float prow = (COL_SCALED && PRESCALE) ? s_prow[8 * warp + r] : 1.0f;
+    f32x2 f[4], f2[4];
+    const float grow1 = ROW_SCALED ? s_grow[8 * warp + r] : 0.0f;
+    const float prow1 = (COL_SCALED && PRESCALE) ? s_prow[8 * warp + r] : 1.0f;
+    const f32x2 grow = pack2(grow1, grow1), prow = pack2(prow1, prow1);
 #pragma unroll
-    for (int c = 0; c < 8; ++c) {
-      const float xv = (c & 1) ? bf16_hi(w[c >> 1]) : bf16_lo(w[c >> 1]);
+    for (int q = 0; q < 4; ++q) {
+      const f32x2 xv = pack2(bf16_lo(w[q]), bf16_hi(w[q]));
       if constexpr (MODE == MODE_ROWS) {
-        f[c] = __fmul_rn(PRESCALE ? __fmul_rn(xv, pc[c]) : xv, grow);
+        f[q] = mul2(PRESCALE ? mul2(xv, pc[q]) : xv, grow);
       } else if constexpr (MODE == MODE_COLS) {
-        f[c] = __fmul_rn(PRESCALE ? __fmul_rn(xv, prow) : xv, gc[c]);
+        f[q] = mul2(PRESCALE ? mul2(xv, prow) : xv, gc[q]);
       } else {
-        f[c] = __fmul_rn(__fmul_rn(xv, pc[c]), grow);
-        f2[c] = __fmul_rn(__fmul_rn(xv, prow), gc[c]);
+        f[q] = mul2(mul2(xv, pc[q]), grow);
+        f2[q] = mul2(mul2(xv, prow), gc[q]);
       }
     }
-    const uint32_t b_lo = fp8x2(f[0], f[1], a.e5m2) | (fp8x2(f[2], f[3], a.e5m2) << 16);
-    const uint32_t b_hi = fp8x2(f[4], f[5], a.e5m2) | (fp8x2(f[6], f[7], a.e5m2) << 16);
-    if (in_cols && codes8)
-      *reinterpret_cast<uint2*>(codes8 + (long long)(row0 + 8 * warp + r) * a.cols + col) = make_uint2(b_lo, b_hi);
-    if constexpr (MODE == MODE_DUAL) {
-      lo4[r] = fp8x2(f2[0], f2[1], a.e5m2) | (fp8x2(f2[2], f2[3], a.e5m2) << 16);
-      hi4[r] = fp8x2(f2[4], f2[5], a.e5m2) | (fp8x2(f2[6], f2[7], a.e5m2) << 16);
-    } else {
-      lo4[r] = b_lo;
-      hi4[r] = b_hi;
-    }
+    const uint2 bytes = fp8x8<E5M2>(f);
+    if (in_cols && codes8) *reinterpret_cast<uint2*>(codes8 + (long long)(row0 + 8 * warp + r) * a.cols + col) = bytes;
+    const uint2 bytes_t = MODE == MODE_DUAL ? fp8x8<E5M2>(f2) : bytes;
+    lo4[r] = bytes_t.x;
+    hi4[r] = bytes_t.y;
   }
   if (a.codes_t) {
     // 8 x 8 byte transpose in registers: column c of this thread's block as the bytes of rows 0..7
@@ -1281,6 +1297,14 @@ encode_fp8_kernel(const EncodeArgs a) {
       for (int h = 0; h < 4; ++h) dst[h] = make_uint4(o[2 * h].x, o[2 * h].y, o[2 * h + 1].x, o[2 * h + 1].y);
     }
   }
+}
+
+template <int MODE, bool PRESCALE>
+void launch_encode_fp8(dim3 grid, cudaStream_t stream, const EncodeArgs& a) {
+  if (a.e5m2)
+    encode_fp8_kernel<MODE, PRESCALE, true><<<grid, ENC_THREADS, 0, stream>>>(a);
+  else
+    encode_fp8_kernel<MODE, PRESCALE, false><<<grid, ENC_THREADS, 0, stream>>>(a);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1752,9 +1776,9 @@ int launch_quantize(fp4_ctx* ctx, cudaStream_t stream, Arena& arena, const void*
       }
       KernelScope scope(ctx, stream, KC_ENCODE, 1);
       if (e4m3 && prescale)
-        encode_fp8_kernel<MODE_ROWS, true><<<tile_grid, ENC_THREADS, 0, stream>>>(ea);
+        launch_encode_fp8<MODE_ROWS, true>(tile_grid, stream, ea);
       else if (e4m3)
-        encode_fp8_kernel<MODE_ROWS, false><<<tile_grid, ENC_THREADS, 0, stream>>>(ea);
+        launch_encode_fp8<MODE_ROWS, false>(tile_grid, stream, ea);
       else if (prescale)
         encode_kernel<MODE_ROWS, false, true><<<tile_grid, ENC_THREADS, 0, stream>>>(ea);
       else
@@ -1772,9 +1796,9 @@ int launch_quantize(fp4_ctx* ctx, cudaStream_t stream, Arena& arena, const void*
       }
       KernelScope scope(ctx, stream, KC_ENCODE, 1);
       if (e4m3 && prescale)
-        encode_fp8_kernel<MODE_COLS, true><<<tile_grid, ENC_THREADS, 0, stream>>>(ea);
+        launch_encode_fp8<MODE_COLS, true>(tile_grid, stream, ea);
       else if (e4m3)
-        encode_fp8_kernel<MODE_COLS, false><<<tile_grid, ENC_THREADS, 0, stream>>>(ea);
+        launch_encode_fp8<MODE_COLS, false>(tile_grid, stream, ea);
       else if (prescale)
         encode_kernel<MODE_COLS, false, true><<<tile_grid, ENC_THREADS, 0, stream>>>(ea);
       else
@@ -1833,7 +1857,7 @@ int launch_quantize_dual(fp4_ctx* ctx, cudaStream_t stream, Arena& arena, const 
   ea.fmax = fp8_max(format);
   KernelScope scope(ctx, stream, KC_ENCODE, 1);
   if (e4m3)
-    encode_fp8_kernel<MODE_DUAL, true><<<tile_grid, ENC_THREADS, 0, stream>>>(ea);
+    launch_encode_fp8<MODE_DUAL, true>(tile_grid, stream, ea);
   else
     encode_kernel<MODE_DUAL, false, true><<<tile_grid, ENC_THREADS, 0, stream>>>(ea);
   FP4_CUDA_TRY(cudaGetLastError());
