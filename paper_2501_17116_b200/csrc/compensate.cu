@@ -397,6 +397,7 @@ comp_wgrad_long_kernel(float* __restrict__ comp, const int* __restrict__ colptr,
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n_long = counts[1], n_blocks = (N + COMP_COLS - 1) / COMP_COLS;
   const int clusters = gridDim.x / LONG_CLUSTER, rank = int(cluster.block_rank());
+  bool read = true;                                 // the sums of the item before have been read by all four blocks
   for (int it = blockIdx.x / LONG_CLUSTER; it < n_long * n_blocks; it += clusters) {
     const int nb = it / n_long, k = list[it - nb * n_long];
     const int n0 = nb * COMP_COLS + 8 * lane;
@@ -404,6 +405,7 @@ comp_wgrad_long_kernel(float* __restrict__ comp, const int* __restrict__ colptr,
     if (n0 < N)
       strided_entries_times_dense(acc, row, val, colptr[k] + rank * LONG_WARPS + warp, colptr[k + 1], LONG_CLUSTER * LONG_WARPS,
                                   dy, N >> 3, n0 >> 3);
+    if (!read) cluster.barrier_wait();
 #pragma unroll
     for (int c = 0; c < 8; ++c) part[warp][lane][c] = acc[c];
     cluster.sync();
@@ -424,8 +426,10 @@ comp_wgrad_long_kernel(float* __restrict__ comp, const int* __restrict__ colptr,
         for (int w = 0; w < LONG_WARPS; ++w) t += p[r][w];
       comp[(long long)k * N + nb * COMP_COLS + o] = t;
     }
-    cluster.sync();                                 // the sums have been read
+    cluster.barrier_arrive();                       // (waited for behind the next item's gathers: backward of 512 x 4096 x 4096 107.2 -> 106.0 us)
+    read = false;
   }
+  if (!read) cluster.barrier_wait();
 }
 
 // Short columns: one warp per (column, 256 outputs), entries in order.  The work items (block of 256
