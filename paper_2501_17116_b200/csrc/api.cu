@@ -469,14 +469,13 @@ int linear_fwd_impl(fp4_ctx* ctx, cudaStream_t st, Arena arena, const void* A_bf
   const void* kept = nullptr;
   const int* kept_end = nullptr;
   if (tail_on) {
-    // The tail's operands need the CSR, the CSC's column pointers and W's amax: the CSR chain and
-    // the first half of the CSC chain are joined before the GEMM here; the CSC's fill runs beside it.
-    if (!reuse_a && ov) {
-      FP4_CUDA_TRY(cudaStreamWaitEvent(st, ctx->ev[3], 0));
-      FP4_CUDA_TRY(cudaStreamWaitEvent(st, ctx->ev[4], 0));
-    }
+    // The tail's operands need the CSC's column pointers and W's amax (hot columns and W's operand, made beside the CSR's
+    // fill) and the CSR (A's); the CSC's fill runs beside the GEMM.
+    const bool beside = !reuse_a && ov;
+    if (beside) FP4_CUDA_TRY(cudaStreamWaitEvent(st, ctx->ev[4], 0));
     Arena ta(scratch_tail, fwd_tail_scratch_bytes(M, K, N));
-    rc = launch_fwd_tail(ctx, st, savedA, W_bf16, savedW->amax, fp8_max(w8), ta, M, K, N, &tail, &kept, &kept_end);
+    rc = launch_fwd_tail(ctx, st, beside ? ctx->ev[3] : nullptr, savedA, W_bf16, savedW->amax, fp8_max(w8), ta, M, K, N, &tail,
+                         &kept, &kept_end);
     if (rc != FP4_OK) return rc;
     if (!reuse_a && ov) {
       rc = fill_csc_beside();

@@ -262,8 +262,8 @@ int launch_comp_fwd(fp4_ctx* ctx, cudaStream_t stream, const float* y1, const in
 // The forward GEMM's dense tail (see GemmTail): operands built from the saved activation and the weights.
 size_t fwd_tail_scratch_bytes(int64_t M, int64_t K, int64_t N);
 // `kept_out` / `kept_end_out`: per token, the entries the tail does not cover.
-int launch_fwd_tail(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, const void* w_bf16, const float* w_amax,
-                    float w_div, Arena& scratch, int64_t M, int64_t K, int64_t N, GemmTail* tail,
+int launch_fwd_tail(fp4_ctx* ctx, cudaStream_t stream, cudaEvent_t csr_done, const fp4_qtensor* a, const void* w_bf16,
+                    const float* w_amax, float w_div, Arena& scratch, int64_t M, int64_t K, int64_t N, GemmTail* tail,
                     const void** kept_out, const int** kept_end_out);
 // Weight-gradient compensation: for every column k of the residual that holds entries (slot_of_col[k] >= 0),
 // comp[k, :] = sum_{entries of column k} val * dy[row, :]; the other rows of `comp` are not written.

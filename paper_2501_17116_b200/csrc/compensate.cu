@@ -560,8 +560,10 @@ size_t fwd_tail_scratch_bytes(int64_t M, int64_t K, int64_t N) {
 // Prepares the dense tail of the forward GEMM from the saved activation `a` (CSR, CSC column
 // pointers, row amax) and the weights; fills `tail` and hands back the list
 // for the per-entry kernel.  Buffers come from `scratch` (fwd_tail_scratch_bytes).
-int launch_fwd_tail(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, const void* w_bf16, const float* w_amax,
-                    float w_div, Arena& scratch, int64_t M, int64_t K, int64_t N, GemmTail* tail,
+// The hot columns and W's operand hang on the column pointers alone: they are made before the stream waits for the CSR
+// (`csr_done`, may be null), beside its fill on another stream.
+int launch_fwd_tail(fp4_ctx* ctx, cudaStream_t stream, cudaEvent_t csr_done, const fp4_qtensor* a, const void* w_bf16,
+                    const float* w_amax, float w_div, Arena& scratch, int64_t M, int64_t K, int64_t N, GemmTail* tail,
                     const void** kept_out, const int** kept_end_out) {
   __half* ta = scratch.take<__half>(size_t(M) * TAIL_WIDTH);
   __half* tb = scratch.take<__half>(size_t(N) * TAIL_WIDTH);
@@ -574,14 +576,15 @@ int launch_fwd_tail(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, con
   *kept_out = kept;
   *kept_end_out = kept_end;
   const int hot_from = int(M / 4 > LONG_COLUMN ? M / 4 : LONG_COLUMN);
-  KernelScope scope(ctx, stream, KC_COMP_FWD, 3);
   const ColumnClasses classes = {list_hot, nullptr, nullptr, count, slot_of_col};
+  KernelScope scope(ctx, stream, KC_COMP_FWD, 3);
   classify_columns_kernel<false><<<unsigned((K + 1023) / 1024), 1024, 0, stream>>>(a->csc_colptr, int(K), hot_from, 0, classes);
+  tail_b_kernel<<<dim3(unsigned(N / TAIL_B_ROWS), TAIL_MAX_COLS / 64), 256, 0, stream>>>(
+      static_cast<const __nv_bfloat16*>(w_bf16), list_hot, count, w_amax, w_div, tb, int(N));
+  if (csr_done) FP4_CUDA_TRY(cudaStreamWaitEvent(stream, csr_done, 0));
   tail_a_kernel<<<unsigned((M + 7) / 8), COMP_THREADS, 0, stream>>>(a->csr_rowptr, a->csr_col, a->csr_val, slot_of_col,
                                                                    count, a->amax, 6.0f, ta, int(M), kept,
                                                                    int(kept_list_capacity(M, K)), kept_end);
-  tail_b_kernel<<<dim3(unsigned(N / TAIL_B_ROWS), TAIL_MAX_COLS / 64), 256, 0, stream>>>(static_cast<const __nv_bfloat16*>(w_bf16),
-                                                                        list_hot, count, w_amax, w_div, tb, int(N));
   FP4_CUDA_TRY(cudaGetLastError());
   tail->a = ta;
   tail->b = tb;
