@@ -616,12 +616,19 @@ int launch_comp_wgrad(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, c
   const int few_max = int(LONG_FEW_ROUNDS * unsigned(ctx->num_sms) / n_blocks);
   classify_columns_kernel<true><<<unsigned((K + 1023) / 1024), 1024, 0, stream>>>(a->csc_colptr, int(K), dense_from, few_max, classes);
   const uint4* dy = static_cast<const uint4*>(dy_bf16);
-  // The long columns (a few blocks, latency) run beside the others.
-  cudaStream_t sl = stream;
+  // The long columns (a few blocks, latency) run beside the others, and beside the dense columns' chain of three launches the
+  // short ones: at a thousand tokens each of these is a few microseconds of latency (backward of 1024 x 2048 x 2048 at alpha
+  // 0.995 40.0 -> 37.5 us, 2048 x 11008 x 1024 94.2 -> 86.6).  At LONG_COLUMN tokens no column is dense unless every token
+  // hits it: the hot ones are long, and the short ones beside them cost more (512 x 4096 x 4096 107 -> 111).
+  cudaStream_t sl = stream, ss = stream;
   if (overlap) {
     sl = overlap->stream;
     FP4_CUDA_TRY(cudaEventRecord(overlap->classified, stream));
     FP4_CUDA_TRY(cudaStreamWaitEvent(sl, overlap->classified, 0));
+    if (dense && M > LONG_COLUMN) {
+      ss = overlap->stream_short;
+      FP4_CUDA_TRY(cudaStreamWaitEvent(ss, overlap->classified, 0));
+    }
   }
   if (dense) {
     const int rc = launch_comp_wgrad_dense_tc(ctx, stream, a, classes.list_dense, classes.counts, dy_bf16, vt, partial, splits,
@@ -639,8 +646,12 @@ int launch_comp_wgrad(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, c
     const long long max_items = (long long)((K + 7) / 8) * n_blocks;
     long long g = 32LL * ctx->num_sms;
     g = g > max_items ? max_items : g;
-    comp_wgrad_short_kernel<<<unsigned(g), COMP_THREADS, 0, stream>>>(comp, a->csc_row, a->csc_val, dy, classes.list_short,
+    comp_wgrad_short_kernel<<<unsigned(g), COMP_THREADS, 0, ss>>>(comp, a->csc_row, a->csc_val, dy, classes.list_short,
                                                                      classes.counts, int(N));
+  }
+  if (ss != stream) {
+    FP4_CUDA_TRY(cudaEventRecord(overlap->short_done, ss));
+    FP4_CUDA_TRY(cudaStreamWaitEvent(stream, overlap->short_done, 0));
   }
   if (sl != stream) {
     FP4_CUDA_TRY(cudaEventRecord(overlap->long_done, sl));
