@@ -557,6 +557,38 @@ def test_residual_with_fewer_entries_than_alpha_allows(lib, M, K, N, kind):
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
 
 
+@pytest.mark.parametrize("mode", ["FP4_QUANTILE_SIGNED", "FP4_QUANTILE_ABS", "FP4_QUANTILE_TOKEN"])
+@pytest.mark.parametrize("M,K,N,wide", [(640, 1280, 1152, False), (1408, 16384, 2176, True)])
+def test_heavy_operand_from_the_activation_and_from_the_entries(lib, M, K, N, wide, mode):
+    """The forward product's operand is made from the activation, with an activation quantised before from its entries
+    (the second size: several slabs, three terms): the same Y, on side streams and on one."""
+    gen = torch.Generator("cuda").manual_seed(K)
+    A = torch.randn((M, K), device="cuda", generator=gen)
+    if wide:
+        A *= torch.where(torch.rand((M, K), device="cuda", generator=gen) < 0.001, 3000.0, 1.0)
+    A = A.to(torch.bfloat16)
+    W = (torch.randn((K, N), device="cuda", generator=gen) * 0.02).to(torch.bfloat16)
+    ctx = lib.Context.for_shape(M, K, N)
+    ctx.set_quantile_mode(getattr(lib.binding, mode))
+    y, sa, sw = lib.fp4_linear_fwd(ctx, A, W, 0.95)
+    reused, _, _ = lib.fp4_linear_fwd(ctx, A, W, 0.95, saved_a=sa, saved_w=sw, reuse_a=True, reuse_w=True)
+    alone = lib.fp4_quantize(ctx, A, 0, alpha=0.95)
+    ctx.set_overlap(False)
+    serial, ss, _ = lib.fp4_linear_fwd(ctx, A, W, 0.95)
+    serial_alone = lib.fp4_quantize(ctx, A, 0, alpha=0.95)
+    torch.cuda.synchronize()
+    assert ctx.read_status() == 0 and int(sa.nnz) > 0.04 * M * K
+    assert torch.equal(y, reused) and torch.equal(y, serial)
+    n = int(sa.nnz)
+    for q in (alone, ss, serial_alone):
+        assert int(q.nnz) == n and torch.equal(q.codes, sa.codes) and torch.equal(q.codes_t, sa.codes_t)
+        for name in ("csr_rowptr", "csc_colptr"):
+            assert torch.equal(getattr(q, name), getattr(sa, name))
+        for name in ("csr_col", "csr_val", "csc_row", "csc_val"):
+            assert torch.equal(getattr(q, name)[:n], getattr(sa, name)[:n])
+    ctx.close()
+
+
 @pytest.mark.parametrize("M,K,N", [(2048, 512, 2048), (8192, 512, 1024), (1920, 5504, 2048)])
 def test_dense_product_of_a_heavy_residual_is_no_less_precise_than_its_gathers(lib, M, K, N):
     """Laplace activations with outliers in single elements: no hot column, every entry is one fused multiply-add in
