@@ -989,9 +989,12 @@ encode_kernel(const EncodeArgs a) {
   constexpr bool ROW_SCALED = MODE != MODE_COLS;      // a row-scaled output exists
   constexpr bool COL_SCALED = MODE != MODE_ROWS;
   uint4 v[8];
-  if (MODE == MODE_COLS) {
-    // The tile is requested ahead of the column scales, so that one latency runs under the other (5120 x 13824, absmax and
-    // codes, 65.8 -> 63.9 us; the other modes have more scales to hold beside it: both axes 145 -> 149).
+  // The tile is requested ahead of the scales, so that one latency runs under the other: by columns (5120 x 13824, absmax and
+  // codes, 65.8 -> 63.9 us) and with the clamp, whose scales come out of three reads and two minima (quantising 16384 x 13824
+  // 300 -> 294, smaller tensors as before).  Rows without the clamp wait for one read only and run slower (4096 x 512 x 5504
+  // forward 29.3 -> 29.8); both axes have more scales to hold beside the tile (145 -> 149).
+  constexpr bool TILE_FIRST = MODE == MODE_COLS || OCC;
+  if (TILE_FIRST) {
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
       v[r] = make_uint4(0, 0, 0, 0);
@@ -1037,7 +1040,7 @@ encode_kernel(const EncodeArgs a) {
 
   const int col = col0 + 8 * lane;                   // first of this thread's 8 columns
   const bool in_cols = col < a.cols;                 // ragged last tile in the column direction
-  if (MODE != MODE_COLS) {
+  if (!TILE_FIRST) {
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
       v[r] = make_uint4(0, 0, 0, 0);
