@@ -663,7 +663,7 @@ static void launch_dense_rows_second(const fp4_ctx* ctx, cudaStream_t stream, co
 int launch_residual_operand(fp4_ctx* ctx, cudaStream_t stream, const ResidualFull& f, int64_t r0) {
   const int64_t rows = f.R - r0 < f.slab ? f.R - r0 : f.slab;
   if (r0 == 0) FP4_CUDA_TRY(cudaMemsetAsync(f.third, 0, 4, stream));
-  KernelScope scope(ctx, stream, f.kernel_class, 2);
+  KernelScope scope(ctx, stream, f.kernel_class, f.act_bf16 ? 2 : 1);
   if (f.act_bf16) {
     DenseActArgs a;
     a.x = static_cast<const uint4*>(f.act_bf16) + r0 * f.C / 8;
@@ -678,9 +678,7 @@ int launch_residual_operand(fp4_ctx* ctx, cudaStream_t stream, const ResidualFul
     dense_act_kernel<false><<<blocks, 256, 0, stream>>>(a);
     dense_act_kernel<true><<<blocks, 256, 0, stream>>>(a);
   } else {
-    const DenseRowsArgs a = dense_rows_args(f, r0, rows);
-    dense_rows_kernel<false><<<unsigned(rows), 256, 0, stream>>>(a);
-    launch_dense_rows_second(ctx, stream, a);
+    dense_rows_kernel<false><<<unsigned(rows), 256, 0, stream>>>(dense_rows_args(f, r0, rows));
   }
   FP4_CUDA_TRY(cudaGetLastError());
   return FP4_OK;
@@ -715,7 +713,14 @@ int launch_residual_product(fp4_ctx* ctx, cudaStream_t stream, const ResidualFul
 int launch_residual_full(fp4_ctx* ctx, cudaStream_t stream, const ResidualFull& f, bool first_operand_ready, cudaEvent_t entries_ready) {
   for (int64_t r0 = 0; r0 < f.R; r0 += f.slab) {
     int rc = r0 == 0 && first_operand_ready ? FP4_OK : launch_residual_operand(ctx, stream, f, r0);
-    if (rc == FP4_OK) rc = launch_residual_product(ctx, stream, f, r0);
+    if (rc != FP4_OK) return rc;
+    if (!f.act_bf16) {
+      // The third term, or where the entries are too few for the product their sums: these read Y1 and store Y, so
+      // this launch stands behind whatever makes Y1, not with the first slab's operand.
+      KernelScope scope(ctx, stream, f.kernel_class, 1);
+      launch_dense_rows_second(ctx, stream, dense_rows_args(f, r0, f.R - r0 < f.slab ? f.R - r0 : f.slab));
+    }
+    rc = launch_residual_product(ctx, stream, f, r0);
     if (rc != FP4_OK) return rc;
   }
   if (!f.act_bf16) return FP4_OK;

@@ -557,6 +557,33 @@ def test_residual_with_fewer_entries_than_alpha_allows(lib, M, K, N, kind):
     assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
 
 
+@pytest.mark.parametrize("M,K,N,alpha", [(1024, 1280, 2176, 0.95), (1920, 5504, 2048, 0.97),
+                                         (1408, 16384, 2176, 0.95)])      # (the last: two slabs of rows)
+@pytest.mark.parametrize("kind", ["three values", "rectified"])
+def test_reused_activation_with_few_entries_and_another_weight(lib, M, K, N, alpha, kind):
+    """An activation whose ties leave none or half of the entries alpha allows, too few for the dense product, quantised
+    with one weight and reused with a second (q, then k and v): the bits of the same call without reuse, on one stream and
+    on side streams.  The call before leaves the first weight's sums in the workspace."""
+    gen = torch.Generator("cuda").manual_seed(M + K)
+    A = torch.randn((M, K), device="cuda", generator=gen)
+    A = (A.round().clamp(-1, 1) if kind == "three values" else A.relu()).to(torch.bfloat16)
+    W, W2 = ((torch.randn((K, N), device="cuda", generator=gen) * 0.02).to(torch.bfloat16) for _ in range(2))
+    size = int(lib.load_library().fp4_workspace_bytes(M, K, N))
+    ctx, tight = lib.Context(0, size), lib.Context(0, size - 256)
+    took = [launches(c, lambda: lib.fp4_linear_fwd(c, A, W2, alpha, out_f32=True)) for c in (ctx, tight)]
+    (want, _, _), per_entry = took[0][0], took[1][0][0]
+    assert took[0][1] != took[1][1]                                    # the dense form's launches, used or not
+    for overlap in (False, True):
+        ctx.set_overlap(overlap)
+        _, sa, _ = lib.fp4_linear_fwd(ctx, A, W, alpha, out_f32=True)
+        got, _, _ = lib.fp4_linear_fwd(ctx, A, W2, alpha, saved_a=sa, reuse_a=True, out_f32=True)
+        torch.cuda.synchronize()
+        assert ctx.read_status() == 0 and int(sa.nnz) <= (0 if kind == "three values" else (1 - alpha) * M * K + 1)
+        assert torch.equal(got, want) and torch.equal(got, per_entry), f"overlap {overlap}"
+    ctx.close()
+    tight.close()
+
+
 @pytest.mark.parametrize("mode", ["FP4_QUANTILE_SIGNED", "FP4_QUANTILE_ABS", "FP4_QUANTILE_TOKEN"])
 @pytest.mark.parametrize("M,K,N,wide", [(640, 1280, 1152, False), (1408, 16384, 2176, True)])
 def test_heavy_operand_from_the_activation_and_from_the_entries(lib, M, K, N, wide, mode):
