@@ -448,6 +448,7 @@ int linear_fwd_impl(fp4_ctx* ctx, cudaStream_t st, Arena arena, const void* A_bf
     if (ov) {
       FP4_CUDA_TRY(cudaEventRecord(ctx->ev[5], st));
       FP4_CUDA_TRY(cudaStreamWaitEvent(so, ctx->ev[5], 0));
+      if (!reuse_a) FP4_CUDA_TRY(cudaStreamWaitEvent(so, ctx->ev[4], 0));      // the number of entries
     }
     rc = launch_residual_operand(ctx, so, f, 0);
     if (rc != FP4_OK) return rc;
@@ -457,7 +458,6 @@ int linear_fwd_impl(fp4_ctx* ctx, cudaStream_t st, Arena arena, const void* A_bf
     if (rc != FP4_OK) return rc;
     if (ov) FP4_CUDA_TRY(cudaStreamWaitEvent(st, ctx->ev[6], 0));
     if (!reuse_a && ov) {
-      FP4_CUDA_TRY(cudaStreamWaitEvent(st, ctx->ev[4], 0));      // the number of entries
       rc = fill_csc_beside();
       if (rc != FP4_OK) return rc;
     }

@@ -316,9 +316,9 @@ struct ResidualFull {
 };
 int residual_full_begin(const fp4_ctx* ctx, ResidualFull& f, Arena& scratch);
 // Slab after slab, operand and product.  The operand of the first slab may have been made before, ahead of Y1 even: it reads
-// V, the thresholds and the number of entries only.  launch_residual_full, which also adds the entries one by one where they
-// are too few for the product, stands behind Y1.  An operand made of `act_bf16` needs the number of entries (ptr[R]) only for
-// the product; `entries_ready` (may be null) says when the rest is there.
+// V or `act_bf16` with the thresholds, and the number of entries (ptr[R]; too few for the product: nothing is made).
+// launch_residual_full, which then adds the entries one by one, stands behind Y1.  With `act_bf16` the entries themselves are
+// needed only there: `entries_ready` (may be null) says when they are complete.
 int launch_residual_operand(fp4_ctx* ctx, cudaStream_t stream, const ResidualFull& f, int64_t r0);
 int launch_residual_full(fp4_ctx* ctx, cudaStream_t stream, const ResidualFull& f, bool first_operand_ready, cudaEvent_t entries_ready);
 

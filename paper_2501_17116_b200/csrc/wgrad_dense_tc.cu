@@ -111,9 +111,9 @@ dense_split_kernel(const int* __restrict__ colptr, const int* __restrict__ row, 
 // term 3 is zero unless a value spans more than 16 bits (500 times the threshold): *third says so, and a second launch
 // then writes it.
 //
-// dense_act_kernel writes it from the activation itself, eight elements per thread: it needs the thresholds only, so it
-// runs beside the FP4 GEMM and the CSR's chain (1920 x 5504 at alpha 0.97: both were ahead of it on the one path).
-// The number of entries is not known to it: where they turn out too few for the product its work is not used.
+// dense_act_kernel writes it from the activation itself, eight elements per thread: it needs the thresholds and the number
+// of entries, so it runs beside the FP4 GEMM and the CSR's fill (1920 x 5504 at alpha 0.97: both were ahead of it on the one
+// path).  Where the entries are too few for the product it does nothing.
 struct DenseActArgs {
   const uint4* x;              // rows row0 .. of the activation
   long long n_vec;             // of the slab
@@ -122,11 +122,13 @@ struct DenseActArgs {
   int thr_per_row;
   uint4* vt;                   // [term][rows][C]
   int* third;
+  const int* entries;          // number of entries (device); fewer than dense_from: nothing to do
+  int dense_from;
 };
 template <bool THIRD>
 __global__ void __launch_bounds__(256)
 dense_act_kernel(const __grid_constant__ DenseActArgs a) {
-  if (THIRD && *a.third == 0) return;
+  if (*a.entries < a.dense_from || (THIRD && *a.third == 0)) return;
   constexpr int FLY = 4;
   const long long i0 = (long long)blockIdx.x * (256 * FLY) + threadIdx.x;
   uint4 v[FLY];
@@ -655,9 +657,13 @@ static DenseRowsArgs dense_rows_args(const ResidualFull& f, int64_t r0, int64_t 
   return ra;
 }
 
+// Idle as a rule: at most four waves of blocks, which calls whose product runs do not show (1920 x 5504 x 2048 at alpha 0.97
+// 149.5 us with one wave, 146 with four, runs 18 apart).  With one wave the gathers' last round was half empty: 3 % of entries
+// there 110 us, 92 with a block per item.
 static void launch_dense_rows_second(const fp4_ctx* ctx, cudaStream_t stream, const DenseRowsArgs& a) {
-  const int some = 5 * ctx->num_sms;                   // (idle as a rule: one wave of blocks)
-  dense_rows_kernel<true><<<unsigned(a.rows < some ? a.rows : some), 256, 0, stream>>>(a);
+  const int64_t items = int64_t(a.rows / 8) * ((a.N + 255) / 256), some = 4 * 5 * ctx->num_sms;
+  const int64_t blocks = items > a.rows ? items : a.rows;
+  dense_rows_kernel<true><<<unsigned(blocks < some ? blocks : some), 256, 0, stream>>>(a);
 }
 
 int launch_residual_operand(fp4_ctx* ctx, cudaStream_t stream, const ResidualFull& f, int64_t r0) {
@@ -674,6 +680,8 @@ int launch_residual_operand(fp4_ctx* ctx, cudaStream_t stream, const ResidualFul
     a.thr_per_row = f.thr_per_row;
     a.vt = static_cast<uint4*>(f.vt);
     a.third = f.third;
+    a.entries = f.ptr + f.R;
+    a.dense_from = f.dense_from;
     const unsigned blocks = unsigned((a.n_vec + 1023) / 1024);
     dense_act_kernel<false><<<blocks, 256, 0, stream>>>(a);
     dense_act_kernel<true><<<blocks, 256, 0, stream>>>(a);
