@@ -288,7 +288,7 @@ constexpr int TAIL_B_ROWS = 64, TAIL_B_PITCH = 192 + 2;      // (halves; an odd 
 __global__ void __launch_bounds__(256)
 tail_b_kernel(const __nv_bfloat16* __restrict__ w, const int* __restrict__ list_hot, const int* __restrict__ count,
               const float* __restrict__ amax_col, float col_div, __half* __restrict__ tb, int N) {
-  __shared__ __half tile[TAIL_B_ROWS * TAIL_B_PITCH];
+  __shared__ __align__(16) __half tile[TAIL_B_ROWS * TAIL_B_PITCH];           // (read by words)
   const int hot = *count, s0 = 64 * blockIdx.y, n0 = TAIL_B_ROWS * blockIdx.x;
   if (s0 >= hot) return;
   const int warp = threadIdx.x >> 5, n = 2 * (threadIdx.x & 31);             // rows n0 + n and the next one
