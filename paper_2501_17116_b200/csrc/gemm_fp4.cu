@@ -494,6 +494,13 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
       }
+      // The even CTA's commits arrive on the empty barriers of both: a CTA of a pair leaves when the arrivals for its last
+      // fills have come, which nobody else waits for.  (They come with the last MMAs, ahead of the last epilogue: no time.)
+      if (PAIR)
+        for (int s = 0; s < STAGES && ok; ++s) {
+          ok = mbar_wait(&empty_bar[stage], phase ^ 1u, abort_flag, args.status, args.wait_limit_ns);
+          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+        }
       if (!ok && PAIR) {
         // Gave up: the peer's copies complete on the even CTA's barriers too, so the copies in flight are given time to land.
         const uint64_t t0 = global_timer_ns();

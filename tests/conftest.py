@@ -20,6 +20,32 @@ def golden_lines(name):
         return [ln.strip() for ln in f if ln.strip() and not ln.lstrip().startswith("#")]
 
 
+def pair_launches(call):
+    """How many of the kernels that `call` launches run as pairs of CTAs (clusters of two asked for at the launch), from a
+    capture of the call; nothing is executed."""
+    import ctypes
+    import torch
+    graph, stream = torch.cuda.CUDAGraph(keep_graph=True), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        graph.capture_begin()
+        call()
+        graph.capture_end()
+    cuda = ctypes.CDLL("libcuda.so.1")
+    handle, n = ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t(0)
+    assert cuda.cuGraphGetNodes(handle, None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert cuda.cuGraphGetNodes(handle, nodes, ctypes.byref(n)) == 0
+    pairs = 0
+    for node in nodes:
+        kind, dims = ctypes.c_int(), (ctypes.c_uint * 16)()                # CUlaunchAttributeValue: 64 bytes
+        assert cuda.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        if kind.value == 0:                                                # a kernel; attribute 4: its cluster's size
+            assert cuda.cuGraphKernelNodeGetAttribute(ctypes.c_void_p(node), 4, dims) == 0
+            pairs += tuple(dims[:3]) == (2, 1, 1)
+    return pairs
+
+
 @pytest.fixture(scope="session")
 def lib():
     """The CUDA library through its Python binding; fails loudly if it is not built."""

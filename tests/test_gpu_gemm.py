@@ -3,6 +3,7 @@ import numpy as np
 import pytest
 import torch
 
+from conftest import pair_launches
 from oracle import fp4_oracle as O
 
 pytestmark = pytest.mark.gpu
@@ -79,6 +80,7 @@ def test_pairs_of_ctas(lib, ctx, kind, shape, f32):
     assert torch.equal(got, want)
     c = lib.Context(0, 1 << 20)
     a, b = torch.from_numpy(O.pack_nibbles(ca)).cuda(), torch.from_numpy(O.pack_nibbles(cb)).cuda()
+    assert pair_launches(lambda: lib.fp4_gemm(c, a, b, gemm_kind=kind, out_f32=f32, out=got)) == 1
     c.debug_set(lib.binding.FP4_DEBUG_WAIT_LIMIT_US, 1000)
     c.debug_set(lib.binding.FP4_DEBUG_SKIP_FILL, 7)
     lib.fp4_gemm(c, a, b, gemm_kind=kind, out_f32=f32)
@@ -106,6 +108,7 @@ def test_both_gradients_by_pairs_of_ctas(lib):
     c = lib.Context.for_shape(M, K, N)
     _, sa, sw = lib.fp4_linear_fwd(c, A, W, 1.0)
     dA, dW = lib.fp4_linear_bwd(c, dY, W, sa, sw)
+    assert pair_launches(lambda: lib.fp4_linear_bwd(c, dY, W, sa, sw, dA=torch.empty_like(dA), dW=torch.empty_like(dW))) == 1
     for k0 in (0, K - 256):
         As, Ws = A[:, k0:k0 + 256].contiguous(), W[k0:k0 + 256].contiguous()
         _, sas, sws = lib.fp4_linear_fwd(c, As, Ws, 1.0)
@@ -116,6 +119,87 @@ def test_both_gradients_by_pairs_of_ctas(lib):
         dAs, _ = lib.fp4_linear_bwd(c, dY[m0:m0 + 256].contiguous(), W, sas, sw)
         assert torch.equal(dA[m0:m0 + 256], dAs)
     assert c.read_status() == 0
+    c.close()
+
+
+@pytest.mark.parametrize("a_fmt,b_fmt", [("e4m3", "e2m1"), ("e2m1", "e4m3"), ("e4m3", "e5m2"), ("e5m2", "e4m3")])
+@pytest.mark.parametrize("shape", [(4224, 4096, 4224), (3200, 2944, 6144)])
+def test_pairs_of_ctas_with_fp8_operands(lib, ctx, a_fmt, b_fmt, shape):
+    """FP8 bytes in a pair: both CTAs' copies count in bytes read, which differ by the operands' formats; an odd number of row
+    blocks and a ragged last tile.  The products are exact, an instruction adds 32 of them into the fp32 accumulator and
+    cuts the sum off: each is off by at most 2^-23 of the summed magnitudes."""
+    I, J, C = shape
+    g = torch.Generator(device="cuda").manual_seed(I + len(a_fmt + b_fmt))
+    types = {"e4m3": torch.float8_e4m3fn, "e5m2": torch.float8_e5m2}
+    val = torch.tensor([0, .5, 1, 1.5, 2, 3, 4, 6, 0, -.5, -1, -1.5, -2, -3, -4, -6], dtype=torch.float64, device="cuda")
+
+    def operand(rows, fmt):
+        if fmt == "e2m1":
+            c = torch.randint(0, 256, (rows, C // 2), dtype=torch.uint8, device="cuda", generator=g)
+            return c, torch.stack([val[(c & 15).long()], val[(c >> 4).long()]], -1).flatten(1)
+        q = torch.randn((rows, C), device="cuda", generator=g).to(types[fmt])
+        return q.view(torch.uint8), q.double()
+
+    (a, va), (b, vb) = operand(I, a_fmt), operand(J, b_fmt)
+    kind = {(True, False): lib.FP4_GEMM_F8F6F4_A8, (False, True): lib.FP4_GEMM_F8F6F4_B8, (True, True): lib.FP4_GEMM_F8F6F4_A8B8}[
+        (a_fmt != "e2m1", b_fmt != "e2m1")]
+    kind |= (lib.binding.FP4_GEMM_A_E5M2 if a_fmt == "e5m2" else 0) | (lib.binding.FP4_GEMM_B_E5M2 if b_fmt == "e5m2" else 0)
+    out = torch.full((I, J), float("nan"), device="cuda")
+    assert pair_launches(lambda: lib.fp4_gemm(ctx, a, b, gemm_kind=kind, out=out)) == 1
+    ctx.status.zero_()
+    lib.fp4_gemm(ctx, a, b, gemm_kind=kind, out=out)
+    torch.cuda.synchronize()
+    assert ctx.read_status() == 0
+    err, mag = (out.double() - va @ vb.T).abs(), va.abs() @ vb.abs().T
+    assert bool((err <= C / 32 * 2.0 ** -23 * mag).all())
+
+
+@pytest.mark.parametrize("hot", [0, 100])
+def test_pairs_of_ctas_with_a_residual(lib, hot):
+    """Pairs with the rows of the weight gradient's compensation and (hot columns) with the forward's dense tail, 63 and 25 row
+    blocks: against the codes' products in float64.  The residual's part may differ by the 4e-6 of its summed magnitudes
+    that the tensor cores' additions are allowed, or by those of an fp32 sum entry by entry, its entries times 2^-24; the
+    two branches are fp32 numbers, four of whose roundings are allowed on top.  The tail is added to the FP4 branch's
+    accumulators: 6 blocks of 4 instructions, each of which cuts at most 2^-23 off the running sum."""
+    M, K, N, alpha = 8064, 3200, 4096, 0.995
+    g = torch.Generator(device="cuda").manual_seed(hot)
+    A = torch.randn((M, K), device="cuda", generator=g)
+    A[:, :32 * hot:32] *= 20.0
+    A, W = A.bfloat16(), (torch.randn((K, N), device="cuda", generator=g) * 0.02).bfloat16()
+    dY = (torch.randn((M, N), device="cuda", generator=g) * 1e-3).bfloat16()
+    c = lib.Context.for_shape(M, K, N)
+    y, sa, sw = lib.fp4_linear_fwd(c, A, W, alpha, out_f32=True)
+    dA, dW = lib.fp4_linear_bwd(c, dY, W, sa, sw, out_f32=True, dge_on=False)
+    again = [torch.empty_like(t) for t in (y, dA, dW)]
+    assert pair_launches(lambda: lib.fp4_linear_fwd(c, A, W, alpha, sa, sw, out=again[0], out_f32=True)) == 1
+    assert pair_launches(lambda: lib.fp4_linear_bwd(c, dY, W, sa, sw, out_f32=True, dge_on=False, dA=again[1], dW=again[2])) == 1
+    six = torch.tensor(6.0, device="cuda")
+    g1 = lib.fp4_quantize(c, dY, 0, prescale=sw.amax / six, codes_t=False)
+    g2 = lib.fp4_quantize(c, dY, 1, prescale=sa.amax / six, codes=False)
+    torch.cuda.synchronize()
+    assert c.read_status() == 0
+    hits = sa.csc_colptr.diff()
+    assert int((hits >= M // 4).sum()) == hot                                   # the columns of the dense forms
+    val = torch.tensor([0, .5, 1, 1.5, 2, 3, 4, 6, 0, -.5, -1, -1.5, -2, -3, -4, -6], dtype=torch.float64, device="cuda")
+    dec = lambda c: torch.stack([val[(c & 15).long()], val[(c >> 4).long()]], -1).flatten(1)        # noqa: E731
+    lo, hi = sa.thresholds.double().tolist()
+    res = A.double() - A.double().clamp(lo, hi)
+
+    def check(got, codes, vectors, residual, dense, entries, cuts=0):
+        fp4 = dec(codes[0]) @ dec(codes[1]).T
+        for v in vectors:
+            fp4 *= v
+        comp = residual @ dense if residual is not None else torch.zeros_like(fp4)
+        allow = 4 * 2.0 ** -24 * (fp4.abs() + comp.abs()) + cuts * 2.0 ** -23 * fp4.abs()
+        if residual is not None:
+            allow += torch.maximum(torch.full_like(entries, 4e-6), (entries + 4) * 2.0 ** -24) * (residual.abs() @ dense.abs())
+        assert bool(((got.double() - fp4 - comp).abs() <= allow).all())
+
+    d_a, d_w, d_1, d_2 = ((q.amax / six).double() for q in (sa, sw, g1, g2))
+    check(y, (sa.codes, sw.codes_t), (d_a[:, None], d_w), res, W.double(), sa.csr_rowptr.diff().double()[:, None],
+          cuts=24 if hot else 0)
+    check(dA, (g1.codes, sw.codes), (d_1[:, None],), None, None, None)
+    check(dW, (sa.codes_t, g2.codes_t), (d_2,), res.T, dY.double(), hits.double()[:, None])
     c.close()
 
 
