@@ -812,7 +812,7 @@ struct TileWidths {
   bool pair;
 };
 struct TileCost {
-  long long tiles;
+  int tiles;                   // (32 bits: the search divides by the thousand, 10.5 us of a backward call in 64, 6.4 so)
   int steady, alone;           // time per tile in a row of tiles; what the last one adds
 };
 TileCost tile_cost(const Fp4GemmDesc& d, int gemm_kind, bool pair, int bn) {
@@ -822,7 +822,7 @@ TileCost tile_cost(const Fp4GemmDesc& d, int gemm_kind, bool pair, int bn) {
                        : 800 + kbs * ((gemm_kind == FP4_GEMM_F8F6F4 ? 130 : 170) + (17 * bn) / 20);
   const bool dge = d.epilogue && d.epilogue->w_bf16;
   const int epi = (dge ? 500 + 40 * bn : (d.out_f32 ? 12 : 10) * bn) + (pair ? 900 : 0);
-  return {((d.I + rows - 1) / rows) * ((d.J + bn - 1) / bn), mma > epi ? mma : epi, mma > epi ? epi : mma};
+  return {int(((d.I + rows - 1) / rows) * ((d.J + bn - 1) / bn)), mma > epi ? mma : epi, mma > epi ? epi : mma};
 }
 TileWidths choose_widths(const fp4_ctx* ctx, const Fp4GemmDesc& p, const Fp4GemmDesc* q, int gemm_kind) {
   constexpr int LEAST = 32, WIDTHS = 15;
@@ -831,7 +831,7 @@ TileWidths choose_widths(const fp4_ctx* ctx, const Fp4GemmDesc& p, const Fp4Gemm
   TileWidths best = {most, most, false};
   long long best_cost = -1;
   for (const bool pair : {false, true}) {
-    const long long G = pair ? ctx->num_sms / 2 : ctx->num_sms;
+    const int G = pair ? ctx->num_sms / 2 : ctx->num_sms;
     if (!G) continue;
     TileCost costs[2][WIDTHS];
     int n = 0;
@@ -843,12 +843,12 @@ TileWidths choose_widths(const fp4_ctx* ctx, const Fp4GemmDesc& p, const Fp4Gemm
       for (int j = 0; j < (q ? n : 1); ++j) {
         const TileCost &c = costs[0][i], &d = costs[1][j];
         // worker r takes tiles r, r + G, ...: the counts change at r = tiles mod G of the first problem and of both
-        const long long all = c.tiles + d.tiles;
-        const long long at[3] = {0, c.tiles % G, all % G};
+        const int all = c.tiles + d.tiles;
+        const int at[3] = {0, c.tiles % G, all % G};
         long long cost = 0;
-        for (const long long r : at) {
-          const long long n1 = (c.tiles - r + G - 1) / G, n2 = (all - r + G - 1) / G - n1;
-          const long long t = n1 * c.steady + n2 * d.steady + (n2 ? d.alone : n1 ? c.alone : 0);
+        for (const int r : at) {
+          const int n1 = (c.tiles - r + G - 1) / G, n2 = (all - r + G - 1) / G - n1;
+          const long long t = (long long)n1 * c.steady + (long long)n2 * d.steady + (n2 ? d.alone : n1 ? c.alone : 0);
           if (t > cost) cost = t;
         }
         if (pair) cost += q ? 2000 : 1000;
