@@ -66,6 +66,18 @@ bool full_product_fits(const Arena& whole, int64_t M, int64_t K, int64_t N) {
   return whole.size >= least_workspace_bytes(M, K, N) + full_scratch_bytes(M, K);
 }
 
+// Whether work of `st` may be put on `side`: a stream that has joined a capture takes work of that capture alone until it ends
+// (any other would be an error, and end the capture as well).
+bool side_is_free(cudaStream_t st, cudaStream_t side) {
+  cudaStreamCaptureStatus status, mine;
+  unsigned long long id = 0, my_id = 0;
+  bool ok = cudaStreamGetCaptureInfo(side, &status, &id) == cudaSuccess;
+  if (ok && status == cudaStreamCaptureStatusNone) return true;
+  ok = ok && status == cudaStreamCaptureStatusActive && cudaStreamGetCaptureInfo(st, &mine, &my_id) == cudaSuccess;
+  if (!ok) cudaGetLastError();                       // the legacy stream while another stream is captured
+  return ok && mine == cudaStreamCaptureStatusActive && my_id == id;
+}
+
 int check_qtensor_dense(const fp4_qtensor* q) {
   if (!q || !q->amax) return FP4_ERR_NULL;
   if (!q->codes && !q->codes_t) return FP4_ERR_NULL;
@@ -256,10 +268,10 @@ int fp4_quantize(fp4_ctx* ctx, void* stream, const void* x_bf16, int64_t rows, i
   key.a = *out;
   return ctx->graphs->run(ctx, static_cast<cudaStream_t>(stream), key, [&](cudaStream_t st) {
     Arena arena(ctx->workspace, ctx->workspace_bytes);
-    // the CSC's fill beside the CSR's
+    // the CSC's fill beside the CSR's, unless a call that is being captured from another stream holds the side stream
     const SparseOverlap so = {nullptr, nullptr, nullptr, ctx->side[0], ctx->ev[7], ctx->ev[4], nullptr};
     return launch_quantize(ctx, st, arena, x_bf16, rows, cols, scale_axis, alpha, prescale, 0.0f, out, status,
-                           ctx->overlap ? &so : nullptr);
+                           ctx->overlap && side_is_free(st, so.stream_csc) ? &so : nullptr);
   });
 }
 

@@ -75,3 +75,53 @@ def test_replays_of_a_captured_step_equal_plain_launches(lib, M, K, N1, N2, alph
     graph.replay()
     check(want2, "replay after plain launches")
     ctx.close()
+
+
+@pytest.mark.parametrize("first", ["quantise", "forward"])
+def test_clamping_on_another_stream_while_a_call_is_captured(lib, first):
+    """Between the capture of a call and its end the same context quantises, with the clamp, on a stream that is not captured,
+    and into a second capture: none of them disturbs another."""
+    M, K, N, alpha = 256, 384, 256, 0.99
+    a_bits, w_bits, _ = WL.small_case(M, K, N, seed=51)
+    b_bits, _, _ = WL.small_case(M, K, N, seed=52)
+    A, B, W = _dev(a_bits), _dev(b_bits), _dev(w_bits)
+    cap = lib.tail_capacity(M, K, alpha)
+    qa, qb, qc = (lib.QTensor(M, K, 0, A.device, cap) for _ in range(3))
+    sw, y = lib.QTensor(K, N, 1, A.device), torch.empty((M, N), dtype=torch.bfloat16, device="cuda")
+    ctx = lib.Context.for_shape(M, K, N)
+    want_a, want_b = (lib.fp4_quantize(ctx, x, 0, alpha=alpha) for x in (A, B))
+    lib.fp4_linear_fwd(ctx, A, W, alpha, qa, sw, out=y)                          # (what a call sets up once)
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    graphs = [torch.cuda.CUDAGraph() for _ in range(2)]
+    torch.cuda.synchronize()
+    with torch.cuda.stream(streams[0]):
+        graphs[0].capture_begin(capture_error_mode="relaxed")
+        if first == "quantise":
+            lib.fp4_quantize(ctx, A, 0, alpha=alpha, out=qa)
+        else:
+            lib.fp4_linear_fwd(ctx, A, W, alpha, qa, sw, out=y)
+        with torch.cuda.stream(streams[1]):
+            for _ in range(4):                                                   # (the third one becomes a graph of its own)
+                lib.fp4_quantize(ctx, B, 0, alpha=alpha, out=qb)
+        if first == "quantise":
+            with torch.cuda.stream(streams[2]):
+                graphs[1].capture_begin(capture_error_mode="relaxed")
+                lib.fp4_quantize(ctx, B, 0, alpha=alpha, out=qc)
+                graphs[1].capture_end()
+            lib.fp4_quantize(ctx, A, 0, alpha=alpha, out=qa)                     # the first capture goes on
+        graphs[0].capture_end()
+    torch.cuda.synchronize()
+    for q in (qa, qc):
+        for name in ("codes", "amax", "csr_val", "csc_val"):
+            getattr(q, name).zero_()
+    torch.cuda.synchronize()
+    for g in graphs[:2 if first == "quantise" else 1]:
+        g.replay()
+        torch.cuda.synchronize()
+    assert ctx.read_status() == 0
+    for q, want in ((qa, want_a), (qb, want_b), (qc, want_b))[:3 if first == "quantise" else 2]:
+        n = int(want.nnz)
+        assert int(q.nnz) == n and torch.equal(q.codes, want.codes) and torch.equal(q.amax, want.amax)
+        for name in ("csr_col", "csr_val", "csc_row", "csc_val"):
+            assert torch.equal(getattr(q, name)[:n], getattr(want, name)[:n])
+    ctx.close()
