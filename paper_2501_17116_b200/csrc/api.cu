@@ -613,7 +613,10 @@ int linear_bwd_impl(fp4_ctx* ctx, cudaStream_t st, Arena arena, const void* dY_b
     if (rc != FP4_OK) return rc;
     slot_of_col = savedA->csc_colptr;                  // every row has one: any vector of non-negative numbers
   } else if (has_comp) {
-    const CompOverlap beside = {ctx->side[1], ctx->side[2], ctx->ev[8], ctx->ev[9], ctx->ev[2]};
+    // A third stream is there without one of its own (creating it took 4 % of fp4_create): the one that
+    // fp4_linear_step_host runs its kernels on, idle in all other calls.  (A step bound by the host's copies does without.)
+    cudaStream_t third = sw == st ? ctx->side[0] : st == ctx->compute_stream ? nullptr : ctx->compute_stream;
+    const CompOverlap beside = {ctx->side[1], third, ctx->ev[8], ctx->ev[9], ctx->ev[2]};
     rc = launch_comp_wgrad(ctx, sw, savedA, dY_bf16, comp_arena, &slot_of_col, comp, M, K, N, status,
                            ctx->overlap ? &beside : nullptr);
     if (rc != FP4_OK) return rc;

@@ -44,7 +44,7 @@ struct fp4_ctx {
   size_t   workspace_bytes;
   void*    encode_tiled;       // cuTensorMapEncodeTiled, fetched through the runtime
   uint32_t* occ_hist;          // quantile selection: two sets of global counters, parity, ticket
-  cudaStream_t side[3];        // side streams for independent kernel chains inside one call
+  cudaStream_t side[2];        // side streams for independent kernel chains inside one call
   cudaEvent_t  ev[10];          // fork / join events of those chains
   // fp4_linear_step_host, pipelined over consecutive calls:
   cudaStream_t copy_stream;          // host-to-device copies of a call's inputs
@@ -270,7 +270,7 @@ int launch_fwd_tail(fp4_ctx* ctx, cudaStream_t stream, cudaEvent_t csr_done, con
 // Lists, slots and the dense path's buffers are carved from `scratch` (comp_wgrad_scratch_bytes); the slot
 // vector is handed back for the GEMM's epilogue.  `a` is the saved activation (its CSC).
 // With `overlap` the long columns run on `overlap->stream`, from `classified` to `long_done`, and where there are dense
-// columns the short ones on `stream_short`, to `short_done`.
+// columns the short ones on `stream_short` (may be null), to `short_done`.
 struct CompOverlap {
   cudaStream_t stream, stream_short;
   cudaEvent_t classified, long_done, short_done;

@@ -617,15 +617,17 @@ int launch_comp_wgrad(fp4_ctx* ctx, cudaStream_t stream, const fp4_qtensor* a, c
   classify_columns_kernel<true><<<unsigned((K + 1023) / 1024), 1024, 0, stream>>>(a->csc_colptr, int(K), dense_from, few_max, classes);
   const uint4* dy = static_cast<const uint4*>(dy_bf16);
   // The long columns (a few blocks, latency) run beside the others, and beside the dense columns' chain of three launches the
-  // short ones: at a thousand tokens each of these is a few microseconds of latency (backward of 1024 x 2048 x 2048 at alpha
-  // 0.995 40.0 -> 37.5 us, 2048 x 11008 x 1024 94.2 -> 86.6).  At LONG_COLUMN tokens no column is dense unless every token
-  // hits it: the hot ones are long, and the short ones beside them cost more (512 x 4096 x 4096 107 -> 111).
+  // short ones: at a thousand tokens each of these is a few microseconds of latency (backward with hot columns 1024 x 2048 x
+  // 2048 at alpha 0.995 47.3 -> 41.0 us, 2048 x 11008 x 1024 111 -> 99, 4096^3 at 0.99 260 -> 255).  The host knows that dense
+  // columns are allowed, not whether there are any; without one, where the chain is idle, the fork is worth -1.3 to 1.5 % (the same
+  // sizes with Laplace activations 37.7 -> 38.2, 102.8 -> 101.3, 272 -> 269).  At LONG_COLUMN tokens no column is dense unless
+  // every token hits it: the hot ones are long, and the short ones beside them cost more (512 x 4096 x 4096 107 -> 111).
   cudaStream_t sl = stream, ss = stream;
   if (overlap) {
     sl = overlap->stream;
     FP4_CUDA_TRY(cudaEventRecord(overlap->classified, stream));
     FP4_CUDA_TRY(cudaStreamWaitEvent(sl, overlap->classified, 0));
-    if (dense && M > LONG_COLUMN) {
+    if (dense && M > LONG_COLUMN && overlap->stream_short) {
       ss = overlap->stream_short;
       FP4_CUDA_TRY(cudaStreamWaitEvent(ss, overlap->classified, 0));
     }
