@@ -585,10 +585,12 @@ def test_reused_activation_with_few_entries_and_another_weight(lib, M, K, N, alp
 
 
 @pytest.mark.parametrize("mode", ["FP4_QUANTILE_SIGNED", "FP4_QUANTILE_ABS", "FP4_QUANTILE_TOKEN"])
-@pytest.mark.parametrize("M,K,N,wide", [(640, 1280, 1152, False), (1408, 16384, 2176, True)])
-def test_heavy_operand_from_the_activation_and_from_the_entries(lib, M, K, N, wide, mode):
+@pytest.mark.parametrize("M,K,N,wide,dense", [(640, 1280, 1152, False, False), (1024, 1280, 2176, False, True),
+                                             (1408, 16384, 2176, True, True)])
+def test_heavy_operand_from_the_activation_and_from_the_entries(lib, M, K, N, wide, dense, mode):
     """The forward product's operand is made from the activation, with an activation quantised before from its entries
-    (the second size: several slabs, three terms): the same Y, on side streams and on one."""
+    (the last size: several slabs, three terms; the first is too small for the product): the same Y, on side streams and
+    on one.  The product's order of additions shows in the bits of Y against a context without room for its operand."""
     gen = torch.Generator("cuda").manual_seed(K)
     A = torch.randn((M, K), device="cuda", generator=gen)
     if wide:
@@ -597,15 +599,19 @@ def test_heavy_operand_from_the_activation_and_from_the_entries(lib, M, K, N, wi
     W = (torch.randn((K, N), device="cuda", generator=gen) * 0.02).to(torch.bfloat16)
     ctx = lib.Context.for_shape(M, K, N)
     ctx.set_quantile_mode(getattr(lib.binding, mode))
-    y, sa, sw = lib.fp4_linear_fwd(ctx, A, W, 0.95)
-    reused, _, _ = lib.fp4_linear_fwd(ctx, A, W, 0.95, saved_a=sa, saved_w=sw, reuse_a=True, reuse_w=True)
+    y, sa, sw = lib.fp4_linear_fwd(ctx, A, W, 0.95, out_f32=True)
+    reused, _, _ = lib.fp4_linear_fwd(ctx, A, W, 0.95, saved_a=sa, saved_w=sw, reuse_a=True, reuse_w=True, out_f32=True)
     alone = lib.fp4_quantize(ctx, A, 0, alpha=0.95)
     ctx.set_overlap(False)
-    serial, ss, _ = lib.fp4_linear_fwd(ctx, A, W, 0.95)
+    serial, ss, _ = lib.fp4_linear_fwd(ctx, A, W, 0.95, out_f32=True)
+    tight = lib.Context(0, ctx.workspace_bytes - 256)
+    tight.set_quantile_mode(getattr(lib.binding, mode))
+    per_entry, _, _ = lib.fp4_linear_fwd(tight, A, W, 0.95, out_f32=True)
     serial_alone = lib.fp4_quantize(ctx, A, 0, alpha=0.95)
     torch.cuda.synchronize()
     assert ctx.read_status() == 0 and int(sa.nnz) > 0.04 * M * K
-    assert torch.equal(y, reused) and torch.equal(y, serial)
+    assert torch.equal(y, reused) and torch.equal(y, serial) and torch.equal(y, per_entry) != dense
+    tight.close()
     n = int(sa.nnz)
     for q in (alone, ss, serial_alone):
         assert int(q.nnz) == n and torch.equal(q.codes, sa.codes) and torch.equal(q.codes_t, sa.codes_t)
