@@ -206,7 +206,7 @@ int fp4_gemm(fp4_ctx* ctx, void* stream, const uint8_t* a_codes, const uint8_t* 
  *   FP16: it matters only for weights ten orders of magnitude below their column's largest).
  *   A residual value
  *   beyond 43 000 times its token's clamped absmax does not fit the FP16 operand: the call
- *   then adds every entry per entry.
+ *   then adds every entry per entry, as with an E5M2 weight, whose scaled values do not fit it either.
  *   A residual that may fill more than 4 % of the activation (by alpha; M >= 512) is multiplied as a
  *   dense matrix where that takes less time for the entries that are there: exact three-term BF16
  *   split, chunks of 64 input channels added in fp32 in order.  Same bound, without the second term.

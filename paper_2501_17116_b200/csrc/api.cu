@@ -375,8 +375,10 @@ int linear_fwd_impl(fp4_ctx* ctx, cudaStream_t st, Arena arena, const void* A_bf
   char* scratch_full = occ && full_room && heavy_residual(savedA, M, K) && full_product_pays(ctx, savedA, M, K, N)
                            ? arena.take<char>(full_bytes) : nullptr;
   const bool full_on = scratch_full != nullptr;
+  // (A hot column holds at least 512 entries.  The tail's weight operand is W / d_W in FP16: an E5M2 weight's reaches 57344,
+  // beyond FP16 with the operand's factor of 4.)
   const bool tail_on = occ && !full_on && savedA->csr_rowptr && savedA->csc_colptr && !heavy_residual(savedA, M, K) &&
-                       residual_entries(savedA) * 100 >= M * K && M >= 512;   // a hot column holds at least 512 entries
+                       residual_entries(savedA) * 100 >= M * K && M >= 512 && savedW->format != FP4_FORMAT_E5M2;
   char* scratch_tail = tail_on ? arena.take<char>(fwd_tail_scratch_bytes(M, K, N)) : nullptr;
   if (!arena.ok) return FP4_ERR_WORKSPACE;
   int rc;

@@ -280,7 +280,7 @@ tail_a_kernel(const int* __restrict__ rowptr, const int* __restrict__ col, const
 
 // B operand of the dense tail: row n holds, for hot column s = 64 j + c, the value
 // x = TAIL_SCALE * W[k_s, n] / d_W[n] as x_hi at 192 j + c, TAIL_BALANCE x_lo at 192 j + 64 + c and
-// x_hi / TAIL_BALANCE at 192 j + 128 + c (|x| <= 6 * 4, or 448 * 4 for an FP8 weight: the weight is at
+// x_hi / TAIL_BALANCE at 192 j + 128 + c (|x| <= 6 * 4, or 448 * 4 for an E4M3 weight; no tail with E5M2, 57344 * 4: the weight is at
 // most amax in magnitude), zero beyond the last hot column of a block of 64; blocks without one are not read.
 // A block of threads makes 64 rows of such a block: whole lines of W in, a shared tile, whole lines out.  (A thread per
 // row and column wrote three halfwords into lines of 768 bytes each: 2048 x 11008 x 1024 at alpha 0.995 forward 117.5 us, 109 now.)

@@ -212,6 +212,39 @@ def test_fp8_accumulation_stays_inside_its_floor(lib, ctx):
     assert (err <= 0.5 * floor + 4 * 2.0 ** -23 * np.abs(want)).all(), f"{np.max(err / floor):.3f} of the floor"
 
 
+@pytest.mark.parametrize("alpha,dense", [(0.99, True), (0.99, False), (0.999, False)])
+@pytest.mark.parametrize("fmt", ["FP4_FORMAT_E4M3", "FP4_FORMAT_E5M2"])
+def test_fp8_weight_beside_a_residual_with_hot_columns(lib, fmt, alpha, dense):
+    """A heavy residual with outlier channels and an FP8 weight: W / d_W reaches 448 (E4M3), which the FP16 operand of the
+    dense tail holds, or 57344 (E5M2), which it does not.  Against float64: the codes' product plus the residual's."""
+    M, K, N = 1024, 640, 1408
+    gen = torch.Generator("cuda").manual_seed(7)
+    A = torch.randn((M, K), device="cuda", generator=gen)
+    if dense:
+        A[:, ::128] *= 20.0
+    A, W = A.bfloat16(), (torch.randn((K, N), device="cuda", generator=gen) * 0.02).bfloat16()
+    fmt_w = getattr(lib.binding, fmt)
+    c = lib.Context.for_shape(M, K, N)
+    y, sa, sw = lib.fp4_linear_fwd(c, A, W, alpha, gemm_kind=lib.binding.FP4_GEMM_F8F6F4, fmt_w=fmt_w, out_f32=True)
+    again, _, _ = lib.fp4_linear_fwd(c, A, W, alpha, gemm_kind=lib.binding.FP4_GEMM_F8F6F4, saved_a=sa, saved_w=sw, reuse_a=True,
+                                     reuse_w=True, out_f32=True)
+    torch.cuda.synchronize()
+    assert c.read_status() == 0 and int((sa.csc_colptr.diff() >= 512).sum()) == (5 if dense else 0)
+    e4m3 = fmt == "FP4_FORMAT_E4M3"
+    val = torch.tensor([0, .5, 1, 1.5, 2, 3, 4, 6, 0, -.5, -1, -1.5, -2, -3, -4, -6], dtype=torch.float64, device="cuda")
+    va = torch.stack([val[(sa.codes & 15).long()], val[(sa.codes >> 4).long()]], -1).flatten(1)
+    vw = sw.codes_t.view(torch.float8_e4m3fn if e4m3 else torch.float8_e5m2).double()
+    unit = (sa.amax / 6.0).double()[:, None] * (sw.amax / (448.0 if e4m3 else 57344.0)).double()
+    lo, hi = sa.thresholds.double().tolist()
+    res = A.double() - A.double().clamp(lo, hi)
+    exact = va @ vw.T * unit + res @ W.double()
+    # K / 32 instructions and 24 of the tail cut 2^-23 off the running sum; 2^-21 for the FP16 splits, or an fp32 sum
+    allow = 2.0 ** -23 * (K // 32 + 24 + 4) * (va.abs() @ vw.abs().T * unit)
+    allow += (4e-6 + 2.0 ** -24 * (res != 0).sum(1, keepdim=True)) * (res.abs() @ W.double().abs())
+    assert bool(((y.double() - exact).abs() <= allow).all()) and torch.equal(y, again)
+    c.close()
+
+
 @pytest.mark.parametrize("fmt_a,dy_fmt", [("FP4_FORMAT_E4M3", "FP4_FORMAT_E5M2"), ("FP4_FORMAT_E2M1", "FP4_FORMAT_E2M1")])
 @pytest.mark.parametrize("M,K,N", [(4096, 2048, 2048), (1024, 4096, 1408)])
 def test_weight_gradient_of_wide_tiles_without_clamp_is_the_same_every_time(lib, fmt_a, dy_fmt, M, K, N):
