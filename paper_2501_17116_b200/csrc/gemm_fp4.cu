@@ -484,9 +484,18 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           ++fills;
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
-        for (int kb = 0; kb < tail_kb && ok; ++kb) {      // dense tail: FP16 columns 64 kb .. 64 kb + 63
+        // Dense tail: FP16 columns 64 kb .. 64 kb + 63.  Then, in a pair, as many waits as the ring has stages: the even CTA's
+        // commits arrive on the empty barriers of both, and a CTA leaves when the arrivals for its last fills have come, which
+        // nobody else waits for.  (A loop of its own behind this one made a launch of 12.9 us, 256 x 1152 x 12544, 13.1, run or
+        // not: its code is what it costs.)
+        const int drain = PAIR && t + workers >= num_tiles ? STAGES : 0;
+        for (int kb = 0; kb < tail_kb + drain && ok; ++kb) {
           ok = mbar_wait(&empty_bar[stage], phase ^ 1u, abort_flag, args.status, args.wait_limit_ns);
           if (!ok) break;
+          if (PAIR && kb >= tail_kb) {
+            if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+            continue;
+          }
           if (rank == 0) mbar_arrive_expect_tx(&full_bar[stage], CTAS * args.tail_tx_bytes);
           tma_load_2d_group<CTAS>(smem + stage * STAGE_BYTES, &map_a2, full0 + 8 * stage, kb * 64, a_row);
           tma_load_2d_group<CTAS>(smem + stage * STAGE_BYTES + A_STAGE_BYTES, &map_b2, full0 + 8 * stage, kb * 64, b_row);
@@ -494,13 +503,6 @@ gemm_fp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
       }
-      // The even CTA's commits arrive on the empty barriers of both: a CTA of a pair leaves when the arrivals for its last
-      // fills have come, which nobody else waits for.  (They come with the last MMAs, ahead of the last epilogue: no time.)
-      if (PAIR)
-        for (int s = 0; s < STAGES && ok; ++s) {
-          ok = mbar_wait(&empty_bar[stage], phase ^ 1u, abort_flag, args.status, args.wait_limit_ns);
-          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
-        }
       if (!ok && PAIR) {
         // Gave up: the peer's copies complete on the even CTA's barriers too, so the copies in flight are given time to land.
         const uint64_t t0 = global_timer_ns();
